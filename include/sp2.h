@@ -92,7 +92,11 @@ typedef enum {
 typedef enum { SP2_F64 = 0, SP2_F32 = 1 } sp2_dtype;
 
 /* Arithmetic of the matrix products (Sec. VI.B).
- *   SP2_MODE_FP64    plain FP64 (CUDA-core DFMA).
+ *   SP2_MODE_FP64    FP64. Products of matrices above N = 257 are formed on the tensor
+ *                    cores from 7 error-free digits of 9 bits per entry (28 exact
+ *                    products summed in integers), with errors below those of an
+ *                    FP64 dot product relative to the norms of its row and column;
+ *                    smaller ones by CUDA-core DFMA.
  *   SP2_MODE_FP32    plain FP32 (CUDA-core FFMA): the paper's "GPU FP32" form.
  *   SP2_MODE_BF16X2  Eq. doubleHalf / Eq. MixPrecMult with bfloat16 hi/lo planes:
  *                    three tensor-core products (hi*hi + hi*lo + lo*hi, lo*lo

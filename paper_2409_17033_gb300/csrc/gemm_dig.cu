@@ -1,0 +1,800 @@
+// FP64 products on the 16-bit tensor cores of sm_103a, by error-free splitting
+// into digits (the scheme of Ozaki, Ogita, Oishi and Rump, "Error-free
+// transformations of matrix multiplication by using fast routines of matrix
+// multiplication and its applications", Numer. Algorithms 59, 2012).
+//
+// Why: GB300's FP64 pipe does about 2 FMA per clock and SM (1.25 TFLOP/s), its
+// 16-bit tensor pipe a thousand times that, so 28 tensor products in place of
+// one FP64 product are still about 40 times faster once a product fills the GPU.
+//
+// Splitting. Row i of a factor is scaled by a power of two 2^ex_i >= its 2-norm
+// and rounded to a 62-bit fixed-point number, which is cut into 7 signed digits
+// of 9 bits: x = 2^(ex - 62) sum_i d_i 2^(54 - 9 i), d_i in [-256, 256]. Digits
+// are exact in bfloat16, a product of two is at most 2^16, and a sum of 256 of
+// them at most 2^24, so the tensor core's FP32 accumulation of a 256-wide K chunk
+// is exact whatever the inputs. The chunks of all digit pairs (i, j) of one
+// weight s = i + j add up in INT32 registers (exact up to K = 4096), and each
+// weight's sum is added to a 64-bit integer T(i, j) of unit 2^(ex_i + ex_j - 62):
+// |C_ij| <= 2^(ex_i + ex_j) by Cauchy-Schwarz, so T never leaves 63 bits. The 28
+// pairs with s <= 6 are formed. What is dropped (s >= 7) and rounded is of the
+// order sqrt(K) 2^-63 of the two rows' norms, below the rounding of an FP64 dot
+// product. Integer additions commute, so a tile's work may be cut into parts (by
+// weight and along K) whose sums meet in T by atomics: the result has the same
+// bits for every cut and every order.
+//
+// Layout. T is stored transposed, T[j * rows + i] for entry (i, j): a warp's lanes
+// hold consecutive rows i, so its 64-bit atomics are whole sectors.
+//
+// Per product: k_digits (each factor; it also clears T), k_gemm_dig, then one
+// pass that turns T into FP64 and applies the recursion's update: k_dig_square
+// (Eq. DM0, with the traces and the step decision), k_dig_symm (Eqs. DM1-DM3) or
+// k_dig_plain.
+//
+// k_gemm_dig is tensor-bound at large N (28 bfloat16 products) and bound by
+// latency and by the number of resident CTA pairs at small N. Tile, pipeline and
+// warp roles are those of the split-precision kernel on CTA pairs: 256 x BN tiles
+// (BN = 256, or 128 where more and smaller tiles fill the GPU better), one
+// tcgen05.mma.cta_group::2 stream per pair, TMA ring, two TMEM chunk buffers
+// drained by 16 warps.
+#include <math.h>
+#include <stdio.h>
+#include <string.h>
+
+#include "decide.cuh"
+#include "sp2_internal.h"
+#include "tc_ptx.cuh"
+
+namespace sp2 {
+
+namespace {
+
+constexpr int kDigits = 7;
+constexpr int kGroups = 7;        // digit-pair weights s = i + j <= 6
+constexpr int kFixBits = 62;      // fixed-point bits of a scaled entry; unit of T
+constexpr int kBadRow = 1 << 20;  // exponent of a row with a NaN or an infinity
+
+constexpr int BM = 128;           // tile rows per CTA
+constexpr int BK = kBoxCols;
+constexpr int KCH = 4;            // k-blocks per TMEM chunk: 256 products, exact in FP32
+constexpr int KSEG_MAX = 64;      // k-blocks an INT32 sum of 7 digit pairs may span (K = 4096)
+constexpr int EPI_WARPS = 16;
+constexpr int NUM_THREADS = 64 + 32 * EPI_WARPS;
+constexpr unsigned long long DRAIN_NS = 200000000ull;
+
+template <int BN>
+struct Geo {
+  static constexpr int A_BYTES = BM * BK * 2;
+  static constexpr int B_ROWS = BN / 2;
+  static constexpr int STAGE_BYTES = A_BYTES + B_ROWS * BK * 2;
+  static constexpr int STAGES = BN == 256 ? 6 : 8;
+  static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 /*align slack*/ + 256 /*barriers*/;
+  static constexpr uint32_t TMEM_COLS = 2 * BN;
+  static constexpr int TCOLS = BN / (EPI_WARPS / 4);
+  // kind::f16: D = F32, A and B bfloat16, K-major, M = 256 over the pair, N = BN
+  static constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) |
+                                    ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(2 * BM >> 4) << 24);
+};
+
+// The weights of part `part` of `parts`: 28 digit pairs split evenly (weight s has s + 1).
+__device__ __forceinline__ uint32_t part_mask(int parts, int part) {
+  if (parts == 1) return 0x7fu;
+  if (parts == 2) return part == 0 ? 0x61u : 0x1eu;                 // {6,5,0}, {4,3,2,1}
+  return part == 0 ? 0x40u : (part == 1 ? 0x21u : (part == 2 ? 0x12u : 0x0cu));
+}
+
+struct DParams {
+  int nkb;             // k-blocks of the K axis (np / 64)
+  int kseg;            // k-blocks of one K part (a multiple of KCH, at most KSEG_MAX)
+  int ksplit;          // K parts
+  int parts;           // weight parts (1, 2 or 4)
+  int64_t rows;        // rows of A (plane stride of its map, leading dimension of T)
+  int64_t np;          // rows of X per plane
+  unsigned long long* T;
+  const Tile* tiles;
+  int nunits;          // tiles x parts x ksplit
+  DevState* st;
+  int step;
+  unsigned long long wait_ns;
+  int withhold;
+};
+
+struct Unit {
+  Tile t;
+  uint32_t mask;
+  int kb0, kb1;
+};
+
+__device__ __forceinline__ Unit unit_of(const DParams& p, int u) {
+  const int per = p.parts * p.ksplit;
+  const int tix = u / per, rem = u - tix * per;
+  const int part = rem / p.ksplit, ks = rem - part * p.ksplit;
+  Unit r;
+  r.t = p.tiles[tix];
+  r.mask = part_mask(p.parts, part);
+  r.kb0 = ks * p.kseg;
+  r.kb1 = r.kb0 + p.kseg < p.nkb ? r.kb0 + p.kseg : p.nkb;
+  return r;
+}
+
+template <int BN>
+__global__ void __launch_bounds__(NUM_THREADS, 1)
+k_gemm_dig(const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUtensorMap bmap,
+           const __grid_constant__ DParams p) {
+  using G = Geo<BN>;
+  constexpr int STAGES = G::STAGES;
+  DevState* st = p.st;
+  {
+    // a pair takes this exit together: stop_at is fixed for the launch
+    const int m = *((volatile const int*)&st->stop_at);
+    if (m != 0 && p.step > m) return;
+  }
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
+                                             ~(uintptr_t)1023);
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + STAGES * G::STAGE_BYTES);
+  uint64_t* empty = full + STAGES;
+  uint64_t* pfull = empty + STAGES;   // rank 0: the peer's stage has landed
+  uint64_t* tfull = pfull + STAGES;   // [2] chunk accumulated in TMEM buffer b
+  uint64_t* tempty = tfull + 2;       // [2] TMEM buffer b drained by both CTAs
+  uint64_t* mdone = tempty + 2;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mdone + 1);
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  int* abortf = &st->abort_flag;
+  const uint32_t rank = cluster_rank();
+  const bool issuer = rank == 0;
+  const int pair = (int)(blockIdx.x >> 1), npairs = (int)(gridDim.x >> 1);
+  const int pairs_per_part = 28 / p.parts;   // digit pairs of a unit
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < STAGES; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
+      mbar_init(&pfull[s], 1);
+    }
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(&tfull[b], 1);
+      mbar_init(&tempty[b], 2 * EPI_WARPS);
+    }
+    mbar_init(mdone, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&amap)) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&bmap)) : "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(tmem_slot)),
+                 "r"(G::TMEM_COLS)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  cluster_sync();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      int64_t g = 0;
+      RingPos<STAGES> rp;
+      bool ok = true;
+      for (int u = pair; u < p.nunits && ok; u += npairs) {
+        const Unit w = unit_of(p, u);
+        const int arow = w.t.row0 + (int)rank * BM;
+        const int brow = w.t.col0 + (int)rank * G::B_ROWS;
+        for (int s = kGroups - 1; s >= 0 && ok; --s) {
+          if (!((w.mask >> s) & 1u)) continue;
+          for (int i = 0; i <= s && ok; ++i) {
+            const int ay = i * (int)p.rows + arow, by = (s - i) * (int)p.np + brow;
+            for (int kx = w.kb0 * BK; kx < w.kb1 * BK; kx += BK, ++g, rp.next()) {
+              if (!mbar_wait<true>(&empty[rp.s], rp.ph ^ 1u, abortf, p.wait_ns)) {
+                ok = false;
+                break;
+              }
+              if (p.withhold && blockIdx.x == 0 && g == 0) continue;  // test hook: never completes
+              uint8_t* sa = smem + rp.s * G::STAGE_BYTES;
+              mbar_arrive_expect_tx(&full[rp.s], G::STAGE_BYTES);
+              tma_load_2d(&amap, &full[rp.s], sa, kx, ay);
+              tma_load_2d(&bmap, &full[rp.s], sa + G::A_BYTES, kx, by);
+            }
+          }
+        }
+      }
+      if (!ok) {
+        // aborted: let the copies already issued land before the CTA exits
+        const int64_t first = g > STAGES ? g - STAGES : 0;
+        for (int64_t q = first; q < g; ++q) {
+          if (p.withhold && blockIdx.x == 0 && q == 0) continue;
+          mbar_wait_drain(&full[q % STAGES], (uint32_t)(q / STAGES) & 1u, DRAIN_NS);
+        }
+      }
+    }
+  } else if (warp == 1) {
+    if (!issuer && lane == 0) {
+      // rank 1: pass each landed stage on to rank 0's MMA issuer
+      const uint32_t pfull_peer = cluster_addr(smem_u32(pfull), 0);
+      RingPos<STAGES> rp;
+      bool ok = true;
+      for (int u = pair; u < p.nunits && ok; u += npairs) {
+        const Unit w = unit_of(p, u);
+        const int n = pairs_per_part * (w.kb1 - w.kb0);
+        for (int q = 0; q < n; ++q, rp.next()) {
+          if (!mbar_wait<true>(&full[rp.s], rp.ph, abortf, p.wait_ns)) {
+            ok = false;
+            break;
+          }
+          mbar_arrive_cluster_release(pfull_peer + (uint32_t)(rp.s * sizeof(uint64_t)));
+        }
+      }
+    } else if (issuer && lane == 0) {
+      bool ok = true;
+      int64_t gc = 0;
+      RingPos<STAGES> rp;
+      const uint64_t adesc0 = sdesc_sw128(smem_u32(smem));
+      for (int u = pair; u < p.nunits && ok; u += npairs) {
+        const Unit w = unit_of(p, u);
+        const int nch = pairs_per_part * ((w.kb1 - w.kb0) / KCH);
+        for (int c = 0; c < nch && ok; ++c, ++gc) {
+          const int b = (int)(gc & 1);
+          if (!mbar_wait<true>(&tempty[b], ((uint32_t)(gc >> 1) & 1u) ^ 1u, abortf, p.wait_ns)) {
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          const uint32_t dtm = tmem + (uint32_t)b * BN;
+#pragma unroll 1
+          for (int kb = 0; kb < KCH; ++kb, rp.next()) {
+            if (!mbar_wait<false>(&full[rp.s], rp.ph, abortf, p.wait_ns) ||
+                !mbar_wait<true>(&pfull[rp.s], rp.ph, abortf, p.wait_ns)) {
+              ok = false;
+              break;
+            }
+            tc_fence_after();
+            const uint64_t adesc = adesc0 + (uint64_t)(rp.s * (G::STAGE_BYTES >> 4));
+            const uint64_t bdesc = adesc + (uint64_t)(G::A_BYTES >> 4);
+#pragma unroll
+            for (int k = 0; k < BK / 16; ++k)
+              umma_f16<2>(dtm, adesc + (uint64_t)(2 * k), bdesc + (uint64_t)(2 * k), G::IDESC,
+                          (kb > 0 || k > 0) ? 1u : 0u);
+            umma_commit_both(&empty[rp.s]);
+          }
+          if (ok) umma_commit_both(&tfull[b]);
+        }
+      }
+      if (!ok) {
+        umma_commit<2>(mdone);
+        mbar_wait_drain(mdone, 0, DRAIN_NS);
+      }
+    }
+  } else {
+    // warp w reads TMEM lanes 32 (w % 4) .. +31 and the columns of group (w - 2) / 4
+    constexpr int TC = G::TCOLS;
+    const int q = warp & 3;
+    const int grp = (warp - 2) >> 2;
+    const int r = (int)rank * BM + q * 32 + lane;
+    const uint32_t trow = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(grp * TC);
+    const uint32_t tempty_peer = !issuer ? cluster_addr(smem_u32(tempty), 0) : 0u;
+    bool ok = true;
+    uint32_t gc = 0;   // chunk counter: buffer gc & 1, phase (gc >> 1) & 1
+    for (int u = pair; u < p.nunits && ok; u += npairs) {
+      uint32_t mask;
+      int kch;
+      unsigned long long* dst;
+      {
+        const Unit w = unit_of(p, u);
+        mask = w.mask;
+        kch = (w.kb1 - w.kb0) / KCH;
+        dst = p.T + (int64_t)(w.t.col0 + grp * TC) * p.rows + (int64_t)w.t.row0 + r;
+      }
+#pragma unroll 1
+      for (int s = kGroups - 1; s >= 0; --s) {
+        if (!((mask >> s) & 1u)) continue;
+        int acc[TC];
+#pragma unroll
+        for (int j = 0; j < TC; ++j) acc[j] = 0;
+#pragma unroll 1
+        for (int c = (s + 1) * kch; c > 0; --c, ++gc) {
+          const uint32_t b = gc & 1u;
+          const bool wt = mbar_wait<true>(&tfull[b], (gc >> 1) & 1u, abortf, p.wait_ns);
+          ok = __all_sync(0xffffffffu, wt);
+          if (!ok) break;
+          tc_fence_after();
+#pragma unroll
+          for (int c0 = 0; c0 < TC; c0 += 16) {
+            uint32_t v[16];
+            tmem_ld16(trow + b * BN + (uint32_t)c0, v);
+#pragma unroll
+            for (int j = 0; j < 16; ++j) acc[c0 + j] += __float2int_rn(__uint_as_float(v[j]));
+          }
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) {
+            if (!issuer)
+              mbar_arrive_cluster(tempty_peer + b * (uint32_t)sizeof(uint64_t));
+            else
+              mbar_arrive(&tempty[b]);
+          }
+        }
+        if (!ok) break;
+        // weight s in T's unit: 2^(108 - 9 s) products' unit over 2^62 (46 - 9 s >= -8)
+        const int sh = 2 * 54 - 9 * s - kFixBits;
+        const int up = sh > 0 ? sh : 0, dn = sh < 0 ? -sh : 0;
+        const int half = dn ? 1 << (dn - 1) : 0;
+        unsigned long long* d = dst;
+#pragma unroll
+        for (int j = 0; j < TC; ++j) {
+          // |acc| < 2^31 - 2^8, so the rounding term cannot overflow
+          const long long v = (long long)((acc[j] + half) >> dn) << up;
+          asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(d),
+                       "l"((unsigned long long)v)
+                       : "memory");
+          d += p.rows;
+        }
+      }
+    }
+  }
+
+  tc_fence_before();
+  __syncthreads();
+  cluster_sync();
+  if (warp == 1) {
+    __syncwarp();
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem),
+                 "r"(G::TMEM_COLS)
+                 : "memory");
+  }
+}
+
+__device__ __forceinline__ bool halted_dig(const DevState* st, int step) {
+  const int m = *((volatile const int*)&st->stop_at);
+  return m != 0 && step > m;
+}
+
+// ------------------------------------------------------------ digits
+// One block per row: the row's power-of-two scale 2^ex >= its 2-norm, then the
+// seven digit planes (plane d of the stack at d * rows * np), and T's share of the
+// product cleared. Integer arithmetic throughout (FP64 conversions run at the slow
+// FP64 rate); the norm in FP32 from the entries' leading 20 bits, relative to the
+// row's largest entry, with a margin above its rounding. HBM-bound at large N: 8
+// bytes read, 14 (and 8 for T) written per entry.
+constexpr int kDigThreads = 128;
+
+__global__ void __launch_bounds__(kDigThreads)
+k_digits(const double* __restrict__ src, int64_t rows, int64_t np, uint16_t* __restrict__ dig,
+         int* __restrict__ ex, unsigned long long* __restrict__ T, const DevState* st, int step) {
+  if (halted_dig(st, step)) return;
+  __shared__ uint32_t smax[kDigThreads / 32];
+  __shared__ float ssum[kDigThreads / 32];
+  const int64_t row = blockIdx.x;
+  const double2* x2 = reinterpret_cast<const double2*>(src + row * np);
+  const int n4 = (int)(np / 4);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint32_t m = 0;
+  for (int c = threadIdx.x; c < n4; c += kDigThreads) {
+    const double2 a = x2[2 * c], b = x2[2 * c + 1];
+    m = max(m, max(max((uint32_t)__double2hiint(a.x) & 0x7fffffffu,
+                       (uint32_t)__double2hiint(a.y) & 0x7fffffffu),
+                   max((uint32_t)__double2hiint(b.x) & 0x7fffffffu,
+                       (uint32_t)__double2hiint(b.y) & 0x7fffffffu)));
+  }
+  m = __reduce_max_sync(0xffffffffu, m);
+  if (lane == 0) smax[warp] = m;
+  __syncthreads();
+  m = smax[0];
+#pragma unroll
+  for (int w = 1; w < kDigThreads / 32; ++w) m = max(m, smax[w]);
+  const int em = (int)(m >> 20);
+  const bool bad = em == 0x7ff;
+  float ss = 0.0f;
+  for (int c = threadIdx.x; c < n4; c += kDigThreads) {
+    const double2 a = x2[2 * c], b = x2[2 * c + 1];
+    const double v[4] = {a.x, a.y, b.x, b.y};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const uint32_t h = (uint32_t)__double2hiint(v[k]) & 0x7fffffffu;
+      const int fe = (int)(h >> 20) - em;   // <= 0
+      // |x| / 2^(em - 1023), truncated to 20 bits; below 2^-60 covered by the margin
+      const float f = fe > -60 ? __uint_as_float((uint32_t)((127 + fe) << 23) | ((h & 0xfffffu) << 3))
+                               : 0.0f;
+      ss = fmaf(f, f, ss);
+    }
+  }
+  for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+  if (lane == 0) ssum[warp] = ss;
+  __syncthreads();
+  ss = 0.0f;
+#pragma unroll
+  for (int w = 0; w < kDigThreads / 32; ++w) ss += ssum[w];
+  // sums of at most 2^14 positive FP32 terms per thread: 1 + 2^-8 covers their
+  // rounding and the truncation of the entries
+  ss = ss * (1.0f + 0.00390625f) + (float)np * 1e-17f;
+  int k2;
+  frexpf(ss, &k2);                      // ss < 2^k2
+  const int q = (k2 + 1) >> 1;          // sqrt(ss) < 2^q
+  const int e = bad ? kBadRow : (m == 0 ? 0 : em - 1023 + q);
+  if (threadIdx.x == 0) ex[row] = e;
+  const int64_t plane = rows * np;
+  constexpr unsigned long long kBias =   // 256 in every digit field below the first
+      (256ull << 45) + (256ull << 36) + (256ull << 27) + (256ull << 18) + (256ull << 9) + 256ull;
+  for (int c = threadIdx.x; c < n4; c += kDigThreads) {
+    const double2 a = x2[2 * c], b = x2[2 * c + 1];
+    const double v[4] = {a.x, a.y, b.x, b.y};
+    uint32_t f[4][kDigits];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const long long bits = __double_as_longlong(v[k]);
+      const int eb = (int)((bits >> 52) & 0x7ff);
+      unsigned long long mant = (unsigned long long)bits & 0xfffffffffffffull;
+      if (eb) mant |= 1ull << 52;
+      const int sh = (eb ? eb : 1) - (1075 - kFixBits) - e;   // at most 10
+      long long I;
+      if (sh >= 0) I = (long long)(mant << sh);
+      else if (sh > -55) I = (long long)((mant + (1ull << (-sh - 1))) >> -sh);
+      else I = 0;
+      if (bits < 0) I = -I;
+      if (bad || m == 0) I = 0;
+      const long long B = I + (long long)kBias;
+      f[k][0] = (uint32_t)((int)(B >> 54) + 256);
+#pragma unroll
+      for (int d = 1; d < kDigits; ++d) f[k][d] = (uint32_t)((unsigned long long)B >> (54 - 9 * d)) & 511u;
+    }
+#pragma unroll
+    for (int d = 0; d < kDigits; ++d) {
+      uint32_t h[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k)   // field - 256 as an FP32 integer; its upper half is the bfloat16
+        h[k] = __float_as_uint(__uint_as_float(0x4B000000u + f[k][d]) - 8388864.0f);
+      uint2 o;
+      o.x = __byte_perm(h[0], h[1], 0x7632);
+      o.y = __byte_perm(h[2], h[3], 0x7632);
+      reinterpret_cast<uint2*>(dig + d * plane + row * np)[c] = o;
+    }
+    if (T) {
+      ulonglong2* t2 = reinterpret_cast<ulonglong2*>(T + row * np);
+      t2[2 * c] = make_ulonglong2(0ull, 0ull);
+      t2[2 * c + 1] = make_ulonglong2(0ull, 0ull);
+    }
+  }
+}
+
+// T's value as FP64 (one rounding), times 2^e. The conversion by magic constants
+// (two FP64 additions) and the scaling by the exponent field keep to FP32-rate
+// integer work otherwise.
+__device__ __forceinline__ double from_fixed(long long t, int ei, int ej) {
+  const int hi = (int)(t >> 32);
+  const uint32_t lo = (uint32_t)t;
+  // 2^84 + 2^63 + hi 2^32, 2^52 + lo
+  const double dh = __hiloint2double(0x45300000, (int)((uint32_t)hi ^ 0x80000000u));
+  const double dl = __hiloint2double(0x43300000, (int)lo);
+  const double off = __hiloint2double(0x45300000, (int)0x80100000u);   // 2^84 + 2^63 + 2^52
+  const double v = (dh - off) + dl;
+  if (ei == kBadRow || ej == kBadRow) return __longlong_as_double(0x7ff8000000000000ll);
+  const int e = ei + ej - kFixBits;
+  const int vh = __double2hiint(v);
+  const int ve = (vh >> 20) & 0x7ff;
+  if (ve == 0) return v;   // zero
+  const int ne = ve + e;
+  if (ne > 0 && ne < 0x7ff) return __hiloint2double(vh + e * (1 << 20), __double2loint(v));
+  return scalbn(v, e);
+}
+
+constexpr int TE = 32;            // tile edge of the passes over T
+constexpr int kPassThreads = 256;
+
+__device__ __forceinline__ void tri_ij(int64_t t, int64_t& I, int64_t& J) {
+  J = (int64_t)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
+  while (J * (J + 1) / 2 > t) --J;
+  while ((J + 1) * (J + 2) / 2 <= t) ++J;
+  I = t - J * (J + 1) / 2;
+}
+
+__device__ __forceinline__ void ld4ll(const unsigned long long* p, long long (&v)[4]) {
+  const longlong2 a = __ldcs(reinterpret_cast<const longlong2*>(p));
+  const longlong2 b = __ldcs(reinterpret_cast<const longlong2*>(p) + 1);
+  v[0] = a.x, v[1] = a.y, v[2] = b.x, v[3] = b.y;
+}
+__device__ __forceinline__ void ld4d(const double* p, double (&v)[4]) {
+  const double2 a = reinterpret_cast<const double2*>(p)[0];
+  const double2 b = reinterpret_cast<const double2*>(p)[1];
+  v[0] = a.x, v[1] = a.y, v[2] = b.x, v[3] = b.y;
+}
+__device__ __forceinline__ void st4d(double* p, const double (&v)[4]) {
+  reinterpret_cast<double2*>(p)[0] = make_double2(v[0], v[1]);
+  reinterpret_cast<double2*>(p)[1] = make_double2(v[2], v[3]);
+}
+
+// X_{n+1} = sigma > 0 ? C : 2 X_n - C from T (C = X_n^2, upper entries), mirrored;
+// partials of Tr, ||.||_F^2 and ||X_n - X_n^2||_F^2 in FP64, and the step decision
+// in the last block. One block per pair of TE x TE tiles (I <= J); T's tile (J, I)
+// holds entries (i, j) of the upper tile with i along its rows. About 8 FP64
+// operations per upper entry bound it (GB300's FP64 pipe).
+__global__ void __launch_bounds__(kPassThreads)
+k_dig_square(const unsigned long long* __restrict__ T, const int* __restrict__ ex,
+             const double* __restrict__ X, double* __restrict__ out, int64_t np, DevState* st,
+             int step, Part3* __restrict__ part, SimtDecide dec) {
+  if (halted_dig(st, step)) return;
+  __shared__ double sm[TE][TE + 1];
+  int64_t I, J;
+  tri_ij(blockIdx.x, I, J);
+  const int r = threadIdx.x >> 3, c4 = (threadIdx.x & 7) * 4;
+  const int64_t gj = J * TE + r, gi0 = I * TE + c4;
+  const int sg = st->sigma[step];
+  double t1 = 0.0, t2 = 0.0, f = 0.0;
+  double y[4];
+  {
+    long long t[4];
+    double x[4];
+    ld4ll(T + gj * np + gi0, t);
+    ld4d(X + gj * np + gi0, x);   // X_n is symmetric
+    const int ej = ex[gj];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int64_t gi = gi0 + k;
+      if (gi > gj) continue;      // below the diagonal of a diagonal tile
+      const double c = from_fixed(t[k], ex[gi], ej);
+      const double v = sg > 0 ? c : 2.0 * x[k] - c;
+      const double d = x[k] - c;
+      y[k] = v;
+      sm[r][c4 + k] = v;
+      if (gi == gj) {
+        t1 += v;
+        t2 += 0.5 * v * v;        // off-diagonal entries count twice, at the end
+        f += 0.5 * d * d;
+      } else {
+        t2 += v * v;
+        f += d * d;
+      }
+    }
+  }
+  __syncthreads();
+  if (I == J) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (gi0 + k > gj) y[k] = sm[c4 + k][r];
+    st4d(out + gj * np + gi0, y);
+  } else {
+    st4d(out + gj * np + gi0, y);
+    double w[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) w[k] = sm[c4 + k][r];   // entry (i, j), i = I TE + r
+    st4d(out + (I * TE + r) * np + J * TE + c4, w);
+  }
+  __syncthreads();
+  t1 = block_sum(t1);
+  __syncthreads();
+  t2 = block_sum(t2);
+  __syncthreads();
+  f = block_sum(f);
+  if (threadIdx.x == 0) part[blockIdx.x] = Part3{t1, 2.0 * t2, 2.0 * f};
+  if (dec.done) {
+    __shared__ int last;
+    if (threadIdx.x == 0) {
+      __threadfence();
+      last = atomicAdd(dec.done, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (last) {
+      __threadfence();
+      decide_block(part, dec.st, dec.p);
+      if (threadIdx.x == 0) *dec.done = 0u;
+    }
+  }
+}
+
+// Y_{n+1} = sigma > 0 ? Z + Z^T : 2 Y_n - (Z + Z^T) for a batch, Z = Y_n X_n from T
+// (ey: exponents of the stacked rows of Y_n, ex: of X_n). One block per tile pair
+// and batch entry.
+__global__ void __launch_bounds__(kPassThreads)
+k_dig_symm(const unsigned long long* __restrict__ T, int64_t rows, const int* __restrict__ ey,
+           const int* __restrict__ ex, const double* __restrict__ yin, double* __restrict__ yout,
+           int64_t np, const DevState* st, int step) {
+  if (halted_dig(st, step)) return;
+  __shared__ double za[TE][TE + 1], zb[TE][TE + 1];
+  int64_t I, J;
+  tri_ij(blockIdx.x, I, J);
+  const int64_t b0 = (int64_t)blockIdx.y * np, base = b0 * np;
+  const int r = threadIdx.x >> 3, c4 = (threadIdx.x & 7) * 4;
+  const int sg = st->sigma[step];
+  {
+    long long ta[4], tb[4];
+    const int64_t gj = J * TE + r, gi = I * TE + r;
+    ld4ll(T + gj * rows + b0 + I * TE + c4, ta);   // z(i, j): j = gj, i along c4
+    ld4ll(T + gi * rows + b0 + J * TE + c4, tb);   // z(j, i): i = gi, j along c4
+    const int xj = ex[gj], xi = ex[gi];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      za[r][c4 + k] = from_fixed(ta[k], ey[b0 + I * TE + c4 + k], xj);
+      zb[r][c4 + k] = from_fixed(tb[k], ey[b0 + J * TE + c4 + k], xi);
+    }
+  }
+  __syncthreads();
+  const int64_t idx = base + (I * TE + r) * np + J * TE + c4;   // entries (I TE + r, J TE + c4 ..)
+  double y[4], yo[4];
+  if (sg < 0) ld4d(yin + idx, yo);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const double sum = za[c4 + k][r] + zb[r][c4 + k];
+    y[k] = sg > 0 ? sum : 2.0 * yo[k] - sum;
+  }
+  st4d(yout + idx, y);
+  if (I == J) return;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) zb[r][c4 + k] = y[k];   // only this thread reads zb[r][c4..] above
+  __syncthreads();
+  double w[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) w[k] = zb[c4 + k][r];
+  st4d(yout + base + (J * TE + r) * np + I * TE + c4, w);
+}
+
+// C = T's value, row-major rows x np
+__global__ void __launch_bounds__(kPassThreads)
+k_dig_plain(const unsigned long long* __restrict__ T, int64_t rows, const int* __restrict__ ea,
+            const int* __restrict__ ex, double* __restrict__ out, int64_t np, const DevState* st,
+            int step) {
+  if (halted_dig(st, step)) return;
+  __shared__ double sm[TE][TE + 1];
+  const int64_t i0 = (int64_t)blockIdx.y * TE, j0 = (int64_t)blockIdx.x * TE;
+  const int r = threadIdx.x >> 3, c4 = (threadIdx.x & 7) * 4;
+  long long t[4];
+  ld4ll(T + (j0 + r) * rows + i0 + c4, t);
+  const int xj = ex[j0 + r];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) sm[r][c4 + k] = from_fixed(t[k], ea[i0 + c4 + k], xj);
+  __syncthreads();
+  double w[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) w[k] = sm[c4 + k][r];
+  st4d(out + (i0 + r) * np + j0 + c4, w);
+}
+
+template <int BN>
+int resident_pairs() {
+  static int n = 0;
+  if (n) return n;
+  auto kern = k_gemm_dig<BN>;
+  int dev = 0, nsm = 0, nc = 0;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           Geo<BN>::SMEM_BYTES) != cudaSuccess ||
+      cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return 0;
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = 2;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.gridDim = dim3((unsigned)(2 * (nsm / 2)));
+  cfg.blockDim = dim3(NUM_THREADS);
+  cfg.dynamicSmemBytes = Geo<BN>::SMEM_BYTES;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  if (cudaOccupancyMaxActiveClusters(&nc, kern, &cfg) != cudaSuccess || nc < 1) return 0;
+  n = nc;
+  return n;
+}
+
+template <int BN>
+cudaError_t launch_bn(const CUtensorMap& am, const CUtensorMap& bm, const DParams& p,
+                      cudaStream_t s) {
+  const int res = resident_pairs<BN>();
+  if (res < 1) return cudaErrorNotSupported;
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = 2;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.gridDim = dim3((unsigned)(2 * (p.nunits < res ? p.nunits : res)));
+  cfg.blockDim = dim3(NUM_THREADS);
+  cfg.dynamicSmemBytes = Geo<BN>::SMEM_BYTES;
+  cfg.stream = s;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_gemm_dig<BN>, am, bm, p);
+}
+
+}  // namespace
+
+int64_t dig_tiles(int64_t rows, int64_t np, int bn, bool upper) {
+  if (!upper) return rows / 256 * (np / bn);
+  int64_t n = 0;   // tiles whose first row is at most their last column
+  for (int64_t r0 = 0; r0 < np; r0 += 256) n += (np - r0 / bn * bn) / bn;
+  return n;
+}
+
+// Tile width and cut of one product: the fewest clocks of the busiest CTA pair by
+// the estimate below.
+DigPlan dig_plan(int64_t rows, int64_t np, bool upper) {
+  const int nkb = (int)(np / BK);
+  const int pairs = 76;
+  DigPlan best;
+  double tbest = 0.0;
+  for (int bn = 256; bn >= 128; bn -= 128) {
+    const int64_t nt = dig_tiles(rows, np, bn, upper);
+    const double chunk = bn == 256 ? 2400.0 : 1600.0, fold = bn == 256 ? 3000.0 : 1500.0;
+    for (int parts = 1; parts <= 4; parts *= 2)
+      for (int ks = (nkb + KSEG_MAX - 1) / KSEG_MAX; ks <= nkb / KCH; ++ks) {
+        const int kseg = ((nkb + ks - 1) / ks + KCH - 1) / KCH * KCH;
+        if ((nkb + kseg - 1) / kseg != ks) continue;
+        const int64_t units = nt * parts * ks;
+        const int64_t waves = (units + pairs - 1) / pairs;
+        const int folds = parts == 1 ? 7 : (parts == 2 ? 4 : 2);
+        const double t = (double)waves * (28.0 / parts * (kseg / KCH) * chunk + folds * fold) + 8000.0;
+        if (tbest == 0.0 || t < tbest) {
+          tbest = t;
+          best.bn = bn;
+          best.parts = parts;
+          best.ksplit = ks;
+          best.kseg = kseg;
+        }
+      }
+  }
+  return best;
+}
+
+cudaError_t launch_digits(const double* src, int64_t rows, int64_t np, const DigOperand& o,
+                          unsigned long long* T, const DevState* st, int step, cudaStream_t s) {
+  k_digits<<<(unsigned)rows, kDigThreads, 0, s>>>(src, rows, np, o.dig, o.ex, T, st, step);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_gemm_dig(const DigOperand& A, int64_t rows, const DigOperand& X, int64_t np,
+                            unsigned long long* T, const Tile* tiles, int ntiles,
+                            const DigPlan& plan, DevState* st, int step, const TcTuning& tune,
+                            cudaStream_t s) {
+  if (np % 256 != 0 || rows % 256 != 0 || kDigits * rows > (int64_t)1 << 30)
+    return cudaErrorInvalidValue;
+  CUtensorMap am, bm;
+  if (!make_map(&am, A.dig, kDigits * rows, np, BM, false) ||
+      !make_map(&bm, X.dig, kDigits * np, np, plan.bn / 2, false))
+    return cudaErrorInvalidValue;
+  DParams p;
+  p.nkb = (int)(np / BK);
+  p.kseg = plan.kseg;
+  p.ksplit = plan.ksplit;
+  p.parts = plan.parts;
+  p.rows = rows;
+  p.np = np;
+  p.T = T;
+  p.tiles = tiles;
+  p.nunits = ntiles * plan.parts * plan.ksplit;
+  p.st = st;
+  p.step = step;
+  p.wait_ns = tune.wait_ns;
+  p.withhold = tune.withhold;
+  return plan.bn == 256 ? launch_bn<256>(am, bm, p, s) : launch_bn<128>(am, bm, p, s);
+}
+
+int64_t dig_square_nparts(int64_t np) { return (np / TE) * (np / TE + 1) / 2; }
+
+cudaError_t launch_dig_square(const unsigned long long* T, const int* ex, const double* X,
+                              double* out, int64_t np, DevState* st, int step, Part3* part,
+                              const SimtDecide* dec, cudaStream_t s) {
+  SimtDecide sd;
+  if (dec) sd = *dec;
+  k_dig_square<<<(unsigned)dig_square_nparts(np), kPassThreads, 0, s>>>(T, ex, X, out, np, st, step,
+                                                                       part, sd);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_dig_symm(const unsigned long long* T, int64_t rows, const int* ey, const int* ex,
+                            const double* yin, double* yout, int64_t np, const DevState* st,
+                            int step, cudaStream_t s) {
+  const dim3 grid((unsigned)dig_square_nparts(np), (unsigned)(rows / np));
+  k_dig_symm<<<grid, kPassThreads, 0, s>>>(T, rows, ey, ex, yin, yout, np, st, step);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_dig_plain(const unsigned long long* T, int64_t rows, const int* ea,
+                             const int* ex, double* out, int64_t np, const DevState* st, int step,
+                             cudaStream_t s) {
+  const dim3 grid((unsigned)(np / TE), (unsigned)(rows / TE));
+  k_dig_plain<<<grid, kPassThreads, 0, s>>>(T, rows, ea, ex, out, np, st, step);
+  return cudaGetLastError();
+}
+
+}  // namespace sp2

@@ -35,6 +35,11 @@ struct sp2_handle_s {
   DevState* d_state = nullptr;
   DevState* h_state = nullptr;  // pinned mirror
   TcTuning tune;                // product-kernel launch settings (sp2_set_option)
+  // The digit buffers of FP64 products ("dig.*") are optional: when device memory or
+  // the workspace limit leaves no room for another buffer they are given back and
+  // the rest of the call's FP64 products run on the CUDA cores (dig_off).
+  bool dig_off = false;
+  const void* dig_x = nullptr;  // the matrix whose digits "dig.x" holds, this step
   // The step loop reads the trailing part of the device state after every step
   // into a pinned ring (kRing slots), each followed by an event; the host waits
   // only for the step kLookahead behind the one it enqueues, so the GPU never
@@ -90,7 +95,9 @@ int fail(sp2_handle_t h, int code, const char* fmt, ...) {
   } while (0)
 
 // --------------------------------------------------------------- workspace
-int ws(sp2_handle_t h, const std::string& name, size_t bytes, void** out) {
+// A named device buffer of at least `bytes`; SP2_ENOMEM with h->err set when there
+// is no room.
+int ws_try(sp2_handle_t h, const std::string& name, size_t bytes, void** out) {
   if (bytes == 0) bytes = 256;
   auto& b = h->bufs[name];
   if (b.bytes >= bytes) {
@@ -118,6 +125,31 @@ int ws(sp2_handle_t h, const std::string& name, size_t bytes, void** out) {
   h->held += bytes;
   *out = p;
   return SP2_OK;
+}
+
+// gives back the digit buffers; true if there were any
+bool drop_digits(sp2_handle_t h) {
+  bool any = false;
+  for (auto& kv : h->bufs)
+    if (kv.first.rfind("dig.", 0) == 0 && kv.second.p) {
+      if (!any) cudaStreamSynchronize(h->stream);
+      any = true;
+      cudaFree(kv.second.p);
+      h->held -= kv.second.bytes;
+      kv.second.p = nullptr;
+      kv.second.bytes = 0;
+    }
+  h->dig_x = nullptr;
+  return any;
+}
+
+int ws(sp2_handle_t h, const std::string& name, size_t bytes, void** out) {
+  int r = ws_try(h, name, bytes, out);
+  if (r == SP2_ENOMEM && drop_digits(h)) {
+    h->dig_off = true;
+    r = ws_try(h, name, bytes, out);
+  }
+  return r;
 }
 
 void ws_free(sp2_handle_t h, const std::string& name) {
@@ -249,9 +281,8 @@ int parts_per_tile(sp2_handle_t h, int mode) { return split_mode(mode) && h->tun
 // time share their operand slices. upper=true keeps only tiles that meet the
 // upper triangle (row0 <= last column), which suffices for symmetric results.
 int tile_list(sp2_handle_t h, int mode, int64_t rows, int64_t np, bool upper, const Tile** d,
-              int* n) {
-  int bm, bn;
-  tile_shape(h, mode, np, &bm, &bn);
+              int* n, int bm = 0, int bn = 0) {
+  if (bm == 0) tile_shape(h, mode, np, &bm, &bn);
   char key[96];
   snprintf(key, sizeof key, "%d/%lld/%lld/%d/%dx%d", mode, (long long)rows, (long long)np,
            (int)upper, bm, bn);
@@ -348,12 +379,117 @@ int tc_common(Ctx& c, TcLaunch* L, int ntiles) {
   return SP2_OK;
 }
 
+// --------------------------------------------------------------- FP64 products by digits
+// FP64 products padded to kPad take the tensor-core form (gemm_dig.cu) as long as
+// its buffers fit: above np = 256, and at np = 256 for a stacked factor of two or
+// more matrices (one 256 x 256 product: 23 us and its passes against 34 us on the
+// CUDA cores; per SP2 step at N = 256, 71 against 59 us alone, 133 against 320 us
+// with 8 responses).
+bool dig_mode(const Ctx& c, int64_t rows) {
+  return c.mode == SP2_MODE_FP64 && c.np % kPad == 0 && !c.h->dig_off &&
+         (c.np > kPad || rows >= 2 * kPad);
+}
+
+// Batch entries whose digits and sums are formed at a time (22 bytes per entry of a
+// stacked factor): at most 2 GiB of them, at least one.
+int64_t dig_chunk(int64_t np, int64_t batch) {
+  const int64_t per = 22 * np * np;
+  const int64_t m = ((int64_t)2 << 30) / per;
+  return m < 1 ? 1 : (m < batch ? m : batch);
+}
+
+struct DigBufs {
+  DigOperand x, a;              // right factor; stacked left factor of `rows` rows
+  unsigned long long* T = nullptr;
+  const Tile* tiles = nullptr;
+  int ntiles = 0;
+  DigPlan plan;
+};
+
+// The buffers of one product of a rows x np left factor (0: the square of the
+// right factor). False when they do not fit: the caller takes the CUDA-core form,
+// as the rest of the call does.
+bool dig_bufs(Ctx& c, int64_t rows, bool upper, DigBufs* b) {
+  sp2_handle_t h = c.h;
+  const size_t el = (size_t)c.np * c.np, ra = (size_t)rows * c.np;
+  const size_t nt = rows ? ra : el;
+  void *xd, *xe, *T, *ad = nullptr, *ae = nullptr;
+  const void* old_x = h->bufs["dig.x"].p;
+  bool ok = ws_try(h, "dig.x", el * 2 * kDigPlanes, &xd) == SP2_OK &&
+            ws_try(h, "dig.xe", (size_t)c.np * sizeof(int), &xe) == SP2_OK &&
+            ws_try(h, "dig.T", nt * 8, &T) == SP2_OK;
+  if (ok && rows)
+    ok = ws_try(h, "dig.a", ra * 2 * kDigPlanes, &ad) == SP2_OK &&
+         ws_try(h, "dig.ae", (size_t)rows * sizeof(int), &ae) == SP2_OK;
+  const int64_t rr = rows ? rows : c.np;
+  if (ok) {
+    b->plan = dig_plan(rr, c.np, upper);
+    ok = tile_list(h, c.mode, rr, c.np, upper, &b->tiles, &b->ntiles, 256, b->plan.bn) == SP2_OK;
+  }
+  if (!ok) {
+    h->err.clear();
+    drop_digits(h);
+    h->dig_off = true;
+    return false;
+  }
+  if (old_x != xd) h->dig_x = nullptr;
+  b->x = DigOperand{static_cast<uint16_t*>(xd), static_cast<int*>(xe)};
+  b->a = rows ? DigOperand{static_cast<uint16_t*>(ad), static_cast<int*>(ae)} : b->x;
+  b->T = static_cast<unsigned long long*>(T);
+  return true;
+}
+
+// work of one digit product: tensor flops of the tiles' 28 digit pairs
+double dig_flops(const Ctx& c, const DigBufs& b) {
+  return 2.0 * 256.0 * b.plan.bn * (double)c.np * 28.0 * b.ntiles;
+}
+
 // X_{n+1} = sigma_n>0 ? X_n^2 : 2 X_n - X_n^2, with trace partials; returns #partials.
 // dec (CUDA-core modes): the step decision with these parameters is taken by the
 // product's last block instead of a separate launch (dec->nparts is set here).
 int square_step(Ctx& c, const MatBuf& xin, const MatBuf& xout, int step, int* nparts,
                 const DecideParams* dec = nullptr) {
   sp2_handle_t h = c.h;
+  DigBufs db;
+  if (dig_mode(c, c.np)) {
+    SimtDecide sd;
+    if (dec) {
+      void* dn;
+      TRY(ws(h, "decide.done", sizeof(unsigned), &dn));
+      sd.p = *dec;
+      sd.p.nparts = (int)dig_square_nparts(c.np);
+      sd.st = c.st;
+      sd.done = static_cast<unsigned*>(dn);
+    }
+    if (dig_bufs(c, 0, true, &db)) {
+      const double* x = static_cast<const double*>(xin.master);
+      // the response product of this step has left X_n's digits, but not a clear T
+      if (h->dig_x == xin.master)
+        CK(cudaMemsetAsync(db.T, 0, (size_t)c.np * c.np * 8, h->stream));
+      else
+        CK(launch_digits(x, c.np, c.np, db.x, db.T, c.st, step, h->stream));
+      h->dig_x = nullptr;
+      cudaEvent_t e0 = nullptr, e1 = nullptr;
+      if (c.timing) {
+        TRY(ev_pair(c, &e0, &e1));
+        CK(cudaEventRecord(e0, h->stream));
+      }
+      CK(launch_gemm_dig(db.x, c.np, db.x, c.np, db.T, db.tiles, db.ntiles, db.plan, c.st, step,
+                         h->tune, h->stream));
+      if (c.timing) {
+        CK(cudaEventRecord(e1, h->stream));
+        c.timed.push_back({step, 0});
+      }
+      CK(launch_dig_square(db.T, db.x.ex, x, static_cast<double*>(xout.master), c.np, c.st, step,
+                           c.part, dec ? &sd : nullptr, h->stream));
+      c.launches++;
+      c.kernels += 3;
+      c.flops += dig_flops(c, db);
+      c.alg += (double)c.n * (double)(c.n + 1) * (double)c.n;
+      *nparts = (int)dig_square_nparts(c.np);
+      return SP2_OK;
+    }
+  }
   const Tile* tl;
   int nt;
   TRY(tile_list(h, c.mode, c.np, c.np, true, &tl, &nt));
@@ -481,6 +617,44 @@ int response_step(Ctx& c, const MatBuf& x, const MatBuf& yin, const MatBuf& yout
   const int64_t rows = batch * c.np;
   const bool split = split_mode(c.mode);
   const bool fused = split && h->tune.fused_response;
+  if (dig_mode(c, rows)) {
+    const int64_t bc = dig_chunk(c.np, batch);
+    DigBufs db;
+    if (dig_bufs(c, bc * c.np, false, &db)) {
+      const double* y = static_cast<const double*>(yin.master);
+      double* yo = static_cast<double*>(yout.master);
+      CK(launch_digits(static_cast<const double*>(x.master), c.np, c.np, db.x, nullptr, c.st, step,
+                       h->stream));
+      h->dig_x = x.master;
+      c.kernels++;
+      for (int64_t b0 = 0; b0 < batch; b0 += bc) {
+        const int64_t nb = batch - b0 < bc ? batch - b0 : bc, r = nb * c.np, off = b0 * c.np * c.np;
+        if (nb != bc) {   // the last, smaller chunk has its own tiles
+          db.plan = dig_plan(r, c.np, false);
+          TRY(tile_list(h, c.mode, r, c.np, false, &db.tiles, &db.ntiles, 256, db.plan.bn));
+        }
+        CK(launch_digits(y + off, r, c.np, db.a, db.T, c.st, step, h->stream));
+        cudaEvent_t e0 = nullptr, e1 = nullptr;
+        if (c.timing) {
+          TRY(ev_pair(c, &e0, &e1));
+          CK(cudaEventRecord(e0, h->stream));
+        }
+        CK(launch_gemm_dig(db.a, r, db.x, c.np, db.T, db.tiles, db.ntiles, db.plan, c.st, step,
+                           h->tune, h->stream));
+        if (c.timing) {
+          CK(cudaEventRecord(e1, h->stream));
+          c.timed.push_back({step, 0});
+        }
+        CK(launch_dig_symm(db.T, r, db.a.ex, db.x.ex, y + off, yo + off, c.np, c.st, step,
+                           h->stream));
+        c.launches++;
+        c.kernels += 3;
+        c.flops += dig_flops(c, db);
+      }
+      c.alg += 2.0 * (double)batch * (double)c.n * (double)c.n * (double)c.n;
+      return SP2_OK;
+    }
+  }
   const Tile* tl;
   int nt;
   TRY(tile_list(h, c.mode, rows, c.np, fused, &tl, &nt));
@@ -602,6 +776,8 @@ int resolve_ckpt(sp2_handle_t h, sp2_opts* o, int64_t np, int64_t batch) {
   const double ms = (double)master_size(o->mode), mat_b = el * (ms + 2.0 * n_planes(o->mode));
   const double b = (double)(batch > 0 ? batch : 1);
   avail -= 2.0 * mat_b + 2.0 * b * mat_b + b * el * ms + (double)(1ull << 30);
+  if (o->mode == SP2_MODE_FP64 && np % kPad == 0)   // digit buffers
+    avail -= el * (14.0 + 22.0 * (double)dig_chunk(np, batch > 0 ? batch : 1));
   const int cap = o->fixed_m > 0 ? o->fixed_m : o->max_iter;
   int k = cap;
   for (int kk = 1; kk <= cap; ++kk) {
@@ -714,6 +890,7 @@ int run_sp2(sp2_handle_t h, const void* Hd, int64_t n, int dtype, double nocc, c
   const int64_t np = c.np;   // the caller's padding (one for every mode a loop may switch to)
   const int mode = o.mode;
   const bool sparse = o.block_sparse != 0;
+  h->dig_x = nullptr;
   if (sparse) {
     if (!split_mode(mode) || !h->tune.pair)
       return fail(h, SP2_EINVAL, "block_sparse: the squares run in the split modes on CTA pairs");
@@ -961,6 +1138,9 @@ int make_ctx(sp2_handle_t h, int mode, int64_t n, int64_t np, bool timing, Ctx* 
   tile_shape(h, mode, np, &bm, &bn);
   int64_t maxp = (np / bm) * (np / bn) * parts_per_tile(h, mode) + 8;
   if (maxp < init_nparts(np)) maxp = init_nparts(np);
+  h->dig_off = false;
+  h->dig_x = nullptr;
+  if (dig_mode(*c, np) && maxp < dig_square_nparts(np)) maxp = dig_square_nparts(np);
   void* p;
   TRY(ws(h, "part", (size_t)maxp * sizeof(Part3), &p));
   c->part = static_cast<Part3*>(p);
@@ -1207,6 +1387,34 @@ int fplanes(Ctx& c, FMat& f) {
 // plus C's max in FP16X2 (planes follow from fplanes when C is an operand)
 int fprod(Ctx& c, FMat& C, const FMat& L, const FMat& R) {
   sp2_handle_t h = c.h;
+  DigBufs db;
+  const bool same = L.m.master == R.m.master;
+  if (dig_mode(c, c.np) && dig_bufs(c, same ? 0 : c.np, false, &db)) {
+    const double* l = static_cast<const double*>(L.m.master);
+    CK(launch_digits(l, c.np, c.np, db.a, db.T, c.st, 0, h->stream));
+    if (!same)
+      CK(launch_digits(static_cast<const double*>(R.m.master), c.np, c.np, db.x, nullptr, c.st, 0,
+                       h->stream));
+    h->dig_x = nullptr;
+    cudaEvent_t e0 = nullptr, e1 = nullptr;
+    if (c.timing) {
+      TRY(ev_pair(c, &e0, &e1));
+      CK(cudaEventRecord(e0, h->stream));
+    }
+    CK(launch_gemm_dig(db.a, c.np, db.x, c.np, db.T, db.tiles, db.ntiles, db.plan, c.st, 0, h->tune,
+                       h->stream));
+    if (c.timing) {
+      CK(cudaEventRecord(e1, h->stream));
+      c.timed.push_back({0, 0});
+    }
+    CK(launch_dig_plain(db.T, c.np, db.a.ex, db.x.ex, static_cast<double*>(C.m.master), c.np, c.st,
+                        0, h->stream));
+    c.launches++;
+    c.kernels += same ? 3 : 4;
+    c.flops += dig_flops(c, db);
+    c.alg += 2.0 * (double)c.n * (double)c.n * (double)c.n;
+    return SP2_OK;
+  }
   const Tile* tl;
   int nt;
   TRY(tile_list(h, c.mode, c.np, c.np, false, &tl, &nt));

@@ -20,8 +20,13 @@ namespace sp2 {
 // 2X - X^2, Y -> YX + XY), so it never touches results.
 constexpr int kPad = 256;
 
+// Above this N FP64 products run by digits on the tensor cores and matrices are
+// padded to kPad (per SP2 step at N = 300: 75 us by digits at np = 512 against 86 us
+// on the CUDA cores at np = 320; at N = 200, 72 against 60).
+constexpr int64_t kDigMinN = 257;
+
 inline int64_t pad_n(int64_t n, int mode) {
-  const int64_t q = mode == SP2_MODE_FP64 ? 64 : (mode == SP2_MODE_FP32 ? 128 : kPad);
+  const int64_t q = mode == SP2_MODE_FP64 && n < kDigMinN ? 64 : (mode == SP2_MODE_FP32 ? 128 : kPad);
   return (n + q - 1) / q * q;
 }
 
@@ -297,6 +302,37 @@ cudaError_t launch_sparse_plan(const SparseBufs& B, int init, int xo, int tl_in,
 cudaError_t launch_zero_blocks(const SparseBufs& B, MatBuf x, int64_t np, int mode,
                                const DevState* st, int step, int init, cudaStream_t s);
 void tc_tile_shape(int pair, int* bm, int* bn);   // output tile of one CTA (pair)
+
+// ---- FP64 products by digits on the tensor cores (gemm_dig.cu), np % 256 == 0
+constexpr int kDigPlanes = 7;
+struct DigOperand {        // digit planes of a rows x np factor and its rows' exponents
+  uint16_t* dig = nullptr; // kDigPlanes x rows x np, bfloat16 integers
+  int* ex = nullptr;       // rows
+};
+struct DigPlan {           // tile width of a CTA pair and the cut of a tile's work
+  int bn = 256, parts = 1, ksplit = 1, kseg = 4;
+};
+DigPlan dig_plan(int64_t rows, int64_t np, bool upper);
+int64_t dig_square_nparts(int64_t np);   // partials of launch_dig_square
+// digits of src (rows x np); T (nullable): np x rows 64-bit sums, cleared
+cudaError_t launch_digits(const double* src, int64_t rows, int64_t np, const DigOperand& o,
+                          unsigned long long* T, const DevState* st, int step, cudaStream_t s);
+// T[j * rows + i] += fixed-point (A X)_ij over the listed 256 x plan.bn tiles
+cudaError_t launch_gemm_dig(const DigOperand& A, int64_t rows, const DigOperand& X, int64_t np,
+                            unsigned long long* T, const Tile* tiles, int ntiles,
+                            const DigPlan& plan, DevState* st, int step, const TcTuning& tune,
+                            cudaStream_t s);
+// the passes from T: the square step with its partials (and, with dec, the step
+// decision), the symmetrised response update of a batch, C = A X
+cudaError_t launch_dig_square(const unsigned long long* T, const int* ex, const double* X,
+                              double* out, int64_t np, DevState* st, int step, Part3* part,
+                              const SimtDecide* dec, cudaStream_t s);
+cudaError_t launch_dig_symm(const unsigned long long* T, int64_t rows, const int* ey, const int* ex,
+                            const double* yin, double* yout, int64_t np, const DevState* st,
+                            int step, cudaStream_t s);
+cudaError_t launch_dig_plain(const unsigned long long* T, int64_t rows, const int* ea,
+                             const int* ex, double* out, int64_t np, const DevState* st, int step,
+                             cudaStream_t s);
 
 // FP16X2 scale of the next symmetric response step: per batch entry, the sum of
 // the EPI_SYMM tile partials (||Y_{n+1}||_F^2) and the plane scale of Y_{n+2},
