@@ -24,47 +24,94 @@ __device__ double block_sum(double v) {
   return v;  // valid in thread 0
 }
 
-// Reads the partials with cache-global loads: in the CUDA-core square they come
-// from the other blocks of the same launch.
-__device__ __noinline__ void decide_block(const Part3* part, DevState* st, const DecideParams& p) {
-  double t1 = 0.0, t2 = 0.0, f = 0.0;
-  for (int i = threadIdx.x; i < p.nparts; i += blockDim.x) {
-    t1 += __ldcg(&part[i].t1);
-    t2 += __ldcg(&part[i].t2);
-    f += __ldcg(&part[i].f);
+// the state's fields the host follows, then (system-wide fence between) the token
+__device__ __forceinline__ void post_snapshot(const DevState* st, const DecideParams& p) {
+  if (!p.snap) return;
+  volatile HostSnap* s = p.snap;
+  s->stop_at = st->stop_at;
+  s->nonfinite = st->nonfinite;
+  s->abort_flag = *((volatile const int*)&st->abort_flag);
+  s->backtracked = st->backtracked;
+  s->stop_step = st->stop_step;
+  s->bounds[0] = st->bounds[0];
+  s->bounds[1] = st->bounds[1];
+  s->alpha = st->alpha;
+  s->beta = st->beta;
+  s->work_kblocks = st->work_kblocks;
+  __threadfence_system();
+  s->token = p.token;
+}
+
+// three block-wide sums at once, each in block_sum's order
+__device__ void block_sum3(double& a, double& b, double& c) {
+  __shared__ double red3[3][32];
+  for (int o = 16; o > 0; o >>= 1) {
+    a += __shfl_xor_sync(0xffffffffu, a, o);
+    b += __shfl_xor_sync(0xffffffffu, b, o);
+    c += __shfl_xor_sync(0xffffffffu, c, o);
   }
-  t1 = block_sum(t1);
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
   __syncthreads();
-  t2 = block_sum(t2);
+  if (l == 0) {
+    red3[0][w] = a;
+    red3[1][w] = b;
+    red3[2][w] = c;
+  }
   __syncthreads();
-  f = block_sum(f);
-  if (threadIdx.x != 0) return;
-  if (st->stop_at != 0) return;  // already stopped: later steps are no-ops
+  if (w != 0) return;
+  const int nw = (blockDim.x + 31) >> 5;
+  a = l < nw ? red3[0][l] : 0.0;
+  b = l < nw ? red3[1][l] : 0.0;
+  c = l < nw ? red3[2][l] : 0.0;
+  for (int o = 16; o > 0; o >>= 1) {
+    a += __shfl_xor_sync(0xffffffffu, a, o);
+    b += __shfl_xor_sync(0xffffffffu, b, o);
+    c += __shfl_xor_sync(0xffffffffu, c, o);
+  }   // valid in thread 0
+}
+
+// One thread's part of the decision: everything it needs of earlier steps is read
+// at once, beside the partials (one memory latency instead of a chain of them).
+struct DecideHist {
+  int stop_at, nbest, plane, sg1, sg2;
+  double fbest, fold, f1, f2, f3, fk;   // f_{s-1}, f_{s-2}, f_{s-3}, f_{s-kStall}
+};
+
+__device__ __forceinline__ void decide_one(DevState* st, const DecideParams& p, const DecideHist& h,
+                                           double t1, double t2, double f) {
+  if (h.stop_at != 0) return;  // already stopped: later steps are no-ops
   const int n = p.n;
+  const int s = n - 1;  // the step that produced X_n (0 for X_1)
   st->t1[n] = t1;
   st->t2[n] = t2;
   if (n >= 2) st->f[n - 1] = f;  // the step that produced X_n measured X_{n-1}
   // split-tail mode: step n (X_n -> X_{n+1}) uses single-plane products while the
   // idempotency error of the last measured iterate exceeds tail_f; once a step
   // has used split products, every later one does
-  if (p.tail_f > 0.0)
-    st->plane1[n] = n == 1 ? 1 : (st->plane1[n - 1] && st->f[n - 1] > p.tail_f ? 1 : 0);
+  if (p.tail_f > 0.0) st->plane1[n] = n == 1 ? 1 : (h.plane && f > p.tail_f ? 1 : 0);
   if (!isfinite(t1) || !isfinite(t2)) {
     st->nonfinite = 1;
     st->stop_at = (n - 1 >= 1) ? n - 1 : -1;
     return;
   }
-  const int s = n - 1;  // the step that produced X_n (0 for X_1)
   // floor candidates: X_s (f known now) with f <= gate and the smallest f so far
-  if (p.fixed_m == 0 && p.floor_gate > 0.0 && s >= 2 && st->f[s] <= p.floor_gate &&
-      (st->nbest == 0 || st->f[s] < st->fbest)) {
-    st->fbest = st->f[s];
+  int nbest = h.nbest;
+  if (p.fixed_m == 0 && p.floor_gate > 0.0 && s >= 2 && f <= p.floor_gate &&
+      (nbest == 0 || f < h.fbest)) {
+    nbest = s;
+    st->fbest = f;
     st->nbest = s;
     st->keep_step = s;
   }
   if (p.fixed_m > 0) {
     if (s == p.fixed_m) st->stop_at = s;
     return;  // branches preset by the host
+  }
+  // the smallest f of the steps before the last kStall
+  double best = h.fold;
+  if (s > kStall) {
+    best = s - kStall == 1 ? h.fk : fmin(h.fold, h.fk);
+    st->fold = best;
   }
   if (s >= 1 && s >= p.min_iter) {
     const double e = fabs(t1 - t2);
@@ -74,19 +121,14 @@ __device__ __noinline__ void decide_block(const Part3* part, DevState* st, const
     //   opposite branches at steps s-2, s-1, f_{s-2} <= gate and f_s >= f_{s-2}; or
     //   min f_1..f_{s-STALL} <= gate and none of f_{s-STALL+1..s} below it
     if (!stop && p.floor_gate > 0.0) {
-      if (s >= 3 && st->sigma[s - 2] != st->sigma[s - 1] && st->f[s - 2] <= p.floor_gate &&
-          st->f[s] >= st->f[s - 2])
-        floor_stop = true;
+      if (s >= 3 && h.sg2 != h.sg1 && h.f2 <= p.floor_gate && f >= h.f2) floor_stop = true;
       // block-sparse recursion: from f <= 1e-4 a pair of opposite steps cuts f at
       // least 600-fold in exact arithmetic; less than twofold is the threshold's floor
-      if (!floor_stop && p.ratio_floor && s >= 3 && st->sigma[s - 2] != st->sigma[s - 1] &&
-          st->f[s - 2] <= kRatioGate && st->f[s] >= 0.5 * st->f[s - 2])
+      if (!floor_stop && p.ratio_floor && s >= 3 && h.sg2 != h.sg1 && h.f2 <= kRatioGate &&
+          f >= 0.5 * h.f2)
         floor_stop = true;
       if (!floor_stop && s > kStall) {
-        double best = st->f[1];
-        for (int k = 2; k <= s - kStall; ++k) best = fmin(best, st->f[k]);
-        double recent = st->f[s - kStall + 1];
-        for (int k = s - kStall + 2; k <= s; ++k) recent = fmin(recent, st->f[k]);
+        const double recent = fmin(fmin(fmin(h.f3, h.f2), h.f1), f);
         if (best <= p.floor_gate && recent >= best) floor_stop = true;
       }
       if (floor_stop) stop = true;
@@ -94,8 +136,8 @@ __device__ __noinline__ void decide_block(const Part3* part, DevState* st, const
     if (stop) {
       st->stop_step = s;
       // at the floor the result is the kept candidate X_nbest (M = nbest - 1 steps)
-      if (floor_stop && st->nbest >= 2 && st->nbest - 1 < s) {
-        st->stop_at = st->nbest - 1;
+      if (floor_stop && nbest >= 2 && nbest - 1 < s) {
+        st->stop_at = nbest - 1;
         st->backtracked = 1;
       } else {
         st->stop_at = s;
@@ -105,6 +147,37 @@ __device__ __noinline__ void decide_block(const Part3* part, DevState* st, const
   }
   // Eq. DM0 branch: the trace after X^2 is t2, after 2X - X^2 it is 2 t1 - t2.
   st->sigma[n] = (fabs(t2 - p.nocc) <= fabs(2.0 * t1 - t2 - p.nocc)) ? 1 : -1;
+}
+
+// Reads the partials with cache-global loads: in the CUDA-core square they come
+// from the other blocks of the same launch.
+__device__ __noinline__ void decide_block(const Part3* part, DevState* st, const DecideParams& p) {
+  static_assert(kStall == 4, "the decision reads f of the last four steps");
+  DecideHist h;
+  if (threadIdx.x == 0) {
+    const int s = p.n - 1;
+    h.stop_at = st->stop_at;
+    h.nbest = st->nbest;
+    h.fbest = st->fbest;
+    h.fold = st->fold;
+    h.plane = st->plane1[s >= 0 ? s : 0];
+    h.sg1 = s >= 1 ? st->sigma[s - 1] : 0;
+    h.sg2 = s >= 2 ? st->sigma[s - 2] : 0;
+    h.f1 = s >= 1 ? st->f[s - 1] : 0.0;
+    h.f2 = s >= 2 ? st->f[s - 2] : 0.0;
+    h.f3 = s >= 3 ? st->f[s - 3] : 0.0;
+    h.fk = s >= kStall ? st->f[s - kStall] : 0.0;
+  }
+  double t1 = 0.0, t2 = 0.0, f = 0.0;
+  for (int i = threadIdx.x; i < p.nparts; i += blockDim.x) {
+    t1 += __ldcg(&part[i].t1);
+    t2 += __ldcg(&part[i].t2);
+    f += __ldcg(&part[i].f);
+  }
+  block_sum3(t1, t2, f);
+  if (threadIdx.x != 0) return;
+  decide_one(st, p, h, t1, t2, f);
+  post_snapshot(st, p);
 }
 
 }  // namespace

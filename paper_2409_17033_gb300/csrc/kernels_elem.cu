@@ -750,7 +750,7 @@ cudaError_t launch_bounds(const void* H, int64_t n, int dtype, double2* part, in
     k_bounds_x4<<<nparts, kRedThreads, 0, s>>>(static_cast<const float*>(H), n, part);
   else
     k_bounds<<<nparts, kRedThreads, 0, s>>>(H, n, dtype, part);
-  k_bounds_final<<<1, 1024, 0, s>>>(part, nparts, st);
+  k_bounds_final<<<1, 128, 0, s>>>(part, nparts, st);
   return cudaGetLastError();
 }
 

@@ -10,6 +10,7 @@
 
 #include <map>
 #include <string>
+#include <thread>
 #include <vector>
 
 #include "sp2_internal.h"
@@ -40,13 +41,13 @@ struct sp2_handle_s {
   // the rest of the call's FP64 products run on the CUDA cores (dig_off).
   bool dig_off = false;
   const void* dig_x = nullptr;  // the matrix whose digits "dig.x" holds, this step
-  // The step loop reads the trailing part of the device state after every step
-  // into a pinned ring (kRing slots), each followed by an event; the host waits
-  // only for the step kLookahead behind the one it enqueues, so the GPU never
-  // idles and at most kLookahead no-op steps follow the stop.
-  static constexpr int kRing = 16, kLookahead = 8;
-  DevState* ring = nullptr;     // pinned, kRing snapshots (tail only)
-  cudaEvent_t ring_ev[kRing] = {};
+  // Every step's decision writes a snapshot into a pinned ring (kRing slots); the
+  // host waits only for the step kLookahead behind the one it enqueues, so the GPU
+  // never idles and at most kLookahead no-op steps follow the stop.
+  static constexpr int kRing = 16, kLookahead = 4;
+  HostSnap* ring = nullptr;         // pinned, kRing snapshots
+  HostSnap late;                    // a snapshot read from the state itself
+  unsigned long long run_id = 0;    // recursions run on this handle (part of the tokens)
   // side stream for host copies that overlap later work of the same call
   cudaStream_t side = nullptr;
   cudaEvent_t side_ev[2] = {};
@@ -845,23 +846,41 @@ int poll_state(sp2_handle_t h) {
   return SP2_OK;
 }
 
-// enqueue a snapshot of the state's trailing part into ring slot `step` % kRing
-int ring_record(sp2_handle_t h, int step) {
-  const int slot = step % sp2_handle_s::kRing;
-  const size_t off = devstate_tail_offset();
-  CK(cudaMemcpyAsync(reinterpret_cast<char*>(h->ring + slot) + off,
-                     reinterpret_cast<const char*>(h->d_state) + off, sizeof(DevState) - off,
-                     cudaMemcpyDeviceToHost, h->stream));
-  CK(cudaEventRecord(h->ring_ev[slot], h->stream));
-  return SP2_OK;
+// the ring slot of `step` and the token its snapshot carries
+void ring_slot(sp2_handle_t h, int step, DecideParams* dp) {
+  dp->snap = h->ring + step % sp2_handle_s::kRing;
+  dp->token = h->run_id * 1024ull + (unsigned long long)step;
 }
 
-// wait for the snapshot of `step` and return it
-int ring_read(sp2_handle_t h, int step, const DevState** out) {
-  const int slot = step % sp2_handle_s::kRing;
-  CK(cudaEventSynchronize(h->ring_ev[slot]));
-  *out = h->ring + slot;
-  return SP2_OK;
+// Wait for the snapshot of `step` and return it. Snapshots are read in step order,
+// none past the one that shows a stop (a stopped recursion's later decisions may
+// not run). When the stream has drained without it (an aborted product never
+// reached its decision), the state itself is read.
+int ring_read(sp2_handle_t h, int step, const HostSnap** out) {
+  HostSnap* s = h->ring + step % sp2_handle_s::kRing;
+  const unsigned long long token = h->run_id * 1024ull + (unsigned long long)step;
+  for (unsigned it = 1;; ++it) {
+    if (__atomic_load_n(&s->token, __ATOMIC_ACQUIRE) == token) {
+      *out = s;
+      return SP2_OK;
+    }
+    if (it % 16384 != 0) continue;
+    const cudaError_t e = cudaStreamQuery(h->stream);
+    if (e == cudaErrorNotReady) {
+      cudaGetLastError();
+      std::this_thread::yield();
+      continue;
+    }
+    CK(e);
+    if (__atomic_load_n(&s->token, __ATOMIC_ACQUIRE) == token) continue;
+    CK(cudaMemcpyAsync(h->h_state, h->d_state, sizeof(DevState), cudaMemcpyDeviceToHost, h->stream));
+    CK(cudaStreamSynchronize(h->stream));
+    const DevState& d = *h->h_state;
+    h->late = HostSnap{token, d.stop_at, d.nonfinite, d.abort_flag, d.backtracked, d.stop_step, 0,
+                       {d.bounds[0], d.bounds[1]}, d.alpha, d.beta, d.work_kblocks};
+    *out = &h->late;
+    return SP2_OK;
+  }
 }
 
 // --------------------------------------------------------------- the SP2 driver
@@ -934,6 +953,7 @@ int run_sp2(sp2_handle_t h, const void* Hd, int64_t n, int dtype, double nocc, c
   c.tail = dp.tail_f > 0.0 ? 1 : 0;
   dp.n = 1;
   dp.nparts = ni;
+  h->run_id++;
   SparseBufs sb;
   if (sparse) {
     // X~_1 = T_tau(X_1); the first square's tiles; X[0]'s content is unknown, so
@@ -989,8 +1009,8 @@ int run_sp2(sp2_handle_t h, const void* Hd, int64_t n, int dtype, double nocc, c
     TRY(ws(h, "decide.done", sizeof(unsigned), &dn));
     CK(cudaMemsetAsync(dn, 0, sizeof(unsigned), h->stream));
   }
-  const DevState* seen = nullptr;   // latest snapshot read
-  int last = 0;                     // last step enqueued
+  const HostSnap* seen = nullptr;   // latest snapshot read
+  int read = 0, last = 0;           // last step whose snapshot was read, last step enqueued
   for (int step = 1; step <= maxit; ++step) {
     const MatBuf& xin = X[step % 2];
     const MatBuf& xo = X[(step + 1) % 2];
@@ -1011,6 +1031,7 @@ int run_sp2(sp2_handle_t h, const void* Hd, int64_t n, int dtype, double nocc, c
       TRY(response_step(c, xin, Y[step % 2], Y[(step + 1) % 2], ybatch, step, sc, step % 2,
                         (step + 1) % 2));
     dp.n = step + 1;
+    ring_slot(h, step, &dp);
     if (sparse) {
       TRY(sparse_square(c, xin, xo, step, sb));
       CK(launch_sparse_plan(sb, 0, (step + 1) % 2, step % 2, (step + 1) % 2, c.part, 0, c.st, step,
@@ -1045,15 +1066,15 @@ int run_sp2(sp2_handle_t h, const void* Hd, int64_t n, int dtype, double nocc, c
       astep = c.alg - a0;
       lstep = c.launches - l0;
     }
-    TRY(ring_record(h, step));
     last = step;
     if (step > sp2_handle_s::kLookahead) {
-      TRY(ring_read(h, step - sp2_handle_s::kLookahead, &seen));
+      TRY(ring_read(h, ++read, &seen));
       if (seen->stop_at != 0 || seen->abort_flag) break;
     }
   }
-  if (!seen || (seen->stop_at == 0 && !seen->abort_flag)) TRY(ring_read(h, last, &seen));
-  const DevState& S = *seen;
+  while (read < last && (!seen || (seen->stop_at == 0 && !seen->abort_flag)))
+    TRY(ring_read(h, ++read, &seen));
+  const HostSnap S = *seen;
   out->alpha = S.alpha;
   out->beta = S.beta;
   out->emin = S.bounds[0];
@@ -1288,17 +1309,23 @@ void drop_pending(sp2_handle_t h) {
 int complete_pending(sp2_handle_t h, sp2_info* info) {
   sp2_handle_s::Pending* p = h->pending;
   h->pending = nullptr;
-  CK(cudaStreamSynchronize(h->stream));
   if (!p) {
+    CK(cudaStreamSynchronize(h->stream));
     if (info) memset(info, 0, sizeof *info);
     return SP2_OK;
   }
   int code = p->status;
   std::string msg = p->msg;
-  cudaError_t e = cudaMemcpy(h->h_state, h->d_state, sizeof(DevState), cudaMemcpyDeviceToHost);
-  int adj_abort = 0;
+  // the state comes with the wait (the recursion's last slot of the ring has been read)
+  volatile int* aflag = &h->ring[0].abort_flag;
+  *aflag = 0;
+  cudaError_t e = cudaMemcpyAsync(h->h_state, h->d_state, sizeof(DevState), cudaMemcpyDeviceToHost,
+                                  h->stream);
   if (e == cudaSuccess && p->adj_state)
-    e = cudaMemcpy(&adj_abort, &p->adj_state->abort_flag, sizeof(int), cudaMemcpyDeviceToHost);
+    e = cudaMemcpyAsync(&h->ring[0].abort_flag, &p->adj_state->abort_flag, sizeof(int),
+                        cudaMemcpyDeviceToHost, h->stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+  const int adj_abort = e == cudaSuccess && p->adj_state ? *aflag : 0;
   if (e != cudaSuccess) {
     delete p;
     return fail(h, SP2_ECUDA, "reading the device state failed: %s", cudaGetErrorString(e));
@@ -1521,18 +1548,11 @@ int sp2_create(sp2_handle_t* out, void* stream, size_t limit) {
     code = SP2_ECUDA;
   }
   if (code == SP2_OK &&
-      cudaMallocHost(&h->ring, sizeof(DevState) * sp2_handle_s::kRing) != cudaSuccess) {
+      cudaMallocHost(&h->ring, sizeof(HostSnap) * sp2_handle_s::kRing) != cudaSuccess) {
     cudaGetLastError();
     code = SP2_ECUDA;
   }
-  for (int i = 0; code == SP2_OK && i < sp2_handle_s::kRing; ++i)
-    if (cudaEventCreateWithFlags(&h->ring_ev[i], cudaEventDisableTiming) != cudaSuccess) {
-      cudaGetLastError();
-      code = SP2_ECUDA;
-    }
   if (code != SP2_OK) {
-    for (int i = 0; i < sp2_handle_s::kRing; ++i)
-      if (h->ring_ev[i]) cudaEventDestroy(h->ring_ev[i]);
     if (h->ring) cudaFreeHost(h->ring);
     if (h->h_state) cudaFreeHost(h->h_state);
     if (h->d_state) cudaFree(h->d_state);
@@ -1540,7 +1560,7 @@ int sp2_create(sp2_handle_t* out, void* stream, size_t limit) {
     return code;
   }
   memset(h->h_state, 0, sizeof(DevState));
-  memset(h->ring, 0, sizeof(DevState) * sp2_handle_s::kRing);
+  memset(h->ring, 0, sizeof(HostSnap) * sp2_handle_s::kRing);
   *out = h;
   return SP2_OK;
 }
@@ -1553,8 +1573,6 @@ int sp2_destroy(sp2_handle_t h) {
   for (auto& kv : h->tiles) cudaFree(kv.second.d);
   if (h->d_state) cudaFree(h->d_state);
   if (h->h_state) cudaFreeHost(h->h_state);
-  for (int i = 0; i < sp2_handle_s::kRing; ++i)
-    if (h->ring_ev[i]) cudaEventDestroy(h->ring_ev[i]);
   if (h->ring) cudaFreeHost(h->ring);
   if (h->side) {
     cudaStreamSynchronize(h->side);

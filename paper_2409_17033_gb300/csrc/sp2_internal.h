@@ -52,9 +52,17 @@ struct DevState {
   int stop_step;                 // the step after which the stop test fired
   double alpha, beta;            // X_1 = alpha I + beta H, from the (widened) bounds
   double work_kblocks;           // block-sparse: 256-wide K blocks the squares ran, all tiles
+  double fold;                   // min f_1..f_{s-kStall} after step s (the stall floor's older part)
 };
-// The host reads the trailing part of DevState (from stop_at on) after every step.
-inline size_t devstate_tail_offset() { return offsetof(DevState, stop_at); }
+
+// What the host learns of a step: written by the step decision into a slot of a
+// pinned host ring, the token last. A copy of the state on the stream after every
+// step (and an event behind it) cost more than a small step's kernels.
+struct HostSnap {
+  unsigned long long token;      // call and step the other fields belong to
+  int stop_at, nonfinite, abort_flag, backtracked, stop_step, pad_;
+  double bounds[2], alpha, beta, work_kblocks;
+};
 
 // Storage of one padded matrix (or a batch of them) in a given mode.
 struct MatBuf {
@@ -177,6 +185,8 @@ struct DecideParams {
   int fixed_m;       // > 0: sigma preset, stop when n - 1 == fixed_m
   double tail_f;     // > 0: single-plane products while f of the last iterate exceeds it
   int ratio_floor = 0;  // block-sparse recursion: the threshold-floor test as well
+  HostSnap* snap = nullptr;  // pinned host slot of this step (nullable) and its token
+  unsigned long long token = 0;
 };
 constexpr double kRatioGate = 1e-4;   // f from which a pair of opposite steps must cut f 600-fold
 cudaError_t launch_decide(const Part3* part, DevState* st, DecideParams p, cudaStream_t s);
