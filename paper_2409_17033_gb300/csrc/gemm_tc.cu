@@ -66,6 +66,7 @@
 
 #include <mutex>
 
+#include "decide.cuh"
 #include "sp2_internal.h"
 #include "tc_ptx.cuh"
 
@@ -74,35 +75,32 @@ namespace sp2 {
 namespace {
 
 constexpr int BM = 128;        // output rows per CTA (a CTA pair's tile has 2 BM)
-constexpr int BN = 256;
+constexpr int BN_FULL = 256;   // tile columns (narrower tiles: 128 and 64, on CTA pairs)
 constexpr int BK = 64;
 constexpr int A_BYTES = BM * BK * 2;
-// Per-CTA ring geometry for CG CTAs per tile: a CTA of a pair holds half of the
-// right factor's rows, so its stage is 32 KB and six stages fit.
-template <int CG>
+// Per-CTA ring geometry for CG CTAs per tile of BN columns: a CTA of a pair holds
+// half of the right factor's rows, so its stage is 32 KB (BN = 256) and six stages fit.
+template <int CG, int BN>
 struct Ring {
   static constexpr int B_ROWS = BN / CG;
   static constexpr int B_BYTES = B_ROWS * BK * 2;
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-  static constexpr int STAGES = CG == 1 ? 4 : 6;
+  static constexpr int STAGES = CG == 1 ? 4 : (BN == 256 ? 6 : 8);
   static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 /*align slack*/ + 256 /*barriers*/;
 };
 constexpr int EPI_WARPS = 16;                    // four warps per TMEM lane quarter
 constexpr int EPI_THREADS = 32 * EPI_WARPS;
 constexpr int NUM_THREADS = 64 + EPI_THREADS;    // TMA warp, MMA warp, epilogue warps
-constexpr uint32_t ACC_COLS = 256;               // one 128 x 256 FP32 accumulator
-constexpr uint32_t TMEM_COLS = 2 * ACC_COLS;     // two chunk buffers
 constexpr int COL_GROUPS = EPI_WARPS / 4;        // column groups of a tile
-constexpr int TCOLS = BN / COL_GROUPS;            // columns per epilogue thread
 constexpr unsigned long long DRAIN_NS = 200000000ull;
 
 // Instruction descriptor, kind::f16: D=F32 (bits 4-5 = 1), A and B format at
 // bits 7-9 / 10-12 (BF16 = 1, F16 = 0; always the same for A and B), both
 // K-major (bits 15,16 = 0), N>>3 at bit 17, M>>4 at bit 24. M is the rows of
 // one instruction: BM, or 2 BM for a CTA pair.
-constexpr uint32_t idesc_for(bool f16, int m) {
+constexpr uint32_t idesc_for(bool f16, int m, int n) {
   return (1u << 4) | ((f16 ? 0u : 1u) << 7) | ((f16 ? 0u : 1u) << 10) |
-         ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
+         ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
 
 // A sum of FP32 terms w x^2 (w a power of two) kept to about 2^-45 of its value
@@ -205,6 +203,7 @@ struct KParams {
   const int* kcnt;
   const uint16_t* klist;
   int nbk;
+  SimtDecide dec;          // narrow square tiles: the last CTA takes the step decision
 };
 
 // Tensor maps of one launch: the left factor's planes with 128-row boxes (A role)
@@ -224,7 +223,7 @@ struct KMaps {
 // is a template parameter, so that each kernel carries only its own code (a
 // smaller kernel keeps the producer's and the MMA issuer's loops in the
 // instruction cache).
-template <int KIND, int EPI>
+template <int KIND, int EPI, int TCOLS>
 __device__ __forceinline__ void tile_end(const KParams& p, float (&acc)[TCOLS], int tix, int pidx,
                                          int it, int e, int lane, int grp, int r, int sg,
                                          double (*red)[3][EPI_WARPS]) {
@@ -390,16 +389,20 @@ __device__ __forceinline__ int sparse_run_end(const uint16_t* kl, int kc, int gs
 // every block listed the chunks, and the results, are the dense kernel's. The
 // sparse loops are separate from the dense ones, which the SPARSE = false
 // kernels alone contain.
-template <int KIND, int EPI, int CG, bool SPARSE = false>
+template <int KIND, int EPI, int CG, int BN = BN_FULL, bool SPARSE = false>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 k_gemm_tc(const __grid_constant__ KMaps maps, const __grid_constant__ KParams p) {
   static_assert(!SPARSE || (EPI == EPI_SQUARE && CG == 2), "block-sparse squares run on pairs");
-  using R = Ring<CG>;
+  static_assert(BN == BN_FULL || CG == 2, "narrow tiles run on pairs");
+  using R = Ring<CG, BN>;
+  constexpr uint32_t ACC_COLS = BN;                // one 128 x BN FP32 accumulator
+  constexpr uint32_t TMEM_COLS = 2 * ACC_COLS;     // two chunk buffers
+  constexpr int TCOLS = BN / COL_GROUPS;           // columns per epilogue thread
   constexpr int STAGES = R::STAGES;
   constexpr int STAGE_BYTES = R::STAGE_BYTES;
   constexpr bool PAIR = CG == 2;
   constexpr bool F16 = KIND == KIND_FP16X2;
-  constexpr uint32_t kIdesc = idesc_for(F16, BM * CG);
+  constexpr uint32_t kIdesc = idesc_for(F16, BM * CG, BN);
   DevState* st = p.st;
   {
     // a pair must take this exit together: stop_at is fixed for the launch, while
@@ -772,7 +775,7 @@ k_gemm_tc(const __grid_constant__ KMaps maps, const __grid_constant__ KParams p)
           }
         }
         if (!ok || *((volatile int*)abortf)) break;
-        tile_end<KIND, EPI>(p, acc, tix, tix * CG + (int)rank, it, e, lane, grp, r, sg, red);
+        tile_end<KIND, EPI, TCOLS>(p, acc, tix, tix * CG + (int)rank, it, e, lane, grp, r, sg, red);
         continue;
       }
       int kb0 = 0;
@@ -810,7 +813,7 @@ k_gemm_tc(const __grid_constant__ KMaps maps, const __grid_constant__ KParams p)
         }
       }
       if (!ok || *((volatile int*)abortf)) break;
-      tile_end<KIND, EPI>(p, acc, tix, tix * CG + (int)rank, it, e, lane, grp, r, sg, red);
+      tile_end<KIND, EPI, TCOLS>(p, acc, tix, tix * CG + (int)rank, it, e, lane, grp, r, sg, red);
     }
   }
 
@@ -831,6 +834,23 @@ k_gemm_tc(const __grid_constant__ KMaps maps, const __grid_constant__ KParams p)
                    "r"(TMEM_COLS)
                    : "memory");
   }
+  if constexpr (EPI == EPI_SQUARE && BN < BN_FULL) {
+    // the last CTA to get here takes the step decision (the wide-tile kernels leave
+    // it to its own launch: its code beside theirs costs them instruction cache)
+    if (p.dec.done) {
+      __shared__ int last;
+      if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicAdd(p.dec.done, 1u) == gridDim.x - 1;
+      }
+      __syncthreads();
+      if (last) {
+        __threadfence();
+        decide_block(p.part, p.dec.st, p.dec.p);
+        if (threadIdx.x == 0) *p.dec.done = 0u;
+      }
+    }
+  }
 }
 
 // The tensor maps of a launch are a function of its plane addresses, shapes and
@@ -842,7 +862,7 @@ k_gemm_tc(const __grid_constant__ KMaps maps, const __grid_constant__ KParams p)
 struct MapKey {
   const void* planes[6];
   int64_t prows, qrows, np;
-  int cg, f16;
+  int cg, bn, f16;
 };
 
 bool cached_maps(const MapKey& k, KMaps* out) {
@@ -862,10 +882,10 @@ bool cached_maps(const MapKey& k, KMaps* out) {
   bool ok = true;
   for (int i = 0; i < 3; ++i) {
     ok = ok && make_map(&m.pa[i], k.planes[i], k.prows, k.np, BM, k.f16) &&
-         make_map(&m.qb[i], k.planes[3 + i], k.qrows, k.np, BN / k.cg, k.f16);
+         make_map(&m.qb[i], k.planes[3 + i], k.qrows, k.np, k.bn / k.cg, k.f16);
     // EPI_SYMM's second half reads X as the left and Y as the right factor
     ok = ok && make_map(&m.qa[i], k.planes[3 + i], k.qrows, k.np, BM, k.f16) &&
-         make_map(&m.pb[i], k.planes[i], k.prows, k.np, BN / k.cg, k.f16);
+         make_map(&m.pb[i], k.planes[i], k.prows, k.np, k.bn / k.cg, k.f16);
   }
   if (!ok) return false;
   keys[next] = k;
@@ -879,11 +899,11 @@ bool cached_maps(const MapKey& k, KMaps* out) {
 // one launch of the (KIND, EPI, CG) kernel over `units` CTAs or CTA pairs (at most
 // the resident ones), with its shared-memory attribute and its resident-pair
 // count queried once
-template <int KIND, int EPI, int CG, bool SPARSE = false>
+template <int KIND, int EPI, int CG, int BN = BN_FULL, bool SPARSE = false>
 cudaError_t launch_kind(const KMaps& maps, const KParams& p, int units, cudaStream_t s) {
   static int resident = 0;
-  auto kern = k_gemm_tc<KIND, EPI, CG, SPARSE>;
-  constexpr int smem = Ring<CG>::SMEM_BYTES;
+  auto kern = k_gemm_tc<KIND, EPI, CG, BN, SPARSE>;
+  constexpr int smem = Ring<CG, BN>::SMEM_BYTES;
   if (!resident) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
@@ -939,12 +959,27 @@ cudaError_t launch_epi(int epi, const KMaps& maps, const KParams& p, int units, 
   return launch_kind<KIND, EPI_PLAIN, CG>(maps, p, units, s);
 }
 
+// narrow tiles (BN < 256) on CTA pairs
+template <int KIND, int BN>
+cudaError_t launch_narrow(int epi, const KMaps& maps, const KParams& p, int units, cudaStream_t s) {
+  if (epi == EPI_SQUARE) return launch_kind<KIND, EPI_SQUARE, 2, BN>(maps, p, units, s);
+  return launch_kind<KIND, EPI_PLAIN, 2, BN>(maps, p, units, s);
+}
+
+template <int BN>
+cudaError_t launch_bn(int kind, int epi, const KMaps& maps, const KParams& p, int units,
+                      cudaStream_t s) {
+  if (kind == KIND_FP16X2) return launch_narrow<KIND_FP16X2, BN>(epi, maps, p, units, s);
+  if (kind == KIND_BF16X3) return launch_narrow<KIND_BF16X3, BN>(epi, maps, p, units, s);
+  return launch_narrow<KIND_BF16X2, BN>(epi, maps, p, units, s);
+}
+
 // the block-sparse square: one launch over every resident pair, the tile count
 // read on the device
 cudaError_t launch_sparse(int kind, const KMaps& maps, const KParams& p, int units, cudaStream_t s) {
-  if (kind == KIND_FP16X2) return launch_kind<KIND_FP16X2, EPI_SQUARE, 2, true>(maps, p, units, s);
-  if (kind == KIND_BF16X3) return launch_kind<KIND_BF16X3, EPI_SQUARE, 2, true>(maps, p, units, s);
-  return launch_kind<KIND_BF16X2, EPI_SQUARE, 2, true>(maps, p, units, s);
+  if (kind == KIND_FP16X2) return launch_kind<KIND_FP16X2, EPI_SQUARE, 2, BN_FULL, true>(maps, p, units, s);
+  if (kind == KIND_BF16X3) return launch_kind<KIND_BF16X3, EPI_SQUARE, 2, BN_FULL, true>(maps, p, units, s);
+  return launch_kind<KIND_BF16X2, EPI_SQUARE, 2, BN_FULL, true>(maps, p, units, s);
 }
 
 template <int CG>
@@ -959,7 +994,33 @@ cudaError_t launch_cg(int kind, int epi, const KMaps& maps, const KParams& p, in
 
 void tc_tile_shape(int pair, int* bm, int* bn) {
   *bm = pair ? 2 * BM : BM;
-  *bn = BN;
+  *bn = BN_FULL;
+}
+
+// Upper tiles (first row at most the last column) or all tiles of a rows x np product.
+static int64_t tile_count(int64_t rows, int64_t np, int bn, bool upper) {
+  if (!upper) return rows / (2 * BM) * (np / bn);
+  int64_t n = 0;
+  for (int64_t r0 = 0; r0 < np; r0 += 2 * BM) n += (np - r0) / bn;
+  return n;
+}
+
+int tc_tile_width(int64_t rows, int64_t np, bool upper) {
+  constexpr int kPairs = 76;
+  const double kb = (double)(np / BK);
+  int best = BN_FULL;
+  double tbest = 0.0;
+  for (int bn = BN_FULL; bn >= 64; bn /= 2) {
+    const int64_t waves = (tile_count(rows, np, bn, upper) + kPairs - 1) / kPairs;
+    const double kclk = bn == 256 ? 600.0 : (bn == 128 ? 400.0 : 320.0);
+    const double end = (upper ? 140.0 : 30.0) * bn;
+    const double t = (double)waves * 3.0 * kb * kclk + end;
+    if (tbest == 0.0 || t < 0.95 * tbest) {
+      tbest = t;
+      best = bn;
+    }
+  }
+  return best;
 }
 
 cudaError_t launch_gemm_tc(const TcLaunch& L, cudaStream_t s, char* errbuf, size_t errlen) {
@@ -990,7 +1051,7 @@ cudaError_t launch_gemm_tc(const TcLaunch& L, cudaStream_t s, char* errbuf, size
        reinterpret_cast<uintptr_t>(Q.hi) | reinterpret_cast<uintptr_t>(Q.lo) |
        reinterpret_cast<uintptr_t>(p_mid) | reinterpret_cast<uintptr_t>(q_mid)) & 15u ||
       np % 256 != 0 || P.rows % np != 0 || Q.rows % np != 0 || P.rows % (BM * cg) != 0 ||
-      Q.rows % BN != 0 || (L.epi == EPI_SYMM && Q.rows != np) ||
+      Q.rows % L.bn != 0 || (L.bn != BN_FULL && (cg != 2 || L.epi == EPI_SYMM || L.dyn_ntiles)) || (L.epi == EPI_SYMM && Q.rows != np) ||
       (L.epi == EPI_SQUARE && P.rows != np) || P.rows > (int64_t)1 << 30) {
     snprintf(errbuf, errlen, "tcgen05 product: operand alignment/shape violates the TMA rules");
     return cudaErrorInvalidValue;
@@ -1008,6 +1069,7 @@ cudaError_t launch_gemm_tc(const TcLaunch& L, cudaStream_t s, char* errbuf, size
   key.qrows = Q.rows;
   key.np = np;
   key.cg = cg;
+  key.bn = L.bn;
   key.f16 = f16 ? 1 : 0;
   if (!cached_maps(key, &maps)) {
     snprintf(errbuf, errlen, "cuTensorMapEncodeTiled failed (driver entry point unavailable?)");
@@ -1058,6 +1120,7 @@ cudaError_t launch_gemm_tc(const TcLaunch& L, cudaStream_t s, char* errbuf, size
   p.kcnt = L.kcnt;
   p.klist = L.klist;
   p.nbk = L.nbk;
+  if (L.dec) p.dec = *L.dec;
   if (L.dyn_ntiles) {
     if (cg != 2 || L.epi != EPI_SQUARE || L.tail || !L.kcnt || !L.klist || L.nbk * 256 != np) {
       snprintf(errbuf, errlen, "tcgen05 product: block-sparse launches are squares on CTA pairs");
@@ -1066,6 +1129,8 @@ cudaError_t launch_gemm_tc(const TcLaunch& L, cudaStream_t s, char* errbuf, size
     return launch_sparse(kind, maps, p, L.ntiles, s);
   }
   // persistent: one CTA (pair) per SM (pair of SMs), the launch's tiles spread over them
+  if (L.bn == 128) return launch_bn<128>(kind, L.epi, maps, p, L.ntiles, s);
+  if (L.bn == 64) return launch_bn<64>(kind, L.epi, maps, p, L.ntiles, s);
   if (cg == 2) return launch_cg<2>(kind, L.epi, maps, p, L.ntiles, s);
   return launch_cg<1>(kind, L.epi, maps, p, L.ntiles, s);
 }

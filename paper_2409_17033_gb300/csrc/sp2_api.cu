@@ -274,6 +274,14 @@ void tile_shape(sp2_handle_t h, int mode, int64_t np, int* bm, int* bn) {
   else simt_tile_shape(mode, np, bm, bn);
 }
 
+// the tile of a square (upper) or plain product: narrower on CTA pairs where 256-wide
+// tiles would not fill the GPU
+void product_tile(sp2_handle_t h, int mode, int64_t rows, int64_t np, bool upper, int* bm,
+                  int* bn) {
+  tile_shape(h, mode, np, bm, bn);
+  if (split_mode(mode) && h->tune.pair) *bn = tc_tile_width(rows, np, upper);
+}
+
 // partials per output tile: a CTA pair's two CTAs each report their own rows
 int parts_per_tile(sp2_handle_t h, int mode) { return split_mode(mode) && h->tune.pair ? 2 : 1; }
 
@@ -445,23 +453,23 @@ double dig_flops(const Ctx& c, const DigBufs& b) {
   return 2.0 * 256.0 * b.plan.bn * (double)c.np * 28.0 * b.ntiles;
 }
 
-// X_{n+1} = sigma_n>0 ? X_n^2 : 2 X_n - X_n^2, with trace partials; returns #partials.
-// dec (CUDA-core modes): the step decision with these parameters is taken by the
-// product's last block instead of a separate launch (dec->nparts is set here).
-int square_step(Ctx& c, const MatBuf& xin, const MatBuf& xout, int step, int* nparts,
+// X_{n+1} = sigma_n>0 ? X_n^2 : 2 X_n - X_n^2, with trace partials; dec: and the step
+// decision with these parameters, by the product's last block, or (wide tensor-core
+// tiles) in a launch of its own (dec->nparts is set here).
+int square_step(Ctx& c, const MatBuf& xin, const MatBuf& xout, int step,
                 const DecideParams* dec = nullptr) {
   sp2_handle_t h = c.h;
   DigBufs db;
+  SimtDecide sd;
+  if (dec) {
+    void* dn;
+    TRY(ws(h, "decide.done", sizeof(unsigned), &dn));
+    sd.p = *dec;
+    sd.st = c.st;
+    sd.done = static_cast<unsigned*>(dn);
+  }
   if (dig_mode(c, c.np)) {
-    SimtDecide sd;
-    if (dec) {
-      void* dn;
-      TRY(ws(h, "decide.done", sizeof(unsigned), &dn));
-      sd.p = *dec;
-      sd.p.nparts = (int)dig_square_nparts(c.np);
-      sd.st = c.st;
-      sd.done = static_cast<unsigned*>(dn);
-    }
+    sd.p.nparts = (int)dig_square_nparts(c.np);
     if (dig_bufs(c, 0, true, &db)) {
       const double* x = static_cast<const double*>(xin.master);
       // the response product of this step has left X_n's digits, but not a clear T
@@ -487,15 +495,15 @@ int square_step(Ctx& c, const MatBuf& xin, const MatBuf& xout, int step, int* np
       c.kernels += 3;
       c.flops += dig_flops(c, db);
       c.alg += (double)c.n * (double)(c.n + 1) * (double)c.n;
-      *nparts = (int)dig_square_nparts(c.np);
       return SP2_OK;
     }
   }
   const Tile* tl;
   int nt;
-  TRY(tile_list(h, c.mode, c.np, c.np, true, &tl, &nt));
   int bm, bn;
-  tile_shape(h, c.mode, c.np, &bm, &bn);
+  product_tile(h, c.mode, c.np, c.np, true, &bm, &bn);
+  TRY(tile_list(h, c.mode, c.np, c.np, true, &tl, &nt, bm, bn));
+  sd.p.nparts = nt * parts_per_tile(h, c.mode);
   TcLaunch L;   // workspace first: nothing is allocated inside the timed interval
   if (split_mode(c.mode)) TRY(tc_common(c, &L, nt));
   cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -512,18 +520,11 @@ int square_step(Ctx& c, const MatBuf& xin, const MatBuf& xout, int step, int* np
     L.prev = static_cast<const float*>(xin.master);
     L.tiles = tl;
     L.step = step;
+    L.bn = bn;
+    if (dec && bn < 256) L.dec = &sd;
     cudaError_t e = launch_gemm_tc(L, h->stream, eb, sizeof eb);
     if (e != cudaSuccess) return fail(h, SP2_ECUDA, "square product: %s %s", cudaGetErrorString(e), eb);
   } else {
-    SimtDecide sd;
-    if (dec) {
-      void* dn;
-      TRY(ws(h, "decide.done", sizeof(unsigned), &dn));
-      sd.p = *dec;
-      sd.p.nparts = nt;
-      sd.st = c.st;
-      sd.done = static_cast<unsigned*>(dn);
-    }
     CK(launch_gemm_simt(c.mode, EPI_SQUARE, xin.master, c.np, xin.master, c.np, xout.master,
                         xin.master, c.part, tl, nt, c.st, step, h->stream, dec ? &sd : nullptr));
   }
@@ -535,7 +536,10 @@ int square_step(Ctx& c, const MatBuf& xin, const MatBuf& xout, int step, int* np
   c.kernels++;
   c.flops += 2.0 * bm * bn * (double)c.np * k_mult(c.mode) * nt;
   c.alg += (double)c.n * (double)(c.n + 1) * (double)c.n * k_mult(c.mode);
-  *nparts = nt * parts_per_tile(h, c.mode);
+  if (dec && split_mode(c.mode) && !L.dec) {
+    CK(launch_decide(c.part, c.st, sd.p, h->stream));
+    c.kernels++;
+  }
   return SP2_OK;
 }
 
@@ -658,9 +662,10 @@ int response_step(Ctx& c, const MatBuf& x, const MatBuf& yin, const MatBuf& yout
   }
   const Tile* tl;
   int nt;
-  TRY(tile_list(h, c.mode, rows, c.np, fused, &tl, &nt));
   int bm, bn;
-  tile_shape(h, c.mode, c.np, &bm, &bn);
+  if (fused) tile_shape(h, c.mode, c.np, &bm, &bn);
+  else product_tile(h, c.mode, rows, c.np, false, &bm, &bn);
+  TRY(tile_list(h, c.mode, rows, c.np, fused, &tl, &nt, bm, bn));
   // workspace first: nothing is allocated inside the timed interval
   TcLaunch L;
   void* yp = nullptr;
@@ -721,6 +726,7 @@ int response_step(Ctx& c, const MatBuf& x, const MatBuf& yin, const MatBuf& yout
     L.out = zo;
     L.tiles = tl;
     L.step = step;
+    L.bn = bn;
     if (f16) {
       L.p_scale = sc.yscale + slot_in * sc.B;
       L.zmax = sc.zmax;
@@ -1003,7 +1009,7 @@ int run_sp2(sp2_handle_t h, const void* Hd, int64_t n, int dtype, double nocc, c
     TRY(ws(h, "Xbest.m", xbytes, &xbest.master));
     if (ybatch > 0) TRY(ws(h, "Ybest.m", (size_t)ybatch * xbytes, &ybest.master));
   }
-  if (!split_mode(mode) && !sparse) {
+  if (!sparse) {
     // the completion counter of the squares' last-block decision starts at zero
     void* dn;
     TRY(ws(h, "decide.done", sizeof(unsigned), &dn));
@@ -1040,17 +1046,8 @@ int run_sp2(sp2_handle_t h, const void* Hd, int64_t n, int dtype, double nocc, c
       c.kernels += 2;
       CK(launch_decide(sb.psum, c.st, dp, h->stream));
       c.kernels++;
-    } else if (!split_mode(mode)) {
-      // CUDA-core square: its last block takes the decision
-      int nparts = 0;
-      TRY(square_step(c, xin, xo, step, &nparts, &dp));
-      dp.nparts = nparts;
     } else {
-      int nparts = 0;
-      TRY(square_step(c, xin, xo, step, &nparts));
-      dp.nparts = nparts;
-      CK(launch_decide(c.part, c.st, dp, h->stream));
-      c.kernels++;
+      TRY(square_step(c, xin, xo, step, &dp));
     }
     if (track) {
       CK(launch_keep_best(xin.master, xbest.master, np * np, mode, c.st, step, h->stream));
@@ -1156,7 +1153,7 @@ int make_ctx(sp2_handle_t h, int mode, int64_t n, int64_t np, bool timing, Ctx* 
   c->timing = timing;
   c->st = h->d_state;
   int bm, bn;
-  tile_shape(h, mode, np, &bm, &bn);
+  product_tile(h, mode, np, np, true, &bm, &bn);
   int64_t maxp = (np / bm) * (np / bn) * parts_per_tile(h, mode) + 8;
   if (maxp < init_nparts(np)) maxp = init_nparts(np);
   h->dig_off = false;
@@ -1243,8 +1240,7 @@ int run_adjoint(sp2_handle_t h, const void* Bd, int64_t batch, int b_diag, int s
       }
     }
     for (int s = s0; s < s1; ++s) {
-      int nparts;
-      TRY(square_step(c, seg[s - s0], seg[s - s0 + 1], s, &nparts));
+      TRY(square_step(c, seg[s - s0], seg[s - s0 + 1], s));
     }
     for (int s = s1; s >= s0; --s) {
       TRY(response_step(c, seg[s - s0], G[gs], G[1 - gs], batch, s, sc, gs, 1 - gs));
@@ -1444,9 +1440,9 @@ int fprod(Ctx& c, FMat& C, const FMat& L, const FMat& R) {
   }
   const Tile* tl;
   int nt;
-  TRY(tile_list(h, c.mode, c.np, c.np, false, &tl, &nt));
   int bm, bn;
-  tile_shape(h, c.mode, c.np, &bm, &bn);
+  product_tile(h, c.mode, c.np, c.np, false, &bm, &bn);
+  TRY(tile_list(h, c.mode, c.np, c.np, false, &tl, &nt, bm, bn));
   TcLaunch T;   // workspace first: nothing is allocated inside the timed interval
   if (split_mode(c.mode)) TRY(tc_common(c, &T, nt));
   cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -1464,6 +1460,7 @@ int fprod(Ctx& c, FMat& C, const FMat& L, const FMat& R) {
     T.out = C.m;
     T.tiles = tl;
     T.step = 0;
+    T.bn = bn;
     if (f16) {
       T.p_scale = L.scale;
       T.q_scale = R.scale;

@@ -280,6 +280,8 @@ struct TcLaunch {
   const int* kcnt = nullptr;
   const uint16_t* klist = nullptr;
   int nbk = 0;                     // K blocks of 256 (np / 256): the stride of klist
+  int bn = 256;                    // tile columns: 256, or 128 / 64 (squares and plain products on pairs)
+  const SimtDecide* dec = nullptr; // squares with bn < 256: take the step decision in the last CTA
 };
 cudaError_t launch_gemm_tc(const TcLaunch& L, cudaStream_t s, char* errbuf, size_t errlen);
 
@@ -312,6 +314,9 @@ cudaError_t launch_sparse_plan(const SparseBufs& B, int init, int xo, int tl_in,
 cudaError_t launch_zero_blocks(const SparseBufs& B, MatBuf x, int64_t np, int mode,
                                const DevState* st, int step, int init, cudaStream_t s);
 void tc_tile_shape(int pair, int* bm, int* bn);   // output tile of one CTA (pair)
+// Tile columns of a product on CTA pairs: narrower tiles where 256-wide ones would
+// leave most pairs idle.
+int tc_tile_width(int64_t rows, int64_t np, bool upper);
 
 // ---- FP64 products by digits on the tensor cores (gemm_dig.cu), np % 256 == 0
 constexpr int kDigPlanes = 7;
