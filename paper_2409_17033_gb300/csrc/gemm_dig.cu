@@ -139,7 +139,7 @@ k_gemm_dig(const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUt
   uint64_t* mdone = tempty + 2;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mdone + 1);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   int* abortf = &st->abort_flag;
   const uint32_t rank = cluster_rank();
   const bool issuer = rank == 0;
@@ -211,52 +211,49 @@ k_gemm_dig(const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUt
       }
     }
   } else if (warp == 1) {
-    if (!issuer && lane == 0) {
-      // rank 1: pass each landed stage on to rank 0's MMA issuer
-      const uint32_t pfull_peer = cluster_addr(smem_u32(pfull), 0);
-      RingPos<STAGES> rp;
-      bool ok = true;
-      for (int u = pair; u < p.nunits && ok; u += npairs) {
-        const Unit w = unit_of(p, u);
-        const int n = pairs_per_part * (w.kb1 - w.kb0);
-        for (int q = 0; q < n; ++q, rp.next()) {
-          if (!mbar_wait<true>(&full[rp.s], rp.ph, abortf, p.wait_ns)) {
-            ok = false;
-            break;
+    if (!issuer) {
+      if (lane == 0) {
+        // rank 1: pass each landed stage on to rank 0's MMA issuer
+        const uint32_t pfull_peer = cluster_addr(smem_u32(pfull), 0);
+        RingPos<STAGES> rp;
+        bool ok = true;
+        for (int u = pair; u < p.nunits && ok; u += npairs) {
+          const Unit w = unit_of(p, u);
+          const int n = pairs_per_part * (w.kb1 - w.kb0);
+          for (int q = 0; q < n; ++q, rp.next()) {
+            if (!mbar_wait<true>(&full[rp.s], rp.ph, abortf, p.wait_ns)) {
+              ok = false;
+              break;
+            }
+            mbar_arrive_cluster_release(pfull_peer + (uint32_t)(rp.s * sizeof(uint64_t)));
           }
-          mbar_arrive_cluster_release(pfull_peer + (uint32_t)(rp.s * sizeof(uint64_t)));
         }
       }
-    } else if (issuer && lane == 0) {
+    } else {
+      // whole warp (the waits by every lane, the instructions by an elected one)
       bool ok = true;
-      int64_t gc = 0;
+      uint32_t gc = 0;
       RingPos<STAGES> rp;
       const uint64_t adesc0 = sdesc_sw128(smem_u32(smem));
       for (int u = pair; u < p.nunits && ok; u += npairs) {
         const Unit w = unit_of(p, u);
         const int nch = pairs_per_part * ((w.kb1 - w.kb0) / KCH);
         for (int c = 0; c < nch && ok; ++c, ++gc) {
-          const int b = (int)(gc & 1);
-          if (!mbar_wait<true>(&tempty[b], ((uint32_t)(gc >> 1) & 1u) ^ 1u, abortf, p.wait_ns)) {
-            ok = false;
-            break;
-          }
+          const uint32_t b = gc & 1u;
+          ok = __all_sync(0xffffffffu, mbar_wait<true>(&tempty[b], ((gc >> 1) & 1u) ^ 1u, abortf,
+                                                      p.wait_ns));
+          if (!ok) break;
           tc_fence_after();
-          const uint32_t dtm = tmem + (uint32_t)b * BN;
+          const uint32_t dtm = tmem + b * BN;
 #pragma unroll 1
           for (int kb = 0; kb < KCH; ++kb, rp.next()) {
-            if (!mbar_wait<false>(&full[rp.s], rp.ph, abortf, p.wait_ns) ||
-                !mbar_wait<true>(&pfull[rp.s], rp.ph, abortf, p.wait_ns)) {
-              ok = false;
-              break;
-            }
+            ok = __all_sync(0xffffffffu, mbar_wait<false>(&full[rp.s], rp.ph, abortf, p.wait_ns) &&
+                                             mbar_wait<true>(&pfull[rp.s], rp.ph, abortf, p.wait_ns));
+            if (!ok) break;
             tc_fence_after();
             const uint64_t adesc = adesc0 + (uint64_t)(rp.s * (G::STAGE_BYTES >> 4));
             const uint64_t bdesc = adesc + (uint64_t)(G::A_BYTES >> 4);
-#pragma unroll
-            for (int k = 0; k < BK / 16; ++k)
-              umma_f16<2>(dtm, adesc + (uint64_t)(2 * k), bdesc + (uint64_t)(2 * k), G::IDESC,
-                          (kb > 0 || k > 0) ? 1u : 0u);
+            umma_kblock<2>(dtm, adesc, bdesc, G::IDESC, kb > 0 ? 1u : 0u);
             umma_commit_both(&empty[rp.s]);
           }
           if (ok) umma_commit_both(&tfull[b]);

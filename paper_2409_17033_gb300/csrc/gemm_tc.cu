@@ -422,7 +422,8 @@ k_gemm_tc(const __grid_constant__ KMaps maps, const __grid_constant__ KParams p)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mdone + 1);
   __shared__ double red[2][3][EPI_WARPS];   // per-tile partials, double-buffered by tile parity
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // (uniform over the warp, also to the compiler)
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   int* abortf = &st->abort_flag;
   // a pair: each CTA loads its own halves of both operands (rows rank*128 .. of the
   // A tile and of the B tile) and drains its own TMEM rows; rank 0 issues the MMAs
@@ -575,7 +576,8 @@ k_gemm_tc(const __grid_constant__ KMaps maps, const __grid_constant__ KParams p)
       }
     }
   } else if (warp == 1) {
-    if (PAIR && !issuer && lane == 0) {
+    if (PAIR && !issuer) {
+     if (lane == 0) {
       // rank 1: pass each landed stage of this CTA on to rank 0's MMA issuer
       const uint32_t pfull_peer = cluster_addr(smem_u32(pfull), 0);
       int64_t total = (int64_t)my_tiles * total_kb;
@@ -588,8 +590,8 @@ k_gemm_tc(const __grid_constant__ KMaps maps, const __grid_constant__ KParams p)
         if (!mbar_wait<PAIR>(&full[rp.s], rp.ph, abortf, p.wait_ns)) break;
         mbar_arrive_cluster_release(pfull_peer + (uint32_t)(rp.s * sizeof(uint64_t)));
       }
+     }
     } else if constexpr (SPARSE) {
-     if (lane == 0 && issuer) {
       bool ok = true;
       int64_t g = 0, gc = 0;
       RingPos<STAGES> rp;
@@ -603,27 +605,21 @@ k_gemm_tc(const __grid_constant__ KMaps maps, const __grid_constant__ KParams p)
           for (int q0 = 0; q0 < kc && ok; ++gc) {
             const int q1 = hh ? q0 + 1 : sparse_run_end(kl, kc, gsz, q0);
             const int b = (int)(gc & 1);
-            if (!mbar_wait<PAIR>(&tempty[b], ((uint32_t)(gc >> 1) & 1u) ^ 1u, abortf, p.wait_ns)) {
-              ok = false;
-              break;
-            }
+            ok = __all_sync(0xffffffffu, mbar_wait<PAIR>(&tempty[b], ((uint32_t)(gc >> 1) & 1u) ^ 1u,
+                                                        abortf, p.wait_ns));
+            if (!ok) break;
             tc_fence_after();
             const uint32_t dtm = tmem + (uint32_t)b * ACC_COLS;
             for (int u = 4 * q0; u < 4 * q1; ++u, ++g, rp.next()) {
               const int s = rp.s;
               const uint32_t ph = rp.ph;
-              if (!mbar_wait<false>(&full[s], ph, abortf, p.wait_ns) ||
-                  !mbar_wait<PAIR>(&pfull[s], ph, abortf, p.wait_ns)) {
-                ok = false;
-                break;
-              }
+              ok = __all_sync(0xffffffffu, mbar_wait<false>(&full[s], ph, abortf, p.wait_ns) &&
+                                               mbar_wait<PAIR>(&pfull[s], ph, abortf, p.wait_ns));
+              if (!ok) break;
               tc_fence_after();
               const uint64_t adesc = adesc0 + (uint64_t)(s * (STAGE_BYTES >> 4));
               const uint64_t bdesc = adesc + (uint64_t)(A_BYTES >> 4);
-#pragma unroll
-              for (int k = 0; k < BK / 16; ++k)
-                umma_f16<CG>(dtm, adesc + (uint64_t)(2 * k), bdesc + (uint64_t)(2 * k), kIdesc,
-                             (u > 4 * q0 || k > 0) ? 1u : 0u);
+              umma_kblock<CG>(dtm, adesc, bdesc, kIdesc, u > 4 * q0 ? 1u : 0u);
               umma_commit_both(&empty[s]);
             }
             if (ok) umma_commit_both(&tfull[b]);
@@ -635,8 +631,8 @@ k_gemm_tc(const __grid_constant__ KMaps maps, const __grid_constant__ KParams p)
         umma_commit<CG>(mdone);
         mbar_wait_drain(mdone, 0, DRAIN_NS);
       }
-     }
-    } else if (lane == 0 && issuer) {
+    } else {
+      // whole warp (the waits by every lane, the instructions by an elected one)
       bool ok = true;
       int64_t g = 0, gc = 0;   // k-block and chunk counters across tiles
       RingPos<STAGES> rp;
@@ -656,10 +652,9 @@ k_gemm_tc(const __grid_constant__ KMaps maps, const __grid_constant__ KParams p)
           }
           const int b = (int)(gc & 1);
           // the epilogue (of both CTAs of a pair) has drained buffer b (chunk gc-2)
-          if (!mbar_wait<PAIR>(&tempty[b], ((uint32_t)(gc >> 1) & 1u) ^ 1u, abortf, p.wait_ns)) {
-            ok = false;
-            break;
-          }
+          ok = __all_sync(0xffffffffu, mbar_wait<PAIR>(&tempty[b], ((uint32_t)(gc >> 1) & 1u) ^ 1u,
+                                                      abortf, p.wait_ns));
+          if (!ok) break;
           tc_fence_after();
           const uint32_t dtm = tmem + (uint32_t)b * ACC_COLS;
           for (int kb = kb0; kb < kb0 + len; ++kb, ++g, rp.next()) {
@@ -667,20 +662,14 @@ k_gemm_tc(const __grid_constant__ KMaps maps, const __grid_constant__ KParams p)
             const uint32_t ph = rp.ph;
             // this CTA's own stage (its own copies: CTA-scope acquire), then, on a
             // pair, the peer's stage as relayed by its warp 1
-            if (!mbar_wait<false>(&full[s], ph, abortf, p.wait_ns) ||
-                (PAIR && !mbar_wait<PAIR>(&pfull[s], ph, abortf, p.wait_ns))) {
-              ok = false;
-              break;
-            }
+            ok = __all_sync(0xffffffffu,
+                            mbar_wait<false>(&full[s], ph, abortf, p.wait_ns) &&
+                                (!PAIR || mbar_wait<PAIR>(&pfull[s], ph, abortf, p.wait_ns)));
+            if (!ok) break;
             tc_fence_after();
             const uint64_t adesc = adesc0 + (uint64_t)(s * (STAGE_BYTES >> 4));
             const uint64_t bdesc = adesc + (uint64_t)(A_BYTES >> 4);
-#pragma unroll
-            for (int k = 0; k < BK / 16; ++k) {
-              // advance 16 elements = 32 bytes along K inside the swizzled row: +2 in 16-byte units
-              umma_f16<CG>(dtm, adesc + (uint64_t)(2 * k), bdesc + (uint64_t)(2 * k), kIdesc,
-                           (kb > kb0 || k > 0) ? 1u : 0u);
-            }
+            umma_kblock<CG>(dtm, adesc, bdesc, kIdesc, kb > kb0 ? 1u : 0u);
             // the stage is free in both CTAs once these MMAs have read it
             if constexpr (PAIR) umma_commit_both(&empty[s]);
             else umma_commit<CG>(&empty[s]);
