@@ -24,22 +24,30 @@ __device__ double block_sum(double v) {
   return v;  // valid in thread 0
 }
 
-// the state's fields the host follows, then (system-wide fence between) the token
-__device__ __forceinline__ void post_snapshot(const DevState* st, const DecideParams& p) {
+// Tells the host of the step: one 8-byte word (token and whether the recursion goes
+// on). Only at its end (a stop, an abort, the last step) the other fields go out
+// first, with a system-wide fence between, which waits for the host's memory.
+__device__ __forceinline__ void post_snapshot(const DevState* st, const DecideParams& p,
+                                              int stop_at) {
   if (!p.snap) return;
   volatile HostSnap* s = p.snap;
-  s->stop_at = st->stop_at;
-  s->nonfinite = st->nonfinite;
-  s->abort_flag = *((volatile const int*)&st->abort_flag);
-  s->backtracked = st->backtracked;
-  s->stop_step = st->stop_step;
-  s->bounds[0] = st->bounds[0];
-  s->bounds[1] = st->bounds[1];
-  s->alpha = st->alpha;
-  s->beta = st->beta;
-  s->work_kblocks = st->work_kblocks;
-  __threadfence_system();
-  s->token = p.token;
+  const int ab = *((volatile const int*)&st->abort_flag);
+  const int last = p.n - 1 >= (p.fixed_m > 0 ? p.fixed_m : p.max_iter);
+  const unsigned long long end = stop_at != 0 || ab || last ? 1ull : 0ull;
+  if (end) {
+    s->stop_at = stop_at;
+    s->nonfinite = st->nonfinite;
+    s->abort_flag = ab;
+    s->backtracked = st->backtracked;
+    s->stop_step = st->stop_step;
+    s->bounds[0] = st->bounds[0];
+    s->bounds[1] = st->bounds[1];
+    s->alpha = st->alpha;
+    s->beta = st->beta;
+    s->work_kblocks = st->work_kblocks;
+    __threadfence_system();
+  }
+  s->word = 2ull * p.token + end;
 }
 
 // three block-wide sums at once, each in block_sum's order
@@ -77,9 +85,10 @@ struct DecideHist {
   double fbest, fold, f1, f2, f3, fk;   // f_{s-1}, f_{s-2}, f_{s-3}, f_{s-kStall}
 };
 
-__device__ __forceinline__ void decide_one(DevState* st, const DecideParams& p, const DecideHist& h,
-                                           double t1, double t2, double f) {
-  if (h.stop_at != 0) return;  // already stopped: later steps are no-ops
+// Returns stop_at.
+__device__ __forceinline__ int decide_one(DevState* st, const DecideParams& p, const DecideHist& h,
+                                          double t1, double t2, double f) {
+  if (h.stop_at != 0) return h.stop_at;  // already stopped: later steps are no-ops
   const int n = p.n;
   const int s = n - 1;  // the step that produced X_n (0 for X_1)
   st->t1[n] = t1;
@@ -92,7 +101,7 @@ __device__ __forceinline__ void decide_one(DevState* st, const DecideParams& p, 
   if (!isfinite(t1) || !isfinite(t2)) {
     st->nonfinite = 1;
     st->stop_at = (n - 1 >= 1) ? n - 1 : -1;
-    return;
+    return (n - 1 >= 1) ? n - 1 : -1;
   }
   // floor candidates: X_s (f known now) with f <= gate and the smallest f so far
   int nbest = h.nbest;
@@ -105,7 +114,7 @@ __device__ __forceinline__ void decide_one(DevState* st, const DecideParams& p, 
   }
   if (p.fixed_m > 0) {
     if (s == p.fixed_m) st->stop_at = s;
-    return;  // branches preset by the host
+    return s == p.fixed_m ? s : 0;  // branches preset by the host
   }
   // the smallest f of the steps before the last kStall
   double best = h.fold;
@@ -136,38 +145,68 @@ __device__ __forceinline__ void decide_one(DevState* st, const DecideParams& p, 
     if (stop) {
       st->stop_step = s;
       // at the floor the result is the kept candidate X_nbest (M = nbest - 1 steps)
-      if (floor_stop && nbest >= 2 && nbest - 1 < s) {
-        st->stop_at = nbest - 1;
-        st->backtracked = 1;
-      } else {
-        st->stop_at = s;
-      }
-      return;
+      const bool back = floor_stop && nbest >= 2 && nbest - 1 < s;
+      if (back) st->backtracked = 1;
+      st->stop_at = back ? nbest - 1 : s;
+      return back ? nbest - 1 : s;
     }
   }
   // Eq. DM0 branch: the trace after X^2 is t2, after 2X - X^2 it is 2 t1 - t2.
   st->sigma[n] = (fabs(t2 - p.nocc) <= fabs(2.0 * t1 - t2 - p.nocc)) ? 1 : -1;
+  return 0;
 }
 
-// Reads the partials with cache-global loads: in the CUDA-core square they come
-// from the other blocks of the same launch.
-__device__ __noinline__ void decide_block(const Part3* part, DevState* st, const DecideParams& p) {
+__device__ __forceinline__ void load_hist(const DevState* st, const DecideParams& p, DecideHist& h) {
   static_assert(kStall == 4, "the decision reads f of the last four steps");
+  const int s = p.n - 1;
+  h.stop_at = st->stop_at;
+  h.nbest = st->nbest;
+  h.fbest = st->fbest;
+  h.fold = st->fold;
+  h.plane = st->plane1[s >= 0 ? s : 0];
+  h.sg1 = s >= 1 ? st->sigma[s - 1] : 0;
+  h.sg2 = s >= 2 ? st->sigma[s - 2] : 0;
+  h.f1 = s >= 1 ? st->f[s - 1] : 0.0;
+  h.f2 = s >= 2 ? st->f[s - 2] : 0.0;
+  h.f3 = s >= 3 ? st->f[s - 3] : 0.0;
+  h.fk = s >= kStall ? st->f[s - kStall] : 0.0;
+}
+
+constexpr int kWarpParts = 512;   // up to this many partials one warp takes the decision
+
+// The decision by the first warp of a block (every thread may call): few partials
+// cost a whole block more in FP64 shuffles (64 clocks a warp and instruction) and
+// barriers than one warp's additions take: 8 us at the end of a product against 2.
+// Reads the partials with cache-global loads: they come from the other blocks of
+// the same launch.
+__device__ __noinline__ void decide_warp(const Part3* part, DevState* st, const DecideParams& p) {
+  if (threadIdx.x >= 32) return;
   DecideHist h;
-  if (threadIdx.x == 0) {
-    const int s = p.n - 1;
-    h.stop_at = st->stop_at;
-    h.nbest = st->nbest;
-    h.fbest = st->fbest;
-    h.fold = st->fold;
-    h.plane = st->plane1[s >= 0 ? s : 0];
-    h.sg1 = s >= 1 ? st->sigma[s - 1] : 0;
-    h.sg2 = s >= 2 ? st->sigma[s - 2] : 0;
-    h.f1 = s >= 1 ? st->f[s - 1] : 0.0;
-    h.f2 = s >= 2 ? st->f[s - 2] : 0.0;
-    h.f3 = s >= 3 ? st->f[s - 3] : 0.0;
-    h.fk = s >= kStall ? st->f[s - kStall] : 0.0;
+  load_hist(st, p, h);
+  double t1 = 0.0, t2 = 0.0, f = 0.0;
+  for (int i = threadIdx.x; i < p.nparts; i += 32) {
+    t1 += __ldcg(&part[i].t1);
+    t2 += __ldcg(&part[i].t2);
+    f += __ldcg(&part[i].f);
   }
+  for (int o = 16; o > 0; o >>= 1) {
+    t1 += __shfl_xor_sync(0xffffffffu, t1, o);
+    t2 += __shfl_xor_sync(0xffffffffu, t2, o);
+    f += __shfl_xor_sync(0xffffffffu, f, o);
+  }
+  if (threadIdx.x != 0) return;
+  const int stop_at = decide_one(st, p, h, t1, t2, f);
+  post_snapshot(st, p, stop_at);
+}
+
+// The same by a whole block (every thread calls).
+__device__ __noinline__ void decide_block(const Part3* part, DevState* st, const DecideParams& p) {
+  if (p.nparts <= kWarpParts) {
+    decide_warp(part, st, p);
+    return;
+  }
+  DecideHist h;
+  if (threadIdx.x == 0) load_hist(st, p, h);
   double t1 = 0.0, t2 = 0.0, f = 0.0;
   for (int i = threadIdx.x; i < p.nparts; i += blockDim.x) {
     t1 += __ldcg(&part[i].t1);
@@ -176,8 +215,8 @@ __device__ __noinline__ void decide_block(const Part3* part, DevState* st, const
   }
   block_sum3(t1, t2, f);
   if (threadIdx.x != 0) return;
-  decide_one(st, p, h, t1, t2, f);
-  post_snapshot(st, p);
+  const int stop_at = decide_one(st, p, h, t1, t2, f);
+  post_snapshot(st, p, stop_at);
 }
 
 }  // namespace

@@ -175,39 +175,35 @@ k_gemm_dig(const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUt
   const uint32_t tmem = *tmem_slot;
 
   if (warp == 0) {
-    if (lane == 0) {
-      int64_t g = 0;
-      RingPos<STAGES> rp;
-      bool ok = true;
-      for (int u = pair; u < p.nunits && ok; u += npairs) {
-        const Unit w = unit_of(p, u);
-        const int arow = w.t.row0 + (int)rank * BM;
-        const int brow = w.t.col0 + (int)rank * G::B_ROWS;
-        for (int s = kGroups - 1; s >= 0 && ok; --s) {
-          if (!((w.mask >> s) & 1u)) continue;
-          for (int i = 0; i <= s && ok; ++i) {
-            const int ay = i * (int)p.rows + arow, by = (s - i) * (int)p.np + brow;
-            for (int kx = w.kb0 * BK; kx < w.kb1 * BK; kx += BK, ++g, rp.next()) {
-              if (!mbar_wait<true>(&empty[rp.s], rp.ph ^ 1u, abortf, p.wait_ns)) {
-                ok = false;
-                break;
-              }
-              if (p.withhold && blockIdx.x == 0 && g == 0) continue;  // test hook: never completes
-              uint8_t* sa = smem + rp.s * G::STAGE_BYTES;
-              mbar_arrive_expect_tx(&full[rp.s], G::STAGE_BYTES);
-              tma_load_2d(&amap, &full[rp.s], sa, kx, ay);
-              tma_load_2d(&bmap, &full[rp.s], sa + G::A_BYTES, kx, by);
-            }
+    // copy issuer: the whole warp (the waits by every lane, the copies by an elected one)
+    int64_t g = 0;
+    RingPos<STAGES> rp;
+    const uint32_t ring = smem_u32(smem);
+    bool ok = true;
+    for (int u = pair; u < p.nunits && ok; u += npairs) {
+      const Unit w = unit_of(p, u);
+      const int arow = w.t.row0 + (int)rank * BM;
+      const int brow = w.t.col0 + (int)rank * G::B_ROWS;
+      for (int s = kGroups - 1; s >= 0 && ok; --s) {
+        if (!((w.mask >> s) & 1u)) continue;
+        for (int i = 0; i <= s && ok; ++i) {
+          const int ay = i * (int)p.rows + arow, by = (s - i) * (int)p.np + brow;
+          for (int kx = w.kb0 * BK; kx < w.kb1 * BK; kx += BK, ++g, rp.next()) {
+            ok = __all_sync(0xffffffffu, mbar_wait<true>(&empty[rp.s], rp.ph ^ 1u, abortf, p.wait_ns));
+            if (!ok) break;
+            if (p.withhold && blockIdx.x == 0 && g == 0) continue;  // test hook: never completes
+            const uint32_t sa = ring + (uint32_t)(rp.s * G::STAGE_BYTES);
+            tma_load_stage(&full[rp.s], G::STAGE_BYTES, &amap, &bmap, sa, sa + G::A_BYTES, kx, ay, by);
           }
         }
       }
-      if (!ok) {
-        // aborted: let the copies already issued land before the CTA exits
-        const int64_t first = g > STAGES ? g - STAGES : 0;
-        for (int64_t q = first; q < g; ++q) {
-          if (p.withhold && blockIdx.x == 0 && q == 0) continue;
-          mbar_wait_drain(&full[q % STAGES], (uint32_t)(q / STAGES) & 1u, DRAIN_NS);
-        }
+    }
+    if (!ok) {
+      // aborted: let the copies already issued land before the CTA exits
+      const int64_t first = g > STAGES ? g - STAGES : 0;
+      for (int64_t q = first; q < g; ++q) {
+        if (p.withhold && blockIdx.x == 0 && q == 0) continue;
+        mbar_wait_drain(&full[q % STAGES], (uint32_t)(q / STAGES) & 1u, DRAIN_NS);
       }
     }
   } else if (warp == 1) {

@@ -46,9 +46,9 @@
 // report drained TMEM buffers there. Same arithmetic and order as one SM.
 //
 // Warp roles:
-//   warp 0  (one thread)  TMA producer
-//   warp 1  (one thread)  tcgen05.mma issuer (pair: rank 1's relays stages); the
-//                         whole warp owns the TMEM allocation
+//   warp 0                TMA producer   } whole warps in uniform control flow, one
+//   warp 1                tcgen05.mma issuer (pair: rank 1's relays stages) } elected
+//                         lane issuing; warp 1 owns the TMEM allocation
 //   warps 2-17            epilogue: tcgen05.ld of each chunk (warp w reads TMEM lanes
 //                         32*(w%4) .. +31, the 64 columns of group (w-2)/4), then
 //                         the epilogue above. With 64 columns per thread the chunk
@@ -103,26 +103,92 @@ constexpr uint32_t idesc_for(bool f16, int m, int n) {
          ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
 
-// A sum of FP32 terms w x^2 (w a power of two) kept to about 2^-45 of its value
-// before it goes to FP64, at FP32 rates (GB300's FP64 rate is a small fraction
-// of its FP32 rate): each square enters as its rounded value plus its fmaf
-// residual (exact), each addition as TwoSum (Knuth) with its rounding error
-// carried in c. The _rn intrinsics keep the compiler from contracting the steps
-// into fused operations, which would lose the error terms.
+// Packed pairs of FP32 values (add / mul / fma.rn.f32x2: each half rounds as the
+// scalar operation does, in half the instructions).
+__device__ __forceinline__ uint64_t pk2(float x, float y) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+  return r;
+}
+__device__ __forceinline__ void upk2(uint64_t v, float& x, float& y) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v));
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+constexpr uint64_t kMinus1x2 = 0xbf800000bf800000ull;   // {-1, -1}
+__device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) { return fma2(b, kMinus1x2, a); }
+
+// A sum of squares of FP32 values kept to about 2^-45 of its value before it goes to
+// FP64, at FP32 rates (GB300's FP64 rate is a small fraction of its FP32 rate), two
+// values at a time: each square enters as its rounded value plus its residual
+// (exact), each addition as TwoSum (Knuth) with its rounding error carried in c. The
+// packed operations are never contracted, which would lose the error terms.
+__device__ __forceinline__ float two_sum(float a, float b, float& err) {
+  const float t = __fadd_rn(a, b), bp = __fsub_rn(t, a);
+  err = __fadd_rn(__fsub_rn(a, __fsub_rn(t, bp)), __fsub_rn(b, bp));   // a + b - t
+  return t;
+}
+// the sum of (hi + lo) over the lanes whose indices differ in the bits W, W/2, .. 1
+template <int W>
+__device__ __forceinline__ void pair_sum(float& hi, float& lo) {
+#pragma unroll
+  for (int o = W; o > 0; o >>= 1) {
+    const float gh = __shfl_xor_sync(0xffffffffu, hi, o), gl = __shfl_xor_sync(0xffffffffu, lo, o);
+    float err;
+    hi = two_sum(hi, gh, err);
+    lo = __fadd_rn(__fadd_rn(lo, gl), err);
+  }
+}
 struct ExactSqSum {
-  float s = 0.0f, c = 0.0f;
-  __device__ __forceinline__ void add_sq(float w, float x) {
-    const float wx = w * x;                 // exact: w is 1 or 2
-    const float p = __fmul_rn(wx, x);
-    const float e = fmaf(wx, x, -p);        // wx x - p exactly
-    const float t = __fadd_rn(s, p);
-    const float bp = __fsub_rn(t, s);
-    const float err = __fadd_rn(__fsub_rn(s, __fsub_rn(t, bp)), __fsub_rn(p, bp));   // s + p - t
-    c = __fadd_rn(c, __fadd_rn(err, e));
+  uint64_t s = 0, c = 0;
+  __device__ __forceinline__ void add_sq(uint64_t x) {
+    const uint64_t p = mul2(x, x);
+    const uint64_t e = fma2(x, x, mul2(p, kMinus1x2));   // x^2 - p exactly
+    const uint64_t t = add2(s, p);
+    const uint64_t bp = sub2(t, s);
+    const uint64_t err = add2(sub2(s, sub2(t, bp)), sub2(p, bp));   // s + p - t
+    c = add2(c, add2(err, e));
     s = t;
   }
-  __device__ __forceinline__ double value() const { return (double)s + (double)c; }
+  // both halves as one sum and its error
+  __device__ __forceinline__ void fold(float& hi, float& lo) const {
+    float s0, s1, c0, c1;
+    upk2(s, s0, s1);
+    upk2(c, c0, c1);
+    float err;
+    hi = two_sum(s0, s1, err);
+    lo = __fadd_rn(__fadd_rn(c0, c1), err);
+  }
 };
+
+// 16-bit planes of two values, packed (the first in the low half): the values'
+// rounding and the residual's are those of split_bf16 / split_fp16 / split_bf16x3
+__device__ __forceinline__ uint32_t cvt_bf16x2(float a, float b) {
+  uint32_t r;
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(b), "f"(a));
+  return r;
+}
+__device__ __forceinline__ uint32_t cvt_f16x2(float a, float b) {
+  uint32_t r;
+  asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(b), "f"(a));
+  return r;
+}
+__device__ __forceinline__ uint64_t bf16x2_floats(uint32_t h) {
+  return pk2(__uint_as_float(h << 16), __uint_as_float(h & 0xffff0000u));
+}
 
 // plane kinds of the product kernel
 constexpr int KIND_BF16X2 = 0, KIND_FP16X2 = 1, KIND_BF16X3 = 2;
@@ -149,28 +215,35 @@ __device__ __forceinline__ void seg_planes(int seg, int nbase, int& pa, int& pb)
   }
 }
 
+// planes of two consecutive values (scale: FP16X2)
 template <int KIND>
-__device__ __forceinline__ void split_store(uint16_t* hi, uint16_t* mid, uint16_t* lo, int64_t idx,
-                                            float v, float scale) {
-  uint16_t h, l;
+__device__ __forceinline__ void split2(float x0, float x1, float scale, uint32_t& h, uint32_t& m,
+                                       uint32_t& l) {
   if constexpr (KIND == KIND_FP16X2) {
-    split_fp16(v, scale, h, l);
-  } else if constexpr (KIND == KIND_BF16X3) {
-    uint16_t m;
-    split_bf16x3(v, h, m, l);
-    mid[idx] = m;
+    const uint64_t v = mul2(pk2(x0, x1), pk2(scale, scale));
+    float a, b;
+    upk2(v, a, b);
+    h = cvt_f16x2(a, b);
+    const float2 hf = __half22float2(*reinterpret_cast<const __half2*>(&h));
+    const uint64_t r = mul2(sub2(v, pk2(hf.x, hf.y)), pk2(kLoScale, kLoScale));
+    upk2(r, a, b);
+    l = cvt_f16x2(a, b);
+    m = 0;
   } else {
-    split_bf16(v, h, l);
+    float a, b;
+    const uint64_t v = pk2(x0, x1);
+    h = cvt_bf16x2(x0, x1);
+    const uint64_t r1 = sub2(v, bf16x2_floats(h));
+    upk2(r1, a, b);
+    if constexpr (KIND == KIND_BF16X3) {
+      m = cvt_bf16x2(a, b);
+      const uint64_t r2 = sub2(r1, bf16x2_floats(m));
+      upk2(r2, a, b);
+    } else {
+      m = 0;
+    }
+    l = cvt_bf16x2(a, b);
   }
-  hi[idx] = h;
-  lo[idx] = l;
-}
-
-template <int KIND>
-__device__ __forceinline__ void store_split(float* m, uint16_t* hi, uint16_t* mid, uint16_t* lo,
-                                            int64_t idx, float v, float scale) {
-  m[idx] = v;
-  split_store<KIND>(hi, mid, lo, idx, v, scale);
 }
 
 struct KParams {
@@ -226,12 +299,12 @@ struct KMaps {
 template <int KIND, int EPI, int TCOLS>
 __device__ __forceinline__ void tile_end(const KParams& p, float (&acc)[TCOLS], int tix, int pidx,
                                          int it, int e, int lane, int grp, int r, int sg,
-                                         double (*red)[3][EPI_WARPS]) {
+                                         float2 (*red)[3][EPI_WARPS]) {
   constexpr bool F16 = KIND == KIND_FP16X2;
   constexpr bool X3 = KIND == KIND_BF16X3;
   const int64_t np = p.np;
   const Tile t = p.tiles[tix];
-  const int64_t bat = EPI == EPI_SQUARE ? 0 : t.row0 / np;   // batch entry (stacked P)
+  const int64_t bat = EPI == EPI_SQUARE ? 0 : t.row0 / (int)np;   // batch entry (stacked P)
   const int64_t gi = t.row0 + r;                               // stacked row
   const int64_t li = gi - bat * np;                            // row within its matrix
   float inv_s = 1.0f;
@@ -266,108 +339,127 @@ __device__ __forceinline__ void tile_end(const KParams& p, float (&acc)[TCOLS], 
     // with their rounding errors (FP64-equivalent); lanes, warps and tiles add in
     // FP64: Tr, ||.||_F^2 and (EPI_SQUARE) ||X_n - X_n^2||_F^2, whose residual is
     // X_n - X_{n+1} up to its sign in either branch. Tr takes the one diagonal
-    // entry a thread's row segment can hold, as it is.
-    float t1 = 0.0f;
+    // entry a thread's row segment can hold, as it is. Entries above the diagonal
+    // count twice, the diagonal once (on2, onf).
+    float t1 = 0.0f, on2 = 0.0f, onf = 0.0f;
     ExactSqSum t2, f;
+    const int wli = (int)li - lane;   // first row of this warp (within its matrix)
 #pragma unroll
     for (int c0 = 0; c0 < TCOLS; c0 += 16) {
-      const int64_t gj0 = t.col0 + grp * TCOLS + c0;
-      if (gj0 + 15 < li) continue;  // whole group below the diagonal
-      float val[16];
+      const int gj0 = t.col0 + grp * TCOLS + c0;
+      if (gj0 + 15 >= wli) {          // else: the whole group below the warp's rows
+        // the diagonal's column within the group: entries before it enter the sums as
+        // zeros and are not stored (negative: the whole row segment is above)
+        const int dj = (int)li - gj0;
+        float val[16];
+        const float* xp = p.prev + gi * np + gj0;
 #pragma unroll
-      for (int j = 0; j < 16; ++j) val[j] = acc[c0 + j] * inv_s;
-      {
-        float xin[16];
-        if (EPI == EPI_SQUARE || sg < 0) {
-          const float* xp = p.prev + gi * np + gj0;
-          ld256f(xp, xin);
-          ld256f(xp + 8, xin + 8);
-          if (sg < 0) {
+        for (int hf = 0; hf < 16; hf += 8) {
+          float xin[8];
+          if (EPI == EPI_SQUARE || sg < 0) ld256f(xp + hf, xin);
 #pragma unroll
-            for (int j = 0; j < 16; ++j) val[j] = 2.0f * xin[j] - val[j];
+          for (int j = 0; j < 8; ++j) {
+            float v = EPI == EPI_SQUARE ? acc[c0 + hf + j] : acc[c0 + hf + j] * inv_s;
+            if (sg < 0) v = 2.0f * xin[j] - v;
+            val[hf + j] = v;
+          }
+#pragma unroll
+          for (int j = 0; j < 8; j += 2) {
+            const int k = hf + j;
+            t2.add_sq(pk2(k > dj ? val[k] : 0.0f, k + 1 > dj ? val[k + 1] : 0.0f));
+            if constexpr (EPI == EPI_SQUARE) {
+              const float r0 = xin[j] - val[k], r1 = xin[j + 1] - val[k + 1];
+              f.add_sq(pk2(k > dj ? r0 : 0.0f, k + 1 > dj ? r1 : 0.0f));
+              onf = k == dj ? r0 : (k + 1 == dj ? r1 : onf);
+            }
+            on2 = k == dj ? val[k] : (k + 1 == dj ? val[k + 1] : on2);
           }
         }
+        uint32_t wh[8], wl[8], wm[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+          split2<KIND>(val[2 * j], val[2 * j + 1], os, wh[j], wm[j], wl[j]);
+        const int64_t o = gi * np + gj0;          // this row segment
+        if (dj <= 0) {
+          st256f(p.out + o, val);
+          st256f(p.out + o + 8, val + 8);
+          st256(p.out_hi + o, wh);
+          st256(p.out_lo + o, wl);
+          if constexpr (X3) st256(p.out_mid + o, wm);
+        } else {
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            const int sh = 16 * (j & 1);
+            if (j >= dj) {
+              p.out[o + j] = val[j];
+              p.out_hi[o + j] = (uint16_t)(wh[j >> 1] >> sh);
+              p.out_lo[o + j] = (uint16_t)(wl[j >> 1] >> sh);
+              if constexpr (X3) p.out_mid[o + j] = (uint16_t)(wm[j >> 1] >> sh);
+            }
+          }
+        }
+        // its mirror, down a column
+        int64_t om = mbase + (int64_t)gj0 * np + li;
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
-          const int64_t gj = gj0 + j;
-          if (gj < li) continue;
-          const float d = val[j], w2 = gj == li ? 1.0f : 2.0f;
-          if (gj == li) t1 += d;
-          t2.add_sq(w2, d);
-          if constexpr (EPI == EPI_SQUARE) f.add_sq(w2, xin[j] - d);
-        }
-      }
-      uint32_t wh[8], wl[8], wm[8];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        uint16_t h0, h1, l0, l1, m0 = 0, m1 = 0;
-        if constexpr (X3) {
-          split_bf16x3(val[2 * j], h0, m0, l0);
-          split_bf16x3(val[2 * j + 1], h1, m1, l1);
-        } else if constexpr (F16) {
-          split_fp16(val[2 * j], os, h0, l0);
-          split_fp16(val[2 * j + 1], os, h1, l1);
-        } else {
-          split_bf16(val[2 * j], h0, l0);
-          split_bf16(val[2 * j + 1], h1, l1);
-        }
-        wh[j] = (uint32_t)h0 | ((uint32_t)h1 << 16);
-        wl[j] = (uint32_t)l0 | ((uint32_t)l1 << 16);
-        wm[j] = (uint32_t)m0 | ((uint32_t)m1 << 16);
-      }
-      if (gj0 >= li) {
-        const int64_t o = gi * np + gj0;
-        st256f(p.out + o, val);
-        st256f(p.out + o + 8, val + 8);
-        st256(p.out_hi + o, wh);
-        st256(p.out_lo + o, wl);
-        if constexpr (X3) st256(p.out_mid + o, wm);
-      } else {
-#pragma unroll
-        for (int j = 0; j < 16; ++j)
-          if (gj0 + j >= li) {
-            const int64_t o = gi * np + gj0 + j;
-            const int sh = 16 * (j & 1);
-            p.out[o] = val[j];
-            p.out_hi[o] = (uint16_t)(wh[j >> 1] >> sh);
-            p.out_lo[o] = (uint16_t)(wl[j >> 1] >> sh);
-            if constexpr (X3) p.out_mid[o] = (uint16_t)(wm[j >> 1] >> sh);
+          const int sh = 16 * (j & 1);
+          if (j > dj) {
+            p.out[om] = val[j];
+            p.out_hi[om] = (uint16_t)(wh[j >> 1] >> sh);
+            p.out_lo[om] = (uint16_t)(wl[j >> 1] >> sh);
+            if constexpr (X3) p.out_mid[om] = (uint16_t)(wm[j >> 1] >> sh);
           }
-      }
-#pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        const int64_t gj = gj0 + j;
-        if (gj <= li) continue;
-        const int64_t o = mbase + gj * np + li;
-        const int sh = 16 * (j & 1);
-        p.out[o] = val[j];
-        p.out_hi[o] = (uint16_t)(wh[j >> 1] >> sh);
-        p.out_lo[o] = (uint16_t)(wl[j >> 1] >> sh);
-        if constexpr (X3) p.out_mid[o] = (uint16_t)(wm[j >> 1] >> sh);
+          om += np;
+        }
       }
     }
-    double d1 = t1, d2 = t2.value(), d3 = f.value();
-    for (int o = 16; o > 0; o >>= 1) {
-      d1 += __shfl_xor_sync(0xffffffffu, d1, o);
-      d2 += __shfl_xor_sync(0xffffffffu, d2, o);
-      d3 += __shfl_xor_sync(0xffffffffu, d3, o);
-    }
+    t1 = on2;
+    // This thread's sums as FP32 pairs (hi + lo), entries above the diagonal twice and
+    // the diagonal's square, exactly, beside them. The warp adds pairs (one exchange
+    // puts ||.||_F^2 into its lower half and f into its upper), and only the tile's sums
+    // over warps are FP64: an FP64 instruction of a warp takes 64 clocks, and the
+    // shuffled additions of 16 warps took a third of a narrow tile's end. A pair keeps
+    // about 2^-46 of its value, as the threads' sums do.
+    float h2, l2, h3, l3;
+    t2.fold(h2, l2);
+    f.fold(h3, l3);
+    h2 *= 2.0f, l2 *= 2.0f, h3 *= 2.0f, l3 *= 2.0f;
+    const bool diag = t.col0 + grp * TCOLS <= wli + 31;   // may hold diagonal entries
+    const bool up = lane >= 16;
     const int pb = it & 1;
-    if (lane == 0) {
-      red[pb][0][e] = d1;
-      red[pb][1][e] = d2;
-      red[pb][2][e] = d3;
+    if (diag) {
+      const float p2 = __fmul_rn(on2, on2), pf = __fmul_rn(onf, onf);
+      float err, l1 = 0.0f;
+      h2 = two_sum(h2, p2, err);
+      l2 = __fadd_rn(l2, __fadd_rn(err, fmaf(on2, on2, -p2)));
+      h3 = two_sum(h3, pf, err);
+      l3 = __fadd_rn(l3, __fadd_rn(err, fmaf(onf, onf, -pf)));
+      pair_sum<16>(t1, l1);
+      if (lane == 0) red[pb][0][e] = make_float2(t1, l1);
+    } else if (lane == 0) {
+      red[pb][0][e] = make_float2(0.0f, 0.0f);
     }
-    // epilogue warps only (named barrier 1): one thread writes the tile's partials
+    {
+      const float gh = __shfl_xor_sync(0xffffffffu, up ? h2 : h3, 16);
+      const float gl = __shfl_xor_sync(0xffffffffu, up ? l2 : l3, 16);
+      float err, h = two_sum(up ? h3 : h2, gh, err);
+      float l = __fadd_rn(__fadd_rn(up ? l3 : l2, gl), err);
+      pair_sum<8>(h, l);
+      if ((lane & 15) == 0) red[pb][up ? 2 : 1][e] = make_float2(h, l);
+    }
+    // epilogue warps only (named barrier 1): one warp adds the tile's partials in FP64
     asm volatile("bar.sync 1, %0;" ::"r"(EPI_THREADS) : "memory");
-    if (e == 0 && lane == 0) {
-      double s1 = 0.0, s2 = 0.0, s3 = 0.0;
-      for (int w = 0; w < EPI_WARPS; ++w) {
-        s1 += red[pb][0][w];
-        s2 += red[pb][1][w];
-        s3 += red[pb][2][w];
+    if (e == 0) {
+      const float2 v = red[pb][up ? 2 : 1][lane & 15];
+      double s = (double)v.x + (double)v.y, s1 = 0.0;
+      for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if (t.col0 < (int)(t.row0 - bat * np) + 2 * BM) {   // the tile meets the diagonal
+        const float2 w = red[pb][0][lane & 15];
+        s1 = (double)w.x + (double)w.y;
+        for (int o = 8; o > 0; o >>= 1) s1 += __shfl_xor_sync(0xffffffffu, s1, o);
       }
-      p.part[pidx] = Part3{s1, s2, s3};
+      const double s3 = __shfl_sync(0xffffffffu, s, 16);
+      if (lane == 0) p.part[pidx] = Part3{s1, s, s3};
     }
   }
 }
@@ -420,7 +512,7 @@ k_gemm_tc(const __grid_constant__ KMaps maps, const __grid_constant__ KParams p)
   uint64_t* tempty = tfull + 2;       // [2] TMEM buffer b drained by the epilogue warps
   uint64_t* mdone = tempty + 2;       // abort path: the MMA issuer's last operations done
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mdone + 1);
-  __shared__ double red[2][3][EPI_WARPS];   // per-tile partials, double-buffered by tile parity
+  __shared__ float2 red[2][3][EPI_WARPS];   // per-tile partials (FP32 pairs), double-buffered by tile parity
 
   // (uniform over the warp, also to the compiler)
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
@@ -493,8 +585,9 @@ k_gemm_tc(const __grid_constant__ KMaps maps, const __grid_constant__ KParams p)
   const uint32_t tmem = *tmem_slot;
 
   if (warp == 0) {
+    // copy issuer: the whole warp (the waits by every lane, the copies by an elected one)
+    const uint32_t ring = smem_u32(smem);
     if constexpr (SPARSE) {
-     if (lane == 0) {
       // block-sparse square: every segment walks the tile's listed K blocks
       int64_t g = 0;
       RingPos<STAGES> rp;
@@ -510,16 +603,13 @@ k_gemm_tc(const __grid_constant__ KMaps maps, const __grid_constant__ KParams p)
           for (int u = 0; u < 4 * kc; ++u, ++g, rp.next()) {
             const int s = rp.s;
             const uint32_t ph = rp.ph;
-            if (!mbar_wait<PAIR>(&empty[s], ph ^ 1u, abortf, p.wait_ns)) {
-              ok = false;
-              break;
-            }
+            ok = __all_sync(0xffffffffu, mbar_wait<PAIR>(&empty[s], ph ^ 1u, abortf, p.wait_ns));
+            if (!ok) break;
             if (p.withhold && blockIdx.x == 0 && g == 0) continue;  // test hook: never completes
             const int kx = (int)kl[u >> 2] * (4 * BK) + (u & 3) * BK;
-            uint8_t* sa = smem + s * STAGE_BYTES;
-            mbar_arrive_expect_tx(&full[s], STAGE_BYTES);
-            tma_load_2d(&maps.pa[pa], &full[s], sa, kx, t.row0 + (int)rank * BM);
-            tma_load_2d(&maps.qb[pb], &full[s], sa + A_BYTES, kx, t.col0 + (int)rank * R::B_ROWS);
+            const uint32_t sa = ring + (uint32_t)(s * STAGE_BYTES);
+            tma_load_stage(&full[s], STAGE_BYTES, &maps.pa[pa], &maps.qb[pb], sa, sa + A_BYTES, kx,
+                           t.row0 + (int)rank * BM, t.col0 + (int)rank * R::B_ROWS);
           }
         }
       }
@@ -530,8 +620,7 @@ k_gemm_tc(const __grid_constant__ KMaps maps, const __grid_constant__ KParams p)
           mbar_wait_drain(&full[q % STAGES], (uint32_t)(q / STAGES) & 1u, DRAIN_NS);
         }
       }
-     }
-    } else if (lane == 0) {
+    } else {
       const int64_t np = p.np;
       const int nkb = p.nkb;
       // k-block counter g runs on across tiles: stage g % STAGES, phase (g / STAGES) & 1
@@ -554,15 +643,11 @@ k_gemm_tc(const __grid_constant__ KMaps maps, const __grid_constant__ KParams p)
           const int brow = (swap ? bat * (int)np + t.col0 : t.col0) + (int)rank * R::B_ROWS;
           for (int kx = 0; kx < nkb * BK; kx += BK, ++g, rp.next()) {
             const int s = rp.s;
-            if (!mbar_wait<PAIR>(&empty[s], rp.ph ^ 1u, abortf, p.wait_ns)) {
-              ok = false;
-              break;
-            }
+            ok = __all_sync(0xffffffffu, mbar_wait<PAIR>(&empty[s], rp.ph ^ 1u, abortf, p.wait_ns));
+            if (!ok) break;
             if (p.withhold && blockIdx.x == 0 && g == 0) continue;  // test hook: never completes
-            uint8_t* sa = smem + s * STAGE_BYTES;
-            mbar_arrive_expect_tx(&full[s], STAGE_BYTES);
-            tma_load_2d(ma, &full[s], sa, kx, arow);
-            tma_load_2d(mb, &full[s], sa + A_BYTES, kx, brow);
+            const uint32_t sa = ring + (uint32_t)(s * STAGE_BYTES);
+            tma_load_stage(&full[s], STAGE_BYTES, ma, mb, sa, sa + A_BYTES, kx, arow, brow);
           }
         }
       }

@@ -858,16 +858,19 @@ void ring_slot(sp2_handle_t h, int step, DecideParams* dp) {
   dp->token = h->run_id * 1024ull + (unsigned long long)step;
 }
 
-// Wait for the snapshot of `step` and return it. Snapshots are read in step order,
-// none past the one that shows a stop (a stopped recursion's later decisions may
-// not run). When the stream has drained without it (an aborted product never
-// reached its decision), the state itself is read.
+// Wait for the word of `step`; *out stays null while the recursion goes on, else it is
+// the snapshot of its end. Words are read in step order, none past the end (a
+// stopped recursion's later decisions may not run). When the stream has drained
+// without it (an aborted product never reached its decision), the state itself is
+// read.
 int ring_read(sp2_handle_t h, int step, const HostSnap** out) {
   HostSnap* s = h->ring + step % sp2_handle_s::kRing;
   const unsigned long long token = h->run_id * 1024ull + (unsigned long long)step;
+  *out = nullptr;
   for (unsigned it = 1;; ++it) {
-    if (__atomic_load_n(&s->token, __ATOMIC_ACQUIRE) == token) {
-      *out = s;
+    const unsigned long long w = __atomic_load_n(&s->word, __ATOMIC_ACQUIRE);
+    if (w >> 1 == token) {
+      if (w & 1ull) *out = s;
       return SP2_OK;
     }
     if (it % 16384 != 0) continue;
@@ -878,12 +881,12 @@ int ring_read(sp2_handle_t h, int step, const HostSnap** out) {
       continue;
     }
     CK(e);
-    if (__atomic_load_n(&s->token, __ATOMIC_ACQUIRE) == token) continue;
+    if (__atomic_load_n(&s->word, __ATOMIC_ACQUIRE) >> 1 == token) continue;
     CK(cudaMemcpyAsync(h->h_state, h->d_state, sizeof(DevState), cudaMemcpyDeviceToHost, h->stream));
     CK(cudaStreamSynchronize(h->stream));
     const DevState& d = *h->h_state;
-    h->late = HostSnap{token, d.stop_at, d.nonfinite, d.abort_flag, d.backtracked, d.stop_step, 0,
-                       {d.bounds[0], d.bounds[1]}, d.alpha, d.beta, d.work_kblocks};
+    h->late = HostSnap{2ull * token + 1ull, d.stop_at, d.nonfinite, d.abort_flag, d.backtracked,
+                       d.stop_step, 0, {d.bounds[0], d.bounds[1]}, d.alpha, d.beta, d.work_kblocks};
     *out = &h->late;
     return SP2_OK;
   }
@@ -1015,8 +1018,8 @@ int run_sp2(sp2_handle_t h, const void* Hd, int64_t n, int dtype, double nocc, c
     TRY(ws(h, "decide.done", sizeof(unsigned), &dn));
     CK(cudaMemsetAsync(dn, 0, sizeof(unsigned), h->stream));
   }
-  const HostSnap* seen = nullptr;   // latest snapshot read
-  int read = 0, last = 0;           // last step whose snapshot was read, last step enqueued
+  const HostSnap* seen = nullptr;   // the snapshot of the recursion's end
+  int read = 0, last = 0;           // last step whose word was read, last step enqueued
   for (int step = 1; step <= maxit; ++step) {
     const MatBuf& xin = X[step % 2];
     const MatBuf& xo = X[(step + 1) % 2];
@@ -1066,11 +1069,11 @@ int run_sp2(sp2_handle_t h, const void* Hd, int64_t n, int dtype, double nocc, c
     last = step;
     if (step > sp2_handle_s::kLookahead) {
       TRY(ring_read(h, ++read, &seen));
-      if (seen->stop_at != 0 || seen->abort_flag) break;
+      if (seen) break;
     }
   }
-  while (read < last && (!seen || (seen->stop_at == 0 && !seen->abort_flag)))
-    TRY(ring_read(h, ++read, &seen));
+  while (!seen && read < last) TRY(ring_read(h, ++read, &seen));
+  if (!seen) return fail(h, SP2_ECUDA, "the recursion's last step reported no end");
   const HostSnap S = *seen;
   out->alpha = S.alpha;
   out->beta = S.beta;

@@ -55,11 +55,12 @@ struct DevState {
   double fold;                   // min f_1..f_{s-kStall} after step s (the stall floor's older part)
 };
 
-// What the host learns of a step: written by the step decision into a slot of a
-// pinned host ring, the token last. A copy of the state on the stream after every
-// step (and an event behind it) cost more than a small step's kernels.
+// What the host learns of a step, in a slot of a pinned host ring written by the step
+// decision. A copy of the state on the stream after every step (and an event behind
+// it) cost more than a small step's kernels.
 struct HostSnap {
-  unsigned long long token;      // call and step the other fields belong to
+  unsigned long long word;       // 2 x token (call and step) + 1 when the recursion ends
+                                 // there and the other fields are valid
   int stop_at, nonfinite, abort_flag, backtracked, stop_step, pad_;
   double bounds[2], alpha, beta, work_kblocks;
 };

@@ -23,12 +23,6 @@ __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
 }
 
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),
-               "r"(bytes)
-               : "memory");
-}
-
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
@@ -119,12 +113,21 @@ __device__ __forceinline__ void mbar_arrive_cluster_release(uint32_t cluster_bar
                : "memory");
 }
 
-__device__ __forceinline__ void tma_load_2d(const CUtensorMap* map, uint64_t* bar, void* dst,
-                                            int x, int y) {
+// One ring stage by the copy issuer's elected lane (whole warp in uniform control
+// flow, as the MMA issuer): arm the stage's barrier with its bytes, then load the
+// left and the right factor's boxes at column x.
+__device__ __forceinline__ void tma_load_stage(uint64_t* bar, uint32_t bytes, const CUtensorMap* ma,
+                                               const CUtensorMap* mb, uint32_t dst_a,
+                                               uint32_t dst_b, int x, int ya, int yb) {
   asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%3, %4}], [%2];" ::"r"(smem_u32(dst)),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar)), "r"(x), "r"(y)
+      "{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
+      "@e mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n\t"
+      "@e cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes"
+      " [%2], [%4, {%6, %7}], [%0];\n\t"
+      "@e cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes"
+      " [%3], [%5, {%6, %8}], [%0];\n\t}" ::"r"(smem_u32(bar)),
+      "r"(bytes), "r"(dst_a), "r"(dst_b), "l"(reinterpret_cast<uint64_t>(ma)),
+      "l"(reinterpret_cast<uint64_t>(mb)), "r"(x), "r"(ya), "r"(yb)
       : "memory");
 }
 
