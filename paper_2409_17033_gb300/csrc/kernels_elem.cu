@@ -633,81 +633,138 @@ __global__ void k_fro_final(const double* part, int nparts, float* scale_out) {
 // ------------------------------------------------------------ contraction
 // out[l,k] = sum_ij P_l[i,j] Q_k[i,j] (Eqs. expectation, direct, dual), FP64
 // accumulation, per-block partials then a fixed-order second pass.
-template <typename T>
-__global__ void k_contract_dense(const T* __restrict__ P, const T* __restrict__ Q, int64_t K,
-                                 int64_t nn, double* part, int nparts, int64_t y0) {
-  const int64_t pair = y0 + blockIdx.y;
-  const int64_t l = pair / K, k = pair % K;
-  const T* p = P + l * nn;
-  const T* q = Q + k * nn;
-  double acc = 0.0;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < nn;
-       t += (int64_t)gridDim.x * blockDim.x)
-    acc += (double)p[t] * (double)q[t];
-  acc = block_sum(acc);
-  if (threadIdx.x == 0) part[pair * nparts + blockIdx.x] = acc;
-}
-
 // FP32 inputs: exact products and sums at FP32 cost. TwoProduct splits a*b into
 // p + e exactly (e = fma(a, b, -p)); TwoSum adds p to the running pair (s, c)
 // without loss; the small terms e and c are summed in FP32, their rounding far
 // below 2^-40 of the magnitudes involved. Each thread converts once to FP64 at
-// the end. A block covers one slice of the N^2 entries for up to kCtrKT
-// perturbations Q_k, so the shared left factor P_l is read once per kCtrKT.
+// the end. FP64 inputs: fma.
+//
+// A block covers one slice of the N^2 entries for up to LT factors P_l and kCtrKT
+// perturbations Q_k, so that every Q_k is read once per LT rows of P and every P_l
+// once per kCtrKT: with one P_l per block (LT = 1) four observables read 17 GB for 64
+// perturbations at N = 4096 where the inputs are 4.6 GB. With LT = 4 the FP32 form is
+// bound by its ten operations per pair and entry.
 constexpr int kCtrKT = 8;
 
 // (the _rn intrinsics are never contracted into FMAs, which would break both
 // error-free transformations)
-__device__ __forceinline__ void acc_exact(float& s, float& c, float a, float b) {
-  const float p = __fmul_rn(a, b);
-  const float e = fmaf(a, b, -p);
-  const float t = __fadd_rn(s, p);
-  const float bp = __fsub_rn(t, s);
-  const float err = __fadd_rn(__fsub_rn(s, __fsub_rn(t, bp)), __fsub_rn(p, bp));
-  c = __fadd_rn(c, __fadd_rn(err, e));
-  s = t;
+struct AccF32 {
+  float s = 0.0f, c = 0.0f;
+  __device__ __forceinline__ void add(float a, float b) {
+    const float p = __fmul_rn(a, b);
+    const float e = fmaf(a, b, -p);
+    const float t = __fadd_rn(s, p);
+    const float bp = __fsub_rn(t, s);
+    const float err = __fadd_rn(__fsub_rn(s, __fsub_rn(t, bp)), __fsub_rn(p, bp));
+    c = __fadd_rn(c, __fadd_rn(err, e));
+    s = t;
+  }
+  __device__ __forceinline__ double value() const { return to_f64(s) + to_f64(c); }
+  // the conversion by integer operations (the FP64 pipe takes 64 clocks for a warp's)
+  static __device__ __forceinline__ double to_f64(float x) {
+    const uint32_t u = __float_as_uint(x), e = (u >> 23) & 0xffu;
+    if (e == 0u || e == 0xffu) return (double)x;
+    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (896u << 20))),
+                            (int)(u << 29));
+  }
+};
+struct AccF64 {
+  double s = 0.0;
+  __device__ __forceinline__ void add(double a, double b) { s = fma(a, b, s); }
+  __device__ __forceinline__ double value() const { return s; }
+};
+template <typename T> struct CtrAcc;
+template <> struct CtrAcc<float> { using type = AccF32; };
+template <> struct CtrAcc<double> { using type = AccF64; };
+
+template <typename T, int VEC> struct CtrVec { T v[VEC]; };
+template <int VEC>
+__device__ __forceinline__ CtrVec<float, VEC> ctr_load(const float* p, int64_t t, bool stream) {
+  CtrVec<float, VEC> r;
+  if constexpr (VEC == 4) {
+    const float4* q = reinterpret_cast<const float4*>(p) + t;
+    const float4 x = stream ? __ldcs(q) : __ldg(q);
+    r.v[0] = x.x, r.v[1] = x.y, r.v[2] = x.z, r.v[3] = x.w;
+  } else {
+    r.v[0] = p[t];
+  }
+  return r;
+}
+template <int VEC>
+__device__ __forceinline__ CtrVec<double, VEC> ctr_load(const double* p, int64_t t, bool stream) {
+  CtrVec<double, VEC> r;
+  if constexpr (VEC == 2) {
+    const double2* q = reinterpret_cast<const double2*>(p) + t;
+    const double2 x = stream ? __ldcs(q) : __ldg(q);
+    r.v[0] = x.x, r.v[1] = x.y;
+  } else {
+    r.v[0] = p[t];
+  }
+  return r;
 }
 
-template <int VEC>
-__global__ void __launch_bounds__(256) k_contract_dense_f32(const float* __restrict__ P,
-                                                           const float* __restrict__ Q, int64_t K,
-                                                           int64_t nn, double* part, int nparts,
-                                                           int64_t y0) {
+// Sums of N values (a power of two up to 32) over a warp: each exchange halves the
+// values a lane still holds, so that N sums cost N - 1 additions and the remaining
+// rounds instead of 5 N. Value i ends in the lanes whose upper bits are i.
+template <int N>
+__device__ __forceinline__ double warp_sums(double (&v)[N], int lane) {
+  int o = 16;
+#pragma unroll
+  for (int n = N; n > 1; n >>= 1, o >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int i = 0; i < n / 2; ++i) {
+      const double send = up ? v[i] : v[i + n / 2], keep = up ? v[i + n / 2] : v[i];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+  for (; o > 0; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+  return v[0];
+}
+
+template <typename T, int VEC, int LT>
+__global__ void __launch_bounds__(256, 2)
+k_contract_dense(const T* __restrict__ P, int64_t L, const T* __restrict__ Q, int64_t K, int64_t nn,
+                 double* part, int nparts, int64_t y0) {
+  using Acc = typename CtrAcc<T>::type;
+  constexpr int NP = LT * kCtrKT;
   const int64_t ktiles = (K + kCtrKT - 1) / kCtrKT;
   const int64_t y = y0 + blockIdx.y;
-  const int64_t l = y / ktiles, k0 = (y % ktiles) * kCtrKT;
+  const int64_t l0 = (y / ktiles) * LT, k0 = (y % ktiles) * kCtrKT;
   const int kn = (int)((K - k0) < kCtrKT ? (K - k0) : kCtrKT);
-  const float* p = P + l * nn;
-  float s[kCtrKT], c[kCtrKT];
-#pragma unroll
-  for (int kk = 0; kk < kCtrKT; ++kk) s[kk] = c[kk] = 0.0f;
+  const int ln = (int)((L - l0) < LT ? (L - l0) : LT);
+  const T* p = P + l0 * nn;
+  Acc acc[LT][kCtrKT];
   const int64_t nv = nn / VEC;
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < nv;
        t += (int64_t)gridDim.x * blockDim.x) {
-    if constexpr (VEC == 4) {
-      const float4 a = __ldg(reinterpret_cast<const float4*>(p) + t);
+    CtrVec<T, VEC> a[LT];
 #pragma unroll
-      for (int kk = 0; kk < kCtrKT; ++kk) {
-        if (kk < kn) {
-          const float4 b = __ldcs(reinterpret_cast<const float4*>(Q + (k0 + kk) * nn) + t);
-          acc_exact(s[kk], c[kk], a.x, b.x);
-          acc_exact(s[kk], c[kk], a.y, b.y);
-          acc_exact(s[kk], c[kk], a.z, b.z);
-          acc_exact(s[kk], c[kk], a.w, b.w);
-        }
-      }
-    } else {
-      const float a = p[t];
+    for (int l = 0; l < LT; ++l) a[l] = ctr_load<VEC>(p + (l < ln ? l : 0) * nn, t, false);
 #pragma unroll
-      for (int kk = 0; kk < kCtrKT; ++kk)
-        if (kk < kn) acc_exact(s[kk], c[kk], a, Q[(k0 + kk) * nn + t]);
+    for (int k = 0; k < kCtrKT; ++k) {
+      if (k >= kn) break;
+      const CtrVec<T, VEC> b = ctr_load<VEC>(Q + (k0 + k) * nn, t, true);
+#pragma unroll
+      for (int l = 0; l < LT; ++l)
+#pragma unroll
+        for (int j = 0; j < VEC; ++j) acc[l][k].add(a[l].v[j], b.v[j]);
     }
   }
+  __shared__ double red[8][NP];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  double v[NP];
 #pragma unroll
-  for (int kk = 0; kk < kCtrKT; ++kk) {
-    if (kk >= kn) break;   // uniform across the block
-    const double v = block_sum((double)s[kk] + (double)c[kk]);
-    if (threadIdx.x == 0) part[(l * K + k0 + kk) * nparts + blockIdx.x] = v;
+  for (int i = 0; i < NP; ++i) v[i] = acc[i / kCtrKT][i % kCtrKT].value();
+  const double s = warp_sums<NP>(v, lane);
+  constexpr int STEP = 32 / NP;   // lanes per value
+  if (lane % STEP == 0) red[warp][lane / STEP] = s;
+  __syncthreads();
+  if (threadIdx.x < NP) {
+    const int l = threadIdx.x / kCtrKT, k = threadIdx.x % kCtrKT;
+    double r = 0.0;
+    for (int w = 0; w < 8; ++w) r += red[w][threadIdx.x];
+    if (l < ln && k < kn) part[((l0 + l) * K + k0 + k) * nparts + blockIdx.x] = r;
   }
 }
 
@@ -885,44 +942,58 @@ int contract_nparts(int64_t n, int q_diag) {
   return (int)g;
 }
 
+namespace {
+template <typename T, int VEC, int LT>
+void contract_rows(const void* P, int64_t L, const void* Q, int64_t K, int64_t nn, double* part,
+                   int nparts, int64_t rows, cudaStream_t s) {
+  // grid rows go out in launches of at most 65535, the limit of gridDim.y
+  constexpr int64_t kMaxY = 65535;
+  for (int64_t y0 = 0; y0 < rows; y0 += kMaxY) {
+    const int64_t ny = (rows - y0) < kMaxY ? (rows - y0) : kMaxY;
+    const dim3 grid((unsigned)nparts, (unsigned)ny);
+    k_contract_dense<T, VEC, LT><<<grid, 256, 0, s>>>(static_cast<const T*>(P), L,
+                                                      static_cast<const T*>(Q), K, nn, part,
+                                                      nparts, y0);
+  }
+}
+// one block row per LT rows of P and kCtrKT perturbations; LT = 4 from three rows of P on
+template <typename T, int VEC>
+void contract_dense(const void* P, int64_t L, const void* Q, int64_t K, int64_t nn, double* part,
+                    int nparts, cudaStream_t s) {
+  const int64_t kt = (K + kCtrKT - 1) / kCtrKT;
+  if (L == 1) contract_rows<T, VEC, 1>(P, L, Q, K, nn, part, nparts, kt, s);
+  else if (L == 2) contract_rows<T, VEC, 2>(P, L, Q, K, nn, part, nparts, kt, s);
+  else contract_rows<T, VEC, 4>(P, L, Q, K, nn, part, nparts, (L + 3) / 4 * kt, s);
+}
+}  // namespace
+
 cudaError_t launch_contract(const void* P, int64_t L, const void* Q, int64_t K, int64_t n,
                             int dtype, int q_diag, double* part, int nparts, double* out,
                             cudaStream_t s) {
-  // grid rows (one per pair, or per observable and group of kCtrKT perturbations)
-  // go out in launches of at most 65535, the limit of gridDim.y
-  constexpr int64_t kMaxY = 65535;
   const int64_t nn = n * n;
-  const bool f32_dense = dtype != SP2_F64 && !q_diag;
-  const int64_t ktiles = (K + kCtrKT - 1) / kCtrKT;
-  const int64_t rows = f32_dense ? L * ktiles : L * K;
-  // float4 path when every matrix starts on a 16-byte boundary
-  const bool v4 = nn % 4 == 0 && ((reinterpret_cast<uintptr_t>(P) |
-                                   reinterpret_cast<uintptr_t>(Q)) & 15u) == 0;
-  for (int64_t y0 = 0; y0 < rows; y0 += kMaxY) {
-    const int64_t ny = (rows - y0) < kMaxY ? (rows - y0) : kMaxY;
-    dim3 grid((unsigned)nparts, (unsigned)ny);
-    if (dtype == SP2_F64) {
-      if (q_diag)
+  // 16-byte loads when every matrix starts on a 16-byte boundary
+  const bool al = ((reinterpret_cast<uintptr_t>(P) | reinterpret_cast<uintptr_t>(Q)) & 15u) == 0;
+  if (q_diag) {
+    constexpr int64_t kMaxY = 65535;
+    const int64_t rows = L * K;
+    for (int64_t y0 = 0; y0 < rows; y0 += kMaxY) {
+      const int64_t ny = (rows - y0) < kMaxY ? (rows - y0) : kMaxY;
+      const dim3 grid((unsigned)nparts, (unsigned)ny);
+      if (dtype == SP2_F64)
         k_contract_diag<double><<<grid, 256, 0, s>>>(static_cast<const double*>(P),
                                                      static_cast<const double*>(Q), K, n, part,
                                                      nparts, y0);
       else
-        k_contract_dense<double><<<grid, 256, 0, s>>>(static_cast<const double*>(P),
-                                                      static_cast<const double*>(Q), K, nn, part,
-                                                      nparts, y0);
-    } else if (q_diag) {
-      k_contract_diag<float><<<grid, 256, 0, s>>>(static_cast<const float*>(P),
-                                                  static_cast<const float*>(Q), K, n, part, nparts,
-                                                  y0);
-    } else if (v4) {
-      k_contract_dense_f32<4><<<grid, 256, 0, s>>>(static_cast<const float*>(P),
-                                                   static_cast<const float*>(Q), K, nn, part,
-                                                   nparts, y0);
-    } else {
-      k_contract_dense_f32<1><<<grid, 256, 0, s>>>(static_cast<const float*>(P),
-                                                   static_cast<const float*>(Q), K, nn, part,
-                                                   nparts, y0);
+        k_contract_diag<float><<<grid, 256, 0, s>>>(static_cast<const float*>(P),
+                                                    static_cast<const float*>(Q), K, n, part,
+                                                    nparts, y0);
     }
+  } else if (dtype == SP2_F64) {
+    if (al && nn % 2 == 0) contract_dense<double, 2>(P, L, Q, K, nn, part, nparts, s);
+    else contract_dense<double, 1>(P, L, Q, K, nn, part, nparts, s);
+  } else {
+    if (al && nn % 4 == 0) contract_dense<float, 4>(P, L, Q, K, nn, part, nparts, s);
+    else contract_dense<float, 1>(P, L, Q, K, nn, part, nparts, s);
   }
   k_contract_final<<<(unsigned)(L * K), 256, 0, s>>>(part, nparts, out);
   return cudaGetLastError();
