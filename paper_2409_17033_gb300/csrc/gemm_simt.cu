@@ -1,5 +1,5 @@
 // CUDA-core product kernels for the plain FP64 and FP32 forms of the SP2 path
-// (the "GPU FP32" arithmetic of Sec. VI.C and an FP64 form for 1e-10 parity).
+// (the "GPU FP32" arithmetic of Sec. VI.C and an FP64 form for small matrices).
 //
 // C = A * X with A a stack of row-major (np x np) matrices and X symmetric, so
 // X is read row-major as the B operand. Epilogues:
@@ -21,7 +21,6 @@ __device__ __forceinline__ bool halted_simt(const DevState* st, int step) {
 }
 
 template <typename T> struct Vec;
-template <> struct Vec<float> { using type = float4; static constexpr int n = 4; };
 template <> struct Vec<double> { using type = double2; static constexpr int n = 2; };
 
 template <typename T, int BM, int BN, int BK, int TM, int TN>
@@ -148,31 +147,262 @@ k_gemm_simt(const T* __restrict__ A, const T* __restrict__ X, int64_t np, int ep
   }
 }
 
+// ------------------------------------------------------------ FP32
+// BM x BN tile, 8 x 8 entries per thread (two 4 x 4 halves in each direction, so that
+// shared memory is read 16 bytes at a time), K steps of BK through two shared-memory
+// buffers with the next step's global loads in registers. The products are packed
+// pairs (fma.rn.f32x2: each half rounds as fmaf), the left factor's entries stored
+// twice side by side so that a pair {a, a} is one load: 38 instructions for 64 fused
+// multiply-adds a thread, where 64 scalar ones waited on 16 scalar shared loads.
+// Each entry's terms are added in the order of k, as by the scalar form.
+__device__ __forceinline__ uint64_t ffma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(uint64_t v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+
+// s + c += x exactly up to the rounding of c (Knuth's TwoSum; the _rn forms are never
+// contracted), and the square of r + er
+struct SumF32 {
+  float s = 0.0f, c = 0.0f;
+  __device__ __forceinline__ void add(float x) {
+    const float t = __fadd_rn(s, x), bp = __fsub_rn(t, s);
+    c = __fadd_rn(c, __fadd_rn(__fsub_rn(s, __fsub_rn(t, bp)), __fsub_rn(x, bp)));
+    s = t;
+  }
+  __device__ __forceinline__ void add_sq(float r, float er = 0.0f) {
+    const float p = __fmul_rn(r, r);
+    add(p);
+    c = __fadd_rn(c, fmaf(2.0f * r, er, fmaf(r, r, -p)));
+  }
+  __device__ __forceinline__ double value() const { return (double)s + (double)c; }
+};
+
+template <int BM, int BN, int BK>
+__global__ void __launch_bounds__(BM / 8 * BN / 8, BM * BN == 128 * 128 ? 2 : (BM == 128 ? 3 : 6))
+k_gemm_f32(const float* __restrict__ A, const float* __restrict__ X, int64_t np, int epi,
+           float* __restrict__ out, const float* __restrict__ xprev, Part3* __restrict__ part,
+           const Tile* __restrict__ tiles, const DevState* st, int step, SimtDecide dec) {
+  constexpr int TX = BN / 8, NT = BM / 8 * TX;
+  constexpr int AS = BM + 2;                       // pairs per k row of the left buffer
+  constexpr int A4 = BM * BK / 4 / NT, B4 = BN * BK / 4 / NT;   // 16-byte loads per thread
+  if (halted_simt(st, step)) return;
+  __shared__ __align__(16) float2 As[2][BK][AS];
+  __shared__ __align__(16) float Bs[2][BK][BN];
+  const Tile t = tiles[blockIdx.x];
+  const int tid = threadIdx.x, tx = tid % TX, ty = tid / TX;
+  const float* ap = A + (int64_t)t.row0 * np;
+  const float* bp = X + t.col0;
+  float4 ra[A4], rb[B4];
+  auto load = [&](int64_t k0) {
+#pragma unroll
+    for (int i = 0; i < A4; ++i) {
+      const int e = tid + i * NT;
+      ra[i] = *reinterpret_cast<const float4*>(ap + (int64_t)(e / (BK / 4)) * np + k0 +
+                                               (e % (BK / 4)) * 4);
+    }
+#pragma unroll
+    for (int i = 0; i < B4; ++i) {
+      const int e = tid + i * NT;
+      rb[i] = *reinterpret_cast<const float4*>(bp + (k0 + e / (BN / 4)) * np + (e % (BN / 4)) * 4);
+    }
+  };
+  auto store = [&](int b) {
+#pragma unroll
+    for (int i = 0; i < A4; ++i) {
+      const int e = tid + i * NT, r = e / (BK / 4), k = (e % (BK / 4)) * 4;
+      As[b][k + 0][r] = make_float2(ra[i].x, ra[i].x);
+      As[b][k + 1][r] = make_float2(ra[i].y, ra[i].y);
+      As[b][k + 2][r] = make_float2(ra[i].z, ra[i].z);
+      As[b][k + 3][r] = make_float2(ra[i].w, ra[i].w);
+    }
+#pragma unroll
+    for (int i = 0; i < B4; ++i) {
+      const int e = tid + i * NT;
+      *reinterpret_cast<float4*>(&Bs[b][e / (BN / 4)][(e % (BN / 4)) * 4]) = rb[i];
+    }
+  };
+  uint64_t acc[8][4];
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
+  load(0);
+  store(0);
+  __syncthreads();
+  int buf = 0;
+  for (int64_t k0 = 0; k0 < np; k0 += BK, buf ^= 1) {
+    const bool more = k0 + BK < np;
+    if (more) load(k0 + BK);
+#pragma unroll
+    for (int kk = 0; kk < BK; ++kk) {
+      uint64_t a[8], b[4];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const ulonglong2* pa =
+            reinterpret_cast<const ulonglong2*>(&As[buf][kk][h * (BM / 2) + ty * 4]);
+        const ulonglong2 a0 = pa[0], a1 = pa[1];
+        a[4 * h] = a0.x, a[4 * h + 1] = a0.y, a[4 * h + 2] = a1.x, a[4 * h + 3] = a1.y;
+        const ulonglong2 bv =
+            *reinterpret_cast<const ulonglong2*>(&Bs[buf][kk][h * (BN / 2) + tx * 4]);
+        b[2 * h] = bv.x, b[2 * h + 1] = bv.y;
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = ffma2(a[i], b[j], acc[i][j]);
+    }
+    if (more) store(buf ^ 1);   // (its readers passed the barrier of the step before)
+    __syncthreads();
+  }
+  // entry (i, j) of this thread: row (i / 4) BM/2 + ty 4 + i % 4, columns likewise
+  const int64_t r0 = t.row0 + ty * 4, c0 = t.col0 + tx * 4;
+  if (epi == EPI_PLAIN) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const float2 u = unpack2(acc[i][2 * h]), v = unpack2(acc[i][2 * h + 1]);
+        *reinterpret_cast<float4*>(out + (r0 + (i >> 2) * (BM / 2) + (i & 3)) * np + c0 +
+                                   h * (BN / 2)) = make_float4(u.x, u.y, v.x, v.y);
+      }
+    return;
+  }
+  const int sg = st->sigma[step];
+  // sums of this thread's entries in FP32 with their rounding errors (FP64
+  // instructions on all 64 entries took 34 us of a tile): entries above the diagonal
+  // (counted twice) and on it
+  SumF32 t1, t2, f, e2, ef;
+#pragma unroll
+  for (int ih = 0; ih < 2; ++ih)
+#pragma unroll
+    for (int jh = 0; jh < 2; ++jh) {
+      const int64_t gi0 = r0 + ih * (BM / 2), gj0 = c0 + jh * (BN / 2);
+      if (gi0 > gj0 + 3) continue;   // the 4 x 4 block lies below the diagonal
+      const bool above = gi0 + 3 < gj0;
+      float v[4][4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float2 u0 = unpack2(acc[4 * ih + i][2 * jh]), u1 = unpack2(acc[4 * ih + i][2 * jh + 1]);
+        const float c[4] = {u0.x, u0.y, u1.x, u1.y};
+        const float4 xv = *reinterpret_cast<const float4*>(xprev + (gi0 + i) * np + gj0);
+        const float x[4] = {xv.x, xv.y, xv.z, xv.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          v[i][j] = sg > 0 ? c[j] : 2.0f * x[j] - c[j];
+          // x - c = r + er exactly
+          const float r = __fsub_rn(x[j], c[j]), bb = __fsub_rn(r, x[j]);
+          const float er = __fsub_rn(__fsub_rn(x[j], __fsub_rn(r, bb)), __fadd_rn(c[j], bb));
+          if (gi0 + i < gj0 + j) {
+            t2.add_sq(v[i][j]);
+            f.add_sq(r, er);
+          } else if (gi0 + i == gj0 + j) {
+            t1.add(v[i][j]);
+            e2.add_sq(v[i][j]);
+            ef.add_sq(r, er);
+          }
+        }
+      }
+      if (above) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          *reinterpret_cast<float4*>(out + (gi0 + i) * np + gj0) =
+              make_float4(v[i][0], v[i][1], v[i][2], v[i][3]);
+          *reinterpret_cast<float4*>(out + (gj0 + i) * np + gi0) =
+              make_float4(v[0][i], v[1][i], v[2][i], v[3][i]);
+        }
+      } else {
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            if (gi0 + i > gj0 + j) continue;
+            out[(gi0 + i) * np + gj0 + j] = v[i][j];
+            if (gi0 + i < gj0 + j) out[(gj0 + j) * np + gi0 + i] = v[i][j];
+          }
+      }
+    }
+  double d1 = t1.value(), d2 = 2.0 * t2.value() + e2.value(), d3 = 2.0 * f.value() + ef.value();
+  constexpr int NW = NT / 32;
+  __shared__ double red[3][NW];
+  for (int o = 16; o > 0; o >>= 1) {
+    d1 += __shfl_xor_sync(0xffffffffu, d1, o);
+    d2 += __shfl_xor_sync(0xffffffffu, d2, o);
+    d3 += __shfl_xor_sync(0xffffffffu, d3, o);
+  }
+  if ((tid & 31) == 0) red[0][tid >> 5] = d1, red[1][tid >> 5] = d2, red[2][tid >> 5] = d3;
+  __syncthreads();
+  if (tid == 0) {
+    double s1 = 0.0, s2 = 0.0, s3 = 0.0;
+    for (int w = 0; w < NW; ++w) s1 += red[0][w], s2 += red[1][w], s3 += red[2][w];
+    part[blockIdx.x] = Part3{s1, s2, s3};
+  }
+  if (dec.done) {
+    __shared__ int last;
+    if (tid == 0) {
+      __threadfence();
+      last = atomicAdd(dec.done, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (last) {
+      __threadfence();
+      decide_block(part, dec.st, dec.p);
+      if (tid == 0) *dec.done = 0u;
+    }
+  }
+}
+
+// Tile of an FP32 product: the least work of the busiest SM, a tile's work weighed by
+// how well the SM's resident warps hide latency (eight or more: fully).
+void f32_tile(int64_t rows, int64_t np, bool upper, int* bm, int* bn) {
+  constexpr int kShapes[3][2] = {{128, 128}, {128, 64}, {64, 64}};
+  double best = 0.0;
+  for (const auto& s : kShapes) {
+    const int64_t m = rows / s[0], n = np / s[1];
+    int64_t nt = m * n;
+    if (upper) {
+      nt = 0;
+      for (int64_t i = 0; i < m; ++i) nt += (np - i * s[0]) / s[1];
+    }
+    const int64_t per = (nt + 151) / 152;
+    const int warps = s[0] * s[1] / 64 / 32;
+    const double w = (double)(per * warps < 8 ? per * warps : 8);
+    const double c = (double)per * s[0] * s[1] / (0.55 + 0.45 * w / 8.0);
+    if (best == 0.0 || c < 0.97 * best) {
+      best = c;
+      *bm = s[0];
+      *bn = s[1];
+    }
+  }
+}
+
 }  // namespace
 
 // FP64 runs at a small fraction of the FP32 rate on GB300, so an FP64 product
 // takes as long as its busiest SM: up to np = 1024 it uses 16 x 16 tiles (136
 // upper tiles at np = 256, where 64 x 64 tiles would keep 10 SMs busy and leave
 // the rest idle), above that 64 x 64.
-void simt_tile_shape(int mode, int64_t np, int* bm, int* bn) {
+void simt_tile_shape(int mode, int64_t rows, int64_t np, bool upper, int* bm, int* bn) {
   if (mode == SP2_MODE_FP64) {
     const int t = np <= 1024 ? 16 : 64;
     *bm = t;
     *bn = t;
   } else {
-    *bm = 128;
-    *bn = 128;
+    f32_tile(rows, np, upper, bm, bn);
   }
 }
 
 cudaError_t launch_gemm_simt(int mode, int epi, const void* A, int64_t a_rows, const void* X,
                              int64_t np, void* out, const void* x_prev, Part3* part,
-                             const Tile* tiles, int ntiles, const DevState* st, int step,
-                             cudaStream_t s, const SimtDecide* dec) {
+                             const Tile* tiles, int ntiles, int bm, int bn, const DevState* st,
+                             int step, cudaStream_t s, const SimtDecide* dec) {
   (void)a_rows;
   if (ntiles <= 0) return cudaSuccess;
-  int bm, bn;
-  simt_tile_shape(mode, np, &bm, &bn);
   SimtDecide sd;
   if (dec && epi == EPI_SQUARE) sd = *dec;
   if (mode == SP2_MODE_FP64 && bm == 16) {
@@ -184,9 +414,15 @@ cudaError_t launch_gemm_simt(int mode, int epi, const void* A, int64_t a_rows, c
         static_cast<const double*>(A), static_cast<const double*>(X), np, epi,
         static_cast<double*>(out), static_cast<const double*>(x_prev), part, tiles, st, step, sd);
   } else {
-    k_gemm_simt<float, 128, 128, 8, 8, 8><<<ntiles, 256, 0, s>>>(
-        static_cast<const float*>(A), static_cast<const float*>(X), np, epi,
-        static_cast<float*>(out), static_cast<const float*>(x_prev), part, tiles, st, step, sd);
+    const float *a = static_cast<const float*>(A), *x = static_cast<const float*>(X);
+    const float* xp = static_cast<const float*>(x_prev);
+    float* o = static_cast<float*>(out);
+    if (bm == 128 && bn == 128)
+      k_gemm_f32<128, 128, 8><<<ntiles, 256, 0, s>>>(a, x, np, epi, o, xp, part, tiles, st, step, sd);
+    else if (bm == 128)
+      k_gemm_f32<128, 64, 16><<<ntiles, 128, 0, s>>>(a, x, np, epi, o, xp, part, tiles, st, step, sd);
+    else
+      k_gemm_f32<64, 64, 16><<<ntiles, 64, 0, s>>>(a, x, np, epi, o, xp, part, tiles, st, step, sd);
   }
   return cudaGetLastError();
 }

@@ -269,17 +269,16 @@ int join_beside(sp2_handle_t h) {
 size_t dsize(int dtype) { return dtype == SP2_F64 ? 8 : 4; }
 
 // --------------------------------------------------------------- tile lists
-void tile_shape(sp2_handle_t h, int mode, int64_t np, int* bm, int* bn) {
-  if (split_mode(mode)) tc_tile_shape(h->tune.pair, bm, bn);
-  else simt_tile_shape(mode, np, bm, bn);
-}
-
-// the tile of a square (upper) or plain product: narrower on CTA pairs where 256-wide
+// the tile of a square (upper) or plain product: on CTA pairs narrower where 256-wide
 // tiles would not fill the GPU
 void product_tile(sp2_handle_t h, int mode, int64_t rows, int64_t np, bool upper, int* bm,
                   int* bn) {
-  tile_shape(h, mode, np, bm, bn);
-  if (split_mode(mode) && h->tune.pair) *bn = tc_tile_width(rows, np, upper);
+  if (!split_mode(mode)) {
+    simt_tile_shape(mode, rows, np, upper, bm, bn);
+    return;
+  }
+  tc_tile_shape(h->tune.pair, bm, bn);
+  if (h->tune.pair) *bn = tc_tile_width(rows, np, upper);
 }
 
 // partials per output tile: a CTA pair's two CTAs each report their own rows
@@ -290,8 +289,7 @@ int parts_per_tile(sp2_handle_t h, int mode) { return split_mode(mode) && h->tun
 // time share their operand slices. upper=true keeps only tiles that meet the
 // upper triangle (row0 <= last column), which suffices for symmetric results.
 int tile_list(sp2_handle_t h, int mode, int64_t rows, int64_t np, bool upper, const Tile** d,
-              int* n, int bm = 0, int bn = 0) {
-  if (bm == 0) tile_shape(h, mode, np, &bm, &bn);
+              int* n, int bm, int bn) {
   char key[96];
   snprintf(key, sizeof key, "%d/%lld/%lld/%d/%dx%d", mode, (long long)rows, (long long)np,
            (int)upper, bm, bn);
@@ -526,7 +524,7 @@ int square_step(Ctx& c, const MatBuf& xin, const MatBuf& xout, int step,
     if (e != cudaSuccess) return fail(h, SP2_ECUDA, "square product: %s %s", cudaGetErrorString(e), eb);
   } else {
     CK(launch_gemm_simt(c.mode, EPI_SQUARE, xin.master, c.np, xin.master, c.np, xout.master,
-                        xin.master, c.part, tl, nt, c.st, step, h->stream, dec ? &sd : nullptr));
+                        xin.master, c.part, tl, nt, bm, bn, c.st, step, h->stream, dec ? &sd : nullptr));
   }
   if (c.timing) {
     CK(cudaEventRecord(e1, h->stream));
@@ -663,7 +661,7 @@ int response_step(Ctx& c, const MatBuf& x, const MatBuf& yin, const MatBuf& yout
   const Tile* tl;
   int nt;
   int bm, bn;
-  if (fused) tile_shape(h, c.mode, c.np, &bm, &bn);
+  if (fused) tc_tile_shape(h->tune.pair, &bm, &bn);
   else product_tile(h, c.mode, rows, c.np, false, &bm, &bn);
   TRY(tile_list(h, c.mode, rows, c.np, fused, &tl, &nt, bm, bn));
   // workspace first: nothing is allocated inside the timed interval
@@ -735,7 +733,7 @@ int response_step(Ctx& c, const MatBuf& x, const MatBuf& yin, const MatBuf& yout
     if (e != cudaSuccess) return fail(h, SP2_ECUDA, "response product: %s %s", cudaGetErrorString(e), eb);
   } else {
     CK(launch_gemm_simt(c.mode, EPI_PLAIN, yin.master, rows, x.master, c.np, z, nullptr, c.part,
-                        tl, nt, c.st, step, h->stream));
+                        tl, nt, bm, bn, c.st, step, h->stream));
   }
   if (c.timing) {
     CK(cudaEventRecord(e1, h->stream));
@@ -1473,7 +1471,7 @@ int fprod(Ctx& c, FMat& C, const FMat& L, const FMat& R) {
     if (e != cudaSuccess) return fail(h, SP2_ECUDA, "finite-T product: %s %s", cudaGetErrorString(e), eb);
   } else {
     CK(launch_gemm_simt(c.mode, EPI_PLAIN, L.m.master, c.np, R.m.master, c.np, C.m.master, nullptr,
-                        c.part, tl, nt, c.st, 0, h->stream));
+                        c.part, tl, nt, bm, bn, c.st, 0, h->stream));
   }
   if (c.timing) {
     CK(cudaEventRecord(e1, h->stream));

@@ -235,9 +235,10 @@ struct SimtDecide {
 // dec (squares only, may be null): take the step decision in the last block.
 cudaError_t launch_gemm_simt(int mode, int epi, const void* A, int64_t a_rows, const void* X,
                              int64_t np, void* out, const void* x_prev, Part3* part,
-                             const Tile* tiles, int ntiles, const DevState* st, int step,
-                             cudaStream_t s, const SimtDecide* dec = nullptr);
-void simt_tile_shape(int mode, int64_t np, int* bm, int* bn);
+                             const Tile* tiles, int ntiles, int bm, int bn, const DevState* st,
+                             int step, cudaStream_t s, const SimtDecide* dec = nullptr);
+// output tile of a square (upper) or plain product of a rows x np left factor
+void simt_tile_shape(int mode, int64_t rows, int64_t np, bool upper, int* bm, int* bn);
 
 // tcgen05 split-precision (BF16X2 / FP16X2 / BF16X3)
 struct TcOperand {   // hi/lo (and BF16X3 mid) planes of a stacked operand, rows x np
