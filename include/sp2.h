@@ -93,7 +93,7 @@ typedef enum { SP2_F64 = 0, SP2_F32 = 1 } sp2_dtype;
 
 /* Arithmetic of the matrix products (Sec. VI.B).
  *   SP2_MODE_FP64    FP64. Products of matrices above N = 257 are formed on the tensor
- *                    cores from 7 error-free digits of 9 bits per entry (28 exact
+ *                    cores from 8 error-free digits of 8 bits per entry (36 exact
  *                    products summed in integers), with errors below those of an
  *                    FP64 dot product relative to the norms of its row and column;
  *                    smaller ones by CUDA-core DFMA.

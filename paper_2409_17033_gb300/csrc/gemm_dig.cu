@@ -4,33 +4,39 @@
 // multiplication and its applications", Numer. Algorithms 59, 2012).
 //
 // Why: GB300's FP64 pipe does about 2 FMA per clock and SM (1.25 TFLOP/s), its
-// 16-bit tensor pipe a thousand times that, so 28 tensor products in place of
-// one FP64 product are still about 40 times faster once a product fills the GPU.
+// 16-bit tensor pipe a thousand times that, so 36 tensor products in place of one
+// FP64 product are still some 30 times faster once a product fills the GPU.
 //
-// Splitting. Row i of a factor is scaled by a power of two 2^ex_i >= its 2-norm
-// and rounded to a 62-bit fixed-point number, which is cut into 7 signed digits
-// of 9 bits: x = 2^(ex - 62) sum_i d_i 2^(54 - 9 i), d_i in [-256, 256]. Digits
-// are exact in bfloat16, a product of two is at most 2^16, and a sum of 256 of
-// them at most 2^24, so the tensor core's FP32 accumulation of a 256-wide K chunk
-// is exact whatever the inputs. The chunks of all digit pairs (i, j) of one
-// weight s = i + j add up in INT32 registers (exact up to K = 4096), and each
-// weight's sum is added to a 64-bit integer T(i, j) of unit 2^(ex_i + ex_j - 62):
-// |C_ij| <= 2^(ex_i + ex_j) by Cauchy-Schwarz, so T never leaves 63 bits. The 28
-// pairs with s <= 6 are formed. What is dropped (s >= 7) and rounded is of the
-// order sqrt(K) 2^-63 of the two rows' norms, below the rounding of an FP64 dot
-// product. Integer additions commute, so a tile's work may be cut into parts (by
-// weight and along K) whose sums meet in T by atomics: the result has the same
-// bits for every cut and every order.
+// Splitting. Row i of a factor is scaled by a power of two 2^ex_i > its 2-norm and
+// rounded to a 63-bit fixed-point number, which is cut into 8 signed digits of 8
+// bits: x = 2^(ex - 63) sum_i d_i 2^(56 - 8 i), d_i in [-128, 128]. Digits are exact
+// in bfloat16, a product of two is at most 2^14, and a sum of 256 of them at most
+// 2^22, so the tensor core's FP32 accumulation of a 256-wide K chunk is exact
+// whatever the inputs, and one FP32 addition of 1.5 2^23 turns it into an integer's
+// bits. The chunks of all digit pairs (i, j) of one weight s = i + j add up in INT32
+// registers (exact to K = 8192) and are stored, one 32-bit plane per weight (and per
+// part of a longer or divided K axis). The passes below add a product's planes into a
+// 64-bit integer T(i, j) of unit 2^(ex_i + ex_j - 62): |C_ij| <= 2^(ex_i + ex_j) by
+// Cauchy-Schwarz, so T never leaves 63 bits. The 36 pairs with s <= 7 are formed. What
+// is dropped (s >= 8) and rounded is of the order sqrt(K) 2^-64 of the two rows'
+// scales, below the rounding of an FP64 dot product. A tile's work may be cut into
+// parts, by weight and along K: integer additions commute, so the result has the same
+// bits for every cut. (Sums that met in T by 64-bit atomics cost 25000 clocks per
+// weight and tile, a third of a product's time at N = 1024.)
 //
-// Layout. T is stored transposed, T[j * rows + i] for entry (i, j): a warp's lanes
-// hold consecutive rows i, so its 64-bit atomics are whole sectors.
+// (7 digits of 9 bits need 28 products, but their chunks reach 2^24, and the
+// conversions to integers (16 a clock and SM) made a chunk's drain as long as its
+// MMAs.)
 //
-// Per product: k_digits (each factor; it also clears T), k_gemm_dig, then one
-// pass that turns T into FP64 and applies the recursion's update: k_dig_square
+// Layout. The planes are stored transposed, G[j * rows + i] for entry (i, j): a warp's
+// lanes hold consecutive rows i, so its stores are whole lines.
+//
+// Per product: k_digits (each factor), k_gemm_dig, then one pass that turns the sums
+// into FP64 and applies the recursion's update: k_dig_square
 // (Eq. DM0, with the traces and the step decision), k_dig_symm (Eqs. DM1-DM3) or
 // k_dig_plain.
 //
-// k_gemm_dig is tensor-bound at large N (28 bfloat16 products) and bound by
+// k_gemm_dig is tensor-bound at large N (36 bfloat16 products) and bound by
 // latency and by the number of resident CTA pairs at small N. Tile, pipeline and
 // warp roles are those of the split-precision kernel on CTA pairs: 256 x BN tiles
 // (BN = 256, or 128 where more and smaller tiles fill the GPU better), one
@@ -48,15 +54,17 @@ namespace sp2 {
 
 namespace {
 
-constexpr int kDigits = 7;
-constexpr int kGroups = 7;        // digit-pair weights s = i + j <= 6
-constexpr int kFixBits = 62;      // fixed-point bits of a scaled entry; unit of T
+constexpr int kDigits = kDigPlanes;
+constexpr int kGroups = 8;        // digit-pair weights s = i + j <= 7
+constexpr int kPairs = kGroups * (kGroups + 1) / 2;
+constexpr int kFixBits = 63;      // fixed-point bits of a scaled entry
+constexpr int kTBits = 62;        // T's unit is 2^(ex_i + ex_j - kTBits)
 constexpr int kBadRow = 1 << 20;  // exponent of a row with a NaN or an infinity
 
 constexpr int BM = 128;           // tile rows per CTA
 constexpr int BK = kBoxCols;
 constexpr int KCH = 4;            // k-blocks per TMEM chunk: 256 products, exact in FP32
-constexpr int KSEG_MAX = 64;      // k-blocks an INT32 sum of 7 digit pairs may span (K = 4096)
+constexpr int KSEG_MAX = 128;     // k-blocks an INT32 sum of 8 digit pairs may span (K = 8192)
 constexpr int EPI_WARPS = 16;
 constexpr int NUM_THREADS = 64 + 32 * EPI_WARPS;
 constexpr unsigned long long DRAIN_NS = 200000000ull;
@@ -75,11 +83,11 @@ struct Geo {
                                     ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(2 * BM >> 4) << 24);
 };
 
-// The weights of part `part` of `parts`: 28 digit pairs split evenly (weight s has s + 1).
+// The weights of part `part` of `parts`: 36 digit pairs split evenly (weight s has s + 1).
 __device__ __forceinline__ uint32_t part_mask(int parts, int part) {
-  if (parts == 1) return 0x7fu;
-  if (parts == 2) return part == 0 ? 0x61u : 0x1eu;                 // {6,5,0}, {4,3,2,1}
-  return part == 0 ? 0x40u : (part == 1 ? 0x21u : (part == 2 ? 0x12u : 0x0cu));
+  if (parts == 1) return 0xffu;
+  if (parts == 2) return part == 0 ? 0xc4u : 0x3bu;                  // {7,6,2}, {5,4,3,1,0}
+  return part == 0 ? 0x81u : (part == 1 ? 0x42u : (part == 2 ? 0x24u : 0x18u));   // {7,0} ..
 }
 
 struct DParams {
@@ -87,9 +95,9 @@ struct DParams {
   int kseg;            // k-blocks of one K part (a multiple of KCH, at most KSEG_MAX)
   int ksplit;          // K parts
   int parts;           // weight parts (1, 2 or 4)
-  int64_t rows;        // rows of A (plane stride of its map, leading dimension of T)
+  int64_t rows;        // rows of A (plane stride of its map, leading dimension of G)
   int64_t np;          // rows of X per plane
-  unsigned long long* T;
+  int* G;              // planes (K part x weight) of np x rows sums
   const Tile* tiles;
   int nunits;          // tiles x parts x ksplit
   DevState* st;
@@ -101,7 +109,7 @@ struct DParams {
 struct Unit {
   Tile t;
   uint32_t mask;
-  int kb0, kb1;
+  int ks, kb0, kb1;
 };
 
 __device__ __forceinline__ Unit unit_of(const DParams& p, int u) {
@@ -111,6 +119,7 @@ __device__ __forceinline__ Unit unit_of(const DParams& p, int u) {
   Unit r;
   r.t = p.tiles[tix];
   r.mask = part_mask(p.parts, part);
+  r.ks = ks;
   r.kb0 = ks * p.kseg;
   r.kb1 = r.kb0 + p.kseg < p.nkb ? r.kb0 + p.kseg : p.nkb;
   return r;
@@ -144,7 +153,7 @@ k_gemm_dig(const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUt
   const uint32_t rank = cluster_rank();
   const bool issuer = rank == 0;
   const int pair = (int)(blockIdx.x >> 1), npairs = (int)(gridDim.x >> 1);
-  const int pairs_per_part = 28 / p.parts;   // digit pairs of a unit
+  const int pairs_per_part = kPairs / p.parts;   // digit pairs of a unit
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
@@ -273,21 +282,24 @@ k_gemm_dig(const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUt
     for (int u = pair; u < p.nunits && ok; u += npairs) {
       uint32_t mask;
       int kch;
-      unsigned long long* dst;
+      int* dst;
       {
         const Unit w = unit_of(p, u);
         mask = w.mask;
         kch = (w.kb1 - w.kb0) / KCH;
-        dst = p.T + (int64_t)(w.t.col0 + grp * TC) * p.rows + (int64_t)w.t.row0 + r;
+        dst = p.G + ((int64_t)w.ks * kGroups * p.np + w.t.col0 + grp * TC) * p.rows +
+              (int64_t)w.t.row0 + r;
       }
 #pragma unroll 1
       for (int s = kGroups - 1; s >= 0; --s) {
         if (!((mask >> s) & 1u)) continue;
-        int acc[TC];
+        // sums of the chunks' bits after the addition of 1.5 2^23, modulo 2^32
+        const int nch = (s + 1) * kch;
+        uint32_t acc[TC];
 #pragma unroll
-        for (int j = 0; j < TC; ++j) acc[j] = 0;
+        for (int j = 0; j < TC; ++j) acc[j] = 0u;
 #pragma unroll 1
-        for (int c = (s + 1) * kch; c > 0; --c, ++gc) {
+        for (int c = nch; c > 0; --c, ++gc) {
           const uint32_t b = gc & 1u;
           const bool wt = mbar_wait<true>(&tfull[b], (gc >> 1) & 1u, abortf, p.wait_ns);
           ok = __all_sync(0xffffffffu, wt);
@@ -298,7 +310,8 @@ k_gemm_dig(const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUt
             uint32_t v[16];
             tmem_ld16(trow + b * BN + (uint32_t)c0, v);
 #pragma unroll
-            for (int j = 0; j < 16; ++j) acc[c0 + j] += __float2int_rn(__uint_as_float(v[j]));
+            for (int j = 0; j < 16; ++j)
+              acc[c0 + j] += __float_as_uint(__uint_as_float(v[j]) + 12582912.0f);
           }
           tc_fence_before();
           __syncwarp();
@@ -310,18 +323,11 @@ k_gemm_dig(const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUt
           }
         }
         if (!ok) break;
-        // weight s in T's unit: 2^(108 - 9 s) products' unit over 2^62 (46 - 9 s >= -8)
-        const int sh = 2 * 54 - 9 * s - kFixBits;
-        const int up = sh > 0 ? sh : 0, dn = sh < 0 ? -sh : 0;
-        const int half = dn ? 1 << (dn - 1) : 0;
-        unsigned long long* d = dst;
+        const uint32_t off = (uint32_t)nch * 0x4b400000u;   // the bits of 1.5 2^23
+        int* d = dst + (int64_t)s * p.np * p.rows;
 #pragma unroll
         for (int j = 0; j < TC; ++j) {
-          // |acc| < 2^31 - 2^8, so the rounding term cannot overflow
-          const long long v = (long long)((acc[j] + half) >> dn) << up;
-          asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(d),
-                       "l"((unsigned long long)v)
-                       : "memory");
+          __stcg(d, (int)(acc[j] - off));
           d += p.rows;
         }
       }
@@ -347,16 +353,15 @@ __device__ __forceinline__ bool halted_dig(const DevState* st, int step) {
 
 // ------------------------------------------------------------ digits
 // One block per row: the row's power-of-two scale 2^ex >= its 2-norm, then the
-// seven digit planes (plane d of the stack at d * rows * np), and T's share of the
-// product cleared. Integer arithmetic throughout (FP64 conversions run at the slow
+// eight digit planes (plane d of the stack at d * rows * np). Integer arithmetic throughout (FP64 conversions run at the slow
 // FP64 rate); the norm in FP32 from the entries' leading 20 bits, relative to the
 // row's largest entry, with a margin above its rounding. HBM-bound at large N: 8
-// bytes read, 14 (and 8 for T) written per entry.
+// bytes read, 16 written per entry.
 constexpr int kDigThreads = 128;
 
 __global__ void __launch_bounds__(kDigThreads)
 k_digits(const double* __restrict__ src, int64_t rows, int64_t np, uint16_t* __restrict__ dig,
-         int* __restrict__ ex, unsigned long long* __restrict__ T, const DevState* st, int step) {
+         int* __restrict__ ex, const DevState* st, int step) {
   if (halted_dig(st, step)) return;
   __shared__ uint32_t smax[kDigThreads / 32];
   __shared__ float ssum[kDigThreads / 32];
@@ -400,17 +405,17 @@ k_digits(const double* __restrict__ src, int64_t rows, int64_t np, uint16_t* __r
   ss = 0.0f;
 #pragma unroll
   for (int w = 0; w < kDigThreads / 32; ++w) ss += ssum[w];
-  // sums of at most 2^14 positive FP32 terms per thread: 1 + 2^-8 covers their
-  // rounding and the truncation of the entries
-  ss = ss * (1.0f + 0.00390625f) + (float)np * 1e-17f;
+  // sums of at most 2^14 positive FP32 terms per thread: 1 + 2^-5 covers their
+  // rounding and the truncation of the entries, and keeps the fixed-point entries (and
+  // the biased ones below) within 63 bits
+  ss = ss * (1.0f + 0.03125f) + (float)np * 1e-17f;
   int k2;
   frexpf(ss, &k2);                      // ss < 2^k2
   const int q = (k2 + 1) >> 1;          // sqrt(ss) < 2^q
   const int e = bad ? kBadRow : (m == 0 ? 0 : em - 1023 + q);
   if (threadIdx.x == 0) ex[row] = e;
   const int64_t plane = rows * np;
-  constexpr unsigned long long kBias =   // 256 in every digit field below the first
-      (256ull << 45) + (256ull << 36) + (256ull << 27) + (256ull << 18) + (256ull << 9) + 256ull;
+  constexpr unsigned long long kBias = 0x0080808080808080ull;   // 128 in every digit below the first
   for (int c = threadIdx.x; c < n4; c += kDigThreads) {
     const double2 a = x2[2 * c], b = x2[2 * c + 1];
     const double v[4] = {a.x, a.y, b.x, b.y};
@@ -421,7 +426,7 @@ k_digits(const double* __restrict__ src, int64_t rows, int64_t np, uint16_t* __r
       const int eb = (int)((bits >> 52) & 0x7ff);
       unsigned long long mant = (unsigned long long)bits & 0xfffffffffffffull;
       if (eb) mant |= 1ull << 52;
-      const int sh = (eb ? eb : 1) - (1075 - kFixBits) - e;   // at most 10
+      const int sh = (eb ? eb : 1) - (1075 - kFixBits) - e;   // at most 11
       long long I;
       if (sh >= 0) I = (long long)(mant << sh);
       else if (sh > -55) I = (long long)((mant + (1ull << (-sh - 1))) >> -sh);
@@ -429,25 +434,49 @@ k_digits(const double* __restrict__ src, int64_t rows, int64_t np, uint16_t* __r
       if (bits < 0) I = -I;
       if (bad || m == 0) I = 0;
       const long long B = I + (long long)kBias;
-      f[k][0] = (uint32_t)((int)(B >> 54) + 256);
+      f[k][0] = (uint32_t)((int)(B >> 56) + 128);
 #pragma unroll
-      for (int d = 1; d < kDigits; ++d) f[k][d] = (uint32_t)((unsigned long long)B >> (54 - 9 * d)) & 511u;
+      for (int d = 1; d < kDigits; ++d) f[k][d] = (uint32_t)((unsigned long long)B >> (56 - 8 * d)) & 255u;
     }
 #pragma unroll
     for (int d = 0; d < kDigits; ++d) {
       uint32_t h[4];
 #pragma unroll
-      for (int k = 0; k < 4; ++k)   // field - 256 as an FP32 integer; its upper half is the bfloat16
-        h[k] = __float_as_uint(__uint_as_float(0x4B000000u + f[k][d]) - 8388864.0f);
+      for (int k = 0; k < 4; ++k)   // field - 128 as an FP32 integer; its upper half is the bfloat16
+        h[k] = __float_as_uint(__uint_as_float(0x4B000000u + f[k][d]) - 8388736.0f);
       uint2 o;
       o.x = __byte_perm(h[0], h[1], 0x7632);
       o.y = __byte_perm(h[2], h[3], 0x7632);
       reinterpret_cast<uint2*>(dig + d * plane + row * np)[c] = o;
     }
-    if (T) {
-      ulonglong2* t2 = reinterpret_cast<ulonglong2*>(T + row * np);
-      t2[2 * c] = make_ulonglong2(0ull, 0ull);
-      t2[2 * c + 1] = make_ulonglong2(0ull, 0ull);
+  }
+}
+
+// A product's sums: planes of `ksplit` K parts x kGroups weights, `plane` entries each.
+struct Sums {
+  const int* g;
+  int64_t plane;
+  int ksplit;
+};
+
+// T of four consecutive entries at o: weight s counts 2^(112 - 8 s) over
+// 2^(2 kFixBits - kTBits) = 2^64, that is 2^(48 - 8 s), the last one rounded
+__device__ __forceinline__ void load_t(const Sums& q, int64_t o, long long (&t)[4]) {
+#pragma unroll
+  for (int k = 0; k < 4; ++k) t[k] = 0;
+  for (int ks = 0; ks < q.ksplit; ++ks) {
+    int4 v[kGroups];
+#pragma unroll
+    for (int s = 0; s < kGroups; ++s)
+      v[s] = __ldcs(reinterpret_cast<const int4*>(q.g + (int64_t)(ks * kGroups + s) * q.plane + o));
+#pragma unroll
+    for (int s = 0; s < kGroups; ++s) {
+      const int x[4] = {v[s].x, v[s].y, v[s].z, v[s].w};
+      const int sh = 2 * 56 - 8 * s - (2 * kFixBits - kTBits);
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        t[k] += sh >= 0 ? (long long)x[k] << (sh > 0 ? sh : 0)
+                        : (long long)((x[k] + (1 << 7)) >> 8);   // at most 2^30
     }
   }
 }
@@ -464,7 +493,7 @@ __device__ __forceinline__ double from_fixed(long long t, int ei, int ej) {
   const double off = __hiloint2double(0x45300000, (int)0x80100000u);   // 2^84 + 2^63 + 2^52
   const double v = (dh - off) + dl;
   if (ei == kBadRow || ej == kBadRow) return __longlong_as_double(0x7ff8000000000000ll);
-  const int e = ei + ej - kFixBits;
+  const int e = ei + ej - kTBits;
   const int vh = __double2hiint(v);
   const int ve = (vh >> 20) & 0x7ff;
   if (ve == 0) return v;   // zero
@@ -483,11 +512,6 @@ __device__ __forceinline__ void tri_ij(int64_t t, int64_t& I, int64_t& J) {
   I = t - J * (J + 1) / 2;
 }
 
-__device__ __forceinline__ void ld4ll(const unsigned long long* p, long long (&v)[4]) {
-  const longlong2 a = __ldcs(reinterpret_cast<const longlong2*>(p));
-  const longlong2 b = __ldcs(reinterpret_cast<const longlong2*>(p) + 1);
-  v[0] = a.x, v[1] = a.y, v[2] = b.x, v[3] = b.y;
-}
 __device__ __forceinline__ void ld4d(const double* p, double (&v)[4]) {
   const double2 a = reinterpret_cast<const double2*>(p)[0];
   const double2 b = reinterpret_cast<const double2*>(p)[1];
@@ -500,67 +524,83 @@ __device__ __forceinline__ void st4d(double* p, const double (&v)[4]) {
 
 // X_{n+1} = sigma > 0 ? C : 2 X_n - C from T (C = X_n^2, upper entries), mirrored;
 // partials of Tr, ||.||_F^2 and ||X_n - X_n^2||_F^2 in FP64, and the step decision
-// in the last block. One block per pair of TE x TE tiles (I <= J); T's tile (J, I)
-// holds entries (i, j) of the upper tile with i along its rows. About 8 FP64
-// operations per upper entry bound it (GB300's FP64 pipe).
+// in the last block. Blocks walk pairs of TE x TE tiles (I <= J); T's tile (J, I)
+// holds entries (i, j) of the upper tile with i along its rows. Bound by its 6 FP64
+// operations per upper entry (an FP64 instruction of a warp takes 64 clocks), so
+// the reductions come once per block, not per tile, ||.||_F^2 and f sharing them.
 __global__ void __launch_bounds__(kPassThreads)
-k_dig_square(const unsigned long long* __restrict__ T, const int* __restrict__ ex,
-             const double* __restrict__ X, double* __restrict__ out, int64_t np, DevState* st,
-             int step, Part3* __restrict__ part, SimtDecide dec) {
+k_dig_square(const Sums q, const int* __restrict__ ex,
+             const double* __restrict__ X, double* __restrict__ out, int64_t np, int ntiles,
+             DevState* st, int step, Part3* __restrict__ part, SimtDecide dec) {
   if (halted_dig(st, step)) return;
-  __shared__ double sm[TE][TE + 1];
-  int64_t I, J;
-  tri_ij(blockIdx.x, I, J);
+  __shared__ double sm[2][TE][TE + 1];
+  __shared__ double red[3][kPassThreads / 32];
   const int r = threadIdx.x >> 3, c4 = (threadIdx.x & 7) * 4;
-  const int64_t gj = J * TE + r, gi0 = I * TE + c4;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int sg = st->sigma[step];
-  double t1 = 0.0, t2 = 0.0, f = 0.0;
-  double y[4];
-  {
-    long long t[4];
-    double x[4];
-    ld4ll(T + gj * np + gi0, t);
-    ld4d(X + gj * np + gi0, x);   // X_n is symmetric
-    const int ej = ex[gj];
+  double t1 = 0.0, t2 = 0.0, f = 0.0;   // t2, f: off-diagonal entries (counted twice below)
+  double e2 = 0.0, ef = 0.0;            // their diagonal entries
+  int buf = 0;
+  for (int64_t tix = blockIdx.x; tix < ntiles; tix += gridDim.x, buf ^= 1) {
+    int64_t I, J;
+    tri_ij(tix, I, J);
+    const int64_t gj = J * TE + r, gi0 = I * TE + c4;
+    double y[4];
+    {
+      long long t[4];
+      double x[4];
+      load_t(q, gj * np + gi0, t);
+      ld4d(X + gj * np + gi0, x);   // X_n is symmetric
+      const int ej = ex[gj];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const int64_t gi = gi0 + k;
-      if (gi > gj) continue;      // below the diagonal of a diagonal tile
-      const double c = from_fixed(t[k], ex[gi], ej);
-      const double v = sg > 0 ? c : 2.0 * x[k] - c;
-      const double d = x[k] - c;
-      y[k] = v;
-      sm[r][c4 + k] = v;
-      if (gi == gj) {
-        t1 += v;
-        t2 += 0.5 * v * v;        // off-diagonal entries count twice, at the end
-        f += 0.5 * d * d;
-      } else {
-        t2 += v * v;
-        f += d * d;
+      for (int k = 0; k < 4; ++k) {
+        const int64_t gi = gi0 + k;
+        if (gi > gj) continue;      // below the diagonal of a diagonal tile
+        const double c = from_fixed(t[k], ex[gi], ej);
+        const double v = sg > 0 ? c : 2.0 * x[k] - c;
+        const double d = x[k] - c;
+        y[k] = v;
+        sm[buf][r][c4 + k] = v;
+        if (gi == gj) {
+          t1 += v;
+          e2 += v * v;
+          ef += d * d;
+        } else {
+          t2 += v * v;
+          f += d * d;
+        }
       }
     }
-  }
-  __syncthreads();
-  if (I == J) {
+    __syncthreads();   // (the other buffer's readers are two tiles back)
+    if (I == J) {
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
-      if (gi0 + k > gj) y[k] = sm[c4 + k][r];
-    st4d(out + gj * np + gi0, y);
-  } else {
-    st4d(out + gj * np + gi0, y);
-    double w[4];
+      for (int k = 0; k < 4; ++k)
+        if (gi0 + k > gj) y[k] = sm[buf][c4 + k][r];
+      st4d(out + gj * np + gi0, y);
+    } else {
+      st4d(out + gj * np + gi0, y);
+      double w[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) w[k] = sm[c4 + k][r];   // entry (i, j), i = I TE + r
-    st4d(out + (I * TE + r) * np + J * TE + c4, w);
+      for (int k = 0; k < 4; ++k) w[k] = sm[buf][c4 + k][r];   // entry (i, j), i = I TE + r
+      st4d(out + (I * TE + r) * np + J * TE + c4, w);
+    }
   }
+  t2 = 2.0 * t2 + e2;
+  f = 2.0 * f + ef;
+  const bool up = lane >= 16;
+  double s = (up ? f : t2) + __shfl_xor_sync(0xffffffffu, up ? t2 : f, 16);
+  for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  for (int o = 16; o > 0; o >>= 1) t1 += __shfl_xor_sync(0xffffffffu, t1, o);
+  if (lane == 0) red[0][warp] = t1, red[1][warp] = s;
+  if (lane == 16) red[2][warp] = s;
   __syncthreads();
-  t1 = block_sum(t1);
-  __syncthreads();
-  t2 = block_sum(t2);
-  __syncthreads();
-  f = block_sum(f);
-  if (threadIdx.x == 0) part[blockIdx.x] = Part3{t1, 2.0 * t2, 2.0 * f};
+  if (warp == 0) {
+    constexpr int NW = kPassThreads / 32;
+    double v = lane < 3 * NW ? red[lane / NW][lane % NW] : 0.0;
+    for (int o = NW / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    const double a2 = __shfl_sync(0xffffffffu, v, NW), af = __shfl_sync(0xffffffffu, v, 2 * NW);
+    if (lane == 0) part[blockIdx.x] = Part3{v, a2, af};
+  }
   if (dec.done) {
     __shared__ int last;
     if (threadIdx.x == 0) {
@@ -580,7 +620,7 @@ k_dig_square(const unsigned long long* __restrict__ T, const int* __restrict__ e
 // (ey: exponents of the stacked rows of Y_n, ex: of X_n). One block per tile pair
 // and batch entry.
 __global__ void __launch_bounds__(kPassThreads)
-k_dig_symm(const unsigned long long* __restrict__ T, int64_t rows, const int* __restrict__ ey,
+k_dig_symm(const Sums q, int64_t rows, const int* __restrict__ ey,
            const int* __restrict__ ex, const double* __restrict__ yin, double* __restrict__ yout,
            int64_t np, const DevState* st, int step) {
   if (halted_dig(st, step)) return;
@@ -593,8 +633,8 @@ k_dig_symm(const unsigned long long* __restrict__ T, int64_t rows, const int* __
   {
     long long ta[4], tb[4];
     const int64_t gj = J * TE + r, gi = I * TE + r;
-    ld4ll(T + gj * rows + b0 + I * TE + c4, ta);   // z(i, j): j = gj, i along c4
-    ld4ll(T + gi * rows + b0 + J * TE + c4, tb);   // z(j, i): i = gi, j along c4
+    load_t(q, gj * rows + b0 + I * TE + c4, ta);   // z(i, j): j = gj, i along c4
+    load_t(q, gi * rows + b0 + J * TE + c4, tb);   // z(j, i): i = gi, j along c4
     const int xj = ex[gj], xi = ex[gi];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
@@ -624,7 +664,7 @@ k_dig_symm(const unsigned long long* __restrict__ T, int64_t rows, const int* __
 
 // C = T's value, row-major rows x np
 __global__ void __launch_bounds__(kPassThreads)
-k_dig_plain(const unsigned long long* __restrict__ T, int64_t rows, const int* __restrict__ ea,
+k_dig_plain(const Sums q, int64_t rows, const int* __restrict__ ea,
             const int* __restrict__ ex, double* __restrict__ out, int64_t np, const DevState* st,
             int step) {
   if (halted_dig(st, step)) return;
@@ -632,7 +672,7 @@ k_dig_plain(const unsigned long long* __restrict__ T, int64_t rows, const int* _
   const int64_t i0 = (int64_t)blockIdx.y * TE, j0 = (int64_t)blockIdx.x * TE;
   const int r = threadIdx.x >> 3, c4 = (threadIdx.x & 7) * 4;
   long long t[4];
-  ld4ll(T + (j0 + r) * rows + i0 + c4, t);
+  load_t(q, (j0 + r) * rows + i0 + c4, t);
   const int xj = ex[j0 + r];
 #pragma unroll
   for (int k = 0; k < 4; ++k) sm[r][c4 + k] = from_fixed(t[k], ea[i0 + c4 + k], xj);
@@ -703,20 +743,22 @@ int64_t dig_tiles(int64_t rows, int64_t np, int bn, bool upper) {
 // the estimate below.
 DigPlan dig_plan(int64_t rows, int64_t np, bool upper) {
   const int nkb = (int)(np / BK);
-  const int pairs = 76;
+  const int resident = 76;
   DigPlan best;
   double tbest = 0.0;
   for (int bn = 256; bn >= 128; bn -= 128) {
     const int64_t nt = dig_tiles(rows, np, bn, upper);
-    const double chunk = bn == 256 ? 2400.0 : 1600.0, fold = bn == 256 ? 3000.0 : 1500.0;
+    const double chunk = bn == 256 ? 2500.0 : 1700.0, fold = bn == 256 ? 6000.0 : 3000.0;
     for (int parts = 1; parts <= 4; parts *= 2)
       for (int ks = (nkb + KSEG_MAX - 1) / KSEG_MAX; ks <= nkb / KCH; ++ks) {
         const int kseg = ((nkb + ks - 1) / ks + KCH - 1) / KCH * KCH;
         if ((nkb + kseg - 1) / kseg != ks) continue;
         const int64_t units = nt * parts * ks;
-        const int64_t waves = (units + pairs - 1) / pairs;
-        const int folds = parts == 1 ? 7 : (parts == 2 ? 4 : 2);
-        const double t = (double)waves * (28.0 / parts * (kseg / KCH) * chunk + folds * fold) + 8000.0;
+        const int64_t waves = (units + resident - 1) / resident;
+        const int folds = parts == 1 ? 8 : (parts == 2 ? 5 : 2);
+        // clocks: the waves, and the pass that reads the sums' planes
+        const double t = (double)waves * ((double)kPairs / parts * (kseg / KCH) * chunk + folds * fold) +
+                         (double)ks * (upper ? 0.5 : 1.0) * (double)rows * (double)np * 32.0 / 3000.0;
         if (tbest == 0.0 || t < tbest) {
           tbest = t;
           best.bn = bn;
@@ -730,14 +772,14 @@ DigPlan dig_plan(int64_t rows, int64_t np, bool upper) {
 }
 
 cudaError_t launch_digits(const double* src, int64_t rows, int64_t np, const DigOperand& o,
-                          unsigned long long* T, const DevState* st, int step, cudaStream_t s) {
-  k_digits<<<(unsigned)rows, kDigThreads, 0, s>>>(src, rows, np, o.dig, o.ex, T, st, step);
+                          const DevState* st, int step, cudaStream_t s) {
+  k_digits<<<(unsigned)rows, kDigThreads, 0, s>>>(src, rows, np, o.dig, o.ex, st, step);
   return cudaGetLastError();
 }
 
 cudaError_t launch_gemm_dig(const DigOperand& A, int64_t rows, const DigOperand& X, int64_t np,
-                            unsigned long long* T, const Tile* tiles, int ntiles,
-                            const DigPlan& plan, DevState* st, int step, const TcTuning& tune,
+                            int* G, const Tile* tiles, int ntiles, const DigPlan& plan,
+                            DevState* st, int step, const TcTuning& tune,
                             cudaStream_t s) {
   if (np % 256 != 0 || rows % 256 != 0 || kDigits * rows > (int64_t)1 << 30)
     return cudaErrorInvalidValue;
@@ -752,7 +794,7 @@ cudaError_t launch_gemm_dig(const DigOperand& A, int64_t rows, const DigOperand&
   p.parts = plan.parts;
   p.rows = rows;
   p.np = np;
-  p.T = T;
+  p.G = G;
   p.tiles = tiles;
   p.nunits = ntiles * plan.parts * plan.ksplit;
   p.st = st;
@@ -762,31 +804,38 @@ cudaError_t launch_gemm_dig(const DigOperand& A, int64_t rows, const DigOperand&
   return plan.bn == 256 ? launch_bn<256>(am, bm, p, s) : launch_bn<128>(am, bm, p, s);
 }
 
-int64_t dig_square_nparts(int64_t np) { return (np / TE) * (np / TE + 1) / 2; }
+static int64_t tri_tiles(int64_t np) { return (np / TE) * (np / TE + 1) / 2; }
 
-cudaError_t launch_dig_square(const unsigned long long* T, const int* ex, const double* X,
+// blocks (and partials) of the square's pass: three per SM
+int64_t dig_square_nparts(int64_t np) {
+  const int64_t n = tri_tiles(np);
+  return n < 456 ? n : 456;
+}
+
+cudaError_t launch_dig_square(const int* G, int ksplit, const int* ex, const double* X,
                               double* out, int64_t np, DevState* st, int step, Part3* part,
                               const SimtDecide* dec, cudaStream_t s) {
   SimtDecide sd;
   if (dec) sd = *dec;
-  k_dig_square<<<(unsigned)dig_square_nparts(np), kPassThreads, 0, s>>>(T, ex, X, out, np, st, step,
-                                                                       part, sd);
+  k_dig_square<<<(unsigned)dig_square_nparts(np), kPassThreads, 0, s>>>(
+      Sums{G, np * np, ksplit}, ex, X, out, np, (int)tri_tiles(np), st, step, part, sd);
   return cudaGetLastError();
 }
 
-cudaError_t launch_dig_symm(const unsigned long long* T, int64_t rows, const int* ey, const int* ex,
+cudaError_t launch_dig_symm(const int* G, int ksplit, int64_t rows, const int* ey, const int* ex,
                             const double* yin, double* yout, int64_t np, const DevState* st,
                             int step, cudaStream_t s) {
-  const dim3 grid((unsigned)dig_square_nparts(np), (unsigned)(rows / np));
-  k_dig_symm<<<grid, kPassThreads, 0, s>>>(T, rows, ey, ex, yin, yout, np, st, step);
+  const dim3 grid((unsigned)tri_tiles(np), (unsigned)(rows / np));
+  k_dig_symm<<<grid, kPassThreads, 0, s>>>(Sums{G, rows * np, ksplit}, rows, ey, ex, yin, yout, np, st,
+                                           step);
   return cudaGetLastError();
 }
 
-cudaError_t launch_dig_plain(const unsigned long long* T, int64_t rows, const int* ea,
+cudaError_t launch_dig_plain(const int* G, int ksplit, int64_t rows, const int* ea,
                              const int* ex, double* out, int64_t np, const DevState* st, int step,
                              cudaStream_t s) {
   const dim3 grid((unsigned)(np / TE), (unsigned)(rows / TE));
-  k_dig_plain<<<grid, kPassThreads, 0, s>>>(T, rows, ea, ex, out, np, st, step);
+  k_dig_plain<<<grid, kPassThreads, 0, s>>>(Sums{G, rows * np, ksplit}, rows, ea, ex, out, np, st, step);
   return cudaGetLastError();
 }
 

@@ -397,17 +397,17 @@ bool dig_mode(const Ctx& c, int64_t rows) {
          (c.np > kPad || rows >= 2 * kPad);
 }
 
-// Batch entries whose digits and sums are formed at a time (22 bytes per entry of a
-// stacked factor): at most 2 GiB of them, at least one.
+// Batch entries whose digits and sums are formed at a time (48 bytes per entry of a
+// stacked factor): at most 4 GiB of them, at least one.
 int64_t dig_chunk(int64_t np, int64_t batch) {
-  const int64_t per = 22 * np * np;
-  const int64_t m = ((int64_t)2 << 30) / per;
+  const int64_t per = 48 * np * np;
+  const int64_t m = ((int64_t)4 << 30) / per;
   return m < 1 ? 1 : (m < batch ? m : batch);
 }
 
 struct DigBufs {
   DigOperand x, a;              // right factor; stacked left factor of `rows` rows
-  unsigned long long* T = nullptr;
+  int* G = nullptr;
   const Tile* tiles = nullptr;
   int ntiles = 0;
   DigPlan plan;
@@ -420,19 +420,18 @@ bool dig_bufs(Ctx& c, int64_t rows, bool upper, DigBufs* b) {
   sp2_handle_t h = c.h;
   const size_t el = (size_t)c.np * c.np, ra = (size_t)rows * c.np;
   const size_t nt = rows ? ra : el;
-  void *xd, *xe, *T, *ad = nullptr, *ae = nullptr;
+  void *xd, *xe, *G, *ad = nullptr, *ae = nullptr;
+  const int64_t rr = rows ? rows : c.np;
+  b->plan = dig_plan(rr, c.np, upper);
   const void* old_x = h->bufs["dig.x"].p;
   bool ok = ws_try(h, "dig.x", el * 2 * kDigPlanes, &xd) == SP2_OK &&
             ws_try(h, "dig.xe", (size_t)c.np * sizeof(int), &xe) == SP2_OK &&
-            ws_try(h, "dig.T", nt * 8, &T) == SP2_OK;
+            ws_try(h, "dig.G", nt * 4 * kDigPlanes * b->plan.ksplit, &G) == SP2_OK;
   if (ok && rows)
     ok = ws_try(h, "dig.a", ra * 2 * kDigPlanes, &ad) == SP2_OK &&
          ws_try(h, "dig.ae", (size_t)rows * sizeof(int), &ae) == SP2_OK;
-  const int64_t rr = rows ? rows : c.np;
-  if (ok) {
-    b->plan = dig_plan(rr, c.np, upper);
+  if (ok)
     ok = tile_list(h, c.mode, rr, c.np, upper, &b->tiles, &b->ntiles, 256, b->plan.bn) == SP2_OK;
-  }
   if (!ok) {
     h->err.clear();
     drop_digits(h);
@@ -442,13 +441,13 @@ bool dig_bufs(Ctx& c, int64_t rows, bool upper, DigBufs* b) {
   if (old_x != xd) h->dig_x = nullptr;
   b->x = DigOperand{static_cast<uint16_t*>(xd), static_cast<int*>(xe)};
   b->a = rows ? DigOperand{static_cast<uint16_t*>(ad), static_cast<int*>(ae)} : b->x;
-  b->T = static_cast<unsigned long long*>(T);
+  b->G = static_cast<int*>(G);
   return true;
 }
 
-// work of one digit product: tensor flops of the tiles' 28 digit pairs
+// work of one digit product: tensor flops of the tiles' 36 digit pairs
 double dig_flops(const Ctx& c, const DigBufs& b) {
-  return 2.0 * 256.0 * b.plan.bn * (double)c.np * 28.0 * b.ntiles;
+  return 2.0 * 256.0 * b.plan.bn * (double)c.np * 36.0 * b.ntiles;
 }
 
 // X_{n+1} = sigma_n>0 ? X_n^2 : 2 X_n - X_n^2, with trace partials; dec: and the step
@@ -470,27 +469,27 @@ int square_step(Ctx& c, const MatBuf& xin, const MatBuf& xout, int step,
     sd.p.nparts = (int)dig_square_nparts(c.np);
     if (dig_bufs(c, 0, true, &db)) {
       const double* x = static_cast<const double*>(xin.master);
-      // the response product of this step has left X_n's digits, but not a clear T
-      if (h->dig_x == xin.master)
-        CK(cudaMemsetAsync(db.T, 0, (size_t)c.np * c.np * 8, h->stream));
-      else
-        CK(launch_digits(x, c.np, c.np, db.x, db.T, c.st, step, h->stream));
+      // (the response product of this step has left X_n's digits)
+      if (h->dig_x != xin.master) {
+        CK(launch_digits(x, c.np, c.np, db.x, c.st, step, h->stream));
+        c.kernels++;
+      }
       h->dig_x = nullptr;
       cudaEvent_t e0 = nullptr, e1 = nullptr;
       if (c.timing) {
         TRY(ev_pair(c, &e0, &e1));
         CK(cudaEventRecord(e0, h->stream));
       }
-      CK(launch_gemm_dig(db.x, c.np, db.x, c.np, db.T, db.tiles, db.ntiles, db.plan, c.st, step,
+      CK(launch_gemm_dig(db.x, c.np, db.x, c.np, db.G, db.tiles, db.ntiles, db.plan, c.st, step,
                          h->tune, h->stream));
       if (c.timing) {
         CK(cudaEventRecord(e1, h->stream));
         c.timed.push_back({step, 0});
       }
-      CK(launch_dig_square(db.T, db.x.ex, x, static_cast<double*>(xout.master), c.np, c.st, step,
+      CK(launch_dig_square(db.G, db.plan.ksplit, db.x.ex, x, static_cast<double*>(xout.master), c.np, c.st, step,
                            c.part, dec ? &sd : nullptr, h->stream));
       c.launches++;
-      c.kernels += 3;
+      c.kernels += 2;
       c.flops += dig_flops(c, db);
       c.alg += (double)c.n * (double)(c.n + 1) * (double)c.n;
       return SP2_OK;
@@ -626,29 +625,33 @@ int response_step(Ctx& c, const MatBuf& x, const MatBuf& yin, const MatBuf& yout
     if (dig_bufs(c, bc * c.np, false, &db)) {
       const double* y = static_cast<const double*>(yin.master);
       double* yo = static_cast<double*>(yout.master);
-      CK(launch_digits(static_cast<const double*>(x.master), c.np, c.np, db.x, nullptr, c.st, step,
+      CK(launch_digits(static_cast<const double*>(x.master), c.np, c.np, db.x, c.st, step,
                        h->stream));
       h->dig_x = x.master;
       c.kernels++;
       for (int64_t b0 = 0; b0 < batch; b0 += bc) {
         const int64_t nb = batch - b0 < bc ? batch - b0 : bc, r = nb * c.np, off = b0 * c.np * c.np;
-        if (nb != bc) {   // the last, smaller chunk has its own tiles
+        if (nb != bc) {   // the last, smaller chunk has its own tiles (and the same K parts:
+                          // the sums' buffer is sized for them)
+          const int ks = db.plan.ksplit, kseg = db.plan.kseg;
           db.plan = dig_plan(r, c.np, false);
+          db.plan.ksplit = ks;
+          db.plan.kseg = kseg;
           TRY(tile_list(h, c.mode, r, c.np, false, &db.tiles, &db.ntiles, 256, db.plan.bn));
         }
-        CK(launch_digits(y + off, r, c.np, db.a, db.T, c.st, step, h->stream));
+        CK(launch_digits(y + off, r, c.np, db.a, c.st, step, h->stream));
         cudaEvent_t e0 = nullptr, e1 = nullptr;
         if (c.timing) {
           TRY(ev_pair(c, &e0, &e1));
           CK(cudaEventRecord(e0, h->stream));
         }
-        CK(launch_gemm_dig(db.a, r, db.x, c.np, db.T, db.tiles, db.ntiles, db.plan, c.st, step,
+        CK(launch_gemm_dig(db.a, r, db.x, c.np, db.G, db.tiles, db.ntiles, db.plan, c.st, step,
                            h->tune, h->stream));
         if (c.timing) {
           CK(cudaEventRecord(e1, h->stream));
           c.timed.push_back({step, 0});
         }
-        CK(launch_dig_symm(db.T, r, db.a.ex, db.x.ex, y + off, yo + off, c.np, c.st, step,
+        CK(launch_dig_symm(db.G, db.plan.ksplit, r, db.a.ex, db.x.ex, y + off, yo + off, c.np, c.st, step,
                            h->stream));
         c.launches++;
         c.kernels += 3;
@@ -782,7 +785,7 @@ int resolve_ckpt(sp2_handle_t h, sp2_opts* o, int64_t np, int64_t batch) {
   const double b = (double)(batch > 0 ? batch : 1);
   avail -= 2.0 * mat_b + 2.0 * b * mat_b + b * el * ms + (double)(1ull << 30);
   if (o->mode == SP2_MODE_FP64 && np % kPad == 0)   // digit buffers
-    avail -= el * (14.0 + 22.0 * (double)dig_chunk(np, batch > 0 ? batch : 1));
+    avail -= el * (16.0 + 48.0 * (double)dig_chunk(np, batch > 0 ? batch : 1));
   const int cap = o->fixed_m > 0 ? o->fixed_m : o->max_iter;
   int k = cap;
   for (int kk = 1; kk <= cap; ++kk) {
@@ -1415,9 +1418,9 @@ int fprod(Ctx& c, FMat& C, const FMat& L, const FMat& R) {
   const bool same = L.m.master == R.m.master;
   if (dig_mode(c, c.np) && dig_bufs(c, same ? 0 : c.np, false, &db)) {
     const double* l = static_cast<const double*>(L.m.master);
-    CK(launch_digits(l, c.np, c.np, db.a, db.T, c.st, 0, h->stream));
+    CK(launch_digits(l, c.np, c.np, db.a, c.st, 0, h->stream));
     if (!same)
-      CK(launch_digits(static_cast<const double*>(R.m.master), c.np, c.np, db.x, nullptr, c.st, 0,
+      CK(launch_digits(static_cast<const double*>(R.m.master), c.np, c.np, db.x, c.st, 0,
                        h->stream));
     h->dig_x = nullptr;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -1425,13 +1428,13 @@ int fprod(Ctx& c, FMat& C, const FMat& L, const FMat& R) {
       TRY(ev_pair(c, &e0, &e1));
       CK(cudaEventRecord(e0, h->stream));
     }
-    CK(launch_gemm_dig(db.a, c.np, db.x, c.np, db.T, db.tiles, db.ntiles, db.plan, c.st, 0, h->tune,
+    CK(launch_gemm_dig(db.a, c.np, db.x, c.np, db.G, db.tiles, db.ntiles, db.plan, c.st, 0, h->tune,
                        h->stream));
     if (c.timing) {
       CK(cudaEventRecord(e1, h->stream));
       c.timed.push_back({0, 0});
     }
-    CK(launch_dig_plain(db.T, c.np, db.a.ex, db.x.ex, static_cast<double*>(C.m.master), c.np, c.st,
+    CK(launch_dig_plain(db.G, db.plan.ksplit, c.np, db.a.ex, db.x.ex, static_cast<double*>(C.m.master), c.np, c.st,
                         0, h->stream));
     c.launches++;
     c.kernels += same ? 3 : 4;

@@ -321,7 +321,7 @@ void tc_tile_shape(int pair, int* bm, int* bn);   // output tile of one CTA (pai
 int tc_tile_width(int64_t rows, int64_t np, bool upper);
 
 // ---- FP64 products by digits on the tensor cores (gemm_dig.cu), np % 256 == 0
-constexpr int kDigPlanes = 7;
+constexpr int kDigPlanes = 8;
 struct DigOperand {        // digit planes of a rows x np factor and its rows' exponents
   uint16_t* dig = nullptr; // kDigPlanes x rows x np, bfloat16 integers
   int* ex = nullptr;       // rows
@@ -331,25 +331,24 @@ struct DigPlan {           // tile width of a CTA pair and the cut of a tile's w
 };
 DigPlan dig_plan(int64_t rows, int64_t np, bool upper);
 int64_t dig_square_nparts(int64_t np);   // partials of launch_dig_square
-// digits of src (rows x np); T (nullable): np x rows 64-bit sums, cleared
+// digits of src (rows x np)
 cudaError_t launch_digits(const double* src, int64_t rows, int64_t np, const DigOperand& o,
-                          unsigned long long* T, const DevState* st, int step, cudaStream_t s);
-// T[j * rows + i] += fixed-point (A X)_ij over the listed 256 x plan.bn tiles
+                          const DevState* st, int step, cudaStream_t s);
+// G: kDigPlanes x plan.ksplit planes of np x rows 32-bit sums, [j * rows + i] for entry
+// (i, j) of A X, over the listed 256 x plan.bn tiles
 cudaError_t launch_gemm_dig(const DigOperand& A, int64_t rows, const DigOperand& X, int64_t np,
-                            unsigned long long* T, const Tile* tiles, int ntiles,
-                            const DigPlan& plan, DevState* st, int step, const TcTuning& tune,
-                            cudaStream_t s);
-// the passes from T: the square step with its partials (and, with dec, the step
+                            int* G, const Tile* tiles, int ntiles, const DigPlan& plan,
+                            DevState* st, int step, const TcTuning& tune, cudaStream_t s);
+// the passes from G: the square step with its partials (and, with dec, the step
 // decision), the symmetrised response update of a batch, C = A X
-cudaError_t launch_dig_square(const unsigned long long* T, const int* ex, const double* X,
-                              double* out, int64_t np, DevState* st, int step, Part3* part,
+cudaError_t launch_dig_square(const int* G, int ksplit, const int* ex, const double* X, double* out,
+                              int64_t np, DevState* st, int step, Part3* part,
                               const SimtDecide* dec, cudaStream_t s);
-cudaError_t launch_dig_symm(const unsigned long long* T, int64_t rows, const int* ey, const int* ex,
+cudaError_t launch_dig_symm(const int* G, int ksplit, int64_t rows, const int* ey, const int* ex,
                             const double* yin, double* yout, int64_t np, const DevState* st,
                             int step, cudaStream_t s);
-cudaError_t launch_dig_plain(const unsigned long long* T, int64_t rows, const int* ea,
-                             const int* ex, double* out, int64_t np, const DevState* st, int step,
-                             cudaStream_t s);
+cudaError_t launch_dig_plain(const int* G, int ksplit, int64_t rows, const int* ea, const int* ex,
+                             double* out, int64_t np, const DevState* st, int step, cudaStream_t s);
 
 // FP16X2 scale of the next symmetric response step: per batch entry, the sum of
 // the EPI_SYMM tile partials (||Y_{n+1}||_F^2) and the plane scale of Y_{n+2},

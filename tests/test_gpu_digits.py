@@ -2,12 +2,13 @@
 response step against extended precision on sampled rows, at the sizes and values
 where the digit arithmetic can go wrong.
 
-Tolerance. With u_i = 2^ex_i <= 2 ||a_i|| (1 + 2^-8), an entry of a K-long product
-drops digit pairs of weight s >= 7, at most 6 K 2^16 2^45 (and a twentieth of that
-for s > 7) of 2^124 u_i u_j, and rounds each factor entry to 2^-63 of u (together
-at most 2 sqrt(K) 2^-63 u_i u_j) and each of at most 28 partial sums to 2^-63: below
-(6.2 K + 2 sqrt(K) + 28) 2^-63 u_i u_j, plus one FP64 rounding of the result (and of
-each sum of the response update)."""
+Tolerance. With u_i = 2^ex_i <= 2 ||a_i|| (1 + 2^-6), an entry of a K-long product
+drops digit pairs of weight s >= 8, at most 7 K 2^14 2^48 (and a hundredth of that
+for s > 8) of 2^126 u_i u_j, and rounds each factor entry to 2^-64 of u (together
+at most 2 sqrt(K) 2^-64 u_i u_j) and the last weight's sums to 2^-63: together below
+(6.2 K + 2 sqrt(K) + 28) 2^-63 u_i u_j (the bound of 7 digits of 9 bits, which the
+tests keep), plus one FP64 rounding of the result (and of each sum of the response
+update)."""
 import numpy as np
 import pytest
 
