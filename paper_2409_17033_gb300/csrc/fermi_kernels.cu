@@ -43,6 +43,7 @@ template <typename T>
 __global__ void __launch_bounds__(256)
     k_combine(T* __restrict__ out, int64_t np, int64_t n, const T* __restrict__ Z1, T z1,
               const T* __restrict__ Z2, T z2, const T* __restrict__ A, T a, T id, float* amax) {
+  dep_sync();
   constexpr int TE = comb_tile<T>();
   constexpr int V = TE / 4, R = 256 / V, P = TE / R;
   const int64_t t = blockIdx.x;
@@ -116,6 +117,7 @@ __global__ void __launch_bounds__(256)
 // out[0] = sum_{i < n} M[i, i] in FP64 (one block, fixed order)
 template <typename T>
 __global__ void k_trace(const T* __restrict__ M, int64_t np, int64_t n, double* out) {
+  dep_sync();
   __shared__ double red[32];
   double s = 0.0;
   for (int64_t i = threadIdx.x; i < n; i += blockDim.x) s += (double)M[i * np + i];
@@ -138,11 +140,11 @@ cudaError_t launch_combine(int mode, void* out, int64_t np, int64_t n, const voi
   const int64_t nb = np / (mode == SP2_MODE_FP64 ? comb_tile<double>() : comb_tile<float>());
   const dim3 grid((unsigned)(nb * (nb + 1) / 2)), block(256);
   if (mode == SP2_MODE_FP64)
-    k_combine<double><<<grid, block, 0, s>>>(
+    launch_dep(k_combine<double>, grid, block, 0, s, 
         static_cast<double*>(out), np, n, static_cast<const double*>(Z1), z1,
         static_cast<const double*>(Z2), z2, static_cast<const double*>(A), a, id, amax);
   else
-    k_combine<float><<<grid, block, 0, s>>>(
+    launch_dep(k_combine<float>, grid, block, 0, s, 
         static_cast<float*>(out), np, n, static_cast<const float*>(Z1), (float)z1,
         static_cast<const float*>(Z2), (float)z2, static_cast<const float*>(A), (float)a,
         (float)id, amax);
@@ -152,9 +154,9 @@ cudaError_t launch_combine(int mode, void* out, int64_t np, int64_t n, const voi
 cudaError_t launch_trace(int mode, const void* M, int64_t np, int64_t n, double* out,
                          cudaStream_t s) {
   if (mode == SP2_MODE_FP64)
-    k_trace<double><<<1, 1024, 0, s>>>(static_cast<const double*>(M), np, n, out);
+    launch_dep(k_trace<double>, 1, 1024, 0, s, static_cast<const double*>(M), np, n, out);
   else
-    k_trace<float><<<1, 1024, 0, s>>>(static_cast<const float*>(M), np, n, out);
+    launch_dep(k_trace<float>, 1, 1024, 0, s, static_cast<const float*>(M), np, n, out);
   return cudaGetLastError();
 }
 

@@ -132,11 +132,6 @@ k_gemm_dig(const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUt
   using G = Geo<BN>;
   constexpr int STAGES = G::STAGES;
   DevState* st = p.st;
-  {
-    // a pair takes this exit together: stop_at is fixed for the launch
-    const int m = *((volatile const int*)&st->stop_at);
-    if (m != 0 && p.step > m) return;
-  }
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~(uintptr_t)1023);
@@ -183,13 +178,19 @@ k_gemm_dig(const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUt
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
+  // nothing of the launches before is read up to here; a halted launch runs no unit
+  // (stop_at is fixed for the launch, so a pair agrees)
+  dep_sync();
+  const int stopped = *((volatile const int*)&st->stop_at);
+  const int nunits = stopped != 0 && p.step > stopped ? 0 : p.nunits;
+
   if (warp == 0) {
     // copy issuer: the whole warp (the waits by every lane, the copies by an elected one)
     int64_t g = 0;
     RingPos<STAGES> rp;
     const uint32_t ring = smem_u32(smem);
     bool ok = true;
-    for (int u = pair; u < p.nunits && ok; u += npairs) {
+    for (int u = pair; u < nunits && ok; u += npairs) {
       const Unit w = unit_of(p, u);
       const int arow = w.t.row0 + (int)rank * BM;
       const int brow = w.t.col0 + (int)rank * G::B_ROWS;
@@ -222,7 +223,7 @@ k_gemm_dig(const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUt
         const uint32_t pfull_peer = cluster_addr(smem_u32(pfull), 0);
         RingPos<STAGES> rp;
         bool ok = true;
-        for (int u = pair; u < p.nunits && ok; u += npairs) {
+        for (int u = pair; u < nunits && ok; u += npairs) {
           const Unit w = unit_of(p, u);
           const int n = pairs_per_part * (w.kb1 - w.kb0);
           for (int q = 0; q < n; ++q, rp.next()) {
@@ -240,7 +241,7 @@ k_gemm_dig(const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUt
       uint32_t gc = 0;
       RingPos<STAGES> rp;
       const uint64_t adesc0 = sdesc_sw128(smem_u32(smem));
-      for (int u = pair; u < p.nunits && ok; u += npairs) {
+      for (int u = pair; u < nunits && ok; u += npairs) {
         const Unit w = unit_of(p, u);
         const int nch = pairs_per_part * ((w.kb1 - w.kb0) / KCH);
         for (int c = 0; c < nch && ok; ++c, ++gc) {
@@ -279,7 +280,7 @@ k_gemm_dig(const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUt
     const uint32_t tempty_peer = !issuer ? cluster_addr(smem_u32(tempty), 0) : 0u;
     bool ok = true;
     uint32_t gc = 0;   // chunk counter: buffer gc & 1, phase (gc >> 1) & 1
-    for (int u = pair; u < p.nunits && ok; u += npairs) {
+    for (int u = pair; u < nunits && ok; u += npairs) {
       uint32_t mask;
       int kch;
       int* dst;
@@ -362,6 +363,7 @@ constexpr int kDigThreads = 128;
 __global__ void __launch_bounds__(kDigThreads)
 k_digits(const double* __restrict__ src, int64_t rows, int64_t np, uint16_t* __restrict__ dig,
          int* __restrict__ ex, const DevState* st, int step) {
+  dep_sync();
   if (halted_dig(st, step)) return;
   __shared__ uint32_t smax[kDigThreads / 32];
   __shared__ float ssum[kDigThreads / 32];
@@ -532,6 +534,7 @@ __global__ void __launch_bounds__(kPassThreads)
 k_dig_square(const Sums q, const int* __restrict__ ex,
              const double* __restrict__ X, double* __restrict__ out, int64_t np, int ntiles,
              DevState* st, int step, Part3* __restrict__ part, SimtDecide dec) {
+  dep_sync();
   if (halted_dig(st, step)) return;
   __shared__ double sm[2][TE][TE + 1];
   __shared__ double red[3][kPassThreads / 32];
@@ -623,6 +626,7 @@ __global__ void __launch_bounds__(kPassThreads)
 k_dig_symm(const Sums q, int64_t rows, const int* __restrict__ ey,
            const int* __restrict__ ex, const double* __restrict__ yin, double* __restrict__ yout,
            int64_t np, const DevState* st, int step) {
+  dep_sync();
   if (halted_dig(st, step)) return;
   __shared__ double za[TE][TE + 1], zb[TE][TE + 1];
   int64_t I, J;
@@ -667,6 +671,7 @@ __global__ void __launch_bounds__(kPassThreads)
 k_dig_plain(const Sums q, int64_t rows, const int* __restrict__ ea,
             const int* __restrict__ ex, double* __restrict__ out, int64_t np, const DevState* st,
             int step) {
+  dep_sync();
   if (halted_dig(st, step)) return;
   __shared__ double sm[TE][TE + 1];
   const int64_t i0 = (int64_t)blockIdx.y * TE, j0 = (int64_t)blockIdx.x * TE;
@@ -716,7 +721,9 @@ cudaError_t launch_bn(const CUtensorMap& am, const CUtensorMap& bm, const DParam
   const int res = resident_pairs<BN>();
   if (res < 1) return cudaErrorNotSupported;
   cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = 2;
   at[0].val.clusterDim.y = 1;
@@ -726,7 +733,7 @@ cudaError_t launch_bn(const CUtensorMap& am, const CUtensorMap& bm, const DParam
   cfg.dynamicSmemBytes = Geo<BN>::SMEM_BYTES;
   cfg.stream = s;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, k_gemm_dig<BN>, am, bm, p);
 }
 
@@ -773,7 +780,7 @@ DigPlan dig_plan(int64_t rows, int64_t np, bool upper) {
 
 cudaError_t launch_digits(const double* src, int64_t rows, int64_t np, const DigOperand& o,
                           const DevState* st, int step, cudaStream_t s) {
-  k_digits<<<(unsigned)rows, kDigThreads, 0, s>>>(src, rows, np, o.dig, o.ex, st, step);
+  launch_dep(k_digits, (unsigned)rows, kDigThreads, 0, s, src, rows, np, o.dig, o.ex, st, step);
   return cudaGetLastError();
 }
 
@@ -817,7 +824,7 @@ cudaError_t launch_dig_square(const int* G, int ksplit, const int* ex, const dou
                               const SimtDecide* dec, cudaStream_t s) {
   SimtDecide sd;
   if (dec) sd = *dec;
-  k_dig_square<<<(unsigned)dig_square_nparts(np), kPassThreads, 0, s>>>(
+  launch_dep(k_dig_square, (unsigned)dig_square_nparts(np), kPassThreads, 0, s, 
       Sums{G, np * np, ksplit}, ex, X, out, np, (int)tri_tiles(np), st, step, part, sd);
   return cudaGetLastError();
 }
@@ -826,7 +833,7 @@ cudaError_t launch_dig_symm(const int* G, int ksplit, int64_t rows, const int* e
                             const double* yin, double* yout, int64_t np, const DevState* st,
                             int step, cudaStream_t s) {
   const dim3 grid((unsigned)tri_tiles(np), (unsigned)(rows / np));
-  k_dig_symm<<<grid, kPassThreads, 0, s>>>(Sums{G, rows * np, ksplit}, rows, ey, ex, yin, yout, np, st,
+  launch_dep(k_dig_symm, grid, kPassThreads, 0, s, Sums{G, rows * np, ksplit}, rows, ey, ex, yin, yout, np, st,
                                            step);
   return cudaGetLastError();
 }
@@ -835,7 +842,7 @@ cudaError_t launch_dig_plain(const int* G, int ksplit, int64_t rows, const int* 
                              const int* ex, double* out, int64_t np, const DevState* st, int step,
                              cudaStream_t s) {
   const dim3 grid((unsigned)(np / TE), (unsigned)(rows / TE));
-  k_dig_plain<<<grid, kPassThreads, 0, s>>>(Sums{G, rows * np, ksplit}, rows, ea, ex, out, np, st, step);
+  launch_dep(k_dig_plain, grid, kPassThreads, 0, s, Sums{G, rows * np, ksplit}, rows, ea, ex, out, np, st, step);
   return cudaGetLastError();
 }
 

@@ -267,6 +267,8 @@ struct KParams {
   const float* q_scale;    // FP16X2: the plane scale of Q (nullable)
   const float* o_scale;    // FP16X2 EPI_SYMM: per batch entry, scale of the output planes
   float* zmax;             // FP16X2 EPI_PLAIN: per batch entry, receives max |C|
+  float* zero;             // EPI_PLAIN: nzero values cleared for the launch that follows
+  int nzero;
   unsigned long long wait_ns;
   int withhold;            // test hook: CTA 0 never issues its first load
   int tail;                // split-tail mode: st->plane1[step] selects the hi planes alone
@@ -496,12 +498,6 @@ k_gemm_tc(const __grid_constant__ KMaps maps, const __grid_constant__ KParams p)
   constexpr bool F16 = KIND == KIND_FP16X2;
   constexpr uint32_t kIdesc = idesc_for(F16, BM * CG, BN);
   DevState* st = p.st;
-  {
-    // a pair must take this exit together: stop_at is fixed for the launch, while
-    // the abort flag may be raised meanwhile (a pair sees it in its waits instead)
-    const int m = *((volatile const int*)&st->stop_at);
-    if ((m != 0 && p.step > m) || (!PAIR && *((volatile const int*)&st->abort_flag))) return;
-  }
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~(uintptr_t)1023);
@@ -525,28 +521,6 @@ k_gemm_tc(const __grid_constant__ KMaps maps, const __grid_constant__ KParams p)
   const bool issuer = rank == 0;
   const int unit = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
   const int nunits = PAIR ? (int)(gridDim.x >> 1) : (int)gridDim.x;
-  // segments of this launch: the split product, or in the split-tail mode's bulk
-  // steps the hi planes alone (one segment; two for the symmetric response)
-  const int nbase = (p.tail && st->plane1[p.step]) ? 1 : p.nbase;
-  const int nseg = EPI == EPI_SYMM ? 2 * nbase : nbase;
-  const int total_kb = nseg * p.nkb;
-  // TMEM chunks: the hi x hi segment of each split product (the last of its
-  // nbase segments; every segment in the split-tail bulk) every ch k-blocks, the
-  // smaller cross terms every ch_lo; both divide nkb, so no chunk spans two segments
-  const int ch_hi = p.ch, ch_lo = nbase == 1 ? p.ch : p.ch_lo;
-  const int nchunks = (nseg / nbase) * (p.nkb / ch_hi + (nbase - 1) * (p.nkb / ch_lo));
-  auto chunk_len = [&](int kb0) {
-    return ((kb0 / p.nkb) % nbase) == nbase - 1 ? ch_hi : ch_lo;
-  };
-  // persistent static schedule: this CTA (pair) handles tiles unit, unit + nunits, ...
-  // (block-sparse: the tile count comes from the device)
-  int ntiles = p.ntiles;
-  if constexpr (SPARSE) ntiles = *((volatile const int*)p.dyn_ntiles);
-  const int my_tiles = unit < ntiles ? (ntiles - 1 - unit) / nunits + 1 : 0;
-  // block-sparse: a cross-term chunk is a run of listed K blocks inside one dense
-  // chunk of ch_lo k-blocks (gsz K blocks of 256)
-  const int gsz = p.ch_lo >> 2;
-
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
       mbar_init(&full[s], 1);
@@ -583,6 +557,39 @@ k_gemm_tc(const __grid_constant__ KMaps maps, const __grid_constant__ KParams p)
   if constexpr (PAIR) cluster_sync();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+
+  // Up to here nothing of the launches before is read: the barriers' and TMEM's setup
+  // (2500 clocks) overlaps their end. A halted launch runs no tile (stop_at is fixed
+  // for the launch, so a pair agrees; the abort flag is seen in the waits).
+  dep_sync();
+  const int stopped = *((volatile const int*)&st->stop_at);
+  const bool halted = stopped != 0 && p.step > stopped;
+  // segments of this launch: the split product, or in the split-tail mode's bulk
+  // steps the hi planes alone (one segment; two for the symmetric response)
+  const int nbase = (p.tail && st->plane1[p.step]) ? 1 : p.nbase;
+  const int nseg = EPI == EPI_SYMM ? 2 * nbase : nbase;
+  const int total_kb = nseg * p.nkb;
+  // TMEM chunks: the hi x hi segment of each split product (the last of its
+  // nbase segments; every segment in the split-tail bulk) every ch k-blocks, the
+  // smaller cross terms every ch_lo; both divide nkb, so no chunk spans two segments
+  const int ch_hi = p.ch, ch_lo = nbase == 1 ? p.ch : p.ch_lo;
+  const int nchunks = (nseg / nbase) * (p.nkb / ch_hi + (nbase - 1) * (p.nkb / ch_lo));
+  auto chunk_len = [&](int kb0) {
+    return ((kb0 / p.nkb) % nbase) == nbase - 1 ? ch_hi : ch_lo;
+  };
+  // persistent static schedule: this CTA (pair) handles tiles unit, unit + nunits, ...
+  // (block-sparse: the tile count comes from the device)
+  int ntiles = p.ntiles;
+  if constexpr (SPARSE) ntiles = *((volatile const int*)p.dyn_ntiles);
+  const int my_tiles = !halted && unit < ntiles ? (ntiles - 1 - unit) / nunits + 1 : 0;
+  // block-sparse: a cross-term chunk is a run of listed K blocks inside one dense
+  // chunk of ch_lo k-blocks (gsz K blocks of 256)
+  const int gsz = p.ch_lo >> 2;
+
+  if constexpr (EPI == EPI_PLAIN) {
+    if (blockIdx.x == 0 && !halted)
+      for (int i = threadIdx.x; i < p.nzero; i += NUM_THREADS) p.zero[i] = 0.0f;
+  }
 
   if (warp == 0) {
     // copy issuer: the whole warp (the waits by every lane, the copies by an elected one)
@@ -911,7 +918,7 @@ k_gemm_tc(const __grid_constant__ KMaps maps, const __grid_constant__ KParams p)
   if constexpr (EPI == EPI_SQUARE && BN < BN_FULL) {
     // the last CTA to get here takes the step decision (the wide-tile kernels leave
     // it to its own launch: its code beside theirs costs them instruction cache)
-    if (p.dec.done) {
+    if (p.dec.done && !halted) {
       __shared__ int last;
       if (threadIdx.x == 0) {
         __threadfence();
@@ -1007,12 +1014,11 @@ cudaError_t launch_kind(const KMaps& maps, const KParams& p, int units, cudaStre
     }
   }
   const int n = units < resident ? units : resident;
-  if (CG == 1) {
-    kern<<<n, NUM_THREADS, smem, s>>>(maps, p);
-    return cudaGetLastError();
-  }
+  if (CG == 1) return launch_dep(kern, n, NUM_THREADS, smem, s, maps, p);
   cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = CG;
   at[0].val.clusterDim.y = 1;
@@ -1022,7 +1028,7 @@ cudaError_t launch_kind(const KMaps& maps, const KParams& p, int units, cudaStre
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = SPARSE ? 1 : 2;   // (block-sparse steps lose by early residency)
   return cudaLaunchKernelEx(&cfg, kern, maps, p);
 }
 
@@ -1186,6 +1192,8 @@ cudaError_t launch_gemm_tc(const TcLaunch& L, cudaStream_t s, char* errbuf, size
   p.q_scale = f16 ? L.q_scale : nullptr;
   p.o_scale = f16 ? L.o_scale : nullptr;
   p.zmax = f16 ? L.zmax : nullptr;
+  p.zero = L.zero;
+  p.nzero = L.zero ? L.nzero : 0;
   p.wait_ns = L.tune.wait_ns;
   p.withhold = L.tune.withhold;
   p.tail = L.tail;

@@ -52,6 +52,7 @@ __device__ double2 block_minmax(double lo, double hi) {
 // Row i contributes H_ii -/+ sum_{j != i} |H_ij| (Sec. II: spectral bound
 // estimates eps_min, eps_max, read as Gershgorin discs).
 __global__ void k_bounds(const void* H, int64_t n, int dtype, double2* part) {
+  dep_sync();
   double lo = INFINITY, hi = -INFINITY;
   for (int64_t i = blockIdx.x; i < n; i += gridDim.x) {
     double r = 0.0, d = 0.0;
@@ -90,6 +91,7 @@ __device__ void set_coefficients(DevState* st, double lo, double hi) {
 }
 
 __global__ void k_bounds_final(const double2* part, int nparts, DevState* st) {
+  dep_sync();
   double lo = INFINITY, hi = -INFINITY;
   for (int i = threadIdx.x; i < nparts; i += blockDim.x) {
     lo = nmin(lo, part[i].x);
@@ -99,18 +101,20 @@ __global__ void k_bounds_final(const double2* part, int nparts, DevState* st) {
   if (threadIdx.x == 0) set_coefficients(st, mm.x, mm.y);
 }
 
-__global__ void k_set_bounds(DevState* st, double lo, double hi) { set_coefficients(st, lo, hi); }
+__global__ void k_set_bounds(DevState* st, double lo, double hi) { dep_sync(); set_coefficients(st, lo, hi); }
 
 struct SigmaArg {
   int8_t s[SP2_MAX_ITER];
 };
 
 __global__ void k_set_sigma(DevState* st, SigmaArg a, int m) {
+  dep_sync();
   for (int i = threadIdx.x; i < m; i += blockDim.x) st->sigma[i + 1] = a.s[i];
 }
 
 // an adjoint recursion runs every step it is given and keeps no floor candidate
 __global__ void k_adjoint_state(DevState* st) {
+  dep_sync();
   st->stop_at = 0;
   st->keep_step = 0;
   st->abort_flag = 0;
@@ -158,6 +162,7 @@ __device__ __forceinline__ void atomic_max_nonneg(float* addr, float v) {
 __global__ void k_init(const void* src, int64_t n, int64_t np, int64_t batch, int dtype,
                        int diag_only, int symmetrize, double alpha, double beta, int mode,
                        MatBuf dst, Part3* part, float* ymax, int coef, const DevState* st) {
+  dep_sync();
   if (coef == INIT_STATE) {
     alpha = st->alpha;
     beta = st->beta;
@@ -205,12 +210,14 @@ __global__ void k_init(const void* src, int64_t n, int64_t np, int64_t batch, in
 
 // ------------------------------------------------------------ decide
 __global__ void k_decide(const Part3* part, DevState* st, DecideParams p) {
+  dep_sync();
   decide_block(part, st, p);
 }
 
 template <typename T>
 __global__ void k_keep_best(const T* __restrict__ src, T* __restrict__ dst, int64_t count,
                             const DevState* st, int step) {
+  dep_sync();
   if (*((volatile const int*)&st->keep_step) != step) return;
   const int64_t n4 = count / 4;   // count is a multiple of np^2, np % 256 == 0
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n4;
@@ -293,6 +300,7 @@ template <typename ZT, int MODE>
 __global__ void __launch_bounds__(kSymThreads)
     k_symm_update(const ZT* __restrict__ Z, MatBuf yin, MatBuf yout, int64_t np,
                   const DevState* st, int step, ScaleBuf sc, int slot_in, int slot_out) {
+  dep_sync();
   if (halted(st, step)) return;
   constexpr int TE = sym_tile<ZT>();
   constexpr int V = TE / 4;                // 4-entry vectors per tile row
@@ -313,10 +321,13 @@ __global__ void __launch_bounds__(kSymThreads)
   float s = 1.0f;
   if (MODE == SP2_MODE_FP16X2) {
     // |Y_{n+1}| <= |Z_ij| + |Z_ji| (+ 2 |Y_n| for sigma<0), elementwise
-    float bound = 2.0f * sc.zmax[b];
+    float bound = 2.0f * sc.zmax[(step & 1) * sc.B + b];
     if (sg < 0) bound += 2.0f * sc.ymax[slot_in * sc.B + b];
     s = pow2_scale(bound);
-    if (t == 0 && threadIdx.x == 0) sc.yscale[slot_out * sc.B + b] = s;
+    if (t == 0 && threadIdx.x == 0) {
+      sc.yscale[slot_out * sc.B + b] = s;
+      sc.zmax[(1 - (step & 1)) * sc.B + b] = 0.0f;   // for the next step's product
+    }
   }
   const int64_t rI = I * TE, rJ = J * TE;
 #pragma unroll
@@ -364,6 +375,7 @@ __global__ void __launch_bounds__(kSymThreads)
 // ------------------------------------------------------------ output copy
 __global__ void k_copy_out(MatBuf src, int64_t n, int64_t np, int64_t batch, int mode,
                            double scale, void* dst, int dtype, const DevState* beta_state) {
+  dep_sync();
   if (beta_state) scale *= beta_state->beta;
   const int64_t total = batch * n * n;
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
@@ -443,6 +455,7 @@ __device__ __forceinline__ void two_sum_add_sq(float& s, float& c, float x) {
 // squares per row segment, added in FP64.
 __global__ void k_init_x4(const float* __restrict__ src, int64_t n, int64_t np, int mode,
                           MatBuf dst, Part3* part, const DevState* st) {
+  dep_sync();
   const double alpha = st->alpha, beta = st->beta;
   const F2 bc = split_coef(beta);
   double t1 = 0.0, t2 = 0.0;
@@ -483,6 +496,7 @@ __global__ void k_init_x4(const float* __restrict__ src, int64_t n, int64_t np, 
 // part of the row with TwoSum in FP32, four 16-byte loads in flight, and moves
 // the sum and its error to FP64 after each group of 16 entries; lanes add in FP64.
 __global__ void k_bounds_x4(const float* __restrict__ H, int64_t n, double2* part) {
+  dep_sync();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int64_t q = n / 4;
   double lo = INFINITY, hi = -INFINITY;
@@ -528,6 +542,7 @@ __global__ void k_bounds_x4(const float* __restrict__ H, int64_t n, double2* par
 // is applied as an FP32 product with the split coefficient (mul_coef)
 __global__ void k_copy_out_x4(const float* __restrict__ src, int64_t n, int64_t np, int64_t batch,
                               double scale, float* __restrict__ dst, const DevState* beta_state) {
+  dep_sync();
   if (beta_state) scale *= beta_state->beta;
   const bool scaled = scale != 1.0;
   const F2 sc = split_coef(scale);
@@ -551,6 +566,7 @@ __global__ void k_copy_out_x4(const float* __restrict__ src, int64_t n, int64_t 
 
 // hi/lo (and BF16X3 mid) planes from the FP32 master; total is a multiple of 4
 __global__ void k_split(MatBuf m, int64_t total, int mode) {
+  dep_sync();
   const int64_t total4 = total / 4;
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total4;
        t += (int64_t)gridDim.x * blockDim.x) {
@@ -570,6 +586,7 @@ __global__ void k_split(MatBuf m, int64_t total, int mode) {
 }
 
 __global__ void k_scales_from_max(ScaleBuf sc, int slot) {
+  dep_sync();
   for (int64_t b = threadIdx.x; b < sc.B; b += blockDim.x)
     sc.yscale[slot * sc.B + b] = pow2_scale(sc.ymax[slot * sc.B + b]);
 }
@@ -577,6 +594,7 @@ __global__ void k_scales_from_max(ScaleBuf sc, int slot) {
 // FP16X2 planes of a batch of sc.B matrices of `per` entries each (per % 4 == 0),
 // each with its slot's power-of-two scale
 __global__ void k_split_scaled(MatBuf m, int64_t per, ScaleBuf sc, int slot) {
+  dep_sync();
   const int64_t total4 = per * sc.B / 4;
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total4;
        t += (int64_t)gridDim.x * blockDim.x) {
@@ -598,6 +616,7 @@ __global__ void k_split_scaled(MatBuf m, int64_t per, ScaleBuf sc, int slot) {
 // therefore fixed by ||Y_{n+1}||_F before the step that writes it.
 __global__ void k_sym_scale(const Part3* part, int ppt, const Tile* tiles, int ntiles, int64_t np,
                             const DevState* st, int step, float* scale_out) {
+  dep_sync();
   if (st) {
     const int m = st->stop_at;
     if ((m != 0 && step > m) || st->abort_flag) return;
@@ -612,6 +631,7 @@ __global__ void k_sym_scale(const Part3* part, int ppt, const Tile* tiles, int n
 }
 
 __global__ void k_fro_part(const float* __restrict__ m, int64_t per, double* part) {
+  dep_sync();
   const float* x = m + blockIdx.y * per;
   double acc = 0.0;
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < per;
@@ -624,6 +644,7 @@ __global__ void k_fro_part(const float* __restrict__ m, int64_t per, double* par
 }
 
 __global__ void k_fro_final(const double* part, int nparts, float* scale_out) {
+  dep_sync();
   double acc = 0.0;
   for (int i = threadIdx.x; i < nparts; i += blockDim.x) acc += part[blockIdx.x * nparts + i];
   acc = block_sum(acc);
@@ -726,6 +747,7 @@ template <typename T, int VEC, int LT>
 __global__ void __launch_bounds__(256, 2)
 k_contract_dense(const T* __restrict__ P, int64_t L, const T* __restrict__ Q, int64_t K, int64_t nn,
                  double* part, int nparts, int64_t y0) {
+  dep_sync();
   using Acc = typename CtrAcc<T>::type;
   constexpr int NP = LT * kCtrKT;
   const int64_t ktiles = (K + kCtrKT - 1) / kCtrKT;
@@ -771,6 +793,7 @@ k_contract_dense(const T* __restrict__ P, int64_t L, const T* __restrict__ Q, in
 template <typename T>
 __global__ void k_contract_diag(const T* __restrict__ P, const T* __restrict__ Q, int64_t K,
                                 int64_t n, double* part, int nparts, int64_t y0) {
+  dep_sync();
   const int64_t pair = y0 + blockIdx.y;
   const int64_t l = pair / K, k = pair % K;
   double acc = 0.0;
@@ -782,6 +805,7 @@ __global__ void k_contract_diag(const T* __restrict__ P, const T* __restrict__ Q
 }
 
 __global__ void k_contract_final(const double* part, int nparts, double* out) {
+  dep_sync();
   const int64_t pair = blockIdx.x;
   double acc = 0.0;
   for (int i = threadIdx.x; i < nparts; i += blockDim.x) acc += part[pair * nparts + i];
@@ -804,10 +828,10 @@ int bounds_nparts(int64_t n) { return (int)(n < 1024 ? (n < 1 ? 1 : n) : 1024); 
 cudaError_t launch_bounds(const void* H, int64_t n, int dtype, double2* part, int nparts,
                           DevState* st, cudaStream_t s) {
   if (dtype == SP2_F32 && n % 4 == 0 && (reinterpret_cast<uintptr_t>(H) & 15u) == 0)
-    k_bounds_x4<<<nparts, kRedThreads, 0, s>>>(static_cast<const float*>(H), n, part);
+    launch_dep(k_bounds_x4, nparts, kRedThreads, 0, s, static_cast<const float*>(H), n, part);
   else
-    k_bounds<<<nparts, kRedThreads, 0, s>>>(H, n, dtype, part);
-  k_bounds_final<<<1, 128, 0, s>>>(part, nparts, st);
+    launch_dep(k_bounds, nparts, kRedThreads, 0, s, H, n, dtype, part);
+  launch_dep(k_bounds_final, 1, 128, 0, s, part, nparts, st);
   return cudaGetLastError();
 }
 
@@ -819,18 +843,18 @@ cudaError_t launch_init(const void* src, int64_t n, int64_t np, int64_t batch, i
                         int coef, const DevState* st) {
   if (coef == INIT_STATE && part && batch == 1 && dtype == SP2_F32 && !diag_only && !symmetrize &&
       !ymax && split_mode(mode) && n % 4 == 0 && (reinterpret_cast<uintptr_t>(src) & 15u) == 0) {
-    k_init_x4<<<nparts, kRedThreads, 0, s>>>(static_cast<const float*>(src), n, np, mode, dst, part,
+    launch_dep(k_init_x4, nparts, kRedThreads, 0, s, static_cast<const float*>(src), n, np, mode, dst, part,
                                              st);
     return cudaGetLastError();
   }
   int grid = part ? nparts : grid_for(batch * np, 1, 4096);
-  k_init<<<grid, kRedThreads, 0, s>>>(src, n, np, batch, dtype, diag_only, symmetrize, alpha,
+  launch_dep(k_init, grid, kRedThreads, 0, s, src, n, np, batch, dtype, diag_only, symmetrize, alpha,
                                       beta, mode, dst, part, ymax, coef, st);
   return cudaGetLastError();
 }
 
 cudaError_t launch_set_bounds(DevState* st, double eps_min, double eps_max, cudaStream_t s) {
-  k_set_bounds<<<1, 1, 0, s>>>(st, eps_min, eps_max);
+  launch_dep(k_set_bounds, 1, 1, 0, s, st, eps_min, eps_max);
   return cudaGetLastError();
 }
 
@@ -838,29 +862,30 @@ cudaError_t launch_set_sigma(DevState* st, const int8_t* sigma, int m, cudaStrea
   if (m < 0 || m > SP2_MAX_ITER) return cudaErrorInvalidValue;
   SigmaArg a;
   for (int i = 0; i < SP2_MAX_ITER; ++i) a.s[i] = i < m ? sigma[i] : 0;
-  k_set_sigma<<<1, 256, 0, s>>>(st, a, m);
+  launch_dep(k_set_sigma, 1, 256, 0, s, st, a, m);
   return cudaGetLastError();
 }
 
 cudaError_t launch_adjoint_state(DevState* st, cudaStream_t s) {
-  k_adjoint_state<<<1, 1, 0, s>>>(st);
+  launch_dep(k_adjoint_state, 1, 1, 0, s, st);
   return cudaGetLastError();
 }
 
 cudaError_t launch_keep_best(const void* src, void* dst, int64_t count, int mode, const DevState* st,
                              int step, cudaStream_t s) {
-  const int grid = 2 * 152 * 4;
+  // two blocks per SM: most launches have nothing to copy
+  const int grid = 2 * 152;
   if (mode == SP2_MODE_FP64)
-    k_keep_best<double><<<grid, 256, 0, s>>>(static_cast<const double*>(src),
+    launch_dep(k_keep_best<double>, grid, 512, 0, s, static_cast<const double*>(src),
                                              static_cast<double*>(dst), count, st, step);
   else
-    k_keep_best<float><<<grid, 256, 0, s>>>(static_cast<const float*>(src), static_cast<float*>(dst),
+    launch_dep(k_keep_best<float>, grid, 512, 0, s, static_cast<const float*>(src), static_cast<float*>(dst),
                                             count, st, step);
   return cudaGetLastError();
 }
 
 cudaError_t launch_decide(const Part3* part, DevState* st, DecideParams p, cudaStream_t s) {
-  k_decide<<<1, kRedThreads, 0, s>>>(part, st, p);
+  launch_dep(k_decide, 1, kRedThreads, 0, s, part, st, p);
   return cudaGetLastError();
 }
 
@@ -871,19 +896,19 @@ cudaError_t launch_symm_update(const void* Z, MatBuf y_in, MatBuf y_out, int64_t
   const int64_t nb = np / (mode == SP2_MODE_FP64 ? sym_tile<double>() : sym_tile<float>());
   dim3 grid((unsigned)(nb * (nb + 1) / 2), (unsigned)batch), block(kSymThreads);
   if (mode == SP2_MODE_FP64)
-    k_symm_update<double, SP2_MODE_FP64><<<grid, block, 0, s>>>(
+    launch_dep(k_symm_update<double, SP2_MODE_FP64>, grid, block, 0, s, 
         static_cast<const double*>(Z), y_in, y_out, np, st, step, sc, slot_in, slot_out);
   else if (mode == SP2_MODE_FP32)
-    k_symm_update<float, SP2_MODE_FP32><<<grid, block, 0, s>>>(
+    launch_dep(k_symm_update<float, SP2_MODE_FP32>, grid, block, 0, s, 
         static_cast<const float*>(Z), y_in, y_out, np, st, step, sc, slot_in, slot_out);
   else if (mode == SP2_MODE_BF16X2)
-    k_symm_update<float, SP2_MODE_BF16X2><<<grid, block, 0, s>>>(
+    launch_dep(k_symm_update<float, SP2_MODE_BF16X2>, grid, block, 0, s, 
         static_cast<const float*>(Z), y_in, y_out, np, st, step, sc, slot_in, slot_out);
   else if (mode == SP2_MODE_BF16X3)
-    k_symm_update<float, SP2_MODE_BF16X3><<<grid, block, 0, s>>>(
+    launch_dep(k_symm_update<float, SP2_MODE_BF16X3>, grid, block, 0, s, 
         static_cast<const float*>(Z), y_in, y_out, np, st, step, sc, slot_in, slot_out);
   else
-    k_symm_update<float, SP2_MODE_FP16X2><<<grid, block, 0, s>>>(
+    launch_dep(k_symm_update<float, SP2_MODE_FP16X2>, grid, block, 0, s, 
         static_cast<const float*>(Z), y_in, y_out, np, st, step, sc, slot_in, slot_out);
   return cudaGetLastError();
 }
@@ -893,31 +918,31 @@ cudaError_t launch_copy_out(MatBuf src, int64_t n, int64_t np, int64_t batch, in
                             const DevState* beta_state) {
   if (mode != SP2_MODE_FP64 && dtype == SP2_F32 && n % 4 == 0 &&
       (reinterpret_cast<uintptr_t>(dst) & 15u) == 0) {
-    k_copy_out_x4<<<grid_for(batch * n, 1, 8192), 256, 0, s>>>(
+    launch_dep(k_copy_out_x4, grid_for(batch * n, 1, 8192), 256, 0, s, 
         static_cast<const float*>(src.master), n, np, batch, scale, static_cast<float*>(dst),
         beta_state);
     return cudaGetLastError();
   }
-  k_copy_out<<<grid_for(batch * n * n, 256, 8192), 256, 0, s>>>(src, n, np, batch, mode, scale,
+  launch_dep(k_copy_out, grid_for(batch * n * n, 256, 8192), 256, 0, s, src, n, np, batch, mode, scale,
                                                                  dst, dtype, beta_state);
   return cudaGetLastError();
 }
 
 cudaError_t launch_split(MatBuf m, int64_t rows, int64_t np, int mode, cudaStream_t s) {
-  k_split<<<grid_for(rows * np / 4, 256, 8192), 256, 0, s>>>(m, rows * np, mode);
+  launch_dep(k_split, grid_for(rows * np / 4, 256, 8192), 256, 0, s, m, rows * np, mode);
   return cudaGetLastError();
 }
 
 cudaError_t launch_split_scaled(MatBuf m, int64_t np, ScaleBuf sc, int slot, cudaStream_t s) {
-  k_scales_from_max<<<1, 256, 0, s>>>(sc, slot);
-  k_split_scaled<<<grid_for(sc.B * np * np / 4, 256, 8192), 256, 0, s>>>(m, np * np, sc, slot);
+  launch_dep(k_scales_from_max, 1, 256, 0, s, sc, slot);
+  launch_dep(k_split_scaled, grid_for(sc.B * np * np / 4, 256, 8192), 256, 0, s, m, np * np, sc, slot);
   return cudaGetLastError();
 }
 
 cudaError_t launch_sym_scale(const Part3* part, int ppt, const Tile* tiles, int ntiles, int64_t np,
                              int64_t batch, const DevState* st, int step, float* scale_out,
                              cudaStream_t s) {
-  k_sym_scale<<<(unsigned)batch, kRedThreads, 0, s>>>(part, ppt, tiles, ntiles, np, st, step,
+  launch_dep(k_sym_scale, (unsigned)batch, kRedThreads, 0, s, part, ppt, tiles, ntiles, np, st, step,
                                                         scale_out);
   return cudaGetLastError();
 }
@@ -927,8 +952,8 @@ int fro_nparts() { return 256; }
 cudaError_t launch_fro_scale(const float* master, int64_t np, int64_t batch, double* part,
                              int nparts, float* scale_out, cudaStream_t s) {
   dim3 grid((unsigned)nparts, (unsigned)batch);
-  k_fro_part<<<grid, kRedThreads, 0, s>>>(master, np * np, part);
-  k_fro_final<<<(unsigned)batch, kRedThreads, 0, s>>>(part, nparts, scale_out);
+  launch_dep(k_fro_part, grid, kRedThreads, 0, s, master, np * np, part);
+  launch_dep(k_fro_final, (unsigned)batch, kRedThreads, 0, s, part, nparts, scale_out);
   return cudaGetLastError();
 }
 
@@ -951,7 +976,7 @@ void contract_rows(const void* P, int64_t L, const void* Q, int64_t K, int64_t n
   for (int64_t y0 = 0; y0 < rows; y0 += kMaxY) {
     const int64_t ny = (rows - y0) < kMaxY ? (rows - y0) : kMaxY;
     const dim3 grid((unsigned)nparts, (unsigned)ny);
-    k_contract_dense<T, VEC, LT><<<grid, 256, 0, s>>>(static_cast<const T*>(P), L,
+    launch_dep(k_contract_dense<T, VEC, LT>, grid, 256, 0, s, static_cast<const T*>(P), L,
                                                       static_cast<const T*>(Q), K, nn, part,
                                                       nparts, y0);
   }
@@ -980,11 +1005,11 @@ cudaError_t launch_contract(const void* P, int64_t L, const void* Q, int64_t K, 
       const int64_t ny = (rows - y0) < kMaxY ? (rows - y0) : kMaxY;
       const dim3 grid((unsigned)nparts, (unsigned)ny);
       if (dtype == SP2_F64)
-        k_contract_diag<double><<<grid, 256, 0, s>>>(static_cast<const double*>(P),
+        launch_dep(k_contract_diag<double>, grid, 256, 0, s, static_cast<const double*>(P),
                                                      static_cast<const double*>(Q), K, n, part,
                                                      nparts, y0);
       else
-        k_contract_diag<float><<<grid, 256, 0, s>>>(static_cast<const float*>(P),
+        launch_dep(k_contract_diag<float>, grid, 256, 0, s, static_cast<const float*>(P),
                                                     static_cast<const float*>(Q), K, n, part,
                                                     nparts, y0);
     }
@@ -995,7 +1020,7 @@ cudaError_t launch_contract(const void* P, int64_t L, const void* Q, int64_t K, 
     if (al && nn % 4 == 0) contract_dense<float, 4>(P, L, Q, K, nn, part, nparts, s);
     else contract_dense<float, 1>(P, L, Q, K, nn, part, nparts, s);
   }
-  k_contract_final<<<(unsigned)(L * K), 256, 0, s>>>(part, nparts, out);
+  launch_dep(k_contract_final, (unsigned)(L * K), 256, 0, s, part, nparts, out);
   return cudaGetLastError();
 }
 

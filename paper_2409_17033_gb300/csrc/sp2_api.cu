@@ -186,7 +186,7 @@ int mat(sp2_handle_t h, const std::string& name, int64_t rows, int64_t np, int m
 // FP16X2 per-matrix scale state for a batch of B response matrices
 int scales(sp2_handle_t h, const std::string& name, int64_t B, ScaleBuf* sc) {
   void* p;
-  TRY(ws(h, name, (size_t)B * 5 * sizeof(float), &p));
+  TRY(ws(h, name, (size_t)B * 6 * sizeof(float), &p));
   float* f = static_cast<float*>(p);
   sc->ymax = f;
   sc->yscale = f + 2 * B;
@@ -718,7 +718,6 @@ int response_step(Ctx& c, const MatBuf& x, const MatBuf& yin, const MatBuf& yout
   }
   if (split) {
     char eb[256] = {0};
-    if (f16) CK(cudaMemsetAsync(sc.zmax, 0, sizeof(float) * batch, h->stream));
     L.epi = EPI_PLAIN;
     L.P = TcOperand{yin.hi, yin.lo, rows, yin.mid};
     L.Q = TcOperand{x.hi, x.lo, c.np, x.mid};
@@ -730,7 +729,10 @@ int response_step(Ctx& c, const MatBuf& x, const MatBuf& yin, const MatBuf& yout
     L.bn = bn;
     if (f16) {
       L.p_scale = sc.yscale + slot_in * sc.B;
-      L.zmax = sc.zmax;
+      // (the update that follows reads this parity's maxima and clears the other's)
+      L.zmax = sc.zmax + (step & 1) * sc.B;
+      L.zero = sc.ymax + slot_out * sc.B;
+      L.nzero = (int)batch;
     }
     cudaError_t e = launch_gemm_tc(L, h->stream, eb, sizeof eb);
     if (e != cudaSuccess) return fail(h, SP2_ECUDA, "response product: %s %s", cudaGetErrorString(e), eb);
@@ -742,7 +744,6 @@ int response_step(Ctx& c, const MatBuf& x, const MatBuf& yin, const MatBuf& yout
     CK(cudaEventRecord(e1, h->stream));
     c.timed.push_back({step, 0});
   }
-  if (f16) CK(cudaMemsetAsync(sc.ymax + slot_out * sc.B, 0, sizeof(float) * batch, h->stream));
   CK(launch_symm_update(z, yin, yout, c.np, batch, c.mode, c.st, step, sc, slot_in, slot_out,
                         h->stream));
   c.launches++;
@@ -988,7 +989,7 @@ int run_sp2(sp2_handle_t h, const void* Hd, int64_t n, int dtype, double nocc, c
     const bool f16 = mode == SP2_MODE_FP16X2;
     if (f16) {
       TRY(scales(h, "Y.scale", ybatch, &sc));
-      CK(cudaMemsetAsync(sc.ymax, 0, sizeof(float) * 2 * ybatch, h->stream));
+      CK(cudaMemsetAsync(sc.ymax, 0, sizeof(float) * 6 * ybatch, h->stream));
     }
     CK(launch_init(Bd, n, np, ybatch, dtype, b_diag, 0, 0.0, 0.0, mode, Y[1], nullptr, 0,
                    f16 ? sc.ymax + 1 * ybatch : nullptr, h->stream, INIT_STATE_BETA, h->d_state));
@@ -1199,7 +1200,7 @@ int run_adjoint(sp2_handle_t h, const void* Bd, int64_t batch, int b_diag, int s
   const bool f16 = mode == SP2_MODE_FP16X2;
   if (f16) {
     TRY(scales(h, "G.scale", batch, &sc));
-    CK(cudaMemsetAsync(sc.ymax, 0, sizeof(float) * 2 * batch, h->stream));
+    CK(cudaMemsetAsync(sc.ymax, 0, sizeof(float) * 6 * batch, h->stream));
   }
   CK(launch_init(Bd, n, np, batch, dtype, b_diag, symmetrize, 0.0, 1.0, mode, G[gs], nullptr, 0,
                  f16 ? sc.ymax + gs * batch : nullptr, h->stream));

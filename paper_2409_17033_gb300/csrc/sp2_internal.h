@@ -128,7 +128,7 @@ __device__ __forceinline__ float pow2_scale(float bound) {
 struct ScaleBuf {
   float* ymax = nullptr;    // [2][B] max |Y| of the matrix in each ping-pong slot
   float* yscale = nullptr;  // [2][B] power-of-two scale of each slot's fp16 planes
-  float* zmax = nullptr;    // [B]    max |Z| of the current step's product Z = Y X
+  float* zmax = nullptr;    // [2][B] max |Z| of a step's product Z = Y X, by step parity
   int64_t B = 0;
 };
 
@@ -148,6 +148,32 @@ struct Tile {       // one output tile of a product kernel
   int row0;         // first output row (within the stacked A operand)
   int col0;         // first output column
 };
+
+// ---------------------------------------------------------------- dependent launches
+// The kernels of a step follow one another within microseconds. Launched as
+// programmatic dependents, a kernel's blocks become resident while the one before
+// still runs, and wait in dep_sync (first thing in every kernel, before any early
+// exit) until it has completed and its writes are visible; as every kernel waits for
+// the one before it, all earlier ones are then complete too.
+__device__ __forceinline__ void dep_sync() {
+  asm volatile("griddepcontrol.launch_dependents;\n\tgriddepcontrol.wait;" ::: "memory");
+}
+
+template <typename... P, typename... A>
+inline cudaError_t launch_dep(void (*kern)(P...), dim3 grid, dim3 block, size_t smem,
+                              cudaStream_t s, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
 
 // ---------------------------------------------------------------- launchers
 // elementwise / reduction kernels (kernels_elem.cu)
@@ -274,6 +300,8 @@ struct TcLaunch {
   const float* q_scale = nullptr;  // FP16X2: the plane scale of Q (nullable)
   const float* o_scale = nullptr;  // FP16X2 EPI_SYMM: per batch entry, scale of the output planes
   float* zmax = nullptr;           // FP16X2 EPI_PLAIN: per batch entry, receives max |C|
+  float* zero = nullptr;           // EPI_PLAIN: nzero floats the launch clears
+  int nzero = 0;
   int tail = 0;                    // split-tail mode (st->plane1 decides per step)
   TcTuning tune;
   // block-sparse square (CTA pairs): tiles, their count and their K-block lists

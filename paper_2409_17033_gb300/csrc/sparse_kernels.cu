@@ -32,6 +32,7 @@ __device__ __forceinline__ bool halted_at(const DevState* st, int step) {
 
 // ||block (I, J)||_F^2 of the master, upper blocks only; one CTA per block
 __global__ void k_block_norms(const float* __restrict__ x, int64_t np, int nb, double* nrm2) {
+  dep_sync();
   int I = 0, rem = blockIdx.x;
   while (rem >= nb - I) {   // blockIdx.x enumerates I <= J row by row
     rem -= nb - I;
@@ -99,6 +100,7 @@ __device__ __forceinline__ void order_ij(int x, int nb, int& I, int& J) {
 }
 
 __global__ void __launch_bounds__(kPlanThreads, 1) k_sparse_plan(PlanArgs a) {
+  dep_sync();
   if (!a.init && halted_at(a.st, a.step)) return;
   const int nb = a.nb;
   const int tid = threadIdx.x;
@@ -224,6 +226,7 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_sparse_plan(PlanArgs a) {
 // zero the listed blocks (and their mirrors) of master and planes
 __global__ void k_zero_blocks(const uint32_t* zero, const int* nzero, MatBuf x, int64_t np,
                               int mode, const DevState* st, int step, int init) {
+  dep_sync();
   if (!init && halted_at(st, step)) return;
   const int n = *nzero;
   const bool x3 = mode == SP2_MODE_BF16X3;
