@@ -79,14 +79,29 @@ struct PlanArgs {
   int step;
 };
 
-__device__ double cta_sum(double v, double* red) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+// N sums over the block, in every thread. The warps' sums are added by one warp each
+// and shared: added by all 1024 threads, their FP64 instructions (64 clocks a warp)
+// took 8 us a sum.
+template <int N>
+__device__ void cta_sums(double (&v)[N], double (*red)[kPlanThreads / 32]) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int i = 0; i < N; ++i)
+    for (int o = 16; o > 0; o >>= 1) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
   __syncthreads();
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  if (lane == 0)
+#pragma unroll
+    for (int i = 0; i < N; ++i) red[i][warp] = v[i];
   __syncthreads();
-  double s = 0.0;
-  for (int w = 0; w < kPlanThreads / 32; ++w) s += red[w];
-  return s;   // in every thread
+  if (warp < N) {
+    double s = red[warp][lane];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    __syncwarp();
+    if (lane == 0) red[warp][0] = s;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < N; ++i) v[i] = red[i][0];
 }
 
 // candidate x of the grouped tile order (groups of 8 block rows sweep the block
@@ -105,9 +120,9 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_sparse_plan(PlanArgs a) {
   const int nb = a.nb;
   const int tid = threadIdx.x;
   __shared__ unsigned long long bits[kMaxSparseBlocks][kWords];   // mask rows of X~_{n+1}
-  __shared__ double red[kPlanThreads / 32];
+  __shared__ double red[4][kPlanThreads / 32];
   __shared__ int scan[kPlanThreads];
-  __shared__ int nz;
+  __shared__ int nz, nwork;
   const int ntin = a.init ? 0 : *a.ntiles_in;
 
   // block norms^2 of the new iterate; -1 marks a block the square did not form
@@ -158,11 +173,13 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_sparse_plan(PlanArgs a) {
       a.zero[z] = ((uint32_t)I << 16) | (uint32_t)J;
     }
   }
-  t1 = cta_sum(t1, red);
-  t2 = cta_sum(t2, red);
-  f = cta_sum(f, red);
-  drop2 = cta_sum(drop2, red);
-  // (cta_sum's barriers also order the mask bits before the listing below)
+  double sums[4] = {t1, t2, f, drop2};
+  cta_sums(sums, red);
+  t1 = sums[0];
+  t2 = sums[1];
+  f = sums[2];
+  drop2 = sums[3];
+  // (cta_sums' barriers also order the mask bits before the listing below)
 
   // the next square: upper tiles with at least one K block, in grouped order;
   // each thread takes a contiguous range of candidates, counts, then writes
@@ -187,7 +204,6 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_sparse_plan(PlanArgs a) {
     __syncthreads();
   }
   int pos = scan[tid] - mine;
-  double work = 0.0;
   for (int x = x0; x < x1; ++x) {
     int I, J;
     order_ij(x, nb, I, J);
@@ -208,9 +224,15 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_sparse_plan(PlanArgs a) {
       ++pos;
     }
   }
-  if (!a.init)
+  if (tid == 0) nwork = 0;
+  __syncthreads();
+  if (!a.init) {
+    int work = 0;   // at most 256^3 / 2 K blocks
     for (int t = tid; t < ntin; t += kPlanThreads) work += a.kcnt_in[t];
-  work = cta_sum(work, red);
+    work = __reduce_add_sync(0xffffffffu, work);
+    if ((tid & 31) == 0) atomicAdd(&nwork, work);
+  }
+  __syncthreads();
   if (tid == 0) {
     *a.ntiles_out = scan[kPlanThreads - 1];
     *a.nzero = nz;
@@ -218,7 +240,7 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_sparse_plan(PlanArgs a) {
     if (!a.init) {
       // the square just done: its share of the upper blocks and its 256-wide K blocks
       if (a.step <= SP2_MAX_ITER) a.st->fill[a.step] = (double)ntin / (0.5 * nb * (nb + 1));
-      a.st->work_kblocks += work;
+      a.st->work_kblocks += (double)nwork;
     }
   }
 }
