@@ -147,17 +147,104 @@ k_gemm_simt(const T* __restrict__ A, const T* __restrict__ X, int64_t np, int ep
   }
 }
 
+// ------------------------------------------------------------ small FP64
+// 8 x 8 tiles for matrices whose 16 x 16 tiles would leave most SMs idle (36 tiles at
+// np = 128), with the K axis halved between two groups of 64 threads: one warp per
+// scheduler, each np / 2 fused multiply-adds long (64 clocks a warp and instruction on
+// the FP64 pipe bound it: 4100 clocks at np = 128, where the 16 x 16 tile takes 16400).
+// The whole K panel of both factors sits in shared memory.
+constexpr int kSmallMaxN = 192;
+
+__global__ void __launch_bounds__(128)
+k_gemm_f64_small(const double* __restrict__ A, const double* __restrict__ X, int64_t np, int epi,
+                 double* __restrict__ out, const double* __restrict__ xprev,
+                 Part3* __restrict__ part, const Tile* __restrict__ tiles, const DevState* st,
+                 int step, SimtDecide dec) {
+  if (halted_simt(st, step)) return;
+  __shared__ __align__(16) double As[8][kSmallMaxN + 2];   // rows of the left factor
+  __shared__ __align__(16) double Bs[kSmallMaxN][8];
+  __shared__ double half[64], r3[3][2];
+  const Tile t = tiles[blockIdx.x];
+  const int n = (int)np, tid = threadIdx.x;
+  for (int e = tid; e < 4 * n; e += 128) {   // 16 bytes at a time: 8 rows of n, n rows of 8
+    const int r = e / (n / 2), k = (e - r * (n / 2)) * 2;
+    const double2 v = *reinterpret_cast<const double2*>(A + (int64_t)(t.row0 + r) * np + k);
+    *reinterpret_cast<double2*>(&As[r][k]) = v;
+    const int kb = e >> 2, c = (e & 3) * 2;
+    *reinterpret_cast<double2*>(&Bs[kb][c]) =
+        *reinterpret_cast<const double2*>(X + (int64_t)kb * np + t.col0 + c);
+  }
+  __syncthreads();
+  const int g = tid >> 6, i = (tid & 63) >> 3, j = tid & 7;
+  double acc = 0.0;
+  const int k1 = (g + 1) * (n / 2);
+#pragma unroll 8
+  for (int k = g * (n / 2); k < k1; ++k) acc = fma(As[i][k], Bs[k][j], acc);
+  if (g == 1) half[tid & 63] = acc;
+  __syncthreads();
+  const int64_t gi = t.row0 + i, gj = t.col0 + j;
+  double t1 = 0.0, t2 = 0.0, f = 0.0;
+  if (g == 0) {
+    const double c = acc + half[tid];
+    if (epi == EPI_PLAIN) {
+      out[gi * np + gj] = c;
+    } else if (gi <= gj) {
+      const int sg = st->sigma[step];
+      const double x = xprev[gi * np + gj];
+      const double v = sg > 0 ? c : 2.0 * x - c;
+      const double r = x - c, w = gi == gj ? 1.0 : 2.0;
+      out[gi * np + gj] = v;
+      if (gi != gj) out[gj * np + gi] = v;
+      t1 = gi == gj ? v : 0.0;
+      t2 = w * v * v;
+      f = w * r * r;
+    }
+  }
+  if (epi == EPI_PLAIN) return;
+  if (g == 0) {
+    for (int o = 16; o > 0; o >>= 1) {
+      t1 += __shfl_xor_sync(0xffffffffu, t1, o);
+      t2 += __shfl_xor_sync(0xffffffffu, t2, o);
+      f += __shfl_xor_sync(0xffffffffu, f, o);
+    }
+    if ((tid & 31) == 0) r3[0][tid >> 5] = t1, r3[1][tid >> 5] = t2, r3[2][tid >> 5] = f;
+  }
+  __syncthreads();
+  if (tid == 0)
+    part[blockIdx.x] = Part3{r3[0][0] + r3[0][1], r3[1][0] + r3[1][1], r3[2][0] + r3[2][1]};
+  if (dec.done) {
+    __shared__ int last;
+    if (tid == 0) {
+      __threadfence();
+      last = atomicAdd(dec.done, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (last) {
+      __threadfence();
+      decide_block(part, dec.st, dec.p);
+      if (tid == 0) *dec.done = 0u;
+    }
+  }
+}
+
 // ------------------------------------------------------------ FP32
-// BM x BN tile, 8 x 8 entries per thread (two 4 x 4 halves in each direction, so that
-// shared memory is read 16 bytes at a time), K steps of BK through two shared-memory
-// buffers with the next step's global loads in registers. The products are packed
-// pairs (fma.rn.f32x2: each half rounds as fmaf), the left factor's entries stored
-// twice side by side so that a pair {a, a} is one load: 38 instructions for 64 fused
-// multiply-adds a thread, where 64 scalar ones waited on 16 scalar shared loads.
-// Each entry's terms are added in the order of k, as by the scalar form.
+// BM x BN tile, 8 x TN entries per thread (4 x 4 blocks, so that shared memory is read
+// 16 bytes at a time; TN = 4 for the smaller tiles, where a tile's warps alone hide the
+// latencies), K steps of BK through two shared-memory buffers with the next step's
+// global loads in registers. The products are packed pairs (fma.rn.f32x2: each half
+// rounds as fmaf): the same rate as scalar ones at half the instructions. Shared-memory
+// reads (four wavefronts for 16 bytes a lane) and the FMA pipe bound it about equally;
+// the left factor's entries are doubled in registers, since pairs stored in shared
+// memory made its reads the bound (N = 1000 square 63 us). Each entry's terms are added
+// in the order of k, as by the scalar form.
 __device__ __forceinline__ uint64_t ffma2(uint64_t a, uint64_t b, uint64_t c) {
   uint64_t r;
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ uint64_t twice(float x) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(x));
   return r;
 }
 __device__ __forceinline__ float2 unpack2(uint64_t v) {
@@ -183,16 +270,16 @@ struct SumF32 {
   __device__ __forceinline__ double value() const { return (double)s + (double)c; }
 };
 
-template <int BM, int BN, int BK>
-__global__ void __launch_bounds__(BM / 8 * BN / 8, BM * BN == 128 * 128 ? 2 : (BM == 128 ? 3 : 6))
+template <int BM, int BN, int BK, int TN>
+__global__ void __launch_bounds__(BM / 8 * BN / TN, BM * BN == 128 * 128 ? 2 : (BM == 128 ? 2 : 4))
 k_gemm_f32(const float* __restrict__ A, const float* __restrict__ X, int64_t np, int epi,
            float* __restrict__ out, const float* __restrict__ xprev, Part3* __restrict__ part,
            const Tile* __restrict__ tiles, const DevState* st, int step, SimtDecide dec) {
-  constexpr int TX = BN / 8, NT = BM / 8 * TX;
-  constexpr int AS = BM + 2;                       // pairs per k row of the left buffer
+  constexpr int TX = BN / TN, NT = BM / 8 * TX, NH = TN / 4;   // column blocks per thread
+  constexpr int AS = BM + 4;                       // entries per k row of the left buffer
   constexpr int A4 = BM * BK / 4 / NT, B4 = BN * BK / 4 / NT;   // 16-byte loads per thread
   if (halted_simt(st, step)) return;
-  __shared__ __align__(16) float2 As[2][BK][AS];
+  __shared__ __align__(16) float As[2][BK][AS];
   __shared__ __align__(16) float Bs[2][BK][BN];
   const Tile t = tiles[blockIdx.x];
   const int tid = threadIdx.x, tx = tid % TX, ty = tid / TX;
@@ -216,10 +303,10 @@ k_gemm_f32(const float* __restrict__ A, const float* __restrict__ X, int64_t np,
 #pragma unroll
     for (int i = 0; i < A4; ++i) {
       const int e = tid + i * NT, r = e / (BK / 4), k = (e % (BK / 4)) * 4;
-      As[b][k + 0][r] = make_float2(ra[i].x, ra[i].x);
-      As[b][k + 1][r] = make_float2(ra[i].y, ra[i].y);
-      As[b][k + 2][r] = make_float2(ra[i].z, ra[i].z);
-      As[b][k + 3][r] = make_float2(ra[i].w, ra[i].w);
+      As[b][k + 0][r] = ra[i].x;
+      As[b][k + 1][r] = ra[i].y;
+      As[b][k + 2][r] = ra[i].z;
+      As[b][k + 3][r] = ra[i].w;
     }
 #pragma unroll
     for (int i = 0; i < B4; ++i) {
@@ -227,11 +314,11 @@ k_gemm_f32(const float* __restrict__ A, const float* __restrict__ X, int64_t np,
       *reinterpret_cast<float4*>(&Bs[b][e / (BN / 4)][(e % (BN / 4)) * 4]) = rb[i];
     }
   };
-  uint64_t acc[8][4];
+  uint64_t acc[8][2 * NH];
 #pragma unroll
   for (int i = 0; i < 8; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
+    for (int j = 0; j < 2 * NH; ++j) acc[i][j] = 0ull;
   load(0);
   store(0);
   __syncthreads();
@@ -241,13 +328,15 @@ k_gemm_f32(const float* __restrict__ A, const float* __restrict__ X, int64_t np,
     if (more) load(k0 + BK);
 #pragma unroll
     for (int kk = 0; kk < BK; ++kk) {
-      uint64_t a[8], b[4];
+      uint64_t a[8], b[2 * NH];
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        const ulonglong2* pa =
-            reinterpret_cast<const ulonglong2*>(&As[buf][kk][h * (BM / 2) + ty * 4]);
-        const ulonglong2 a0 = pa[0], a1 = pa[1];
-        a[4 * h] = a0.x, a[4 * h + 1] = a0.y, a[4 * h + 2] = a1.x, a[4 * h + 3] = a1.y;
+        const float4 v = *reinterpret_cast<const float4*>(&As[buf][kk][h * (BM / 2) + ty * 4]);
+        a[4 * h] = twice(v.x), a[4 * h + 1] = twice(v.y);
+        a[4 * h + 2] = twice(v.z), a[4 * h + 3] = twice(v.w);
+      }
+#pragma unroll
+      for (int h = 0; h < NH; ++h) {
         const ulonglong2 bv =
             *reinterpret_cast<const ulonglong2*>(&Bs[buf][kk][h * (BN / 2) + tx * 4]);
         b[2 * h] = bv.x, b[2 * h + 1] = bv.y;
@@ -255,7 +344,7 @@ k_gemm_f32(const float* __restrict__ A, const float* __restrict__ X, int64_t np,
 #pragma unroll
       for (int i = 0; i < 8; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = ffma2(a[i], b[j], acc[i][j]);
+        for (int j = 0; j < 2 * NH; ++j) acc[i][j] = ffma2(a[i], b[j], acc[i][j]);
     }
     if (more) store(buf ^ 1);   // (its readers passed the barrier of the step before)
     __syncthreads();
@@ -266,7 +355,7 @@ k_gemm_f32(const float* __restrict__ A, const float* __restrict__ X, int64_t np,
 #pragma unroll
     for (int i = 0; i < 8; ++i)
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
+      for (int h = 0; h < NH; ++h) {
         const float2 u = unpack2(acc[i][2 * h]), v = unpack2(acc[i][2 * h + 1]);
         *reinterpret_cast<float4*>(out + (r0 + (i >> 2) * (BM / 2) + (i & 3)) * np + c0 +
                                    h * (BN / 2)) = make_float4(u.x, u.y, v.x, v.y);
@@ -281,7 +370,7 @@ k_gemm_f32(const float* __restrict__ A, const float* __restrict__ X, int64_t np,
 #pragma unroll
   for (int ih = 0; ih < 2; ++ih)
 #pragma unroll
-    for (int jh = 0; jh < 2; ++jh) {
+    for (int jh = 0; jh < NH; ++jh) {
       const int64_t gi0 = r0 + ih * (BM / 2), gj0 = c0 + jh * (BN / 2);
       if (gi0 > gj0 + 3) continue;   // the 4 x 4 block lies below the diagonal
       const bool above = gi0 + 3 < gj0;
@@ -370,9 +459,10 @@ void f32_tile(int64_t rows, int64_t np, bool upper, int* bm, int* bn) {
       for (int64_t i = 0; i < m; ++i) nt += (np - i * s[0]) / s[1];
     }
     const int64_t per = (nt + 151) / 152;
-    const int warps = s[0] * s[1] / 64 / 32;
+    const int warps = s[0] * s[1] / (s[1] == 128 ? 64 : 32) / 32;
     const double w = (double)(per * warps < 8 ? per * warps : 8);
-    const double c = (double)per * s[0] * s[1] / (0.55 + 0.45 * w / 8.0);
+    // (the narrow tiles read more shared memory per multiply-add)
+    const double c = (double)per * s[0] * s[1] / (0.55 + 0.45 * w / 8.0) / (s[1] == 128 ? 1.0 : 0.85);
     if (best == 0.0 || c < 0.97 * best) {
       best = c;
       *bm = s[0];
@@ -384,12 +474,13 @@ void f32_tile(int64_t rows, int64_t np, bool upper, int* bm, int* bn) {
 }  // namespace
 
 // FP64 runs at a small fraction of the FP32 rate on GB300, so an FP64 product
-// takes as long as its busiest SM: up to np = 1024 it uses 16 x 16 tiles (136
-// upper tiles at np = 256, where 64 x 64 tiles would keep 10 SMs busy and leave
-// the rest idle), above that 64 x 64.
+// takes as long as its busiest SM: 8 x 8 tiles up to np = 192 for a square or a
+// single product (at np = 128 16 x 16 tiles keep 36 SMs busy), 16 x 16 up to
+// np = 1024 (136 upper tiles at np = 256, where 64 x 64 would keep 10 SMs busy),
+// above that 64 x 64.
 void simt_tile_shape(int mode, int64_t rows, int64_t np, bool upper, int* bm, int* bn) {
   if (mode == SP2_MODE_FP64) {
-    const int t = np <= 1024 ? 16 : 64;
+    const int t = np <= kSmallMaxN && rows == np ? 8 : (np <= 1024 ? 16 : 64);
     *bm = t;
     *bn = t;
   } else {
@@ -407,7 +498,11 @@ cudaError_t launch_gemm_simt(int mode, int epi, const void* A, int64_t a_rows, c
   if (ntiles <= 0) return cudaSuccess;
   SimtDecide sd;
   if (dec && epi == EPI_SQUARE) sd = *dec;
-  if (mode == SP2_MODE_FP64 && bm == 16) {
+  if (mode == SP2_MODE_FP64 && bm == 8) {
+    k_gemm_f64_small<<<ntiles, 128, 0, s>>>(
+        static_cast<const double*>(A), static_cast<const double*>(X), np, epi,
+        static_cast<double*>(out), static_cast<const double*>(x_prev), part, tiles, st, step, sd);
+  } else if (mode == SP2_MODE_FP64 && bm == 16) {
     k_gemm_simt<double, 16, 16, 32, 1, 1><<<ntiles, 256, 0, s>>>(static_cast<const double*>(A), static_cast<const double*>(X), np, epi,
         static_cast<double*>(out), static_cast<const double*>(x_prev), part, tiles, st, step, sd);
   } else if (mode == SP2_MODE_FP64) {
@@ -418,11 +513,11 @@ cudaError_t launch_gemm_simt(int mode, int epi, const void* A, int64_t a_rows, c
     const float* xp = static_cast<const float*>(x_prev);
     float* o = static_cast<float*>(out);
     if (bm == 128 && bn == 128)
-      k_gemm_f32<128, 128, 8><<<ntiles, 256, 0, s>>>(a, x, np, epi, o, xp, part, tiles, st, step, sd);
+      k_gemm_f32<128, 128, 8, 8><<<ntiles, 256, 0, s>>>(a, x, np, epi, o, xp, part, tiles, st, step, sd);
     else if (bm == 128)
-      k_gemm_f32<128, 64, 16><<<ntiles, 128, 0, s>>>(a, x, np, epi, o, xp, part, tiles, st, step, sd);
+      k_gemm_f32<128, 64, 16, 4><<<ntiles, 256, 0, s>>>(a, x, np, epi, o, xp, part, tiles, st, step, sd);
     else
-      k_gemm_f32<64, 64, 16><<<ntiles, 64, 0, s>>>(a, x, np, epi, o, xp, part, tiles, st, step, sd);
+      k_gemm_f32<64, 64, 16, 4><<<ntiles, 128, 0, s>>>(a, x, np, epi, o, xp, part, tiles, st, step, sd);
   }
   return cudaGetLastError();
 }
