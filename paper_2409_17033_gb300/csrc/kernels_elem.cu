@@ -492,6 +492,54 @@ __global__ void k_init_x4(const float* __restrict__ src, int64_t n, int64_t np, 
   if (threadIdx.x == 0) part[blockIdx.x] = Part3{t1, t2, 0.0};
 }
 
+// Y_1 = beta B of a batch (dense or diagonals) in FP32 inputs and a split or FP32 mode,
+// N % 4 == 0: the padded masters four entries at a time, beta as hi + lo, and (FP16X2)
+// each matrix's max. Diagonals write their zeros as whole vectors; 742 us for four
+// 4096 x 4096 masters with per-entry index arithmetic and FP64. HBM-bound: 4 bytes
+// written (and 4 read) per entry.
+__global__ void k_init_batch_x4(const float* __restrict__ src, int64_t n, int64_t np, int64_t batch,
+                                int diag_only, double beta, int mode, MatBuf dst, float* ymax,
+                                int planes, int coef, const DevState* st) {
+  dep_sync();
+  const F2 bc = split_coef(coef == INIT_STATE_BETA ? st->beta : beta);
+  const int q = (int)(np / 4);
+  const int64_t rows = batch * np;
+  for (int64_t r = blockIdx.x; r < rows; r += gridDim.x) {
+    const int64_t b = r / np;
+    const int i = (int)(r - b * np);
+    float m = 0.0f;
+    for (int c = threadIdx.x; c < q; c += blockDim.x) {
+      const int j = 4 * c;
+      float x[4] = {0.f, 0.f, 0.f, 0.f};
+      if (i < n && j < n) {   // n % 4 == 0: the whole group is inside
+        if (!diag_only) {
+          const float4 h = __ldcs(reinterpret_cast<const float4*>(src + (b * n + i) * n + j));
+          x[0] = h.x;
+          x[1] = h.y;
+          x[2] = h.z;
+          x[3] = h.w;
+        } else if (i >= j && i < j + 4) {
+          const float d = src[b * n + i];
+#pragma unroll
+          for (int k = 0; k < 4; ++k) x[k] = i == j + k ? d : 0.0f;
+        }
+      }
+      float f[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        f[k] = mul_coef(x[k], bc);
+        m = fmaxf(m, fabsf(f[k]));
+      }
+      reinterpret_cast<float4*>(dst.master)[r * q + c] = make_float4(f[0], f[1], f[2], f[3]);
+      if (planes) store_planes4(dst, mode, r * q + c, f);
+    }
+    if (ymax) {
+      for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+      if ((threadIdx.x & 31) == 0 && m > 0.0f) atomic_max_nonneg(&ymax[b], m);
+    }
+  }
+}
+
 // Gershgorin discs of an FP32 H, one warp per row: each lane sums |h| of its
 // part of the row with TwoSum in FP32, four 16-byte loads in flight, and moves
 // the sum and its error to FP64 after each group of 16 entries; lanes add in FP64.
@@ -698,32 +746,6 @@ template <typename T> struct CtrAcc;
 template <> struct CtrAcc<float> { using type = AccF32; };
 template <> struct CtrAcc<double> { using type = AccF64; };
 
-template <typename T, int VEC> struct CtrVec { T v[VEC]; };
-template <int VEC>
-__device__ __forceinline__ CtrVec<float, VEC> ctr_load(const float* p, int64_t t, bool stream) {
-  CtrVec<float, VEC> r;
-  if constexpr (VEC == 4) {
-    const float4* q = reinterpret_cast<const float4*>(p) + t;
-    const float4 x = stream ? __ldcs(q) : __ldg(q);
-    r.v[0] = x.x, r.v[1] = x.y, r.v[2] = x.z, r.v[3] = x.w;
-  } else {
-    r.v[0] = p[t];
-  }
-  return r;
-}
-template <int VEC>
-__device__ __forceinline__ CtrVec<double, VEC> ctr_load(const double* p, int64_t t, bool stream) {
-  CtrVec<double, VEC> r;
-  if constexpr (VEC == 2) {
-    const double2* q = reinterpret_cast<const double2*>(p) + t;
-    const double2 x = stream ? __ldcs(q) : __ldg(q);
-    r.v[0] = x.x, r.v[1] = x.y;
-  } else {
-    r.v[0] = p[t];
-  }
-  return r;
-}
-
 // Sums of N values (a power of two up to 32) over a warp: each exchange halves the
 // values a lane still holds, so that N sums cost N - 1 additions and the remaining
 // rounds instead of 5 N. Value i ends in the lanes whose upper bits are i.
@@ -743,34 +765,96 @@ __device__ __forceinline__ double warp_sums(double (&v)[N], int lane) {
   return v[0];
 }
 
+// 16 bytes from global to this thread's own place in shared memory, asynchronously
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                   (uint32_t)__cvta_generic_to_shared(dst)),
+               "l"(src)
+               : "memory");
+}
+
+// VEC: entries per load; 16-byte loads go through two shared-memory stages of the
+// thread's own vectors (LT + kCtrKT of them), so that a stage's loads are in flight
+// while the stage before is added: with loads into registers a thread waited out the
+// memory's latency four times per 16 x 4 x 8 additions.
 template <typename T, int VEC, int LT>
 __global__ void __launch_bounds__(256, 2)
 k_contract_dense(const T* __restrict__ P, int64_t L, const T* __restrict__ Q, int64_t K, int64_t nn,
                  double* part, int nparts, int64_t y0) {
   dep_sync();
   using Acc = typename CtrAcc<T>::type;
-  constexpr int NP = LT * kCtrKT;
+  constexpr int NP = LT * kCtrKT, NV = LT + kCtrKT;
   const int64_t ktiles = (K + kCtrKT - 1) / kCtrKT;
   const int64_t y = y0 + blockIdx.y;
   const int64_t l0 = (y / ktiles) * LT, k0 = (y % ktiles) * kCtrKT;
   const int kn = (int)((K - k0) < kCtrKT ? (K - k0) : kCtrKT);
   const int ln = (int)((L - l0) < LT ? (L - l0) : LT);
   const T* p = P + l0 * nn;
+  const T* q = Q + k0 * nn;
   Acc acc[LT][kCtrKT];
-  const int64_t nv = nn / VEC;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < nv;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    CtrVec<T, VEC> a[LT];
+  const int64_t nv = nn / VEC, stride = (int64_t)gridDim.x * blockDim.x;
+  int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if constexpr (VEC * sizeof(T) == 16) {
+    extern __shared__ __align__(16) uint8_t ctr_smem[];
+    struct Vec {
+      T v[VEC];
+    };
+    Vec* mine = reinterpret_cast<Vec*>(ctr_smem) + threadIdx.x;   // [stage][vector][thread]
+    auto fetch = [&](int st, int64_t tt) {
+      if (tt < nv) {
 #pragma unroll
-    for (int l = 0; l < LT; ++l) a[l] = ctr_load<VEC>(p + (l < ln ? l : 0) * nn, t, false);
+        for (int l = 0; l < LT; ++l)
+          if (l < ln) cp_async16(mine + (st * NV + l) * 256, p + l * nn + tt * VEC);
 #pragma unroll
-    for (int k = 0; k < kCtrKT; ++k) {
-      if (k >= kn) break;
-      const CtrVec<T, VEC> b = ctr_load<VEC>(Q + (k0 + k) * nn, t, true);
+        for (int k = 0; k < kCtrKT; ++k)
+          if (k < kn) cp_async16(mine + (st * NV + LT + k) * 256, q + k * nn + tt * VEC);
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    fetch(0, t);
+    for (int st = 0; t < nv; t += stride, st ^= 1) {
+      fetch(st ^ 1, t + stride);
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+      Vec a[LT];
 #pragma unroll
-      for (int l = 0; l < LT; ++l)
+      for (int l = 0; l < LT; ++l) a[l] = mine[(st * NV + (l < ln ? l : 0)) * 256];
+      if (kn == kCtrKT) {   // (no exits between the perturbations: their chains interleave)
 #pragma unroll
-        for (int j = 0; j < VEC; ++j) acc[l][k].add(a[l].v[j], b.v[j]);
+        for (int k2 = 0; k2 < kCtrKT; k2 += 2) {
+          const Vec b0 = mine[(st * NV + LT + k2) * 256], b1 = mine[(st * NV + LT + k2 + 1) * 256];
+#pragma unroll
+          for (int j = 0; j < VEC; ++j)
+#pragma unroll
+            for (int l = 0; l < LT; ++l) {
+              acc[l][k2].add(a[l].v[j], b0.v[j]);
+              acc[l][k2 + 1].add(a[l].v[j], b1.v[j]);
+            }
+        }
+      } else {
+#pragma unroll
+        for (int k = 0; k < kCtrKT; ++k) {
+          if (k >= kn) break;
+          const Vec b = mine[(st * NV + LT + k) * 256];
+#pragma unroll
+          for (int l = 0; l < LT; ++l)
+#pragma unroll
+            for (int j = 0; j < VEC; ++j) acc[l][k].add(a[l].v[j], b.v[j]);
+        }
+      }
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+  } else {
+    for (; t < nv; t += stride) {
+      T a[LT];
+#pragma unroll
+      for (int l = 0; l < LT; ++l) a[l] = p[(l < ln ? l : 0) * nn + t];
+#pragma unroll
+      for (int k = 0; k < kCtrKT; ++k) {
+        if (k >= kn) break;
+        const T b = q[k * nn + t];
+#pragma unroll
+        for (int l = 0; l < LT; ++l) acc[l][k].add(a[l], b);
+      }
     }
   }
   __shared__ double red[8][NP];
@@ -845,6 +929,15 @@ cudaError_t launch_init(const void* src, int64_t n, int64_t np, int64_t batch, i
       !ymax && split_mode(mode) && n % 4 == 0 && (reinterpret_cast<uintptr_t>(src) & 15u) == 0) {
     launch_dep(k_init_x4, nparts, kRedThreads, 0, s, static_cast<const float*>(src), n, np, mode, dst, part,
                                              st);
+    return cudaGetLastError();
+  }
+  if (!part && alpha == 0.0 && coef != INIT_STATE && dtype == SP2_F32 && mode != SP2_MODE_FP64 &&
+      !symmetrize && n % 4 == 0 && (diag_only || (reinterpret_cast<uintptr_t>(src) & 15u) == 0)) {
+    // (FP16X2 with ymax: the planes follow from the maxima; FP32 has none)
+    const int planes = split_mode(mode) && !(mode == SP2_MODE_FP16X2 && ymax) ? 1 : 0;
+    launch_dep(k_init_batch_x4, grid_for(batch * np, 1, 152 * 16), 256, 0, s,
+               static_cast<const float*>(src), n, np, batch, diag_only, beta, mode, dst, ymax,
+               planes, coef, st);
     return cudaGetLastError();
   }
   int grid = part ? nparts : grid_for(batch * np, 1, 4096);
@@ -973,12 +1066,15 @@ void contract_rows(const void* P, int64_t L, const void* Q, int64_t K, int64_t n
                    int nparts, int64_t rows, cudaStream_t s) {
   // grid rows go out in launches of at most 65535, the limit of gridDim.y
   constexpr int64_t kMaxY = 65535;
+  constexpr size_t smem = VEC * sizeof(T) == 16 ? (size_t)2 * (LT + kCtrKT) * 256 * 16 : 0;
+  if (smem > 48 * 1024)
+    cudaFuncSetAttribute(k_contract_dense<T, VEC, LT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)smem);
   for (int64_t y0 = 0; y0 < rows; y0 += kMaxY) {
     const int64_t ny = (rows - y0) < kMaxY ? (rows - y0) : kMaxY;
     const dim3 grid((unsigned)nparts, (unsigned)ny);
-    launch_dep(k_contract_dense<T, VEC, LT>, grid, 256, 0, s, static_cast<const T*>(P), L,
-                                                      static_cast<const T*>(Q), K, nn, part,
-                                                      nparts, y0);
+    launch_dep(k_contract_dense<T, VEC, LT>, grid, 256, smem, s, static_cast<const T*>(P), L,
+               static_cast<const T*>(Q), K, nn, part, nparts, y0);
   }
 }
 // one block row per LT rows of P and kCtrKT perturbations; LT = 4 from three rows of P on
