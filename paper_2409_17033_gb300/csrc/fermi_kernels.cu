@@ -10,10 +10,15 @@ __device__ __forceinline__ void atomic_max_nonneg_f(float* addr, float v) {
   atomicMax(reinterpret_cast<int*>(addr), __float_as_int(v));
 }
 
-// out = z1 (Z1 + Z1^T) + z2 (Z2 + Z2^T) + a A + id I (I restricted to the
-// caller's n x n block). Null operands are skipped. One block of 256 threads per
-// upper-triangle tile pair (I <= J) of TE x TE tiles, from a linear block index;
-// both tiles written with 16-byte accesses, each element from its own inputs.
+// out = z1 (Z1 + Z1^T) + z2 (Z2 + Z2^T) + a A + id I (I restricted to the caller's
+// n x n block) for a batch (grid.y), with the planes the next product reads. Null
+// operands are skipped. One block of 256 threads per upper-triangle tile pair (I <= J)
+// of TE x TE tiles, from a linear block index; both tiles written with 16-byte
+// accesses, each element from its own inputs. FP16X2: the planes' scale comes from the
+// bound 2 |z1| max|Z1| + 2 |z2| max|Z2| + |a| max|A| + |id| on an entry, at most a few
+// binades above the result's max, so the planes need no pass of their own (a max of the
+// result, a scale and a split: two more launches and 8 more bytes an entry). Bound by
+// memory: 4 bytes an entry of each operand read, 4 (FP16X2, BF16X2: 8) written.
 template <typename T>
 constexpr int comb_tile() { return sizeof(T) == 4 ? 64 : 32; }
 
@@ -39,10 +44,11 @@ __device__ __forceinline__ void st4(T* p, const T (&v)[4]) {
   }
 }
 
-template <typename T>
+template <typename T, int MODE>
 __global__ void __launch_bounds__(256)
-    k_combine(T* __restrict__ out, int64_t np, int64_t n, const T* __restrict__ Z1, T z1,
-              const T* __restrict__ Z2, T z2, const T* __restrict__ A, T a, T id, float* amax) {
+    k_combine(MatBuf out, int64_t np, int64_t n, const T* __restrict__ Z1, T z1,
+              const T* __restrict__ Z2, T z2, const T* __restrict__ A, T a, T id, int planes,
+              CombineScale cs) {
   dep_sync();
   constexpr int TE = comb_tile<T>();
   constexpr int V = TE / 4, R = 256 / V, P = TE / R;
@@ -54,7 +60,18 @@ __global__ void __launch_bounds__(256)
   const bool diag = I == J;
   __shared__ T sa[TE][TE + 1], sb[TE][TE + 1];
   const int c4 = (threadIdx.x % V) * 4, r0 = threadIdx.x / V;
-  const int64_t rI = I * TE, rJ = J * TE;
+  const int64_t rI = I * TE, rJ = J * TE, base = (int64_t)blockIdx.y * np * np;
+  float s = 1.0f;
+  if constexpr (MODE == SP2_MODE_FP16X2) {
+    if (planes) {
+      float bound = fabsf((float)id);
+      if (Z1) bound += 2.0f * fabsf((float)z1) * cs.z1max[blockIdx.y];
+      if (Z2) bound += 2.0f * fabsf((float)z2) * cs.z2max[blockIdx.y];
+      if (A) bound += fabsf((float)a) * cs.amax[blockIdx.y];
+      s = pow2_scale(bound);
+      if (t == 0 && threadIdx.x == 0) cs.scale[blockIdx.y] = s;
+    }
+  }
   T v[P][4], w[P][4];   // out tile (I,J) and, off the diagonal, tile (J,I)
 #pragma unroll
   for (int p = 0; p < P; ++p)
@@ -69,8 +86,8 @@ __global__ void __launch_bounds__(256)
     for (int p = 0; p < P; ++p) {
       const int r = r0 + p * R;
       T x[4], y[4];
-      ld4(Z + (rI + r) * np + rJ + c4, x);
-      ld4(Z + (rJ + r) * np + rI + c4, y);
+      ld4(Z + base + (rI + r) * np + rJ + c4, x);
+      ld4(Z + base + (rJ + r) * np + rI + c4, y);
 #pragma unroll
       for (int j = 0; j < 4; ++j) sa[r][c4 + j] = x[j], sb[r][c4 + j] = y[j];
     }
@@ -96,7 +113,7 @@ __global__ void __launch_bounds__(256)
       for (int j = 0; j < 4; ++j) o[j] = pass == 0 ? v[p][j] : w[p][j];
       if (A) {
         T x[4];
-        ld4(A + gi * np + gj0, x);
+        ld4(A + base + gi * np + gj0, x);
 #pragma unroll
         for (int j = 0; j < 4; ++j) o[j] += a * x[j];
       }
@@ -105,58 +122,63 @@ __global__ void __launch_bounds__(256)
         if (gi == gj0 + j && gi < n) o[j] += id;
         m = fmaxf(m, fabsf((float)o[j]));
       }
-      st4(out + gi * np + gj0, o);
+      const int64_t idx = base + gi * np + gj0;
+      if (planes) store_y4<T, MODE>(out, idx, o, s);
+      else st4(static_cast<T*>(out.master) + idx, o);
     }
   }
-  if (amax) {
+  if (cs.omax) {
     for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0 && m > 0.0f) atomic_max_nonneg_f(amax, m);
+    if ((threadIdx.x & 31) == 0 && m > 0.0f) atomic_max_nonneg_f(&cs.omax[blockIdx.y], m);
   }
 }
 
-// out[0] = sum_{i < n} M[i, i] in FP64 (one block, fixed order)
+// out[b] = sum_{i < n} M_b[i, i] in FP64 (one block per batch entry, fixed order)
 template <typename T>
 __global__ void k_trace(const T* __restrict__ M, int64_t np, int64_t n, double* out) {
   dep_sync();
   __shared__ double red[32];
   double s = 0.0;
-  for (int64_t i = threadIdx.x; i < n; i += blockDim.x) s += (double)M[i * np + i];
+  for (int64_t i = threadIdx.x; i < n; i += blockDim.x) s += (double)M[(int64_t)blockIdx.x * np * np + i * np + i];
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
   __syncthreads();
   if (threadIdx.x == 0) {
     double t = 0.0;
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-    out[0] = t;
+    out[blockIdx.x] = t;
   }
 }
 
 }  // namespace
 
-cudaError_t launch_combine(int mode, void* out, int64_t np, int64_t n, const void* Z1, double z1,
-                           const void* Z2, double z2, const void* A, double a, double id,
-                           float* amax, cudaStream_t s) {
-  // np is a multiple of 256, so both tile edges divide it
+cudaError_t launch_combine(int mode, MatBuf out, int64_t np, int64_t n, int64_t batch,
+                           const void* Z1, double z1, const void* Z2, double z2, const void* A,
+                           double a, double id, bool planes, const CombineScale& cs,
+                           cudaStream_t s) {
+  // np is a multiple of 64, so both tile edges divide it
   const int64_t nb = np / (mode == SP2_MODE_FP64 ? comb_tile<double>() : comb_tile<float>());
-  const dim3 grid((unsigned)(nb * (nb + 1) / 2)), block(256);
-  if (mode == SP2_MODE_FP64)
-    launch_dep(k_combine<double>, grid, block, 0, s, 
-        static_cast<double*>(out), np, n, static_cast<const double*>(Z1), z1,
-        static_cast<const double*>(Z2), z2, static_cast<const double*>(A), a, id, amax);
-  else
-    launch_dep(k_combine<float>, grid, block, 0, s, 
-        static_cast<float*>(out), np, n, static_cast<const float*>(Z1), (float)z1,
-        static_cast<const float*>(Z2), (float)z2, static_cast<const float*>(A), (float)a,
-        (float)id, amax);
+  const dim3 grid((unsigned)(nb * (nb + 1) / 2), (unsigned)batch), block(256);
+  auto go = [&](auto kern, auto zero) {
+    using T = decltype(zero);
+    return launch_dep(kern, grid, block, 0, s, out, np, n, static_cast<const T*>(Z1), (T)z1,
+                      static_cast<const T*>(Z2), (T)z2, static_cast<const T*>(A), (T)a, (T)id,
+                      planes ? 1 : 0, cs);
+  };
+  if (mode == SP2_MODE_FP64) go(k_combine<double, SP2_MODE_FP64>, 0.0);
+  else if (mode == SP2_MODE_FP32) go(k_combine<float, SP2_MODE_FP32>, 0.0f);
+  else if (mode == SP2_MODE_BF16X2) go(k_combine<float, SP2_MODE_BF16X2>, 0.0f);
+  else if (mode == SP2_MODE_BF16X3) go(k_combine<float, SP2_MODE_BF16X3>, 0.0f);
+  else go(k_combine<float, SP2_MODE_FP16X2>, 0.0f);
   return cudaGetLastError();
 }
 
-cudaError_t launch_trace(int mode, const void* M, int64_t np, int64_t n, double* out,
+cudaError_t launch_trace(int mode, const void* M, int64_t np, int64_t n, int64_t batch, double* out,
                          cudaStream_t s) {
   if (mode == SP2_MODE_FP64)
-    launch_dep(k_trace<double>, 1, 1024, 0, s, static_cast<const double*>(M), np, n, out);
+    launch_dep(k_trace<double>, (unsigned)batch, 1024, 0, s, static_cast<const double*>(M), np, n, out);
   else
-    launch_dep(k_trace<float>, 1, 1024, 0, s, static_cast<const float*>(M), np, n, out);
+    launch_dep(k_trace<float>, (unsigned)batch, 1024, 0, s, static_cast<const float*>(M), np, n, out);
   return cudaGetLastError();
 }
 

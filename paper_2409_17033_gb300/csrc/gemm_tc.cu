@@ -20,7 +20,7 @@
 //   EPI_SQUARE  X_{n+1} = sigma_n > 0 ? X_n^2 : 2 X_n - X_n^2 (Eq. DM0), upper
 //               tiles only, mirrored; partials of Tr X_{n+1}, ||X_{n+1}||_F^2 and
 //               ||X_n - X_n^2||_F^2 for the branch and stop decisions.
-//   EPI_PLAIN   C = P Q stored as it is (FP32).
+//   EPI_PLAIN   C = P Q stored as it is, or each batch entry transposed (FP32).
 //   EPI_SYMM    Y_{n+1} = sigma_n > 0 ? Y_n X_n + X_n Y_n : 2 Y_n - (Y_n X_n + X_n Y_n)
 //               (Eqs. DM1, DM2, DM3) for a stacked batch of symmetric Y. With X
 //               and Y symmetric, (X Y)(I, J) = X(I, :) Y(:, J), so each upper tile
@@ -269,6 +269,7 @@ struct KParams {
   float* zmax;             // FP16X2 EPI_PLAIN: per batch entry, receives max |C|
   float* zero;             // EPI_PLAIN: nzero values cleared for the launch that follows
   int nzero;
+  int trans;               // EPI_PLAIN: store each batch entry of C transposed
   unsigned long long wait_ns;
   int withhold;            // test hook: CTA 0 never issues its first load
   int tail;                // split-tail mode: st->plane1[step] selects the hi planes alone
@@ -324,6 +325,15 @@ __device__ __forceinline__ void tile_end(const KParams& p, float (&acc)[TCOLS], 
       for (int j = 0; j < 16; ++j) {
         v[j] = acc[c0 + j] * inv_s;
         zm = fmaxf(zm, fabsf(v[j]));
+      }
+      if (p.trans) {   // down a column: consecutive rows (lanes) are consecutive addresses
+        float* dt = p.out + bat * np * np + (int64_t)(t.col0 + grp * TCOLS + c0) * np + li;
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+          *dt = v[j];
+          dt += np;
+        }
+        continue;
       }
       st256f(dst, v);
       st256f(dst + 8, v + 8);
@@ -1194,6 +1204,7 @@ cudaError_t launch_gemm_tc(const TcLaunch& L, cudaStream_t s, char* errbuf, size
   p.zmax = f16 ? L.zmax : nullptr;
   p.zero = L.zero;
   p.nzero = L.zero ? L.nzero : 0;
+  p.trans = L.trans;
   p.wait_ns = L.tune.wait_ns;
   p.withhold = L.tune.withhold;
   p.tail = L.tail;

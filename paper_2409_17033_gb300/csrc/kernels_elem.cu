@@ -255,43 +255,6 @@ __device__ __forceinline__ void ld4_stream<double>(const double* p, double (&v)[
   v[0] = a.x, v[1] = a.y, v[2] = b.x, v[3] = b.y;
 }
 
-// four consecutive entries of Y_{n+1} (idx a multiple of 4): master and, in the split
-// modes, the hi/lo planes as one 8-byte store each
-template <typename ZT, int MODE>
-__device__ __forceinline__ void store_y4(MatBuf y, int64_t idx, const ZT (&v)[4], float s) {
-  if constexpr (sizeof(ZT) == 4) {
-    *reinterpret_cast<float4*>(static_cast<float*>(y.master) + idx) =
-        make_float4((float)v[0], (float)v[1], (float)v[2], (float)v[3]);
-  } else {
-    double2* d = reinterpret_cast<double2*>(static_cast<double*>(y.master) + idx);
-    d[0] = make_double2((double)v[0], (double)v[1]);
-    d[1] = make_double2((double)v[2], (double)v[3]);
-  }
-  if (MODE == SP2_MODE_BF16X3) {
-    uint16_t h[4], m[4], l[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) split_bf16x3((float)v[j], h[j], m[j], l[j]);
-    *reinterpret_cast<uint2*>(y.hi + idx) =
-        make_uint2(h[0] | ((uint32_t)h[1] << 16), h[2] | ((uint32_t)h[3] << 16));
-    *reinterpret_cast<uint2*>(y.mid + idx) =
-        make_uint2(m[0] | ((uint32_t)m[1] << 16), m[2] | ((uint32_t)m[3] << 16));
-    *reinterpret_cast<uint2*>(y.lo + idx) =
-        make_uint2(l[0] | ((uint32_t)l[1] << 16), l[2] | ((uint32_t)l[3] << 16));
-  }
-  if (MODE == SP2_MODE_BF16X2 || MODE == SP2_MODE_FP16X2) {
-    uint16_t h[4], l[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      if (MODE == SP2_MODE_BF16X2) split_bf16((float)v[j], h[j], l[j]);
-      else split_fp16((float)v[j], s, h[j], l[j]);
-    }
-    *reinterpret_cast<uint2*>(y.hi + idx) =
-        make_uint2(h[0] | ((uint32_t)h[1] << 16), h[2] | ((uint32_t)h[3] << 16));
-    *reinterpret_cast<uint2*>(y.lo + idx) =
-        make_uint2(l[0] | ((uint32_t)l[1] << 16), l[2] | ((uint32_t)l[3] << 16));
-  }
-}
-
 constexpr int kSymThreads = 256;
 template <typename ZT>
 constexpr int sym_tile() { return sizeof(ZT) == 4 ? 64 : 32; }   // 33 / 17 KB of shared memory

@@ -1377,49 +1377,68 @@ int finish_call(sp2_handle_t h, sp2_handle_s::Pending* p, sp2_info* info, bool w
 // --------------------------------------------------------------- finite temperature
 // A padded matrix of the finite-temperature recursion with its plane scale
 // (FP16X2: a power of two from its max; 1 otherwise) and max accumulator.
+// (a batch of them, stacked, for the responses of several perturbations).
 struct FMat {
   MatBuf m;
-  float* scale = nullptr;  // device float (FP16X2)
-  float* amax = nullptr;   // device float (FP16X2)
+  float* scale = nullptr;  // device floats, one per batch entry (FP16X2)
+  float* amax = nullptr;   // device floats, one per batch entry (FP16X2)
+  int64_t B = 1;
 };
 
-int fmat(sp2_handle_t h, const std::string& name, int64_t np, int mode, FMat* f) {
-  TRY(mat(h, name, np, np, mode, &f->m));
+int fmat(sp2_handle_t h, const std::string& name, int64_t np, int mode, FMat* f, int64_t B = 1) {
+  f->B = B;
+  TRY(mat(h, name, B * np, np, mode, &f->m));
   if (mode == SP2_MODE_FP16X2) {
     void* p;
-    TRY(ws(h, name + ".s", 2 * sizeof(float), &p));
+    TRY(ws(h, name + ".s", (size_t)B * 2 * sizeof(float), &p));
     f->scale = static_cast<float*>(p);
-    f->amax = f->scale + 1;
+    f->amax = f->scale + B;
   }
   return SP2_OK;
+}
+
+// batch entry b of f
+FMat fentry(const FMat& f, int64_t b, int64_t np, int mode) {
+  const int64_t off = b * np * np;
+  FMat e = f;
+  e.B = 1;
+  e.m.master = static_cast<char*>(f.m.master) + (size_t)off * master_size(mode);
+  if (f.m.hi) e.m.hi = f.m.hi + off;
+  if (f.m.lo) e.m.lo = f.m.lo + off;
+  if (f.m.mid) e.m.mid = f.m.mid + off;
+  if (f.scale) e.scale = f.scale + b;
+  if (f.amax) e.amax = f.amax + b;
+  return e;
 }
 
 // hi/lo planes of f from its master (FP16X2: scale from f->amax)
 int fplanes(Ctx& c, FMat& f) {
   sp2_handle_t h = c.h;
   if (c.mode == SP2_MODE_BF16X2 || c.mode == SP2_MODE_BF16X3) {
-    CK(launch_split(f.m, c.np, c.np, c.mode, h->stream));
+    CK(launch_split(f.m, f.B * c.np, c.np, c.mode, h->stream));
     c.kernels++;
   } else if (c.mode == SP2_MODE_FP16X2) {
     ScaleBuf sc;
     sc.ymax = f.amax;
     sc.yscale = f.scale;
-    sc.B = 1;
+    sc.B = f.B;
     CK(launch_split_scaled(f.m, c.np, sc, 0, h->stream));
     c.kernels += 2;
   }
   return SP2_OK;
 }
 
-// C = L R for symmetric R (R's rows are the K-major operand); master only,
-// plus C's max in FP16X2 (planes follow from fplanes when C is an operand)
-int fprod(Ctx& c, FMat& C, const FMat& L, const FMat& R) {
+// C = L R for symmetric R (R's rows are the K-major operand), L one matrix or a stacked
+// batch (then C is one too); master only, plus C's max in FP16X2 (planes follow from
+// fplanes when C is an operand). trans (split modes): each entry of C transposed.
+int fprod(Ctx& c, FMat& C, const FMat& L, const FMat& R, bool trans = false) {
   sp2_handle_t h = c.h;
   DigBufs db;
-  const bool same = L.m.master == R.m.master;
-  if (dig_mode(c, c.np) && dig_bufs(c, same ? 0 : c.np, false, &db)) {
+  const bool same = L.m.master == R.m.master && L.B == 1;
+  const int64_t rows = L.B * c.np;
+  if (dig_mode(c, rows) && dig_bufs(c, same ? 0 : rows, false, &db)) {
     const double* l = static_cast<const double*>(L.m.master);
-    CK(launch_digits(l, c.np, c.np, db.a, c.st, 0, h->stream));
+    CK(launch_digits(l, rows, c.np, db.a, c.st, 0, h->stream));
     if (!same)
       CK(launch_digits(static_cast<const double*>(R.m.master), c.np, c.np, db.x, c.st, 0,
                        h->stream));
@@ -1429,25 +1448,25 @@ int fprod(Ctx& c, FMat& C, const FMat& L, const FMat& R) {
       TRY(ev_pair(c, &e0, &e1));
       CK(cudaEventRecord(e0, h->stream));
     }
-    CK(launch_gemm_dig(db.a, c.np, db.x, c.np, db.G, db.tiles, db.ntiles, db.plan, c.st, 0, h->tune,
+    CK(launch_gemm_dig(db.a, rows, db.x, c.np, db.G, db.tiles, db.ntiles, db.plan, c.st, 0, h->tune,
                        h->stream));
     if (c.timing) {
       CK(cudaEventRecord(e1, h->stream));
       c.timed.push_back({0, 0});
     }
-    CK(launch_dig_plain(db.G, db.plan.ksplit, c.np, db.a.ex, db.x.ex, static_cast<double*>(C.m.master), c.np, c.st,
+    CK(launch_dig_plain(db.G, db.plan.ksplit, rows, db.a.ex, db.x.ex, static_cast<double*>(C.m.master), c.np, c.st,
                         0, h->stream));
     c.launches++;
     c.kernels += same ? 3 : 4;
     c.flops += dig_flops(c, db);
-    c.alg += 2.0 * (double)c.n * (double)c.n * (double)c.n;
+    c.alg += 2.0 * (double)L.B * (double)c.n * (double)c.n * (double)c.n;
     return SP2_OK;
   }
   const Tile* tl;
   int nt;
   int bm, bn;
-  product_tile(h, c.mode, c.np, c.np, false, &bm, &bn);
-  TRY(tile_list(h, c.mode, c.np, c.np, false, &tl, &nt, bm, bn));
+  product_tile(h, c.mode, rows, c.np, false, &bm, &bn);
+  TRY(tile_list(h, c.mode, rows, c.np, false, &tl, &nt, bm, bn));
   TcLaunch T;   // workspace first: nothing is allocated inside the timed interval
   if (split_mode(c.mode)) TRY(tc_common(c, &T, nt));
   cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -1457,15 +1476,16 @@ int fprod(Ctx& c, FMat& C, const FMat& L, const FMat& R) {
   }
   if (split_mode(c.mode)) {
     const bool f16 = c.mode == SP2_MODE_FP16X2;
-    if (f16) CK(cudaMemsetAsync(C.amax, 0, sizeof(float), h->stream));
+    if (f16) CK(cudaMemsetAsync(C.amax, 0, sizeof(float) * L.B, h->stream));
     char eb[256] = {0};
     T.epi = EPI_PLAIN;
-    T.P = TcOperand{L.m.hi, L.m.lo, c.np, L.m.mid};
+    T.P = TcOperand{L.m.hi, L.m.lo, rows, L.m.mid};
     T.Q = TcOperand{R.m.hi, R.m.lo, c.np, R.m.mid};
     T.out = C.m;
     T.tiles = tl;
     T.step = 0;
     T.bn = bn;
+    T.trans = trans ? 1 : 0;
     if (f16) {
       T.p_scale = L.scale;
       T.q_scale = R.scale;
@@ -1474,7 +1494,7 @@ int fprod(Ctx& c, FMat& C, const FMat& L, const FMat& R) {
     cudaError_t e = launch_gemm_tc(T, h->stream, eb, sizeof eb);
     if (e != cudaSuccess) return fail(h, SP2_ECUDA, "finite-T product: %s %s", cudaGetErrorString(e), eb);
   } else {
-    CK(launch_gemm_simt(c.mode, EPI_PLAIN, L.m.master, c.np, R.m.master, c.np, C.m.master, nullptr,
+    CK(launch_gemm_simt(c.mode, EPI_PLAIN, L.m.master, rows, R.m.master, c.np, C.m.master, nullptr,
                         c.part, tl, nt, bm, bn, c.st, 0, h->stream));
   }
   if (c.timing) {
@@ -1484,21 +1504,25 @@ int fprod(Ctx& c, FMat& C, const FMat& L, const FMat& R) {
   c.launches++;
   c.kernels++;
   c.flops += 2.0 * bm * bn * (double)c.np * k_mult(c.mode) * nt;
-  c.alg += 2.0 * (double)c.n * (double)c.n * (double)c.n * k_mult(c.mode);
+  c.alg += 2.0 * (double)L.B * (double)c.n * (double)c.n * (double)c.n * k_mult(c.mode);
   return SP2_OK;
 }
 
-// out = z1 (Z1 + Z1^T) + z2 (Z2 + Z2^T) + a A + id I, then planes when `planes`
+// out = z1 (Z1 + Z1^T) + z2 (Z2 + Z2^T) + a A + id I (of every batch entry), with its
+// planes when `planes`
 int fcomb(Ctx& c, FMat& out, const FMat* Z1, double z1, const FMat* Z2, double z2,
           const FMat* A, double a, double id, bool planes) {
   sp2_handle_t h = c.h;
-  const bool f16 = c.mode == SP2_MODE_FP16X2;
-  if (f16) CK(cudaMemsetAsync(out.amax, 0, sizeof(float), h->stream));
-  CK(launch_combine(c.mode, out.m.master, c.np, c.n, Z1 ? Z1->m.master : nullptr, z1,
-                    Z2 ? Z2->m.master : nullptr, z2, A ? A->m.master : nullptr, a, id,
-                    f16 ? out.amax : nullptr, h->stream));
+  CombineScale cs;
+  if (c.mode == SP2_MODE_FP16X2 && planes) {
+    CK(cudaMemsetAsync(out.amax, 0, sizeof(float) * out.B, h->stream));
+    cs = CombineScale{Z1 ? Z1->amax : nullptr, Z2 ? Z2->amax : nullptr, A ? A->amax : nullptr,
+                      out.scale, out.amax};
+  }
+  CK(launch_combine(c.mode, out.m, c.np, c.n, out.B, Z1 ? Z1->m.master : nullptr, z1,
+                    Z2 ? Z2->m.master : nullptr, z2, A ? A->m.master : nullptr, a, id, planes, cs,
+                    h->stream));
   c.kernels++;
-  if (planes) TRY(fplanes(c, out));
   return SP2_OK;
 }
 
@@ -1832,16 +1856,19 @@ struct FermiState {
   bool canonical = false;
   std::vector<FMat> dl, W;   // delta_0..delta_n, W_0..W_{n-1}
   FMat P, S, T, U, Z2[2];    // scratch of the forward pass and the responses
-  FMat dd[2], E, F1, dW, G1, RI;
+  FMat dd[2], E, F1, dW, G1, RI;   // (batches of B response matrices but for RI)
+  int64_t B = 1;
   double trI = 0.0;
-  void* tr = nullptr;        // 2 device doubles
+  void* tr = nullptr;        // B device doubles
+  void* ones = nullptr;      // the identity's diagonal, on the device
 };
 
-int fermi_response(Ctx& c, FermiState& fs, const void* src, int dtype, int diag, bool isI,
-                   FMat** result);
+int fermi_responses(Ctx& c, FermiState& fs, const void* ones, const void* src, int64_t K, int dtype,
+                    int diag, FMat* result);
+int fermi_batch(Ctx& c, FermiState& fs, int64_t want, int64_t* B);
 
 int fermi_setup(Ctx& c, FermiState& fs, const void* Hd, int64_t N, int dtype, double mu, double kT,
-                int n_doublings, bool canonical, bool responses) {
+                int n_doublings, bool canonical, bool responses, bool defer_i = false) {
   sp2_handle_t h = c.h;
   const int mode = c.mode;
   const int64_t np = c.np;
@@ -1911,84 +1938,131 @@ int fermi_setup(Ctx& c, FermiState& fs, const void* Hd, int64_t N, int dtype, do
     b = 2.0 * b / (1.0 + 4.0 * b * b);
   }
   if (!responses) return SP2_OK;
-  TRY(fmat(h, "ft.dd0", np, mode, &fs.dd[0]));
-  TRY(fmat(h, "ft.dd1", np, mode, &fs.dd[1]));
-  TRY(fmat(h, "ft.E", np, mode, &fs.E));
-  TRY(fmat(h, "ft.F1", np, mode, &fs.F1));
-  TRY(fmat(h, "ft.dW", np, mode, &fs.dW));
-  TRY(fmat(h, "ft.G1", np, mode, &fs.G1));
-  TRY(ws(h, "ft.tr", 2 * sizeof(double), &fs.tr));
+  int64_t one;
+  TRY(fermi_batch(c, fs, 1, &one));
   if (canonical) {
     TRY(fmat(h, "ft.RI", np, mode, &fs.RI));
-    void* ones = nullptr;
-    TRY(ws(h, "ft.ones", (size_t)N * dsize(dtype), &ones));
+    TRY(ws(h, "ft.ones", (size_t)N * dsize(dtype), &fs.ones));
     std::vector<double> h1(N, 1.0);
     std::vector<float> h1f(N, 1.0f);
-    CK(cudaMemcpyAsync(ones, dtype == SP2_F64 ? (const void*)h1.data() : (const void*)h1f.data(),
+    CK(cudaMemcpyAsync(fs.ones, dtype == SP2_F64 ? (const void*)h1.data() : (const void*)h1f.data(),
                        (size_t)N * dsize(dtype), cudaMemcpyHostToDevice, h->stream));
     CK(cudaStreamSynchronize(h->stream));
-    FMat* r;
-    TRY(fermi_response(c, fs, ones, dtype, 1, true, &r));   // the response to I first
+    // the response to I first, or (defer_i) with the first batch of responses
+    if (!defer_i) TRY(fermi_responses(c, fs, fs.ones, nullptr, 0, dtype, 1, nullptr));
   }
   return SP2_OK;
 }
 
-// First-order response of f(H) to B (chain rule of every doubling); canonical
-// adds -(Tr D1 / Tr R_I) R_I. *result points at the FMat holding it (scratch
-// of fs, valid until the next response).
-int fermi_response(Ctx& c, FermiState& fs, const void* src, int dtype, int diag, bool isI,
-                   FMat** result) {
+// Scratch for batches of up to `want` responses; *B: how many fit. A batch shares each
+// product's launch (one 2048 x 2048 product keeps 64 of 76 CTA pairs busy for one tile:
+// 42 us) and the launches of the passes between them: 4 perturbations at N = 2048,
+// FP16X2, 39.7 -> 31.9 ms with the planes written by k_combine. At most 2^25 entries
+// (2.4 GB of scratch), from where on one matrix's product fills the GPU for several
+// waves. Where memory or the workspace limit leaves no room, smaller batches.
+int fermi_batch(Ctx& c, FermiState& fs, int64_t want, int64_t* B) {
+  sp2_handle_t h = c.h;
+  const int64_t cap = ((int64_t)1 << 25) / (c.np * c.np);
+  int64_t b = want < cap ? want : cap;
+  // (under a workspace limit FP64 leaves the room to the digits of its products)
+  if (b < 1 || (h->limit && c.mode == SP2_MODE_FP64)) b = 1;
+  struct Buf {
+    const char* name;
+    FMat* f;
+  };
+  const Buf bufs[] = {{"ft.dd0", &fs.dd[0]}, {"ft.dd1", &fs.dd[1]}, {"ft.E", &fs.E}, {"ft.F1", &fs.F1},
+                      {"ft.dW", &fs.dW}, {"ft.G1", &fs.G1}, {"ft.P", &fs.P}, {"ft.T", &fs.T},
+                      {"ft.U", &fs.U}};
+  for (;; b = (b + 1) / 2) {
+    int r = SP2_OK;
+    for (const Buf& q : bufs)
+      if (r == SP2_OK) r = fmat(h, q.name, c.np, c.mode, q.f, b);
+    if (r == SP2_OK) r = ws(h, "ft.tr", (size_t)b * sizeof(double), &fs.tr);
+    if (r == SP2_OK) break;
+    if (r != SP2_ENOMEM || b == 1) return r;
+    // (all of them: some may have grown)
+    CK(cudaStreamSynchronize(h->stream));
+    for (const Buf& q : bufs)
+      for (const char* part : {".m", ".h", ".l", ".d", ".s"}) ws_free(h, std::string(q.name) + part);
+    h->err.clear();
+  }
+  fs.B = b;
+  *B = b;
+  return SP2_OK;
+}
+
+// First-order responses of f(H) to K perturbations (chain rule of every doubling);
+// canonical adds -(Tr D1 / Tr R_I) R_I to each. *result: the batch holding them
+// (scratch of fs, valid until the next responses). ones (canonical): the response R_I to
+// the identity, given by its diagonal, is computed in the same batch, kept with its
+// trace. K + (ones ? 1 : 0) is at most the batch of fermi_batch.
+int fermi_responses(Ctx& c, FermiState& fs, const void* ones, const void* src, int64_t K, int dtype,
+                    int diag, FMat* result) {
   sp2_handle_t h = c.h;
   const int mode = c.mode;
   const int n = fs.n;
+  const int64_t e0 = ones ? 1 : 0, B = K + e0, el = c.np * c.np;
+  for (FMat* f : {&fs.dd[0], &fs.dd[1], &fs.E, &fs.F1, &fs.dW, &fs.G1, &fs.P, &fs.T, &fs.U}) f->B = B;
   double* tr = static_cast<double*>(fs.tr);
   int cur = 0;
   FMat& d0 = fs.dd[0];
-  if (mode == SP2_MODE_FP16X2) CK(cudaMemsetAsync(d0.amax, 0, sizeof(float), h->stream));
-  CK(launch_init(src, c.n, c.np, 1, dtype, diag, 0, 0.0, -fs.cst, mode, d0.m, nullptr, 0,
-                 mode == SP2_MODE_FP16X2 ? d0.amax : nullptr, h->stream));
-  c.kernels++;
-  if (mode == SP2_MODE_FP16X2) TRY(fplanes(c, d0));
+  const bool f16 = mode == SP2_MODE_FP16X2;
+  if (f16) CK(cudaMemsetAsync(d0.amax, 0, sizeof(float) * B, h->stream));
+  if (ones) {
+    CK(launch_init(ones, c.n, c.np, 1, dtype, 1, 0, 0.0, -fs.cst, mode, d0.m, nullptr, 0,
+                   f16 ? d0.amax : nullptr, h->stream));
+    c.kernels++;
+  }
+  if (K > 0) {
+    const FMat dk = fentry(d0, e0, c.np, mode);
+    CK(launch_init(src, c.n, c.np, K, dtype, diag, 0, 0.0, -fs.cst, mode, dk.m, nullptr, 0,
+                   f16 ? dk.amax : nullptr, h->stream));
+    c.kernels++;
+  }
+  if (f16) TRY(fplanes(c, d0));
   for (int j = 0; j < n; ++j) {
     FMat& din = fs.dd[cur];
-    FMat& dout = (j == n - 1 && isI) ? fs.RI : fs.dd[1 - cur];
+    FMat& dout = fs.dd[1 - cur];
     // E = d delta delta + delta d delta = Z1 + Z1^T, Z1 = d delta * delta
     TRY(fprod(c, fs.P, din, fs.dl[j]));
     TRY(fcomb(c, fs.E, &fs.P, 1.0, nullptr, 0.0, nullptr, 0.0, 0.0, true));
-    // dW = -4 W E W = -2 (F2 + F2^T), F2 = (W E) W
-    TRY(fprod(c, fs.F1, fs.W[j], fs.E));
+    // dW = -4 W E W = -2 (F2 + F2^T), F2 = F1 W, F1 = W E = (E W)^T
+    if (split_mode(mode)) {
+      TRY(fprod(c, fs.F1, fs.E, fs.W[j], true));
+    } else {
+      for (int64_t b = 0; b < B; ++b) {
+        FMat f1 = fentry(fs.F1, b, c.np, mode);
+        TRY(fprod(c, f1, fs.W[j], fentry(fs.E, b, c.np, mode)));
+      }
+    }
     TRY(fplanes(c, fs.F1));
     TRY(fprod(c, fs.U, fs.F1, fs.W[j]));
     TRY(fcomb(c, fs.dW, &fs.U, -2.0, nullptr, 0.0, nullptr, 0.0, 0.0, true));
-    // d delta' = 2 (d delta W + delta dW) = (G1 + G1^T) + (G2 + G2^T)
+    // d delta' = 2 (d delta W + delta dW) = (G1 + G1^T) + (G2 + G2^T), G2 = dW delta
     TRY(fprod(c, fs.G1, din, fs.W[j]));
-    TRY(fprod(c, fs.T, fs.dl[j], fs.dW));
+    TRY(fprod(c, fs.T, fs.dW, fs.dl[j]));
     TRY(fcomb(c, dout, &fs.G1, 1.0, &fs.T, 1.0, nullptr, 0.0, 0.0, j < n - 1));
     cur = 1 - cur;
   }
-  if (isI) {
-    CK(launch_trace(mode, fs.RI.m.master, c.np, c.n, tr + 1, h->stream));
-    CK(cudaMemcpyAsync(&h->h_state->bounds[1], tr + 1, sizeof(double), cudaMemcpyDeviceToHost,
-                       h->stream));
-    CK(cudaStreamSynchronize(h->stream));
-    fs.trI = h->h_state->bounds[1];
-    c.kernels++;
-    *result = &fs.RI;
-    return SP2_OK;
-  }
   FMat& res = fs.dd[cur];
-  *result = &res;
   if (fs.canonical) {
-    CK(launch_trace(mode, res.m.master, c.np, c.n, tr, h->stream));
-    CK(cudaMemcpyAsync(&h->h_state->bounds[0], tr, sizeof(double), cudaMemcpyDeviceToHost,
-                       h->stream));
-    CK(cudaStreamSynchronize(h->stream));
-    const double trk = h->h_state->bounds[0];
+    std::vector<double> trk((size_t)B);
+    CK(launch_trace(mode, res.m.master, c.np, c.n, B, tr, h->stream));
+    CK(cudaMemcpyAsync(trk.data(), tr, sizeof(double) * B, cudaMemcpyDeviceToHost, h->stream));
     c.kernels++;
+    if (ones)
+      CK(cudaMemcpyAsync(fs.RI.m.master, res.m.master, (size_t)el * master_size(mode),
+                         cudaMemcpyDeviceToDevice, h->stream));
+    CK(cudaStreamSynchronize(h->stream));
+    if (ones) fs.trI = trk[0];
     // res - (trk / trI) RI, written as (a/2)(RI + RI^T) + res (RI is exactly symmetric)
-    TRY(fcomb(c, fs.G1, &fs.RI, -0.5 * trk / fs.trI, nullptr, 0.0, &res, 1.0, 0.0, false));
-    *result = &fs.G1;
+    for (int64_t k = e0; k < B; ++k) {
+      FMat g = fentry(fs.G1, k, c.np, mode);
+      const FMat rk = fentry(res, k, c.np, mode);
+      TRY(fcomb(c, g, &fs.RI, -0.5 * trk[k] / fs.trI, nullptr, 0.0, &rk, 1.0, 0.0, false));
+    }
   }
+  if (result && K > 0) *result = fentry(fs.canonical ? fs.G1 : res, e0, c.np, mode);
   return SP2_OK;
 }
 
@@ -2026,7 +2100,7 @@ int sp2_fermi(sp2_handle_t h, const void* H, int64_t N, int dtype, double mu, do
   Ctx c;
   TRY(make_ctx(h, mode, N, np, o.time_kernels != 0, &c));
   FermiState fs;
-  TRY(fermi_setup(c, fs, Hd, N, dtype, mu, kT, n_doublings, canonical != 0, K > 0));
+  TRY(fermi_setup(c, fs, Hd, N, dtype, mu, kT, n_doublings, canonical != 0, K > 0, true));
   // D = I/2 + delta_n
   if (D) {
     TRY(fcomb(c, fs.P, nullptr, 0.0, nullptr, 0.0, &fs.dl[fs.n], 1.0, 0.5, false));
@@ -2034,15 +2108,28 @@ int sp2_fermi(sp2_handle_t h, const void* H, int64_t N, int dtype, double mu, do
     c.kernels++;
     TRY(finish_out(h, od));
   }
+  // batches from the last perturbation back (the responses may overwrite B), the first
+  // with the response to I
   const int64_t per = b_diag_only ? N : N * N;
-  for (int64_t kk = K - 1; kk >= 0; --kk) {
-    FMat* r;
-    TRY(fermi_response(c, fs, static_cast<const char*>(Bd) + (size_t)kk * per * dsize(dtype), dtype,
-                       b_diag_only, false, &r));
-    CK(launch_copy_out(r->m, N, np, 1, mode, 1.0,
-                       static_cast<char*>(oy.dev) + (size_t)kk * N * N * dsize(dtype), dtype,
+  int64_t batch = 1;
+  if (K > 0) TRY(fermi_batch(c, fs, K + (fs.canonical ? 1 : 0), &batch));
+  bool need_i = fs.canonical;
+  for (int64_t k1 = K; k1 > 0;) {
+    if (need_i && batch == 1) {
+      TRY(fermi_responses(c, fs, fs.ones, nullptr, 0, dtype, 1, nullptr));
+      need_i = false;
+    }
+    const int64_t room = batch - (need_i ? 1 : 0), nk = k1 < room ? k1 : room, k0 = k1 - nk;
+    FMat r;
+    TRY(fermi_responses(c, fs, need_i ? fs.ones : nullptr,
+                        static_cast<const char*>(Bd) + (size_t)k0 * per * dsize(dtype), nk, dtype,
+                        b_diag_only, &r));
+    CK(launch_copy_out(r.m, N, np, nk, mode, 1.0,
+                       static_cast<char*>(oy.dev) + (size_t)k0 * N * N * dsize(dtype), dtype,
                        h->stream));
     c.kernels++;
+    need_i = false;
+    k1 = k0;
   }
   if (K > 0) TRY(finish_out(h, oy));
   CK(cudaStreamSynchronize(h->stream));
@@ -2096,7 +2183,7 @@ int dist_to_identity(Ctx& c, const FMat& T, double* out) {
   TRY(ws(h, "no.part", (size_t)np_ * sizeof(double), &part));
   CK(launch_contract(T.m.master, 1, T.m.master, 1, c.np, mdt, 0, static_cast<double*>(part), np_,
                      d, h->stream));
-  CK(launch_trace(c.mode, T.m.master, c.np, c.n, d + 1, h->stream));
+  CK(launch_trace(c.mode, T.m.master, c.np, c.n, 1, d + 1, h->stream));
   double hv[2];
   CK(cudaMemcpyAsync(hv, d, 2 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
   CK(cudaStreamSynchronize(h->stream));
@@ -2556,9 +2643,9 @@ int sp2_scf_response(sp2_handle_t h, const void* H, int64_t N, int dtype, double
       // one finite-temperature response per field through the kept history
       const size_t per = (size_t)N * dsize(dtype);
       for (int64_t f = 0; f < F; ++f) {
-        FMat* r;
-        TRY(fermi_response(c, fs, static_cast<const char*>(pub) + f * per, dtype, 1, false, &r));
-        CK(launch_site_charges(r->m.master, o.mode, 1, ns, norb, np, qo + f * ns, h->stream));
+        FMat r;
+        TRY(fermi_responses(c, fs, nullptr, static_cast<const char*>(pub) + f * per, 1, dtype, 1, &r));
+        CK(launch_site_charges(r.m.master, o.mode, 1, ns, norb, np, qo + f * ns, h->stream));
         c.kernels++;
       }
     } else {

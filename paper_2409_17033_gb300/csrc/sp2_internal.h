@@ -124,6 +124,43 @@ __device__ __forceinline__ float pow2_scale(float bound) {
   return ldexpf(1.0f, k);
 }
 
+// four consecutive entries of a matrix (idx a multiple of 4): master and, in the split
+// modes, the planes as one 8-byte store each
+template <typename ZT, int MODE>
+__device__ __forceinline__ void store_y4(MatBuf y, int64_t idx, const ZT (&v)[4], float s) {
+  if constexpr (sizeof(ZT) == 4) {
+    *reinterpret_cast<float4*>(static_cast<float*>(y.master) + idx) =
+        make_float4((float)v[0], (float)v[1], (float)v[2], (float)v[3]);
+  } else {
+    double2* d = reinterpret_cast<double2*>(static_cast<double*>(y.master) + idx);
+    d[0] = make_double2((double)v[0], (double)v[1]);
+    d[1] = make_double2((double)v[2], (double)v[3]);
+  }
+  if (MODE == SP2_MODE_BF16X3) {
+    uint16_t h[4], m[4], l[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) split_bf16x3((float)v[j], h[j], m[j], l[j]);
+    *reinterpret_cast<uint2*>(y.hi + idx) =
+        make_uint2(h[0] | ((uint32_t)h[1] << 16), h[2] | ((uint32_t)h[3] << 16));
+    *reinterpret_cast<uint2*>(y.mid + idx) =
+        make_uint2(m[0] | ((uint32_t)m[1] << 16), m[2] | ((uint32_t)m[3] << 16));
+    *reinterpret_cast<uint2*>(y.lo + idx) =
+        make_uint2(l[0] | ((uint32_t)l[1] << 16), l[2] | ((uint32_t)l[3] << 16));
+  }
+  if (MODE == SP2_MODE_BF16X2 || MODE == SP2_MODE_FP16X2) {
+    uint16_t h[4], l[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      if (MODE == SP2_MODE_BF16X2) split_bf16((float)v[j], h[j], l[j]);
+      else split_fp16((float)v[j], s, h[j], l[j]);
+    }
+    *reinterpret_cast<uint2*>(y.hi + idx) =
+        make_uint2(h[0] | ((uint32_t)h[1] << 16), h[2] | ((uint32_t)h[3] << 16));
+    *reinterpret_cast<uint2*>(y.lo + idx) =
+        make_uint2(l[0] | ((uint32_t)l[1] << 16), l[2] | ((uint32_t)l[3] << 16));
+  }
+}
+
 // Per-matrix scale state of a batch of B response matrices (FP16X2 only).
 struct ScaleBuf {
   float* ymax = nullptr;    // [2][B] max |Y| of the matrix in each ping-pong slot
@@ -302,6 +339,7 @@ struct TcLaunch {
   float* zmax = nullptr;           // FP16X2 EPI_PLAIN: per batch entry, receives max |C|
   float* zero = nullptr;           // EPI_PLAIN: nzero floats the launch clears
   int nzero = 0;
+  int trans = 0;                   // EPI_PLAIN: store each batch entry of C transposed
   int tail = 0;                    // split-tail mode (st->plane1 decides per step)
   TcTuning tune;
   // block-sparse square (CTA pairs): tiles, their count and their K-block lists
@@ -391,14 +429,24 @@ cudaError_t launch_fro_scale(const float* master, int64_t np, int64_t batch, dou
 int fro_nparts();
 
 // finite temperature (fermi_kernels.cu)
-// out = z1 (Z1 + Z1^T) + z2 (Z2 + Z2^T) + a A + id I on the padded np x np
-// matrices (null operands skipped, I only on the caller's n x n block);
-// amax (nullable) receives max |out| (must start at 0).
-cudaError_t launch_combine(int mode, void* out, int64_t np, int64_t n, const void* Z1, double z1,
-                           const void* Z2, double z2, const void* A, double a, double id,
-                           float* amax, cudaStream_t s);
-// out[0] = Tr of the caller's n x n block, FP64
-cudaError_t launch_trace(int mode, const void* M, int64_t np, int64_t n, double* out,
+// Max magnitudes of the operands (per batch entry) that fix the FP16X2 plane scale of a
+// combination, and where that scale and the result's own max go; null elsewhere.
+struct CombineScale {
+  const float* z1max = nullptr;
+  const float* z2max = nullptr;
+  const float* amax = nullptr;
+  float* scale = nullptr;
+  float* omax = nullptr;     // (must start at 0)
+};
+// out = z1 (Z1 + Z1^T) + z2 (Z2 + Z2^T) + a A + id I for a batch of padded np x np
+// matrices (null operands skipped, I only on the caller's n x n block), with its
+// planes when `planes`.
+cudaError_t launch_combine(int mode, MatBuf out, int64_t np, int64_t n, int64_t batch,
+                           const void* Z1, double z1, const void* Z2, double z2, const void* A,
+                           double a, double id, bool planes, const CombineScale& cs,
+                           cudaStream_t s);
+// out[b] = Tr of the caller's n x n block of batch entry b, FP64
+cudaError_t launch_trace(int mode, const void* M, int64_t np, int64_t n, int64_t batch, double* out,
                          cudaStream_t s);
 
 // self-consistent response and MLP (scf_kernels.cu)

@@ -1,0 +1,169 @@
+"""The forms a call's sizes choose between: CUDA-core product tiles, narrow tensor-core
+tiles, contraction kernels, and batches of finite-temperature responses, each at the
+sizes where it can go wrong."""
+import ctypes as C
+
+import numpy as np
+import pytest
+import torch
+
+import workloads
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def sp2():
+    import __graft_entry__ as g
+    g.build()
+    import paper_2409_17033_gb300 as p
+    return p
+
+
+def _sym(n, rng, scale=1.0):
+    g = rng.standard_normal((n, n)) * scale
+    return g + g.T
+
+
+# A K-long sum of products in arithmetic of unit roundoff u is off by at most
+# (K + 2) u |a| . |b| <= (K + 2) u ||a|| ||b||; the response adds two such sums, and the
+# update's own roundings of 4 u of its terms.
+@pytest.mark.parametrize("mode,n", [("fp64", 2), ("fp64", 64), ("fp64", 129), ("fp64", 190),
+                                    ("fp64", 200), ("fp32", 2), ("fp32", 127), ("fp32", 300),
+                                    ("fp32", 700), ("fp32", 1026), ("fp32", 1500)])
+@pytest.mark.parametrize("diag", [False, True])
+def test_cuda_core_products(sp2, mode, n, diag):
+    rng = np.random.default_rng(n)
+    dt = np.float64 if mode == "fp64" else np.float32
+    u = 2.0 ** -53 if mode == "fp64" else 2.0 ** -24
+    h = _sym(n, rng).astype(dt)
+    b = np.stack([rng.standard_normal(n) if diag else _sym(n, rng) for _ in range(2)]).astype(dt)
+    for sig in (1, -1):
+        # bounds (-1, 0): X_1 = -H, Y_1 = -B; one step
+        d1, d, _ = sp2.sp2_response(torch.from_numpy(h).cuda(), max(n // 2, 1),
+                                    torch.from_numpy(b).cuda(), diag_only=diag, mode=mode,
+                                    sigma=[sig], bounds=(-1.0, 0.0), want_density=True,
+                                    handle=sp2.Handle(), allow_noconv=True)
+        d1, d = d1.cpu().numpy(), d.cpu().numpy()
+        x = -h.astype(np.float64)
+        nx = np.linalg.norm(x, axis=1)
+        c = x @ x
+        ref = c if sig > 0 else 2.0 * x - c
+        tol = (2 * n + 6) * u * (nx[:, None] * nx[None, :] + np.abs(x))
+        assert np.array_equal(d, d.T) and np.all(np.abs(d - ref) <= tol)
+        for k in range(2):
+            y = -b[k].astype(np.float64)
+            y = np.diag(y) if diag else y
+            ny = np.linalg.norm(y, axis=1)
+            s = y @ x + x @ y
+            ref = s if sig > 0 else 2.0 * y - s
+            cross = ny[:, None] * nx[None, :]
+            tol = (2 * n + 6) * u * (cross + cross.T + np.abs(y))
+            assert np.array_equal(d1[k], d1[k].T) and np.all(np.abs(d1[k] - ref) <= tol)
+
+
+@pytest.mark.parametrize("mode", ["bf16x2", "fp16x2", "bf16x3"])
+@pytest.mark.parametrize("n", [96, 256, 300, 770, 1030])
+def test_narrow_tiles_keep_the_bits(sp2, mode, n):
+    """Tiles of a CTA pair as narrow as the size makes them against 128 x 256 tiles of
+    one SM: the same arithmetic per entry, so the same bits. The recursion's branches are
+    given, since the traces' sums depend on the tiles in their last bits."""
+    p = workloads.random_spectrum(n, nocc=n // 2, k=2, seed=n)
+    H = torch.from_numpy(p.H.astype(np.float32)).cuda()
+    B = torch.from_numpy(p.H1[:2].astype(np.float32)).cuda()
+    out = []
+    for pair in (1, 0):
+        h = sp2.Handle()
+        h.set_option("pair_tiles", pair)
+        d1, d, _ = sp2.sp2_response(H, p.nocc, B, mode=mode, sigma=[1, -1, -1, 1, 1],
+                                    want_density=True, handle=h, allow_noconv=True)
+        out.append((d1.clone(), d.clone()))
+    assert torch.equal(out[0][1], out[1][1]) and torch.equal(out[0][0], out[1][0])
+
+
+# FP32 entries' products are summed exactly up to 2^-40 of their magnitudes (bound
+# 1e-12), FP64 ones by a fused multiply-add each over at most N^2 terms.
+@pytest.mark.parametrize("L,K,n,shift", [(1, 1, 1, 0), (1, 8, 64, 0), (2, 9, 65, 0), (3, 8, 64, 0),
+                                         (3, 7, 130, 0), (5, 17, 101, 0), (4, 16, 96, 1),
+                                         (9, 3, 66, 0)])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
+def test_contraction_forms(sp2, L, K, n, shift, dtype):
+    g = torch.Generator().manual_seed(L * 100 + K)
+    def make(rows):   # shift: the matrices do not start on a 16-byte boundary
+        buf = torch.empty(rows * n * n + shift, dtype=dtype, device="cuda")
+        v = buf[shift:].view(rows, n, n)
+        v.copy_(torch.randn(rows, n, n, generator=g, dtype=torch.float64))
+        return v
+    P, Q = make(L), make(K)
+    out = sp2.response_contract(P, Q, handle=sp2.Handle()).cpu().numpy()
+    p, q = P.double().cpu().numpy().reshape(L, -1), Q.double().cpu().numpy().reshape(K, -1)
+    ref = (p.astype(np.longdouble) @ q.astype(np.longdouble).T)
+    mag = np.abs(p) @ np.abs(q).T
+    tol = (1e-12 if dtype == torch.float32 else (n * n + 40) * 2.0 ** -53) * mag
+    assert np.all(np.abs(out - ref).astype(float) <= tol)
+
+
+def test_contraction_in_a_graph(sp2):
+    """The allocation-free contraction captured behind a copy and a kernel, replayed on
+    other inputs."""
+    from paper_2409_17033_gb300 import _lib
+    lib = _lib.load()
+    P = torch.randn(3, 96, 96, device="cuda")
+    Q = torch.randn(9, 96, 96, device="cuda")
+    src = torch.randn_like(Q)
+    out = torch.zeros(3, 9, dtype=torch.float64, device="cuda")
+
+    def call(stream):
+        return lib.response_contract_noalloc(
+            C.c_void_p(P.data_ptr()), 3, C.c_void_p(Q.data_ptr()), 9, 96, 1, 0,
+            C.c_void_p(out.data_ptr()), C.c_void_p(stream.cuda_stream))
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(s):
+        assert call(s) == 0
+        P.mul_(1.0)
+    s.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=s):
+        Q.copy_(src)
+        assert call(torch.cuda.current_stream()) == 0
+        P.mul_(2.0)
+        assert call(torch.cuda.current_stream()) == 0
+    for _ in range(2):
+        src.normal_()
+        p0 = P.double()
+        torch.cuda.synchronize()
+        graph.replay()
+        torch.cuda.synchronize()
+        ref = torch.einsum("lij,kij->lk", 2.0 * p0, src.double())
+        assert torch.allclose(out, ref, rtol=1e-11, atol=1e-9)
+
+
+@pytest.mark.parametrize("mode,n,k,diag,canonical,limit", [
+    ("fp16x2", 96, 1, False, True, 0), ("fp16x2", 300, 5, True, True, 0),
+    ("fp16x2", 300, 5, False, True, 160 << 20), ("fp16x2", 301, 3, False, False, 0),
+    ("bf16x2", 513, 3, False, True, 0), ("bf16x3", 300, 2, True, False, 0),
+    ("fp32", 130, 3, False, True, 0), ("fp64", 100, 4, True, True, 0),
+    ("fp64", 300, 3, False, True, 0), ("fp64", 300, 3, False, True, 200 << 20)])
+def test_fermi_batches(sp2, mode, n, k, diag, canonical, limit):
+    """Responses computed as a batch against one perturbation at a time: the same
+    arithmetic per entry (FP64: the same error-free products, or sums in another order,
+    whose rounding the doublings carry: 1e-10)."""
+    rng = np.random.default_rng(n)
+    dt = torch.float64 if mode == "fp64" else torch.float32
+    H = torch.from_numpy(_sym(n, rng, 0.3 / np.sqrt(n))).to(dt).cuda()
+    b = rng.standard_normal((k, n)) if diag else np.stack([_sym(n, rng) for _ in range(k)])
+    b *= 10.0 ** (2 * np.arange(k)).reshape((k,) + (1,) * (b.ndim - 1))
+    B = torch.from_numpy(b).to(dt).cuda()
+    kw = dict(diag_only=diag, canonical=canonical, mode=mode, n_doublings=12)
+    h = sp2.Handle(limit) if limit else sp2.Handle()
+    D1, D, _ = sp2.sp2_fermi(H, 0.05, 0.1, B, handle=h, **kw)
+    one = sp2.Handle()
+    for i in range(k):
+        r, d, _ = sp2.sp2_fermi(H, 0.05, 0.1, B[i:i + 1].contiguous(), handle=one, **kw)
+        assert torch.equal(D, d)
+        assert (torch.equal(D1[i], D1[i].T) if mode != "fp64" else True)
+        if mode == "fp64":
+            assert (D1[i] - r[0]).norm() <= 1e-10 * r[0].norm()
+        else:
+            assert torch.equal(D1[i], r[0])
