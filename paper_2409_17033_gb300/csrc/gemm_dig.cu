@@ -31,6 +31,11 @@
 // Layout. The planes are stored transposed, G[j * rows + i] for entry (i, j): a warp's
 // lanes hold consecutive rows i, so its stores are whole lines.
 //
+// A step that carries responses forms Y_n X_n and X_n^2 in one launch, X_n stacked below
+// the batch Y_n (upper tiles only): its digits are made once, and at small N the square's
+// tiles run on CTA pairs that the response's leave idle (SCF of 16 fields at N = 256,
+// where the square took 30 us of a step on the CUDA cores: 28.7 -> 21.4 ms).
+//
 // Per product: k_digits (each factor), k_gemm_dig, then one pass that turns the sums
 // into FP64 and applies the recursion's update: k_dig_square
 // (Eq. DM0, with the traces and the step decision), k_dig_symm (Eqs. DM1-DM3) or
@@ -96,7 +101,9 @@ struct DParams {
   int ksplit;          // K parts
   int parts;           // weight parts (1, 2 or 4)
   int64_t rows;        // rows of A (plane stride of its map, leading dimension of G)
-  int64_t np;          // rows of X per plane
+  int64_t np;
+  int64_t xrows;       // rows of X's map per plane, and the first of X's own
+  int xoff;
   int* G;              // planes (K part x weight) of np x rows sums
   const Tile* tiles;
   int nunits;          // tiles x parts x ksplit
@@ -197,7 +204,7 @@ k_gemm_dig(const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUt
       for (int s = kGroups - 1; s >= 0 && ok; --s) {
         if (!((w.mask >> s) & 1u)) continue;
         for (int i = 0; i <= s && ok; ++i) {
-          const int ay = i * (int)p.rows + arow, by = (s - i) * (int)p.np + brow;
+          const int ay = i * (int)p.rows + arow, by = (s - i) * (int)p.xrows + p.xoff + brow;
           for (int kx = w.kb0 * BK; kx < w.kb1 * BK; kx += BK, ++g, rp.next()) {
             ok = __all_sync(0xffffffffu, mbar_wait<true>(&empty[rp.s], rp.ph ^ 1u, abortf, p.wait_ns));
             if (!ok) break;
@@ -353,22 +360,24 @@ __device__ __forceinline__ bool halted_dig(const DevState* st, int step) {
 }
 
 // ------------------------------------------------------------ digits
-// One block per row: the row's power-of-two scale 2^ex >= its 2-norm, then the
-// eight digit planes (plane d of the stack at d * rows * np). Integer arithmetic throughout (FP64 conversions run at the slow
-// FP64 rate); the norm in FP32 from the entries' leading 20 bits, relative to the
+// One block per row (of two stacked matrices): the row's power-of-two scale 2^ex >= its 2-norm, then the
+// eight digit planes (plane d of the stack at d * rows * np). Integer arithmetic
+// throughout (FP64 conversions run at the slow FP64 rate); the norm in FP32 from the entries' leading 20 bits, relative to the
 // row's largest entry, with a margin above its rounding. HBM-bound at large N: 8
 // bytes read, 16 written per entry.
 constexpr int kDigThreads = 128;
 
 __global__ void __launch_bounds__(kDigThreads)
-k_digits(const double* __restrict__ src, int64_t rows, int64_t np, uint16_t* __restrict__ dig,
-         int* __restrict__ ex, const DevState* st, int step) {
+k_digits(const double* __restrict__ src, int64_t rows1, const double* __restrict__ src2,
+         int64_t rows, int64_t np, uint16_t* __restrict__ dig, int* __restrict__ ex,
+         const DevState* st, int step) {
   dep_sync();
   if (halted_dig(st, step)) return;
   __shared__ uint32_t smax[kDigThreads / 32];
   __shared__ float ssum[kDigThreads / 32];
   const int64_t row = blockIdx.x;
-  const double2* x2 = reinterpret_cast<const double2*>(src + row * np);
+  const double2* x2 =
+      reinterpret_cast<const double2*>(row < rows1 ? src + row * np : src2 + (row - rows1) * np);
   const int n4 = (int)(np / 4);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   uint32_t m = 0;
@@ -466,6 +475,7 @@ struct Sums {
 __device__ __forceinline__ void load_t(const Sums& q, int64_t o, long long (&t)[4]) {
 #pragma unroll
   for (int k = 0; k < 4; ++k) t[k] = 0;
+  long long last[4] = {0, 0, 0, 0};   // the last weight's sum over the K parts, rounded once
   for (int ks = 0; ks < q.ksplit; ++ks) {
     int4 v[kGroups];
 #pragma unroll
@@ -476,11 +486,14 @@ __device__ __forceinline__ void load_t(const Sums& q, int64_t o, long long (&t)[
       const int x[4] = {v[s].x, v[s].y, v[s].z, v[s].w};
       const int sh = 2 * 56 - 8 * s - (2 * kFixBits - kTBits);
 #pragma unroll
-      for (int k = 0; k < 4; ++k)
-        t[k] += sh >= 0 ? (long long)x[k] << (sh > 0 ? sh : 0)
-                        : (long long)((x[k] + (1 << 7)) >> 8);   // at most 2^30
+      for (int k = 0; k < 4; ++k) {
+        if (sh >= 0) t[k] += (long long)x[k] << (sh > 0 ? sh : 0);
+        else last[k] += x[k];
+      }
     }
   }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) t[k] += (last[k] + (1 << 7)) >> 8;
 }
 
 // T's value as FP64 (one rounding), times 2^e. The conversion by magic constants
@@ -526,12 +539,12 @@ __device__ __forceinline__ void st4d(double* p, const double (&v)[4]) {
 
 // X_{n+1} = sigma > 0 ? C : 2 X_n - C from T (C = X_n^2, upper entries), mirrored;
 // partials of Tr, ||.||_F^2 and ||X_n - X_n^2||_F^2 in FP64, and the step decision
-// in the last block. Blocks walk pairs of TE x TE tiles (I <= J); T's tile (J, I)
+// in the last block. G has leading dimension ld. Blocks walk pairs of TE x TE tiles (I <= J); T's tile (J, I)
 // holds entries (i, j) of the upper tile with i along its rows. Bound by its 6 FP64
 // operations per upper entry (an FP64 instruction of a warp takes 64 clocks), so
 // the reductions come once per block, not per tile, ||.||_F^2 and f sharing them.
 __global__ void __launch_bounds__(kPassThreads)
-k_dig_square(const Sums q, const int* __restrict__ ex,
+k_dig_square(const Sums q, int64_t ld, const int* __restrict__ ex,
              const double* __restrict__ X, double* __restrict__ out, int64_t np, int ntiles,
              DevState* st, int step, Part3* __restrict__ part, SimtDecide dec) {
   dep_sync();
@@ -552,7 +565,7 @@ k_dig_square(const Sums q, const int* __restrict__ ex,
     {
       long long t[4];
       double x[4];
-      load_t(q, gj * np + gi0, t);
+      load_t(q, gj * ld + gi0, t);
       ld4d(X + gj * np + gi0, x);   // X_n is symmetric
       const int ej = ex[gj];
 #pragma unroll
@@ -620,7 +633,8 @@ k_dig_square(const Sums q, const int* __restrict__ ex,
 }
 
 // Y_{n+1} = sigma > 0 ? Z + Z^T : 2 Y_n - (Z + Z^T) for a batch, Z = Y_n X_n from T
-// (ey: exponents of the stacked rows of Y_n, ex: of X_n). One block per tile pair
+// (ey: exponents of the stacked rows of Y_n, ex: of X_n; rows: G's leading dimension).
+// One block per tile pair
 // and batch entry.
 __global__ void __launch_bounds__(kPassThreads)
 k_dig_symm(const Sums q, int64_t rows, const int* __restrict__ ey,
@@ -748,13 +762,14 @@ int64_t dig_tiles(int64_t rows, int64_t np, int bn, bool upper) {
 
 // Tile width and cut of one product: the fewest clocks of the busiest CTA pair by
 // the estimate below.
-DigPlan dig_plan(int64_t rows, int64_t np, bool upper) {
+DigPlan dig_plan(int64_t rows, int64_t np, bool upper, bool with_x) {
   const int nkb = (int)(np / BK);
   const int resident = 76;
   DigPlan best;
   double tbest = 0.0;
   for (int bn = 256; bn >= 128; bn -= 128) {
-    const int64_t nt = dig_tiles(rows, np, bn, upper);
+    const int64_t nt = dig_tiles(rows, np, bn, upper) + (with_x ? dig_tiles(np, np, bn, true) : 0);
+    const double sums = ((upper ? 0.5 : 1.0) * (double)rows + (with_x ? 0.5 * (double)np : 0.0)) * (double)np;
     const double chunk = bn == 256 ? 2500.0 : 1700.0, fold = bn == 256 ? 6000.0 : 3000.0;
     for (int parts = 1; parts <= 4; parts *= 2)
       for (int ks = (nkb + KSEG_MAX - 1) / KSEG_MAX; ks <= nkb / KCH; ++ks) {
@@ -765,7 +780,7 @@ DigPlan dig_plan(int64_t rows, int64_t np, bool upper) {
         const int folds = parts == 1 ? 8 : (parts == 2 ? 5 : 2);
         // clocks: the waves, and the pass that reads the sums' planes
         const double t = (double)waves * ((double)kPairs / parts * (kseg / KCH) * chunk + folds * fold) +
-                         (double)ks * (upper ? 0.5 : 1.0) * (double)rows * (double)np * 32.0 / 3000.0;
+                         (double)ks * sums * 32.0 / 3000.0;
         if (tbest == 0.0 || t < tbest) {
           tbest = t;
           best.bn = bn;
@@ -778,9 +793,11 @@ DigPlan dig_plan(int64_t rows, int64_t np, bool upper) {
   return best;
 }
 
-cudaError_t launch_digits(const double* src, int64_t rows, int64_t np, const DigOperand& o,
-                          const DevState* st, int step, cudaStream_t s) {
-  launch_dep(k_digits, (unsigned)rows, kDigThreads, 0, s, src, rows, np, o.dig, o.ex, st, step);
+cudaError_t launch_digits(const double* src, int64_t rows, const double* src2, int64_t rows2,
+                          int64_t np, const DigOperand& o, const DevState* st, int step,
+                          cudaStream_t s) {
+  launch_dep(k_digits, (unsigned)(rows + rows2), kDigThreads, 0, s, src, rows, src2, rows + rows2, np,
+             o.dig, o.ex, st, step);
   return cudaGetLastError();
 }
 
@@ -788,11 +805,12 @@ cudaError_t launch_gemm_dig(const DigOperand& A, int64_t rows, const DigOperand&
                             int* G, const Tile* tiles, int ntiles, const DigPlan& plan,
                             DevState* st, int step, const TcTuning& tune,
                             cudaStream_t s) {
-  if (np % 256 != 0 || rows % 256 != 0 || kDigits * rows > (int64_t)1 << 30)
+  if (np % 256 != 0 || rows % 256 != 0 || X.rows < X.off + np || X.off % 256 != 0 ||
+      kDigits * rows > (int64_t)1 << 30 || kDigits * X.rows > (int64_t)1 << 30)
     return cudaErrorInvalidValue;
   CUtensorMap am, bm;
   if (!make_map(&am, A.dig, kDigits * rows, np, BM, false) ||
-      !make_map(&bm, X.dig, kDigits * np, np, plan.bn / 2, false))
+      !make_map(&bm, X.dig, kDigits * X.rows, np, plan.bn / 2, false))
     return cudaErrorInvalidValue;
   DParams p;
   p.nkb = (int)(np / BK);
@@ -801,6 +819,8 @@ cudaError_t launch_gemm_dig(const DigOperand& A, int64_t rows, const DigOperand&
   p.parts = plan.parts;
   p.rows = rows;
   p.np = np;
+  p.xrows = X.rows;
+  p.xoff = (int)X.off;
   p.G = G;
   p.tiles = tiles;
   p.nunits = ntiles * plan.parts * plan.ksplit;
@@ -819,20 +839,20 @@ int64_t dig_square_nparts(int64_t np) {
   return n < 456 ? n : 456;
 }
 
-cudaError_t launch_dig_square(const int* G, int ksplit, const int* ex, const double* X,
-                              double* out, int64_t np, DevState* st, int step, Part3* part,
+cudaError_t launch_dig_square(const int* G, int ksplit, int64_t ld, int64_t off, const int* ex,
+                              const double* X, double* out, int64_t np, DevState* st, int step, Part3* part,
                               const SimtDecide* dec, cudaStream_t s) {
   SimtDecide sd;
   if (dec) sd = *dec;
   launch_dep(k_dig_square, (unsigned)dig_square_nparts(np), kPassThreads, 0, s, 
-      Sums{G, np * np, ksplit}, ex, X, out, np, (int)tri_tiles(np), st, step, part, sd);
+      Sums{G + off, np * ld, ksplit}, ld, ex, X, out, np, (int)tri_tiles(np), st, step, part, sd);
   return cudaGetLastError();
 }
 
-cudaError_t launch_dig_symm(const int* G, int ksplit, int64_t rows, const int* ey, const int* ex,
-                            const double* yin, double* yout, int64_t np, const DevState* st,
-                            int step, cudaStream_t s) {
-  const dim3 grid((unsigned)tri_tiles(np), (unsigned)(rows / np));
+cudaError_t launch_dig_symm(const int* G, int ksplit, int64_t rows, int64_t batch, const int* ey,
+                            const int* ex, const double* yin, double* yout, int64_t np,
+                            const DevState* st, int step, cudaStream_t s) {
+  const dim3 grid((unsigned)tri_tiles(np), (unsigned)batch);
   launch_dep(k_dig_symm, grid, kPassThreads, 0, s, Sums{G, rows * np, ksplit}, rows, ey, ex, yin, yout, np, st,
                                            step);
   return cudaGetLastError();

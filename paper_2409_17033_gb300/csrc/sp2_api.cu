@@ -40,6 +40,7 @@ struct sp2_handle_s {
   // the workspace limit leaves no room for another buffer they are given back and
   // the rest of the call's FP64 products run on the CUDA cores (dig_off).
   bool dig_off = false;
+  bool dig_apart = false;       // no room for a step's two products in one launch
   const void* dig_x = nullptr;  // the matrix whose digits "dig.x" holds, this step
   // Every step's decision writes a snapshot into a pinned ring (kRing slots); the
   // host waits only for the step kLookahead behind the one it enqueues, so the GPU
@@ -288,11 +289,12 @@ int parts_per_tile(sp2_handle_t h, int mode) { return split_mode(mode) && h->tun
 // row blocks sweep the column blocks together, so CTAs resident at the same
 // time share their operand slices. upper=true keeps only tiles that meet the
 // upper triangle (row0 <= last column), which suffices for symmetric results.
+// Of the rows from upper_from on (if any) only those tiles are kept in any case.
 int tile_list(sp2_handle_t h, int mode, int64_t rows, int64_t np, bool upper, const Tile** d,
-              int* n, int bm, int bn) {
-  char key[96];
-  snprintf(key, sizeof key, "%d/%lld/%lld/%d/%dx%d", mode, (long long)rows, (long long)np,
-           (int)upper, bm, bn);
+              int* n, int bm, int bn, int64_t upper_from = -1) {
+  char key[128];
+  snprintf(key, sizeof key, "%d/%lld/%lld/%d/%dx%d/%lld", mode, (long long)rows, (long long)np,
+           (int)upper, bm, bn, (long long)upper_from);
   auto it = h->tiles.find(key);
   if (it != h->tiles.end()) {
     *d = it->second.d;
@@ -307,7 +309,8 @@ int tile_list(sp2_handle_t h, int mode, int64_t rows, int64_t np, bool upper, co
     for (int64_t cn = 0; cn < nn; ++cn)
       for (int64_t m = g0; m < g0 + gs; ++m) {
         const int64_t r0 = m * bm, c0 = cn * bn;
-        if (upper && r0 % np > c0 + bn - 1) continue;   // row within its batch entry
+        const bool up = upper || (upper_from >= 0 && r0 >= upper_from);
+        if (up && r0 % np > c0 + bn - 1) continue;   // row within its batch entry
         v.push_back(Tile{(int)r0, (int)c0});
       }
   }
@@ -389,9 +392,9 @@ int tc_common(Ctx& c, TcLaunch* L, int ntiles) {
 // --------------------------------------------------------------- FP64 products by digits
 // FP64 products padded to kPad take the tensor-core form (gemm_dig.cu) as long as
 // its buffers fit: above np = 256, and at np = 256 for a stacked factor of two or
-// more matrices (one 256 x 256 product: 23 us and its passes against 34 us on the
-// CUDA cores; per SP2 step at N = 256, 71 against 59 us alone, 133 against 320 us
-// with 8 responses).
+// more matrices (a batch of responses with X_n below it, 512 rows or more: the SCF's
+// step of 16 fields 87 -> 65 us; one 256 x 256 product alone is faster on the CUDA
+// cores: per SP2 step at N = 256 without responses, 71 against 59 us).
 bool dig_mode(const Ctx& c, int64_t rows) {
   return c.mode == SP2_MODE_FP64 && c.np % kPad == 0 && !c.h->dig_off &&
          (c.np > kPad || rows >= 2 * kPad);
@@ -414,33 +417,36 @@ struct DigBufs {
 };
 
 // The buffers of one product of a rows x np left factor (0: the square of the
-// right factor). False when they do not fit: the caller takes the CUDA-core form,
+// right factor; with_x: the right factor stacked below the left one, and its square
+// formed as well). False when they do not fit: the caller takes the CUDA-core form,
 // as the rest of the call does.
-bool dig_bufs(Ctx& c, int64_t rows, bool upper, DigBufs* b) {
+bool dig_bufs(Ctx& c, int64_t rows, bool upper, DigBufs* b, bool with_x = false) {
   sp2_handle_t h = c.h;
-  const size_t el = (size_t)c.np * c.np, ra = (size_t)rows * c.np;
+  const int64_t left = rows + (with_x ? c.np : 0);   // rows of the stacked left factor
+  const size_t el = (size_t)c.np * c.np, ra = (size_t)left * c.np;
   const size_t nt = rows ? ra : el;
-  void *xd, *xe, *G, *ad = nullptr, *ae = nullptr;
-  const int64_t rr = rows ? rows : c.np;
-  b->plan = dig_plan(rr, c.np, upper);
+  void *xd = nullptr, *xe = nullptr, *G, *ad = nullptr, *ae = nullptr;
+  b->plan = dig_plan(rows ? rows : c.np, c.np, upper, with_x);
   const void* old_x = h->bufs["dig.x"].p;
-  bool ok = ws_try(h, "dig.x", el * 2 * kDigPlanes, &xd) == SP2_OK &&
-            ws_try(h, "dig.xe", (size_t)c.np * sizeof(int), &xe) == SP2_OK &&
+  bool ok = (with_x || (ws_try(h, "dig.x", el * 2 * kDigPlanes, &xd) == SP2_OK &&
+                        ws_try(h, "dig.xe", (size_t)c.np * sizeof(int), &xe) == SP2_OK)) &&
             ws_try(h, "dig.G", nt * 4 * kDigPlanes * b->plan.ksplit, &G) == SP2_OK;
   if (ok && rows)
     ok = ws_try(h, "dig.a", ra * 2 * kDigPlanes, &ad) == SP2_OK &&
-         ws_try(h, "dig.ae", (size_t)rows * sizeof(int), &ae) == SP2_OK;
+         ws_try(h, "dig.ae", (size_t)left * sizeof(int), &ae) == SP2_OK;
   if (ok)
-    ok = tile_list(h, c.mode, rr, c.np, upper, &b->tiles, &b->ntiles, 256, b->plan.bn) == SP2_OK;
+    ok = tile_list(h, c.mode, rows ? left : c.np, c.np, upper, &b->tiles, &b->ntiles, 256, b->plan.bn,
+                   with_x ? rows : -1) == SP2_OK;
   if (!ok) {
     h->err.clear();
     drop_digits(h);
-    h->dig_off = true;
+    (with_x ? h->dig_apart : h->dig_off) = true;
     return false;
   }
-  if (old_x != xd) h->dig_x = nullptr;
-  b->x = DigOperand{static_cast<uint16_t*>(xd), static_cast<int*>(xe)};
-  b->a = rows ? DigOperand{static_cast<uint16_t*>(ad), static_cast<int*>(ae)} : b->x;
+  if (with_x || old_x != xd) h->dig_x = nullptr;
+  b->x = DigOperand{static_cast<uint16_t*>(xd), static_cast<int*>(xe), c.np, 0};
+  b->a = rows ? DigOperand{static_cast<uint16_t*>(ad), static_cast<int*>(ae), left, 0} : b->x;
+  if (with_x) b->x = DigOperand{b->a.dig, b->a.ex, left, rows};
   b->G = static_cast<int*>(G);
   return true;
 }
@@ -448,6 +454,55 @@ bool dig_bufs(Ctx& c, int64_t rows, bool upper, DigBufs* b) {
 // work of one digit product: tensor flops of the tiles' 36 digit pairs
 double dig_flops(const Ctx& c, const DigBufs& b) {
   return 2.0 * 256.0 * b.plan.bn * (double)c.np * 36.0 * b.ntiles;
+}
+
+int last_block_decides(Ctx& c, const DecideParams& dec, SimtDecide* sd) {
+  void* dn;
+  TRY(ws(c.h, "decide.done", sizeof(unsigned), &dn));
+  sd->p = dec;
+  sd->st = c.st;
+  sd->done = static_cast<unsigned*>(dn);
+  return SP2_OK;
+}
+
+// One FP64 step with responses by digits, Y_n X_n and X_n^2 in one product launch, and
+// the step decision. *done stays false where it does not apply (other modes, a batch
+// that is cut, no room): the caller takes the steps one by one.
+int dig_step(Ctx& c, const MatBuf& xin, const MatBuf& xout, const MatBuf& yin, const MatBuf& yout,
+             int64_t batch, int step, const DecideParams* dec, bool* done) {
+  sp2_handle_t h = c.h;
+  const int64_t rows = batch * c.np;
+  DigBufs db;
+  if (!dig_mode(c, rows + c.np) || h->dig_apart || dig_chunk(c.np, batch + 1) <= batch) return SP2_OK;
+  if (!dig_bufs(c, rows, false, &db, true)) return SP2_OK;
+  SimtDecide sd;
+  TRY(last_block_decides(c, *dec, &sd));
+  sd.p.nparts = (int)dig_square_nparts(c.np);
+  const double *x = static_cast<const double*>(xin.master), *y = static_cast<const double*>(yin.master);
+  const int64_t left = rows + c.np;
+  CK(launch_digits(y, rows, x, c.np, c.np, db.a, c.st, step, h->stream));
+  cudaEvent_t e0 = nullptr, e1 = nullptr;
+  if (c.timing) {
+    TRY(ev_pair(c, &e0, &e1));
+    CK(cudaEventRecord(e0, h->stream));
+  }
+  CK(launch_gemm_dig(db.a, left, db.x, c.np, db.G, db.tiles, db.ntiles, db.plan, c.st, step, h->tune,
+                     h->stream));
+  if (c.timing) {
+    CK(cudaEventRecord(e1, h->stream));
+    c.timed.push_back({step, 0});
+  }
+  const int* xe = db.a.ex + rows;
+  CK(launch_dig_symm(db.G, db.plan.ksplit, left, batch, db.a.ex, xe, y,
+                     static_cast<double*>(yout.master), c.np, c.st, step, h->stream));
+  CK(launch_dig_square(db.G, db.plan.ksplit, left, rows, xe, x, static_cast<double*>(xout.master),
+                       c.np, c.st, step, c.part, &sd, h->stream));
+  c.launches++;
+  c.kernels += 4;
+  c.flops += dig_flops(c, db);
+  c.alg += (double)c.n * (double)c.n * (2.0 * (double)batch * (double)c.n + (double)(c.n + 1));
+  *done = true;
+  return SP2_OK;
 }
 
 // X_{n+1} = sigma_n>0 ? X_n^2 : 2 X_n - X_n^2, with trace partials; dec: and the step
@@ -458,20 +513,14 @@ int square_step(Ctx& c, const MatBuf& xin, const MatBuf& xout, int step,
   sp2_handle_t h = c.h;
   DigBufs db;
   SimtDecide sd;
-  if (dec) {
-    void* dn;
-    TRY(ws(h, "decide.done", sizeof(unsigned), &dn));
-    sd.p = *dec;
-    sd.st = c.st;
-    sd.done = static_cast<unsigned*>(dn);
-  }
+  if (dec) TRY(last_block_decides(c, *dec, &sd));
   if (dig_mode(c, c.np)) {
     sd.p.nparts = (int)dig_square_nparts(c.np);
     if (dig_bufs(c, 0, true, &db)) {
       const double* x = static_cast<const double*>(xin.master);
       // (the response product of this step has left X_n's digits)
       if (h->dig_x != xin.master) {
-        CK(launch_digits(x, c.np, c.np, db.x, c.st, step, h->stream));
+        CK(launch_digits(x, c.np, nullptr, 0, c.np, db.x, c.st, step, h->stream));
         c.kernels++;
       }
       h->dig_x = nullptr;
@@ -486,7 +535,7 @@ int square_step(Ctx& c, const MatBuf& xin, const MatBuf& xout, int step,
         CK(cudaEventRecord(e1, h->stream));
         c.timed.push_back({step, 0});
       }
-      CK(launch_dig_square(db.G, db.plan.ksplit, db.x.ex, x, static_cast<double*>(xout.master), c.np, c.st, step,
+      CK(launch_dig_square(db.G, db.plan.ksplit, c.np, 0, db.x.ex, x, static_cast<double*>(xout.master), c.np, c.st, step,
                            c.part, dec ? &sd : nullptr, h->stream));
       c.launches++;
       c.kernels += 2;
@@ -625,7 +674,7 @@ int response_step(Ctx& c, const MatBuf& x, const MatBuf& yin, const MatBuf& yout
     if (dig_bufs(c, bc * c.np, false, &db)) {
       const double* y = static_cast<const double*>(yin.master);
       double* yo = static_cast<double*>(yout.master);
-      CK(launch_digits(static_cast<const double*>(x.master), c.np, c.np, db.x, c.st, step,
+      CK(launch_digits(static_cast<const double*>(x.master), c.np, nullptr, 0, c.np, db.x, c.st, step,
                        h->stream));
       h->dig_x = x.master;
       c.kernels++;
@@ -639,7 +688,7 @@ int response_step(Ctx& c, const MatBuf& x, const MatBuf& yin, const MatBuf& yout
           db.plan.kseg = kseg;
           TRY(tile_list(h, c.mode, r, c.np, false, &db.tiles, &db.ntiles, 256, db.plan.bn));
         }
-        CK(launch_digits(y + off, r, c.np, db.a, c.st, step, h->stream));
+        CK(launch_digits(y + off, r, nullptr, 0, c.np, db.a, c.st, step, h->stream));
         cudaEvent_t e0 = nullptr, e1 = nullptr;
         if (c.timing) {
           TRY(ev_pair(c, &e0, &e1));
@@ -651,7 +700,7 @@ int response_step(Ctx& c, const MatBuf& x, const MatBuf& yin, const MatBuf& yout
           CK(cudaEventRecord(e1, h->stream));
           c.timed.push_back({step, 0});
         }
-        CK(launch_dig_symm(db.G, db.plan.ksplit, r, db.a.ex, db.x.ex, y + off, yo + off, c.np, c.st, step,
+        CK(launch_dig_symm(db.G, db.plan.ksplit, r, nb, db.a.ex, db.x.ex, y + off, yo + off, c.np, c.st, step,
                            h->stream));
         c.launches++;
         c.kernels += 3;
@@ -786,7 +835,7 @@ int resolve_ckpt(sp2_handle_t h, sp2_opts* o, int64_t np, int64_t batch) {
   const double b = (double)(batch > 0 ? batch : 1);
   avail -= 2.0 * mat_b + 2.0 * b * mat_b + b * el * ms + (double)(1ull << 30);
   if (o->mode == SP2_MODE_FP64 && np % kPad == 0)   // digit buffers
-    avail -= el * (16.0 + 48.0 * (double)dig_chunk(np, batch > 0 ? batch : 1));
+    avail -= el * (16.0 + 48.0 * (double)dig_chunk(np, batch > 0 ? batch + 1 : 1));
   const int cap = o->fixed_m > 0 ? o->fixed_m : o->max_iter;
   int k = cap;
   for (int kk = 1; kk <= cap; ++kk) {
@@ -1038,12 +1087,17 @@ int run_sp2(sp2_handle_t h, const void* Hd, int64_t n, int dtype, double nocc, c
         CK(cudaMemcpyAsync(ck, xin.master, xbytes, cudaMemcpyDeviceToDevice, h->stream));
       }
     }
-    if (ybatch > 0)
-      TRY(response_step(c, xin, Y[step % 2], Y[(step + 1) % 2], ybatch, step, sc, step % 2,
-                        (step + 1) % 2));
     dp.n = step + 1;
     ring_slot(h, step, &dp);
-    if (sparse) {
+    bool squared = false;
+    if (ybatch > 0)
+      TRY(dig_step(c, xin, xo, Y[step % 2], Y[(step + 1) % 2], ybatch, step, &dp, &squared));
+    if (ybatch > 0 && !squared)
+      TRY(response_step(c, xin, Y[step % 2], Y[(step + 1) % 2], ybatch, step, sc, step % 2,
+                        (step + 1) % 2));
+    if (squared) {
+      // (both products of the step are under way)
+    } else if (sparse) {
       TRY(sparse_square(c, xin, xo, step, sb));
       CK(launch_sparse_plan(sb, 0, (step + 1) % 2, step % 2, (step + 1) % 2, c.part, 0, c.st, step,
                             h->stream));
@@ -1162,6 +1216,7 @@ int make_ctx(sp2_handle_t h, int mode, int64_t n, int64_t np, bool timing, Ctx* 
   int64_t maxp = (np / bm) * (np / bn) * parts_per_tile(h, mode) + 8;
   if (maxp < init_nparts(np)) maxp = init_nparts(np);
   h->dig_off = false;
+  h->dig_apart = false;
   h->dig_x = nullptr;
   if (dig_mode(*c, np) && maxp < dig_square_nparts(np)) maxp = dig_square_nparts(np);
   void* p;
@@ -1438,9 +1493,9 @@ int fprod(Ctx& c, FMat& C, const FMat& L, const FMat& R, bool trans = false) {
   const int64_t rows = L.B * c.np;
   if (dig_mode(c, rows) && dig_bufs(c, same ? 0 : rows, false, &db)) {
     const double* l = static_cast<const double*>(L.m.master);
-    CK(launch_digits(l, rows, c.np, db.a, c.st, 0, h->stream));
+    CK(launch_digits(l, rows, nullptr, 0, c.np, db.a, c.st, 0, h->stream));
     if (!same)
-      CK(launch_digits(static_cast<const double*>(R.m.master), c.np, c.np, db.x, c.st, 0,
+      CK(launch_digits(static_cast<const double*>(R.m.master), c.np, nullptr, 0, c.np, db.x, c.st, 0,
                        h->stream));
     h->dig_x = nullptr;
     cudaEvent_t e0 = nullptr, e1 = nullptr;

@@ -391,28 +391,34 @@ constexpr int kDigPlanes = 8;
 struct DigOperand {        // digit planes of a rows x np factor and its rows' exponents
   uint16_t* dig = nullptr; // kDigPlanes x rows x np, bfloat16 integers
   int* ex = nullptr;       // rows
+  int64_t rows = 0, off = 0;   // rows of a plane, and the operand's first (a right factor
+                               // may be the last matrix of a stacked left one)
 };
 struct DigPlan {           // tile width of a CTA pair and the cut of a tile's work
   int bn = 256, parts = 1, ksplit = 1, kseg = 4;
 };
-DigPlan dig_plan(int64_t rows, int64_t np, bool upper);
+// with_x: np more rows, of which only the upper tiles are formed
+DigPlan dig_plan(int64_t rows, int64_t np, bool upper, bool with_x = false);
 int64_t dig_square_nparts(int64_t np);   // partials of launch_dig_square
-// digits of src (rows x np)
-cudaError_t launch_digits(const double* src, int64_t rows, int64_t np, const DigOperand& o,
-                          const DevState* st, int step, cudaStream_t s);
+// digits of src (rows x np) and, below it, of src2 (rows2 x np; rows2 may be 0)
+cudaError_t launch_digits(const double* src, int64_t rows, const double* src2, int64_t rows2,
+                          int64_t np, const DigOperand& o, const DevState* st, int step,
+                          cudaStream_t s);
 // G: kDigPlanes x plan.ksplit planes of np x rows 32-bit sums, [j * rows + i] for entry
 // (i, j) of A X, over the listed 256 x plan.bn tiles
 cudaError_t launch_gemm_dig(const DigOperand& A, int64_t rows, const DigOperand& X, int64_t np,
                             int* G, const Tile* tiles, int ntiles, const DigPlan& plan,
                             DevState* st, int step, const TcTuning& tune, cudaStream_t s);
 // the passes from G: the square step with its partials (and, with dec, the step
-// decision), the symmetrised response update of a batch, C = A X
-cudaError_t launch_dig_square(const int* G, int ksplit, const int* ex, const double* X, double* out,
+// decision), the symmetrised response update of a batch, C = A X. The square's and the
+// response's sums may lie in a larger G: its leading dimension and the first row.
+cudaError_t launch_dig_square(const int* G, int ksplit, int64_t ld, int64_t off, const int* ex,
+                              const double* X, double* out,
                               int64_t np, DevState* st, int step, Part3* part,
                               const SimtDecide* dec, cudaStream_t s);
-cudaError_t launch_dig_symm(const int* G, int ksplit, int64_t rows, const int* ey, const int* ex,
-                            const double* yin, double* yout, int64_t np, const DevState* st,
-                            int step, cudaStream_t s);
+cudaError_t launch_dig_symm(const int* G, int ksplit, int64_t rows, int64_t batch, const int* ey,
+                            const int* ex, const double* yin, double* yout, int64_t np,
+                            const DevState* st, int step, cudaStream_t s);
 cudaError_t launch_dig_plain(const int* G, int ksplit, int64_t rows, const int* ea, const int* ex,
                              double* out, int64_t np, const DevState* st, int step, cudaStream_t s);
 

@@ -167,3 +167,35 @@ def test_fermi_batches(sp2, mode, n, k, diag, canonical, limit):
             assert (D1[i] - r[0]).norm() <= 1e-10 * r[0].norm()
         else:
             assert torch.equal(D1[i], r[0])
+
+
+@pytest.mark.parametrize("n,batch,diag", [(200, 1, False), (256, 2, True), (257, 1, False),
+                                          (300, 4, True), (600, 2, False)])
+def test_fp64_step_in_one_launch(sp2, n, batch, diag):
+    """Both products of a step in one launch against the same products apart (a square
+    without responses): the same integers, so the same bits from np = 512 on, where both
+    sides use them; and against the recursion in FP64 sums."""
+    p = workloads.random_spectrum(n, nocc=n // 2, k=batch, seed=n)
+    H = torch.from_numpy(np.ascontiguousarray(p.H)).cuda()
+    b = np.stack([np.diag(p.H1[i]) if diag else p.H1[i] for i in range(batch)])
+    B = torch.from_numpy(np.ascontiguousarray(b)).cuda()
+    kw = dict(mode="fp64", sigma=[1, -1, -1, 1], allow_noconv=True)
+    d1, d, _ = sp2.sp2_response(H, p.nocc, B, diag_only=diag, want_density=True,
+                                handle=sp2.Handle(), **kw)
+    dens, _ = sp2.sp2_density(H, p.nocc, handle=sp2.Handle(), **kw)
+    if n > 256:
+        assert torch.equal(d, dens)
+    # the recursion's four steps in FP64 sums
+    _, info = sp2.sp2_density(H, p.nocc, handle=sp2.Handle(), **kw)
+    x = info["alpha"] * np.eye(n) + info["beta"] * p.H
+    ys = [info["beta"] * (np.diag(v) if diag else v) for v in b]
+    for s in (1, -1, -1, 1):
+        ys = [(y @ x + x @ y) if s > 0 else 2.0 * y - (y @ x + x @ y) for y in ys]
+        x = x @ x if s > 0 else 2.0 * x - x @ x
+    # each step rounds sums of n products of entries' row and column norms (at most 1
+    # for X, ||Y||_F for Y) and doubles what came before
+    u = 64.0 * (n + 4) * 2.0 ** -53
+    assert np.abs(d.cpu().numpy() - x).max() <= u
+    for k in range(batch):
+        y0 = np.linalg.norm(info["beta"] * b[k])
+        assert np.abs(d1[k].cpu().numpy() - ys[k]).max() <= u * 16.0 * y0
