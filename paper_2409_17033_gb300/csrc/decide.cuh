@@ -219,5 +219,47 @@ __device__ __noinline__ void decide_block(const Part3* part, DevState* st, const
   post_snapshot(st, p, stop_at);
 }
 
+// After the decision, by the same block: X_s into the candidate's place when step s made
+// it the best so far. Only a few steps do, near the end, and a launch of its own for
+// every step (k_keep_best) took 2 us of a small step: FP64 density at N = 128 590 -> 550
+// us. One block copies 128 KB in some 8 us but 1 MB in 17 (BF16X2 at N = 300, where a
+// recursion has more candidates, 783 -> 850 us), and in the larger products' kernels
+// this code costs registers (FP32 forward chi at N = 1500 5 % slower): the small FP64
+// square alone has it, up to kKeepSmall.
+__device__ __forceinline__ void keep_candidate(const DevState* st, const DecideParams& p) {
+  if (p.keep_n == 0) return;
+  __syncthreads();
+  if (*((volatile const int*)&st->keep_step) != p.n - 1) return;
+  const uint4* src = static_cast<const uint4*>(p.keep_src);
+  uint4* dst = static_cast<uint4*>(p.keep_dst);
+  constexpr int U = 8;
+  for (int i0 = threadIdx.x; i0 < p.keep_n; i0 += U * blockDim.x) {
+    uint4 v[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (i0 + u * (int)blockDim.x < p.keep_n) v[u] = src[i0 + u * blockDim.x];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (i0 + u * (int)blockDim.x < p.keep_n) dst[i0 + u * blockDim.x] = v[u];
+  }
+}
+
+// The end of a square: its last block takes the step decision (every thread of every
+// block calls, its partials stored). KEEP: and keeps a small candidate.
+template <bool KEEP = false>
+__device__ __forceinline__ void last_block_decides(const Part3* part, const SimtDecide& dec) {
+  __shared__ int last;
+  if (threadIdx.x == 0) {
+    __threadfence();
+    last = atomicAdd(dec.done, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  decide_block(part, dec.st, dec.p);
+  if (threadIdx.x == 0) *dec.done = 0u;
+  if constexpr (KEEP) keep_candidate(dec.st, dec.p);
+}
+
 }  // namespace
 }  // namespace sp2

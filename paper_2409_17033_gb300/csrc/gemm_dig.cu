@@ -617,19 +617,7 @@ k_dig_square(const Sums q, int64_t ld, const int* __restrict__ ex,
     const double a2 = __shfl_sync(0xffffffffu, v, NW), af = __shfl_sync(0xffffffffu, v, 2 * NW);
     if (lane == 0) part[blockIdx.x] = Part3{v, a2, af};
   }
-  if (dec.done) {
-    __shared__ int last;
-    if (threadIdx.x == 0) {
-      __threadfence();
-      last = atomicAdd(dec.done, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (last) {
-      __threadfence();
-      decide_block(part, dec.st, dec.p);
-      if (threadIdx.x == 0) *dec.done = 0u;
-    }
-  }
+  if (dec.done) last_block_decides(part, dec);
 }
 
 // Y_{n+1} = sigma > 0 ? Z + Z^T : 2 Y_n - (Z + Z^T) for a batch, Z = Y_n X_n from T

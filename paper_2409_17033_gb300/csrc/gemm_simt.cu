@@ -130,21 +130,7 @@ k_gemm_simt(const T* __restrict__ A, const T* __restrict__ X, int64_t np, int ep
     for (int w = 0; w < 8; ++w) { s1 += r1[w]; s2 += r2[w]; s3 += r3[w]; }
     part[blockIdx.x] = Part3{s1, s2, s3};
   }
-  if (dec.done) {
-    // the last block to finish reduces every block's partials (fixed order, as the
-    // decision kernel does) and takes the step decision
-    __shared__ int last;
-    if (tid == 0) {
-      __threadfence();
-      last = atomicAdd(dec.done, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (last) {
-      __threadfence();
-      decide_block(part, dec.st, dec.p);
-      if (tid == 0) *dec.done = 0u;
-    }
-  }
+  if (dec.done) last_block_decides(part, dec);   // (partials in fixed order, as the decision kernel)
 }
 
 // ------------------------------------------------------------ small FP64
@@ -212,19 +198,7 @@ k_gemm_f64_small(const double* __restrict__ A, const double* __restrict__ X, int
   __syncthreads();
   if (tid == 0)
     part[blockIdx.x] = Part3{r3[0][0] + r3[0][1], r3[1][0] + r3[1][1], r3[2][0] + r3[2][1]};
-  if (dec.done) {
-    __shared__ int last;
-    if (tid == 0) {
-      __threadfence();
-      last = atomicAdd(dec.done, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (last) {
-      __threadfence();
-      decide_block(part, dec.st, dec.p);
-      if (tid == 0) *dec.done = 0u;
-    }
-  }
+  if (dec.done) last_block_decides<true>(part, dec);
 }
 
 // ------------------------------------------------------------ FP32
@@ -431,19 +405,7 @@ k_gemm_f32(const float* __restrict__ A, const float* __restrict__ X, int64_t np,
     for (int w = 0; w < NW; ++w) s1 += red[0][w], s2 += red[1][w], s3 += red[2][w];
     part[blockIdx.x] = Part3{s1, s2, s3};
   }
-  if (dec.done) {
-    __shared__ int last;
-    if (tid == 0) {
-      __threadfence();
-      last = atomicAdd(dec.done, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (last) {
-      __threadfence();
-      decide_block(part, dec.st, dec.p);
-      if (tid == 0) *dec.done = 0u;
-    }
-  }
+  if (dec.done) last_block_decides(part, dec);
 }
 
 // Tile of an FP32 product: the least work of the busiest SM, a tile's work weighed by

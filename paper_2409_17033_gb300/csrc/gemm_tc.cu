@@ -928,19 +928,7 @@ k_gemm_tc(const __grid_constant__ KMaps maps, const __grid_constant__ KParams p)
   if constexpr (EPI == EPI_SQUARE && BN < BN_FULL) {
     // the last CTA to get here takes the step decision (the wide-tile kernels leave
     // it to its own launch: its code beside theirs costs them instruction cache)
-    if (p.dec.done && !halted) {
-      __shared__ int last;
-      if (threadIdx.x == 0) {
-        __threadfence();
-        last = atomicAdd(p.dec.done, 1u) == gridDim.x - 1;
-      }
-      __syncthreads();
-      if (last) {
-        __threadfence();
-        decide_block(p.part, p.dec.st, p.dec.p);
-        if (threadIdx.x == 0) *p.dec.done = 0u;
-      }
-    }
+    if (p.dec.done && !halted) last_block_decides(p.part, p.dec);
   }
 }
 

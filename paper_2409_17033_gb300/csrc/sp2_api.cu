@@ -392,9 +392,9 @@ int tc_common(Ctx& c, TcLaunch* L, int ntiles) {
 // --------------------------------------------------------------- FP64 products by digits
 // FP64 products padded to kPad take the tensor-core form (gemm_dig.cu) as long as
 // its buffers fit: above np = 256, and at np = 256 for a stacked factor of two or
-// more matrices (a batch of responses with X_n below it, 512 rows or more: the SCF's
-// step of 16 fields 87 -> 65 us; one 256 x 256 product alone is faster on the CUDA
-// cores: per SP2 step at N = 256 without responses, 71 against 59 us).
+// more matrices (a batch of responses with X_n below it: SCF of 16 fields at N = 256 28.7 -> 21.4
+// ms; one 256 x 256 product alone is faster on the CUDA cores: per SP2 step at N = 256
+// without responses, 71 against 59 us).
 bool dig_mode(const Ctx& c, int64_t rows) {
   return c.mode == SP2_MODE_FP64 && c.np % kPad == 0 && !c.h->dig_off &&
          (c.np > kPad || rows >= 2 * kPad);
@@ -456,7 +456,7 @@ double dig_flops(const Ctx& c, const DigBufs& b) {
   return 2.0 * 256.0 * b.plan.bn * (double)c.np * 36.0 * b.ntiles;
 }
 
-int last_block_decides(Ctx& c, const DecideParams& dec, SimtDecide* sd) {
+int decide_args(Ctx& c, const DecideParams& dec, SimtDecide* sd) {
   void* dn;
   TRY(ws(c.h, "decide.done", sizeof(unsigned), &dn));
   sd->p = dec;
@@ -476,7 +476,7 @@ int dig_step(Ctx& c, const MatBuf& xin, const MatBuf& xout, const MatBuf& yin, c
   if (!dig_mode(c, rows + c.np) || h->dig_apart || dig_chunk(c.np, batch + 1) <= batch) return SP2_OK;
   if (!dig_bufs(c, rows, false, &db, true)) return SP2_OK;
   SimtDecide sd;
-  TRY(last_block_decides(c, *dec, &sd));
+  TRY(decide_args(c, *dec, &sd));
   sd.p.nparts = (int)dig_square_nparts(c.np);
   const double *x = static_cast<const double*>(xin.master), *y = static_cast<const double*>(yin.master);
   const int64_t left = rows + c.np;
@@ -513,7 +513,7 @@ int square_step(Ctx& c, const MatBuf& xin, const MatBuf& xout, int step,
   sp2_handle_t h = c.h;
   DigBufs db;
   SimtDecide sd;
-  if (dec) TRY(last_block_decides(c, *dec, &sd));
+  if (dec) TRY(decide_args(c, *dec, &sd));
   if (dig_mode(c, c.np)) {
     sd.p.nparts = (int)dig_square_nparts(c.np);
     if (dig_bufs(c, 0, true, &db)) {
@@ -1069,6 +1069,8 @@ int run_sp2(sp2_handle_t h, const void* Hd, int64_t n, int dtype, double nocc, c
     TRY(ws(h, "decide.done", sizeof(unsigned), &dn));
     CK(cudaMemsetAsync(dn, 0, sizeof(unsigned), h->stream));
   }
+  // a small candidate is kept by the block that takes the decision (see keep_candidate)
+  const bool keep_small = track && mode == SP2_MODE_FP64 && xbytes <= kKeepSmall;
   const HostSnap* seen = nullptr;   // the snapshot of the recursion's end
   int read = 0, last = 0;           // last step whose word was read, last step enqueued
   for (int step = 1; step <= maxit; ++step) {
@@ -1089,6 +1091,11 @@ int run_sp2(sp2_handle_t h, const void* Hd, int64_t n, int dtype, double nocc, c
     }
     dp.n = step + 1;
     ring_slot(h, step, &dp);
+    if (keep_small) {
+      dp.keep_src = xin.master;
+      dp.keep_dst = xbest.master;
+      dp.keep_n = (int)(xbytes / 16);
+    }
     bool squared = false;
     if (ybatch > 0)
       TRY(dig_step(c, xin, xo, Y[step % 2], Y[(step + 1) % 2], ybatch, step, &dp, &squared));
@@ -1109,8 +1116,10 @@ int run_sp2(sp2_handle_t h, const void* Hd, int64_t n, int dtype, double nocc, c
       TRY(square_step(c, xin, xo, step, &dp));
     }
     if (track) {
-      CK(launch_keep_best(xin.master, xbest.master, np * np, mode, c.st, step, h->stream));
-      c.kernels++;
+      if (!keep_small) {
+        CK(launch_keep_best(xin.master, xbest.master, np * np, mode, c.st, step, h->stream));
+        c.kernels++;
+      }
       if (ybatch > 0) {
         CK(launch_keep_best(Y[step % 2].master, ybest.master, ybatch * np * np, mode, c.st, step,
                             h->stream));

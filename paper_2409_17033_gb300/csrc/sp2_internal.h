@@ -251,7 +251,11 @@ struct DecideParams {
   int ratio_floor = 0;  // block-sparse recursion: the threshold-floor test as well
   HostSnap* snap = nullptr;  // pinned host slot of this step (nullable) and its token
   unsigned long long token = 0;
+  const void* keep_src = nullptr;    // small FP64 X_s: the block that takes the decision
+  void* keep_dst = nullptr;          // keeps a floor candidate, keep_n vectors of 16 bytes
+  int keep_n = 0;
 };
+constexpr size_t kKeepSmall = (size_t)128 << 10;   // FP64 matrices up to np = 128
 constexpr double kRatioGate = 1e-4;   // f from which a pair of opposite steps must cut f 600-fold
 cudaError_t launch_decide(const Part3* part, DevState* st, DecideParams p, cudaStream_t s);
 // copy `count` entries of the master src -> dst when st->keep_step == step (the

@@ -199,3 +199,18 @@ def test_fp64_step_in_one_launch(sp2, n, batch, diag):
     for k in range(batch):
         y0 = np.linalg.norm(info["beta"] * b[k])
         assert np.abs(d1[k].cpu().numpy() - ys[k]).max() <= u * 16.0 * y0
+
+
+@pytest.mark.parametrize("n", [33, 128, 129, 190])
+def test_fp64_floor_candidate(sp2, n):
+    """The recursion run to its precision floor returns the kept candidate (X_n kept by
+    the square's last block up to np = 128, by a copy kernel above)."""
+    p = workloads.random_spectrum(n, nocc=n // 2, k=1, seed=n)
+    H = torch.from_numpy(np.ascontiguousarray(p.H)).cuda()
+    D, info = sp2.sp2_density(H, p.nocc, mode="fp64", handle=sp2.Handle())
+    e, v = np.linalg.eigh(p.H)
+    ref = v[:, :p.nocc] @ v[:, :p.nocc].T
+    D = D.cpu().numpy()
+    # N-long FP64 sums through some 30 steps, each at most doubling an error off the gap
+    assert info["converged"] and np.linalg.norm(D - ref) <= 1e-10 * np.sqrt(n)
+    assert np.linalg.norm(D @ D - D) <= 1e-11 * np.sqrt(n)
