@@ -103,34 +103,6 @@ constexpr uint32_t idesc_for(bool f16, int m, int n) {
          ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
 
-// Packed pairs of FP32 values (add / mul / fma.rn.f32x2: each half rounds as the
-// scalar operation does, in half the instructions).
-__device__ __forceinline__ uint64_t pk2(float x, float y) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
-  return r;
-}
-__device__ __forceinline__ void upk2(uint64_t v, float& x, float& y) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v));
-}
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
-  uint64_t r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
-  uint64_t r;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-constexpr uint64_t kMinus1x2 = 0xbf800000bf800000ull;   // {-1, -1}
-__device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) { return fma2(b, kMinus1x2, a); }
-
 // A sum of squares of FP32 values kept to about 2^-45 of its value before it goes to
 // FP64, at FP32 rates (GB300's FP64 rate is a small fraction of its FP32 rate), two
 // values at a time: each square enters as its rounded value plus its residual

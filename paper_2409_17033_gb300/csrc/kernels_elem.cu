@@ -4,6 +4,8 @@
 // All reductions accumulate in FP64 in a fixed order (deterministic).
 #include <math.h>
 
+#include <type_traits>
+
 #include "sp2_internal.h"
 #include "decide.cuh"
 
@@ -675,7 +677,7 @@ __global__ void k_fro_final(const double* part, int nparts, float* scale_out) {
 // perturbations Q_k, so that every Q_k is read once per LT rows of P and every P_l
 // once per kCtrKT: with one P_l per block (LT = 1) four observables read 17 GB for 64
 // perturbations at N = 4096 where the inputs are 4.6 GB. With LT = 4 the FP32 form is
-// bound by its ten operations per pair and entry.
+// bound by its ten operations per pair and entry (two rows of P packed).
 constexpr int kCtrKT = 8;
 
 // (the _rn intrinsics are never contracted into FMAs, which would break both
@@ -698,6 +700,28 @@ struct AccF32 {
     if (e == 0u || e == 0xffu) return (double)x;
     return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (896u << 20))),
                             (int)(u << 29));
+  }
+};
+// The same for two rows of P at once, in packed operations: each half rounds as above
+// (a difference is an fma with -1), at half the instructions: 4 x 64 pairs at N = 4096
+// 1.66 -> 1.60 ms, where the FMA pipe's ten operations take 1.16 at its nominal rate.
+struct AccF32x2 {
+  uint64_t s = 0, c = 0;
+  __device__ __forceinline__ void add(uint64_t a, uint64_t b, uint64_t nb) {
+    const uint64_t np = mul2(a, nb);                // -p
+    const uint64_t e = fma2(a, b, np);
+    const uint64_t t = sub2(s, np);
+    const uint64_t bp = sub2(t, s);
+    const uint64_t err = sub2(sub2(s, sub2(t, bp)), add2(np, bp));
+    c = add2(c, add2(err, e));
+    s = t;
+  }
+  __device__ __forceinline__ void values(double& v0, double& v1) const {
+    float s0, s1, c0, c1;
+    upk2(s, s0, s1);
+    upk2(c, c0, c1);
+    v0 = AccF32::to_f64(s0) + AccF32::to_f64(c0);
+    v1 = AccF32::to_f64(s1) + AccF32::to_f64(c1);
   }
 };
 struct AccF64 {
@@ -754,7 +778,9 @@ k_contract_dense(const T* __restrict__ P, int64_t L, const T* __restrict__ Q, in
   const int ln = (int)((L - l0) < LT ? (L - l0) : LT);
   const T* p = P + l0 * nn;
   const T* q = Q + k0 * nn;
-  Acc acc[LT][kCtrKT];
+  constexpr bool PK = sizeof(T) == 4 && VEC == 4 && LT > 1;   // rows of P in packed pairs
+  Acc acc[PK ? 1 : LT][PK ? 1 : kCtrKT];
+  AccF32x2 acc2[PK ? LT / 2 : 1][PK ? kCtrKT : 1];
   const int64_t nv = nn / VEC, stride = (int64_t)gridDim.x * blockDim.x;
   int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if constexpr (VEC * sizeof(T) == 16) {
@@ -781,27 +807,55 @@ k_contract_dense(const T* __restrict__ P, int64_t L, const T* __restrict__ Q, in
       Vec a[LT];
 #pragma unroll
       for (int l = 0; l < LT; ++l) a[l] = mine[(st * NV + (l < ln ? l : 0)) * 256];
-      if (kn == kCtrKT) {   // (no exits between the perturbations: their chains interleave)
+      if constexpr (PK) {
+        auto add_k = [&](int k, auto two) {   // perturbation k (and k + 1)
+          constexpr int NK = decltype(two)::value ? 2 : 1;
+          Vec b[NK];
 #pragma unroll
-        for (int k2 = 0; k2 < kCtrKT; k2 += 2) {
-          const Vec b0 = mine[(st * NV + LT + k2) * 256], b1 = mine[(st * NV + LT + k2 + 1) * 256];
+          for (int i = 0; i < NK; ++i) b[i] = mine[(st * NV + LT + k + i) * 256];
 #pragma unroll
           for (int j = 0; j < VEC; ++j)
 #pragma unroll
-            for (int l = 0; l < LT; ++l) {
-              acc[l][k2].add(a[l].v[j], b0.v[j]);
-              acc[l][k2 + 1].add(a[l].v[j], b1.v[j]);
+            for (int l = 0; l < LT / 2; ++l) {
+              const uint64_t ap = pk2(a[2 * l].v[j], a[2 * l + 1].v[j]);
+#pragma unroll
+              for (int i = 0; i < NK; ++i)
+                acc2[l][k + i].add(ap, pk2(b[i].v[j], b[i].v[j]), pk2(-b[i].v[j], -b[i].v[j]));
             }
+        };
+        if (kn == kCtrKT) {   // (no exits between the perturbations: their chains interleave)
+#pragma unroll
+          for (int k = 0; k < kCtrKT; k += 2) add_k(k, std::true_type());
+        } else {
+#pragma unroll
+          for (int k = 0; k < kCtrKT; ++k) {
+            if (k >= kn) break;
+            add_k(k, std::false_type());
+          }
         }
       } else {
+        if (kn == kCtrKT) {   // (no exits between the perturbations: their chains interleave)
 #pragma unroll
-        for (int k = 0; k < kCtrKT; ++k) {
-          if (k >= kn) break;
-          const Vec b = mine[(st * NV + LT + k) * 256];
+          for (int k2 = 0; k2 < kCtrKT; k2 += 2) {
+            const Vec b0 = mine[(st * NV + LT + k2) * 256], b1 = mine[(st * NV + LT + k2 + 1) * 256];
 #pragma unroll
-          for (int l = 0; l < LT; ++l)
+            for (int j = 0; j < VEC; ++j)
 #pragma unroll
-            for (int j = 0; j < VEC; ++j) acc[l][k].add(a[l].v[j], b.v[j]);
+              for (int l = 0; l < LT; ++l) {
+                acc[l][k2].add(a[l].v[j], b0.v[j]);
+                acc[l][k2 + 1].add(a[l].v[j], b1.v[j]);
+              }
+          }
+        } else {
+#pragma unroll
+          for (int k = 0; k < kCtrKT; ++k) {
+            if (k >= kn) break;
+            const Vec b = mine[(st * NV + LT + k) * 256];
+#pragma unroll
+            for (int l = 0; l < LT; ++l)
+#pragma unroll
+              for (int j = 0; j < VEC; ++j) acc[l][k].add(a[l].v[j], b.v[j]);
+          }
         }
       }
     }
@@ -823,8 +877,15 @@ k_contract_dense(const T* __restrict__ P, int64_t L, const T* __restrict__ Q, in
   __shared__ double red[8][NP];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   double v[NP];
+  if constexpr (PK) {
 #pragma unroll
-  for (int i = 0; i < NP; ++i) v[i] = acc[i / kCtrKT][i % kCtrKT].value();
+    for (int i = 0; i < NP / 2; ++i)
+      acc2[i / kCtrKT][i % kCtrKT].values(v[i / kCtrKT * 2 * kCtrKT + i % kCtrKT],
+                                          v[(i / kCtrKT * 2 + 1) * kCtrKT + i % kCtrKT]);
+  } else {
+#pragma unroll
+    for (int i = 0; i < NP; ++i) v[i] = acc[i / kCtrKT][i % kCtrKT].value();
+  }
   const double s = warp_sums<NP>(v, lane);
   constexpr int STEP = 32 / NP;   // lanes per value
   if (lane % STEP == 0) red[warp][lane / STEP] = s;

@@ -186,6 +186,34 @@ struct Tile {       // one output tile of a product kernel
   int col0;         // first output column
 };
 
+// Packed pairs of FP32 values (add / mul / fma.rn.f32x2: each half rounds as the
+// scalar operation does, in half the instructions).
+__device__ __forceinline__ uint64_t pk2(float x, float y) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+  return r;
+}
+__device__ __forceinline__ void upk2(uint64_t v, float& x, float& y) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v));
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+constexpr uint64_t kMinus1x2 = 0xbf800000bf800000ull;   // {-1, -1}
+__device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) { return fma2(b, kMinus1x2, a); }
+
 // ---------------------------------------------------------------- dependent launches
 // The kernels of a step follow one another within microseconds. Launched as
 // programmatic dependents, a kernel's blocks become resident while the one before
