@@ -505,6 +505,76 @@ __global__ void k_init_batch_x4(const float* __restrict__ src, int64_t n, int64_
   }
 }
 
+// The same for beta (B + B^T) / 2 of dense matrices: one block per upper pair of 64 x 64
+// tiles, each tile read once in 16-byte vectors and transposed through shared memory
+// (k_init reads B^T down its columns and works in FP64: 92 us at N = 2048, an autograd
+// step 4.54 -> 4.43 ms). Bound by memory: 4 bytes read, 4 written (8 with planes) per
+// entry. Half the sum is kept
+// with its rounding error, so that an entry is rounded once, as from FP64.
+template <int MODE>
+__global__ void __launch_bounds__(256)
+k_init_sym_x4(const float* __restrict__ src, int64_t n, int64_t np, double beta, MatBuf dst,
+              float* ymax, int planes, int coef, const DevState* st) {
+  dep_sync();
+  constexpr int TE = 64, R = 16, P = TE / R;
+  const F2 bc = split_coef(coef == INIT_STATE_BETA ? st->beta : beta);
+  const int64_t t = blockIdx.x, b = blockIdx.y;
+  int64_t J = (int64_t)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
+  while (J * (J + 1) / 2 > t) --J;
+  while ((J + 1) * (J + 2) / 2 <= t) ++J;
+  const int64_t I = t - J * (J + 1) / 2, rI = I * TE, rJ = J * TE, base = b * np * np;
+  const int c4 = (threadIdx.x % 16) * 4, r0 = threadIdx.x / 16;
+  __shared__ float za[TE][TE + 1], zb[TE][TE + 1];
+  const float* m = src + b * n * n;
+  float v[P][4];
+#pragma unroll
+  for (int p = 0; p < P; ++p) {
+    const int r = r0 + p * R;
+    const bool ia = rI + r < n && rJ + c4 < n, ib = rJ + r < n && rI + c4 < n;   // (n % 4 == 0)
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    const float4 x = ia ? *reinterpret_cast<const float4*>(m + (rI + r) * n + rJ + c4) : zero;
+    const float4 y = ib ? *reinterpret_cast<const float4*>(m + (rJ + r) * n + rI + c4) : zero;
+    v[p][0] = x.x, v[p][1] = x.y, v[p][2] = x.z, v[p][3] = x.w;
+    zb[r][c4] = y.x, zb[r][c4 + 1] = y.y, zb[r][c4 + 2] = y.z, zb[r][c4 + 3] = y.w;
+  }
+  __syncthreads();
+  float mx = 0.0f;
+  auto store = [&](int64_t idx, const float (&f)[4]) {
+    if (planes) store_y4<float, MODE>(dst, idx, f, 1.0f);
+    else store_y4<float, SP2_MODE_FP32>(dst, idx, f, 1.0f);
+  };
+#pragma unroll
+  for (int p = 0; p < P; ++p) {
+    const int r = r0 + p * R;
+    float f[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const float x = 0.5f * v[p][j], y = 0.5f * zb[c4 + j][r];
+      float s = 0.0f, e = 0.0f;
+      two_sum_add(s, e, x);
+      two_sum_add(s, e, y);   // s + e = x + y
+      f[j] = fmaf(s, bc.hi, fmaf(s, bc.lo, e * bc.hi));
+      za[r][c4 + j] = f[j];
+      mx = fmaxf(mx, fabsf(f[j]));
+    }
+    store(base + (rI + r) * np + rJ + c4, f);
+  }
+  if (ymax) {
+    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if ((threadIdx.x & 31) == 0 && mx > 0.0f) atomic_max_nonneg(&ymax[b], mx);
+  }
+  if (I == J) return;
+  __syncthreads();
+#pragma unroll
+  for (int p = 0; p < P; ++p) {
+    const int r = r0 + p * R;
+    float f[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) f[j] = za[c4 + j][r];
+    store(base + (rJ + r) * np + rI + c4, f);
+  }
+}
+
 // Gershgorin discs of an FP32 H, one warp per row: each lane sums |h| of its
 // part of the row with TwoSum in FP32, four 16-byte loads in flight, and moves
 // the sum and its error to FP64 after each group of 16 entries; lanes add in FP64.
@@ -962,6 +1032,22 @@ cudaError_t launch_init(const void* src, int64_t n, int64_t np, int64_t batch, i
     launch_dep(k_init_batch_x4, grid_for(batch * np, 1, 152 * 16), 256, 0, s,
                static_cast<const float*>(src), n, np, batch, diag_only, beta, mode, dst, ymax,
                planes, coef, st);
+    return cudaGetLastError();
+  }
+  if (symmetrize && !diag_only && !part && alpha == 0.0 && coef != INIT_STATE && dtype == SP2_F32 &&
+      mode != SP2_MODE_FP64 && n % 4 == 0 && batch <= 65535 &&
+      (reinterpret_cast<uintptr_t>(src) & 15u) == 0) {
+    const int planes = split_mode(mode) && !(mode == SP2_MODE_FP16X2 && ymax) ? 1 : 0;
+    const int64_t nb = np / 64;
+    const dim3 tiles((unsigned)(nb * (nb + 1) / 2), (unsigned)batch);
+    auto go = [&](auto kern) {
+      launch_dep(kern, tiles, 256, 0, s, static_cast<const float*>(src), n, np, beta, dst, ymax, planes,
+                 coef, st);
+    };
+    if (mode == SP2_MODE_FP32) go(k_init_sym_x4<SP2_MODE_FP32>);
+    else if (mode == SP2_MODE_BF16X2) go(k_init_sym_x4<SP2_MODE_BF16X2>);
+    else if (mode == SP2_MODE_BF16X3) go(k_init_sym_x4<SP2_MODE_BF16X3>);
+    else go(k_init_sym_x4<SP2_MODE_FP16X2>);
     return cudaGetLastError();
   }
   int grid = part ? nparts : grid_for(batch * np, 1, 4096);

@@ -214,3 +214,22 @@ def test_fp64_floor_candidate(sp2, n):
     # N-long FP64 sums through some 30 steps, each at most doubling an error off the gap
     assert info["converged"] and np.linalg.norm(D - ref) <= 1e-10 * np.sqrt(n)
     assert np.linalg.norm(D @ D - D) <= 1e-11 * np.sqrt(n)
+
+
+@pytest.mark.parametrize("mode", ["fp32", "bf16x2", "bf16x3", "fp16x2"])
+@pytest.mark.parametrize("n", [60, 64, 300, 301])
+def test_dense_incoming_gradient(sp2, mode, n):
+    """The adjoint takes the symmetric part of a dense gradient, rounded once from its
+    exact value: the same result as from that part itself."""
+    p = workloads.random_spectrum(n, nocc=n // 2, k=1, seed=n)
+    H = torch.from_numpy(p.H.astype(np.float32)).cuda()
+    g = torch.Generator().manual_seed(n)
+    W = torch.randn(n, n, generator=g).cuda()
+    half = 0.5 * (W.double() + W.double().T)
+    out = []
+    for w in (W, half.float()):
+        x = H.clone().requires_grad_(True)
+        d = sp2.sp2_density_autograd(x, p.nocc, mode=mode, handle=sp2.Handle())
+        (grad,) = torch.autograd.grad((w * d).sum(), x)
+        out.append(grad)
+    assert torch.equal(out[0], out[1]) and out[0].abs().max() > 0
