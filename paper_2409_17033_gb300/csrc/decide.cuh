@@ -246,12 +246,14 @@ __device__ __forceinline__ void keep_candidate(const DevState* st, const DecideP
 
 // The end of a square: its last block takes the step decision (every thread of every
 // block calls, its partials stored). KEEP: and keeps a small candidate.
+// nblocks: how many blocks call (0: the whole grid).
 template <bool KEEP = false>
-__device__ __forceinline__ void last_block_decides(const Part3* part, const SimtDecide& dec) {
+__device__ __forceinline__ void last_block_decides(const Part3* part, const SimtDecide& dec,
+                                                   unsigned nblocks = 0) {
   __shared__ int last;
   if (threadIdx.x == 0) {
     __threadfence();
-    last = atomicAdd(dec.done, 1u) == gridDim.x - 1;
+    last = atomicAdd(dec.done, 1u) == (nblocks ? nblocks : gridDim.x) - 1;
   }
   __syncthreads();
   if (!last) return;

@@ -37,7 +37,7 @@
 // where the square took 30 us of a step on the CUDA cores: 28.7 -> 21.4 ms).
 //
 // Per product: k_digits (each factor), k_gemm_dig, then one pass that turns the sums
-// into FP64 and applies the recursion's update: k_dig_square
+// into FP64 and applies the recursion's update: k_dig_step, or k_dig_square
 // (Eq. DM0, with the traces and the step decision), k_dig_symm (Eqs. DM1-DM3) or
 // k_dig_plain.
 //
@@ -367,6 +367,7 @@ __device__ __forceinline__ bool halted_dig(const DevState* st, int step) {
 // bytes read, 16 written per entry.
 constexpr int kDigThreads = 128;
 
+template <bool TWO>   // (the choice of the source costs a single matrix's pass registers and time)
 __global__ void __launch_bounds__(kDigThreads)
 k_digits(const double* __restrict__ src, int64_t rows1, const double* __restrict__ src2,
          int64_t rows, int64_t np, uint16_t* __restrict__ dig, int* __restrict__ ex,
@@ -376,8 +377,8 @@ k_digits(const double* __restrict__ src, int64_t rows1, const double* __restrict
   __shared__ uint32_t smax[kDigThreads / 32];
   __shared__ float ssum[kDigThreads / 32];
   const int64_t row = blockIdx.x;
-  const double2* x2 =
-      reinterpret_cast<const double2*>(row < rows1 ? src + row * np : src2 + (row - rows1) * np);
+  const double2* x2 = reinterpret_cast<const double2*>(
+      !TWO || row < rows1 ? src + row * np : src2 + (row - rows1) * np);
   const int n4 = (int)(np / 4);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   uint32_t m = 0;
@@ -475,7 +476,8 @@ struct Sums {
 __device__ __forceinline__ void load_t(const Sums& q, int64_t o, long long (&t)[4]) {
 #pragma unroll
   for (int k = 0; k < 4; ++k) t[k] = 0;
-  long long last[4] = {0, 0, 0, 0};   // the last weight's sum over the K parts, rounded once
+  // the last weight's sum over the K parts, x = 256 hi + lo, rounded once
+  int hi[4] = {0, 0, 0, 0}, lo[4] = {0, 0, 0, 0};
   for (int ks = 0; ks < q.ksplit; ++ks) {
     int4 v[kGroups];
 #pragma unroll
@@ -488,12 +490,12 @@ __device__ __forceinline__ void load_t(const Sums& q, int64_t o, long long (&t)[
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
         if (sh >= 0) t[k] += (long long)x[k] << (sh > 0 ? sh : 0);
-        else last[k] += x[k];
+        else hi[k] += x[k] >> 8, lo[k] += x[k] & 255;
       }
     }
   }
 #pragma unroll
-  for (int k = 0; k < 4; ++k) t[k] += (last[k] + (1 << 7)) >> 8;
+  for (int k = 0; k < 4; ++k) t[k] += hi[k] + ((lo[k] + (1 << 7)) >> 8);
 }
 
 // T's value as FP64 (one rounding), times 2^e. The conversion by magic constants
@@ -543,13 +545,25 @@ __device__ __forceinline__ void st4d(double* p, const double (&v)[4]) {
 // holds entries (i, j) of the upper tile with i along its rows. Bound by its 6 FP64
 // operations per upper entry (an FP64 instruction of a warp takes 64 clocks), so
 // the reductions come once per block, not per tile, ||.||_F^2 and f sharing them.
-__global__ void __launch_bounds__(kPassThreads)
-k_dig_square(const Sums q, int64_t ld, const int* __restrict__ ex,
-             const double* __restrict__ X, double* __restrict__ out, int64_t np, int ntiles,
-             DevState* st, int step, Part3* __restrict__ part, SimtDecide dec) {
-  dep_sync();
-  if (halted_dig(st, step)) return;
-  __shared__ double sm[2][TE][TE + 1];
+struct SquareArgs {
+  Sums q;
+  int64_t ld;
+  const int* ex;
+  const double* X;
+  double* out;
+  int ntiles, nblocks;
+  Part3* part;
+  SimtDecide dec;
+};
+using PassTile = double[2][TE][TE + 1];
+
+__device__ __forceinline__ void square_pass(const SquareArgs& a, int block, int64_t np, DevState* st,
+                                            int step, PassTile& sm) {
+  const Sums& q = a.q;
+  const int64_t ld = a.ld;
+  const int* __restrict__ ex = a.ex;
+  const double* __restrict__ X = a.X;
+  double* __restrict__ out = a.out;
   __shared__ double red[3][kPassThreads / 32];
   const int r = threadIdx.x >> 3, c4 = (threadIdx.x & 7) * 4;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -557,7 +571,7 @@ k_dig_square(const Sums q, int64_t ld, const int* __restrict__ ex,
   double t1 = 0.0, t2 = 0.0, f = 0.0;   // t2, f: off-diagonal entries (counted twice below)
   double e2 = 0.0, ef = 0.0;            // their diagonal entries
   int buf = 0;
-  for (int64_t tix = blockIdx.x; tix < ntiles; tix += gridDim.x, buf ^= 1) {
+  for (int64_t tix = block; tix < a.ntiles; tix += a.nblocks, buf ^= 1) {
     int64_t I, J;
     tri_ij(tix, I, J);
     const int64_t gj = J * TE + r, gi0 = I * TE + c4;
@@ -615,25 +629,43 @@ k_dig_square(const Sums q, int64_t ld, const int* __restrict__ ex,
     double v = lane < 3 * NW ? red[lane / NW][lane % NW] : 0.0;
     for (int o = NW / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     const double a2 = __shfl_sync(0xffffffffu, v, NW), af = __shfl_sync(0xffffffffu, v, 2 * NW);
-    if (lane == 0) part[blockIdx.x] = Part3{v, a2, af};
+    if (lane == 0) a.part[block] = Part3{v, a2, af};
   }
-  if (dec.done) last_block_decides(part, dec);
+  if (a.dec.done) last_block_decides(a.part, a.dec, (unsigned)a.nblocks);
+}
+
+__global__ void __launch_bounds__(kPassThreads)
+k_dig_square(const __grid_constant__ SquareArgs a, int64_t np, DevState* st, int step) {
+  dep_sync();
+  if (halted_dig(st, step)) return;
+  __shared__ PassTile sm;
+  square_pass(a, (int)blockIdx.x, np, st, step, sm);
 }
 
 // Y_{n+1} = sigma > 0 ? Z + Z^T : 2 Y_n - (Z + Z^T) for a batch, Z = Y_n X_n from T
 // (ey: exponents of the stacked rows of Y_n, ex: of X_n; rows: G's leading dimension).
 // One block per tile pair
 // and batch entry.
-__global__ void __launch_bounds__(kPassThreads)
-k_dig_symm(const Sums q, int64_t rows, const int* __restrict__ ey,
-           const int* __restrict__ ex, const double* __restrict__ yin, double* __restrict__ yout,
-           int64_t np, const DevState* st, int step) {
-  dep_sync();
-  if (halted_dig(st, step)) return;
-  __shared__ double za[TE][TE + 1], zb[TE][TE + 1];
+struct SymmArgs {
+  Sums q;
+  int64_t rows;
+  const int *ey, *ex;
+  const double* yin;
+  double* yout;
+};
+
+__device__ __forceinline__ void symm_pass(const SymmArgs& a, int64_t tile, int64_t entry, int64_t np,
+                                          const DevState* st, int step, PassTile& sm) {
+  const Sums& q = a.q;
+  const int64_t rows = a.rows;
+  const int *__restrict__ ey = a.ey, *__restrict__ ex = a.ex;
+  const double* __restrict__ yin = a.yin;
+  double* __restrict__ yout = a.yout;
+  double(&za)[TE][TE + 1] = sm[0];
+  double(&zb)[TE][TE + 1] = sm[1];
   int64_t I, J;
-  tri_ij(blockIdx.x, I, J);
-  const int64_t b0 = (int64_t)blockIdx.y * np, base = b0 * np;
+  tri_ij(tile, I, J);
+  const int64_t b0 = entry * np, base = b0 * np;
   const int r = threadIdx.x >> 3, c4 = (threadIdx.x & 7) * 4;
   const int sg = st->sigma[step];
   {
@@ -666,6 +698,28 @@ k_dig_symm(const Sums q, int64_t rows, const int* __restrict__ ey,
 #pragma unroll
   for (int k = 0; k < 4; ++k) w[k] = zb[c4 + k][r];
   st4d(yout + base + (J * TE + r) * np + I * TE + c4, w);
+}
+
+__global__ void __launch_bounds__(kPassThreads)
+k_dig_symm(const __grid_constant__ SymmArgs a, int64_t np, const DevState* st, int step) {
+  dep_sync();
+  if (halted_dig(st, step)) return;
+  __shared__ PassTile sm;
+  symm_pass(a, blockIdx.x, blockIdx.y, np, st, step, sm);
+}
+
+// Both of a step whose products ran together. The square's blocks come first: they end in
+// the decision, a chain of latencies that the response's blocks cover (SCF of 16 fields at
+// N = 256, whose square has 36 blocks: 21.4 -> 19.0 ms).
+__global__ void __launch_bounds__(kPassThreads)
+k_dig_step(const __grid_constant__ SquareArgs a, const __grid_constant__ SymmArgs y, int tiles,
+           int64_t np, DevState* st, int step) {
+  dep_sync();
+  if (halted_dig(st, step)) return;
+  __shared__ PassTile sm;
+  const int b = (int)blockIdx.x - a.nblocks;
+  if (b < 0) square_pass(a, (int)blockIdx.x, np, st, step, sm);
+  else symm_pass(y, b % tiles, b / tiles, np, st, step, sm);
 }
 
 // C = T's value, row-major rows x np
@@ -784,8 +838,12 @@ DigPlan dig_plan(int64_t rows, int64_t np, bool upper, bool with_x) {
 cudaError_t launch_digits(const double* src, int64_t rows, const double* src2, int64_t rows2,
                           int64_t np, const DigOperand& o, const DevState* st, int step,
                           cudaStream_t s) {
-  launch_dep(k_digits, (unsigned)(rows + rows2), kDigThreads, 0, s, src, rows, src2, rows + rows2, np,
-             o.dig, o.ex, st, step);
+  auto go = [&](auto kern) {
+    launch_dep(kern, (unsigned)(rows + rows2), kDigThreads, 0, s, src, rows, src2, rows + rows2, np, o.dig,
+               o.ex, st, step);
+  };
+  if (rows2 > 0) go(k_digits<true>);
+  else go(k_digits<false>);
   return cudaGetLastError();
 }
 
@@ -827,22 +885,41 @@ int64_t dig_square_nparts(int64_t np) {
   return n < 456 ? n : 456;
 }
 
-cudaError_t launch_dig_square(const int* G, int ksplit, int64_t ld, int64_t off, const int* ex,
-                              const double* X, double* out, int64_t np, DevState* st, int step, Part3* part,
+static SquareArgs square_args(const int* G, int ksplit, int64_t ld, int64_t off, const int* ex,
+                              const double* X, double* out, int64_t np, Part3* part,
+                              const SimtDecide* dec) {
+  SquareArgs a{Sums{G + off, np * ld, ksplit}, ld, ex, X, out, (int)tri_tiles(np),
+               (int)dig_square_nparts(np), part, SimtDecide()};
+  if (dec) a.dec = *dec;
+  return a;
+}
+
+cudaError_t launch_dig_square(const int* G, int ksplit, const int* ex, const double* X, double* out,
+                              int64_t np, DevState* st, int step, Part3* part,
                               const SimtDecide* dec, cudaStream_t s) {
-  SimtDecide sd;
-  if (dec) sd = *dec;
-  launch_dep(k_dig_square, (unsigned)dig_square_nparts(np), kPassThreads, 0, s, 
-      Sums{G + off, np * ld, ksplit}, ld, ex, X, out, np, (int)tri_tiles(np), st, step, part, sd);
+  const SquareArgs a = square_args(G, ksplit, np, 0, ex, X, out, np, part, dec);
+  launch_dep(k_dig_square, (unsigned)a.nblocks, kPassThreads, 0, s, a, np, st, step);
   return cudaGetLastError();
 }
 
-cudaError_t launch_dig_symm(const int* G, int ksplit, int64_t rows, int64_t batch, const int* ey,
-                            const int* ex, const double* yin, double* yout, int64_t np,
-                            const DevState* st, int step, cudaStream_t s) {
-  const dim3 grid((unsigned)tri_tiles(np), (unsigned)batch);
-  launch_dep(k_dig_symm, grid, kPassThreads, 0, s, Sums{G, rows * np, ksplit}, rows, ey, ex, yin, yout, np, st,
-                                           step);
+cudaError_t launch_dig_symm(const int* G, int ksplit, int64_t rows, const int* ey, const int* ex,
+                            const double* yin, double* yout, int64_t np, const DevState* st,
+                            int step, cudaStream_t s) {
+  const dim3 grid((unsigned)tri_tiles(np), (unsigned)(rows / np));
+  launch_dep(k_dig_symm, grid, kPassThreads, 0, s,
+             SymmArgs{Sums{G, rows * np, ksplit}, rows, ey, ex, yin, yout}, np, st, step);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_dig_step(const int* G, int ksplit, int64_t batch, const int* ex, const double* yin,
+                            double* yout, const double* X, double* out, int64_t np, DevState* st,
+                            int step, Part3* part, const SimtDecide* dec, cudaStream_t s) {
+  const int64_t rows = batch * np, ld = rows + np;
+  const SquareArgs a = square_args(G, ksplit, ld, rows, ex + rows, X, out, np, part, dec);
+  const SymmArgs y{Sums{G, ld * np, ksplit}, ld, ex, ex + rows, yin, yout};
+  const int tiles = (int)tri_tiles(np);
+  launch_dep(k_dig_step, (unsigned)(a.nblocks + tiles * batch), kPassThreads, 0, s, a, y, tiles, np, st,
+             step);
   return cudaGetLastError();
 }
 

@@ -492,13 +492,10 @@ int dig_step(Ctx& c, const MatBuf& xin, const MatBuf& xout, const MatBuf& yin, c
     CK(cudaEventRecord(e1, h->stream));
     c.timed.push_back({step, 0});
   }
-  const int* xe = db.a.ex + rows;
-  CK(launch_dig_symm(db.G, db.plan.ksplit, left, batch, db.a.ex, xe, y,
-                     static_cast<double*>(yout.master), c.np, c.st, step, h->stream));
-  CK(launch_dig_square(db.G, db.plan.ksplit, left, rows, xe, x, static_cast<double*>(xout.master),
-                       c.np, c.st, step, c.part, &sd, h->stream));
+  CK(launch_dig_step(db.G, db.plan.ksplit, batch, db.a.ex, y, static_cast<double*>(yout.master), x,
+                     static_cast<double*>(xout.master), c.np, c.st, step, c.part, &sd, h->stream));
   c.launches++;
-  c.kernels += 4;
+  c.kernels += 3;
   c.flops += dig_flops(c, db);
   c.alg += (double)c.n * (double)c.n * (2.0 * (double)batch * (double)c.n + (double)(c.n + 1));
   *done = true;
@@ -535,7 +532,7 @@ int square_step(Ctx& c, const MatBuf& xin, const MatBuf& xout, int step,
         CK(cudaEventRecord(e1, h->stream));
         c.timed.push_back({step, 0});
       }
-      CK(launch_dig_square(db.G, db.plan.ksplit, c.np, 0, db.x.ex, x, static_cast<double*>(xout.master), c.np, c.st, step,
+      CK(launch_dig_square(db.G, db.plan.ksplit, db.x.ex, x, static_cast<double*>(xout.master), c.np, c.st, step,
                            c.part, dec ? &sd : nullptr, h->stream));
       c.launches++;
       c.kernels += 2;
@@ -700,7 +697,7 @@ int response_step(Ctx& c, const MatBuf& x, const MatBuf& yin, const MatBuf& yout
           CK(cudaEventRecord(e1, h->stream));
           c.timed.push_back({step, 0});
         }
-        CK(launch_dig_symm(db.G, db.plan.ksplit, r, nb, db.a.ex, db.x.ex, y + off, yo + off, c.np, c.st, step,
+        CK(launch_dig_symm(db.G, db.plan.ksplit, r, db.a.ex, db.x.ex, y + off, yo + off, c.np, c.st, step,
                            h->stream));
         c.launches++;
         c.kernels += 3;

@@ -442,15 +442,17 @@ cudaError_t launch_gemm_dig(const DigOperand& A, int64_t rows, const DigOperand&
                             int* G, const Tile* tiles, int ntiles, const DigPlan& plan,
                             DevState* st, int step, const TcTuning& tune, cudaStream_t s);
 // the passes from G: the square step with its partials (and, with dec, the step
-// decision), the symmetrised response update of a batch, C = A X. The square's and the
-// response's sums may lie in a larger G: its leading dimension and the first row.
-cudaError_t launch_dig_square(const int* G, int ksplit, int64_t ld, int64_t off, const int* ex,
-                              const double* X, double* out,
+// decision), the symmetrised response update of a batch, both from one G of the batch's
+// rows and X's below them (ex: the exponents likewise), C = A X
+cudaError_t launch_dig_square(const int* G, int ksplit, const int* ex, const double* X, double* out,
                               int64_t np, DevState* st, int step, Part3* part,
                               const SimtDecide* dec, cudaStream_t s);
-cudaError_t launch_dig_symm(const int* G, int ksplit, int64_t rows, int64_t batch, const int* ey,
-                            const int* ex, const double* yin, double* yout, int64_t np,
-                            const DevState* st, int step, cudaStream_t s);
+cudaError_t launch_dig_symm(const int* G, int ksplit, int64_t rows, const int* ey, const int* ex,
+                            const double* yin, double* yout, int64_t np, const DevState* st,
+                            int step, cudaStream_t s);
+cudaError_t launch_dig_step(const int* G, int ksplit, int64_t batch, const int* ex, const double* yin,
+                            double* yout, const double* X, double* out, int64_t np, DevState* st,
+                            int step, Part3* part, const SimtDecide* dec, cudaStream_t s);
 cudaError_t launch_dig_plain(const int* G, int ksplit, int64_t rows, const int* ea, const int* ex,
                              double* out, int64_t np, const DevState* st, int step, cudaStream_t s);
 
