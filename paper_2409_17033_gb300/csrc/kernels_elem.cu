@@ -968,6 +968,21 @@ k_contract_dense(const T* __restrict__ P, int64_t L, const T* __restrict__ Q, in
   }
 }
 
+// One pair (l, k) per block row: FP64 matrices too small to fill the GPU in groups.
+__global__ void k_contract_pair(const double* __restrict__ P, const double* __restrict__ Q, int64_t K,
+                                int64_t nn, double* part, int nparts, int64_t y0) {
+  dep_sync();
+  const int64_t pair = y0 + blockIdx.y;
+  const double* p = P + pair / K * nn;
+  const double* q = Q + pair % K * nn;
+  double acc = 0.0;
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < nn;
+       t += (int64_t)gridDim.x * blockDim.x)
+    acc = fma(p[t], q[t], acc);
+  acc = block_sum(acc);
+  if (threadIdx.x == 0) part[pair * nparts + blockIdx.x] = acc;
+}
+
 template <typename T>
 __global__ void k_contract_diag(const T* __restrict__ P, const T* __restrict__ Q, int64_t K,
                                 int64_t n, double* part, int nparts, int64_t y0) {
@@ -1187,13 +1202,31 @@ void contract_rows(const void* P, int64_t L, const void* Q, int64_t K, int64_t n
                static_cast<const T*>(Q), K, nn, part, nparts, y0);
   }
 }
-// one block row per LT rows of P and kCtrKT perturbations; LT = 4 from three rows of P on
+// One block row per LT rows of P and kCtrKT perturbations. FP32: LT = 4 from three rows
+// of P on. FP64 is bound by its pipe, which a row formed for nothing would keep busy, so
+// LT divides L (3 x 40 pairs at N = 2000 0.95 ms by pairs, 0.85 so); and with fewer than
+// eight blocks per SM some SMs have a block more than others for a good part of the
+// time: there every pair has its own block row (2 x 5 pairs at N = 700 47 us; a drawn
+// case of this kind took 200 us in groups and 171 by pairs).
 template <typename T, int VEC>
 void contract_dense(const void* P, int64_t L, const void* Q, int64_t K, int64_t nn, double* part,
                     int nparts, cudaStream_t s) {
   const int64_t kt = (K + kCtrKT - 1) / kCtrKT;
-  if (L == 1) contract_rows<T, VEC, 1>(P, L, Q, K, nn, part, nparts, kt, s);
-  else if (L == 2) contract_rows<T, VEC, 2>(P, L, Q, K, nn, part, nparts, kt, s);
+  int64_t lt = L == 1 ? 1 : (L == 2 ? 2 : 4);
+  if constexpr (sizeof(T) == 8) {
+    lt = L % 4 == 0 ? 4 : (L % 2 == 0 ? 2 : 1);
+    if (nparts * (L / lt) * kt < 8 * 152) {
+      constexpr int64_t kMaxY = 65535;
+      for (int64_t y0 = 0; y0 < L * K; y0 += kMaxY) {
+        const int64_t ny = L * K - y0 < kMaxY ? L * K - y0 : kMaxY;
+        launch_dep(k_contract_pair, dim3((unsigned)nparts, (unsigned)ny), 256, 0, s,
+                   static_cast<const double*>(P), static_cast<const double*>(Q), K, nn, part, nparts, y0);
+      }
+      return;
+    }
+  }
+  if (lt == 1) contract_rows<T, VEC, 1>(P, L, Q, K, nn, part, nparts, L * kt, s);
+  else if (lt == 2) contract_rows<T, VEC, 2>(P, L, Q, K, nn, part, nparts, L / 2 * kt, s);
   else contract_rows<T, VEC, 4>(P, L, Q, K, nn, part, nparts, (L + 3) / 4 * kt, s);
 }
 }  // namespace
