@@ -92,7 +92,8 @@ typedef enum {
 typedef enum { SP2_F64 = 0, SP2_F32 = 1 } sp2_dtype;
 
 /* Arithmetic of the matrix products (Sec. VI.B).
- *   SP2_MODE_FP64    FP64. Products of matrices above N = 257 are formed on the tensor
+ *   SP2_MODE_FP64    FP64. Products of matrices from N = 257 on (in steps with responses
+ *                    from N = 193, where they are padded to 256) are formed on the tensor
  *                    cores from 8 error-free digits of 8 bits per entry (36 exact
  *                    products summed in integers), with errors below those of an
  *                    FP64 dot product relative to the norms of its row and column;

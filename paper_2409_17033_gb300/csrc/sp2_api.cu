@@ -1918,7 +1918,6 @@ struct FermiState {
   std::vector<FMat> dl, W;   // delta_0..delta_n, W_0..W_{n-1}
   FMat P, S, T, U, Z2[2];    // scratch of the forward pass and the responses
   FMat dd[2], E, F1, dW, G1, RI;   // (batches of B response matrices but for RI)
-  int64_t B = 1;
   double trI = 0.0;
   void* tr = nullptr;        // B device doubles
   void* ones = nullptr;      // the identity's diagonal, on the device
@@ -2047,7 +2046,6 @@ int fermi_batch(Ctx& c, FermiState& fs, int64_t want, int64_t* B) {
       for (const char* part : {".m", ".h", ".l", ".d", ".s"}) ws_free(h, std::string(q.name) + part);
     h->err.clear();
   }
-  fs.B = b;
   *B = b;
   return SP2_OK;
 }
