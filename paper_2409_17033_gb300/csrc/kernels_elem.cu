@@ -746,8 +746,9 @@ __global__ void k_fro_final(const double* part, int nparts, float* scale_out) {
 // A block covers one slice of the N^2 entries for up to LT factors P_l and kCtrKT
 // perturbations Q_k, so that every Q_k is read once per LT rows of P and every P_l
 // once per kCtrKT: with one P_l per block (LT = 1) four observables read 17 GB for 64
-// perturbations at N = 4096 where the inputs are 4.6 GB. With LT = 4 the FP32 form is
-// bound by its ten operations per pair and entry (two rows of P packed).
+// perturbations at N = 4096 where the inputs are 4.6 GB (4.01 ms, 1.51 with LT = 4). With
+// LT = 4 the FP32 form is bound by its ten operations per pair and entry (two rows of P
+// packed).
 constexpr int kCtrKT = 8;
 
 // (the _rn intrinsics are never contracted into FMAs, which would break both
@@ -786,12 +787,11 @@ struct AccF32x2 {
     c = add2(c, add2(err, e));
     s = t;
   }
-  __device__ __forceinline__ void values(double& v0, double& v1) const {
+  __device__ __forceinline__ double value(int half) const {
     float s0, s1, c0, c1;
     upk2(s, s0, s1);
     upk2(c, c0, c1);
-    v0 = AccF32::to_f64(s0) + AccF32::to_f64(c0);
-    v1 = AccF32::to_f64(s1) + AccF32::to_f64(c1);
+    return half ? AccF32::to_f64(s1) + AccF32::to_f64(c1) : AccF32::to_f64(s0) + AccF32::to_f64(c0);
   }
 };
 struct AccF64 {
@@ -830,61 +830,132 @@ __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
                : "memory");
 }
 
-// VEC: entries per load; 16-byte loads go through two shared-memory stages of the
-// thread's own vectors (LT + kCtrKT of them), so that a stage's loads are in flight
-// while the stage before is added: with loads into registers a thread waited out the
-// memory's latency four times per 16 x 4 x 8 additions.
-template <typename T, int VEC, int LT>
+// one entry the same way, or a zero
+template <typename T>
+__device__ __forceinline__ void cp_async_entry(T* dst, const T* src, bool in) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(
+                   (uint32_t)__cvta_generic_to_shared(dst)),
+               "l"(src), "n"((int)sizeof(T)), "r"(in ? (int)sizeof(T) : 0)
+               : "memory");
+}
+
+// A block's sums of its LT x KN pairs (KN >= kn, the perturbations it has) into the
+// partials: by warp, then over the 8 warps.
+template <int LT, int KN, typename V>
+__device__ __forceinline__ void contract_sums(const V& value, int ln, int kn, double (*red)[32],
+                                              double* part, int64_t K, int nparts) {
+  constexpr int NP = LT * KN, STEP = 32 / NP;   // lanes per value
+  double v[NP];
+#pragma unroll
+  for (int i = 0; i < NP; ++i) v[i] = value(i / KN, i % KN);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const double s = warp_sums<NP>(v, lane);
+  if (lane % STEP == 0) red[warp][lane / STEP] = s;
+  __syncthreads();
+  if (threadIdx.x < NP) {
+    const int l = threadIdx.x / KN, k = threadIdx.x % KN;
+    double r = 0.0;
+    for (int w = 0; w < 8; ++w) r += red[w][threadIdx.x];
+    if (l < ln && k < kn) part[(l * K + k) * nparts] = r;
+  }
+}
+
+// Every thread adds V entries (16 bytes) of each matrix at a time, through two
+// shared-memory stages of its own entries of LT + KT matrices, so that a stage's loads
+// are in flight while the stage before is added: with loads into registers a thread
+// waited out the memory's latency four times per 16 x 4 x 8 additions. VEC: V
+// consecutive entries by one 16-byte copy, for matrices that start on 16 bytes; else
+// (odd N, offset buffers) V entries 256 apart, each by a copy of its own: in FP32 4 x 64
+// pairs at N = 4093 take 2.06 ms and 1 x 64 0.92, where one P_l per block took 4.61 and
+// 1.18, and a loop that loads one entry a time 6.97 and 4.22. KT = 2: for one or two
+// perturbations, whose block would spend as long on the FP64 sums of pairs that it does not
+// have as on its entries (3 x 1 pairs at N = 2000 100 us, now 54). One instance has one
+// size of sums: several cost instruction cache (2 x 64 pairs at N = 4096 0.83 against 0.80).
+template <typename T, bool VEC, int LT, int KT>
 __global__ void __launch_bounds__(256, 2)
 k_contract_dense(const T* __restrict__ P, int64_t L, const T* __restrict__ Q, int64_t K, int64_t nn,
                  double* part, int nparts, int64_t y0) {
   dep_sync();
   using Acc = typename CtrAcc<T>::type;
-  constexpr int NP = LT * kCtrKT, NV = LT + kCtrKT;
-  const int64_t ktiles = (K + kCtrKT - 1) / kCtrKT;
+  constexpr int NV = LT + KT, V = 16 / (int)sizeof(T);
+  const int64_t ktiles = (K + KT - 1) / KT;
   const int64_t y = y0 + blockIdx.y;
-  const int64_t l0 = (y / ktiles) * LT, k0 = (y % ktiles) * kCtrKT;
-  const int kn = (int)((K - k0) < kCtrKT ? (K - k0) : kCtrKT);
+  const int64_t l0 = (y / ktiles) * LT, k0 = (y % ktiles) * KT;
+  const int kn = (int)((K - k0) < KT ? (K - k0) : KT);
   const int ln = (int)((L - l0) < LT ? (L - l0) : LT);
   const T* p = P + l0 * nn;
   const T* q = Q + k0 * nn;
-  constexpr bool PK = sizeof(T) == 4 && VEC == 4 && LT > 1;   // rows of P in packed pairs
-  Acc acc[PK ? 1 : LT][PK ? 1 : kCtrKT];
-  AccF32x2 acc2[PK ? LT / 2 : 1][PK ? kCtrKT : 1];
-  const int64_t nv = nn / VEC, stride = (int64_t)gridDim.x * blockDim.x;
-  int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if constexpr (VEC * sizeof(T) == 16) {
-    extern __shared__ __align__(16) uint8_t ctr_smem[];
-    struct Vec {
-      T v[VEC];
-    };
-    Vec* mine = reinterpret_cast<Vec*>(ctr_smem) + threadIdx.x;   // [stage][vector][thread]
-    auto fetch = [&](int st, int64_t tt) {
-      if (tt < nv) {
+  constexpr bool PK = sizeof(T) == 4 && LT > 1;   // rows of P in packed pairs
+  Acc acc[PK ? 1 : LT][PK ? 1 : KT];
+  AccF32x2 acc2[PK ? LT / 2 : 1][PK ? KT : 1];
+  extern __shared__ __align__(16) uint8_t ctr_smem[];
+  struct alignas(16) Vec {
+    T v[V];
+  };
+  Vec* mine = reinterpret_cast<Vec*>(ctr_smem) + threadIdx.x;   // VEC: [stage][matrix][thread]
+  T* single = reinterpret_cast<T*>(ctr_smem) + threadIdx.x;     // else [stage][matrix][entry][thread]
+  // a block's group of 256 V entries: c, c + gridDim.x, ...
+  const int64_t groups = (nn + 256 * V - 1) / (256 * V);
+  auto fetch = [&](int st, int64_t c, int m) {   // m: the block's perturbations
+    if constexpr (VEC) {
+      const int64_t o = (c * 256 + threadIdx.x) * V;
+      if (o < nn) {   // (nn is a multiple of V)
 #pragma unroll
         for (int l = 0; l < LT; ++l)
-          if (l < ln) cp_async16(mine + (st * NV + l) * 256, p + l * nn + tt * VEC);
+          if (l < ln) cp_async16(mine + (st * NV + l) * 256, p + l * nn + o);
 #pragma unroll
-        for (int k = 0; k < kCtrKT; ++k)
-          if (k < kn) cp_async16(mine + (st * NV + LT + k) * 256, q + k * nn + tt * VEC);
+        for (int k = 0; k < KT; ++k)
+          if (k < m) cp_async16(mine + (st * NV + LT + k) * 256, q + k * nn + o);
       }
-      asm volatile("cp.async.commit_group;" ::: "memory");
-    };
-    fetch(0, t);
-    for (int st = 0; t < nv; t += stride, st ^= 1) {
-      fetch(st ^ 1, t + stride);
+    } else if (c < groups) {
+      T* d = single + st * NV * V * 256;
+      const int64_t o = c * 256 * V + threadIdx.x;
+#pragma unroll
+      for (int j = 0; j < V; ++j) {
+        const bool in = o + j * 256 < nn;
+        const int64_t oj = in ? o + j * 256 : 0;   // (past the end: zeros)
+#pragma unroll
+        for (int l = 0; l < LT; ++l)
+          if (l < ln) cp_async_entry(d + (l * V + j) * 256, p + l * nn + oj, in);
+#pragma unroll
+        for (int k = 0; k < KT; ++k)
+          if (k < m) cp_async_entry(d + ((LT + k) * V + j) * 256, q + k * nn + oj, in);
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  auto entries = [&](int st, int i) {   // this thread's entries of matrix i
+    if constexpr (VEC) {
+      return mine[(st * NV + i) * 256];
+    } else {
+      Vec r;
+#pragma unroll
+      for (int j = 0; j < V; ++j) r.v[j] = single[((st * NV + i) * V + j) * 256];
+      return r;
+    }
+  };
+  auto more = [&](int64_t c) {
+    return VEC ? (c * 256 + threadIdx.x) * V < nn : c < groups;
+  };
+  // KN: the block's perturbations, or 0: up to KT, tested one by one
+  auto run = [&](auto kn_c) {
+    constexpr int KN = decltype(kn_c)::value;
+    int64_t c = blockIdx.x;
+    fetch(0, c, KN > 0 ? KN : kn);
+    for (int st = 0; more(c); c += gridDim.x, st ^= 1) {
+      fetch(st ^ 1, c + gridDim.x, KN > 0 ? KN : kn);
       asm volatile("cp.async.wait_group 1;" ::: "memory");
       Vec a[LT];
 #pragma unroll
-      for (int l = 0; l < LT; ++l) a[l] = mine[(st * NV + (l < ln ? l : 0)) * 256];
-      if constexpr (PK) {
-        auto add_k = [&](int k, auto two) {   // perturbation k (and k + 1)
-          constexpr int NK = decltype(two)::value ? 2 : 1;
-          Vec b[NK];
+      for (int l = 0; l < LT; ++l) a[l] = entries(st, l < ln ? l : 0);
+      auto add_k = [&](int k, auto two) {   // perturbation k (and k + 1: their chains interleave)
+        constexpr int NK = decltype(two)::value ? 2 : 1;
+        Vec b[NK];
 #pragma unroll
-          for (int i = 0; i < NK; ++i) b[i] = mine[(st * NV + LT + k + i) * 256];
+        for (int i = 0; i < NK; ++i) b[i] = entries(st, LT + k + i);
 #pragma unroll
-          for (int j = 0; j < VEC; ++j)
+        for (int j = 0; j < V; ++j) {
+          if constexpr (PK) {
 #pragma unroll
             for (int l = 0; l < LT / 2; ++l) {
               const uint64_t ap = pk2(a[2 * l].v[j], a[2 * l + 1].v[j]);
@@ -892,83 +963,63 @@ k_contract_dense(const T* __restrict__ P, int64_t L, const T* __restrict__ Q, in
               for (int i = 0; i < NK; ++i)
                 acc2[l][k + i].add(ap, pk2(b[i].v[j], b[i].v[j]), pk2(-b[i].v[j], -b[i].v[j]));
             }
-        };
-        if (kn == kCtrKT) {   // (no exits between the perturbations: their chains interleave)
-#pragma unroll
-          for (int k = 0; k < kCtrKT; k += 2) add_k(k, std::true_type());
-        } else {
-#pragma unroll
-          for (int k = 0; k < kCtrKT; ++k) {
-            if (k >= kn) break;
-            add_k(k, std::false_type());
-          }
-        }
-      } else {
-        if (kn == kCtrKT) {   // (no exits between the perturbations: their chains interleave)
-#pragma unroll
-          for (int k2 = 0; k2 < kCtrKT; k2 += 2) {
-            const Vec b0 = mine[(st * NV + LT + k2) * 256], b1 = mine[(st * NV + LT + k2 + 1) * 256];
-#pragma unroll
-            for (int j = 0; j < VEC; ++j)
-#pragma unroll
-              for (int l = 0; l < LT; ++l) {
-                acc[l][k2].add(a[l].v[j], b0.v[j]);
-                acc[l][k2 + 1].add(a[l].v[j], b1.v[j]);
-              }
-          }
-        } else {
-#pragma unroll
-          for (int k = 0; k < kCtrKT; ++k) {
-            if (k >= kn) break;
-            const Vec b = mine[(st * NV + LT + k) * 256];
+          } else {
 #pragma unroll
             for (int l = 0; l < LT; ++l)
 #pragma unroll
-              for (int j = 0; j < VEC; ++j) acc[l][k].add(a[l].v[j], b.v[j]);
+              for (int i = 0; i < NK; ++i) acc[l][k + i].add(a[l].v[j], b[i].v[j]);
           }
+        }
+      };
+      if constexpr (KN > 0) {
+#pragma unroll
+        for (int k = 0; k + 1 < KN; k += 2) add_k(k, std::true_type());
+        if constexpr (KN % 2 != 0) add_k(KN - 1, std::false_type());
+      } else {
+#pragma unroll
+        for (int k = 0; k < KT; ++k) {
+          if (k >= kn) break;
+          add_k(k, std::false_type());
         }
       }
     }
-    asm volatile("cp.async.wait_all;" ::: "memory");
-  } else {
-    for (; t < nv; t += stride) {
-      T a[LT];
-#pragma unroll
-      for (int l = 0; l < LT; ++l) a[l] = p[(l < ln ? l : 0) * nn + t];
-#pragma unroll
-      for (int k = 0; k < kCtrKT; ++k) {
-        if (k >= kn) break;
-        const T b = q[k * nn + t];
-#pragma unroll
-        for (int l = 0; l < LT; ++l) acc[l][k].add(a[l], b);
+  };
+  if constexpr (sizeof(T) == 8) {
+    // (an FP64 instruction that a test inside the loop switches off takes its 64 clocks)
+    if constexpr (KT < kCtrKT) {
+      if (kn == 1) run(std::integral_constant<int, 1>());
+      else run(std::integral_constant<int, KT>());
+    } else {
+      switch (kn) {
+        case 1: run(std::integral_constant<int, 1>()); break;
+        case 2: run(std::integral_constant<int, 2>()); break;
+        case 3: run(std::integral_constant<int, 3>()); break;
+        case 4: run(std::integral_constant<int, 4>()); break;
+        case 5: run(std::integral_constant<int, 5>()); break;
+        case 6: run(std::integral_constant<int, 6>()); break;
+        case 7: run(std::integral_constant<int, 7>()); break;
+        default: run(std::integral_constant<int, KT>());
       }
     }
-  }
-  __shared__ double red[8][NP];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  double v[NP];
-  if constexpr (PK) {
-#pragma unroll
-    for (int i = 0; i < NP / 2; ++i)
-      acc2[i / kCtrKT][i % kCtrKT].values(v[i / kCtrKT * 2 * kCtrKT + i % kCtrKT],
-                                          v[(i / kCtrKT * 2 + 1) * kCtrKT + i % kCtrKT]);
   } else {
-#pragma unroll
-    for (int i = 0; i < NP; ++i) v[i] = acc[i / kCtrKT][i % kCtrKT].value();
+    if (kn == KT) run(std::integral_constant<int, KT>());
+    else run(std::integral_constant<int, 0>());
   }
-  const double s = warp_sums<NP>(v, lane);
-  constexpr int STEP = 32 / NP;   // lanes per value
-  if (lane % STEP == 0) red[warp][lane / STEP] = s;
-  __syncthreads();
-  if (threadIdx.x < NP) {
-    const int l = threadIdx.x / kCtrKT, k = threadIdx.x % kCtrKT;
-    double r = 0.0;
-    for (int w = 0; w < 8; ++w) r += red[w][threadIdx.x];
-    if (l < ln && k < kn) part[((l0 + l) * K + k0 + k) * nparts + blockIdx.x] = r;
-  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  __shared__ double red[8][32];
+  auto value = [&](int l, int k) {
+    if constexpr (PK) {
+      return acc2[l / 2][k].value(l % 2);
+    } else {
+      return acc[l][k].value();
+    }
+  };
+  double* out = part + (l0 * K + k0) * nparts + blockIdx.x;
+  contract_sums<LT, KT>(value, ln, kn, red, out, K, nparts);
 }
 
-// One pair (l, k) per block row: FP64 matrices too small to fill the GPU in groups.
+// One pair (l, k) per block row: FP64 matrices too small to fill the GPU in groups, and
+// groups of a pair or two.
 __global__ void k_contract_pair(const double* __restrict__ P, const double* __restrict__ Q, int64_t K,
                                 int64_t nn, double* part, int nparts, int64_t y0) {
   dep_sync();
@@ -1186,36 +1237,42 @@ int contract_nparts(int64_t n, int q_diag) {
 }
 
 namespace {
-template <typename T, int VEC, int LT>
+template <typename T, bool VEC, int LT, int KT>
 void contract_rows(const void* P, int64_t L, const void* Q, int64_t K, int64_t nn, double* part,
-                   int nparts, int64_t rows, cudaStream_t s) {
+                   int nparts, cudaStream_t s) {
+  const int64_t rows = (L + LT - 1) / LT * ((K + KT - 1) / KT);
   // grid rows go out in launches of at most 65535, the limit of gridDim.y
   constexpr int64_t kMaxY = 65535;
-  constexpr size_t smem = VEC * sizeof(T) == 16 ? (size_t)2 * (LT + kCtrKT) * 256 * 16 : 0;
-  if (smem > 48 * 1024)
-    cudaFuncSetAttribute(k_contract_dense<T, VEC, LT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)smem);
+  // (single entries come through L1: at three blocks per SM their stages leave it too
+  // little, FP64 1 x 64 pairs at N = 2749 1125 us against 850 at two)
+  constexpr size_t stages = (size_t)2 * (LT + KT) * 256 * 16, two = (size_t)80 << 10;
+  constexpr size_t smem = VEC || stages > two ? stages : two;
+  cudaFuncSetAttribute(k_contract_dense<T, VEC, LT, KT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       (int)smem);
   for (int64_t y0 = 0; y0 < rows; y0 += kMaxY) {
     const int64_t ny = (rows - y0) < kMaxY ? (rows - y0) : kMaxY;
     const dim3 grid((unsigned)nparts, (unsigned)ny);
-    launch_dep(k_contract_dense<T, VEC, LT>, grid, 256, smem, s, static_cast<const T*>(P), L,
+    launch_dep(k_contract_dense<T, VEC, LT, KT>, grid, 256, smem, s, static_cast<const T*>(P), L,
                static_cast<const T*>(Q), K, nn, part, nparts, y0);
   }
 }
-// One block row per LT rows of P and kCtrKT perturbations. FP32: LT = 4 from three rows
-// of P on. FP64 is bound by its pipe, which a row formed for nothing would keep busy, so
-// LT divides L (3 x 40 pairs at N = 2000 0.95 ms by pairs, 0.85 so); and with fewer than
-// eight blocks per SM some SMs have a block more than others for a good part of the
-// time: there every pair has its own block row (2 x 5 pairs at N = 700 47 us; a drawn
-// case of this kind took 200 us in groups and 171 by pairs).
-template <typename T, int VEC>
+// One block row per LT rows of P and kCtrKT perturbations. FP32: LT = 4 where it divides
+// L, and for three rows (two packed pairs in any case); else 2, as four would form up to
+// three rows for nothing (5 x 40 pairs at N = 2000 541 us, by twos 404). FP64 is bound by
+// its pipe, which a row formed for nothing would keep busy, so LT divides L
+// (3 x 40 pairs at N = 2000 0.95 ms by pairs, 0.85 so); and with fewer than eight blocks
+// per SM some SMs have a block more than others for a good part of the time: there every
+// pair has its own block row (2 x 5 pairs at N = 700 47 us in groups, 39 by pairs), as
+// where a group shares next to nothing: 1 x 1 at N = 2000 41 and 40 us; of matrices that
+// are not aligned also two pairs, 9 x 2 at N = 2749 314 and 281 us. K <= 2: see KT.
+template <typename T, bool VEC>
 void contract_dense(const void* P, int64_t L, const void* Q, int64_t K, int64_t nn, double* part,
                     int nparts, cudaStream_t s) {
   const int64_t kt = (K + kCtrKT - 1) / kCtrKT;
-  int64_t lt = L == 1 ? 1 : (L == 2 ? 2 : 4);
+  int64_t lt = L == 1 ? 1 : (L == 3 || L % 4 == 0 ? 4 : 2);
   if constexpr (sizeof(T) == 8) {
     lt = L % 4 == 0 ? 4 : (L % 2 == 0 ? 2 : 1);
-    if (nparts * (L / lt) * kt < 8 * 152) {
+    if (nparts * (L / lt) * kt < 8 * 152 || lt * K <= (VEC ? 1 : 2)) {
       constexpr int64_t kMaxY = 65535;
       for (int64_t y0 = 0; y0 < L * K; y0 += kMaxY) {
         const int64_t ny = L * K - y0 < kMaxY ? L * K - y0 : kMaxY;
@@ -1225,9 +1282,14 @@ void contract_dense(const void* P, int64_t L, const void* Q, int64_t K, int64_t 
       return;
     }
   }
-  if (lt == 1) contract_rows<T, VEC, 1>(P, L, Q, K, nn, part, nparts, L * kt, s);
-  else if (lt == 2) contract_rows<T, VEC, 2>(P, L, Q, K, nn, part, nparts, L / 2 * kt, s);
-  else contract_rows<T, VEC, 4>(P, L, Q, K, nn, part, nparts, (L + 3) / 4 * kt, s);
+  auto go = [&](auto kt_c) {
+    constexpr int KT = decltype(kt_c)::value;
+    if (lt == 1) contract_rows<T, VEC, 1, KT>(P, L, Q, K, nn, part, nparts, s);
+    else if (lt == 2) contract_rows<T, VEC, 2, KT>(P, L, Q, K, nn, part, nparts, s);
+    else contract_rows<T, VEC, 4, KT>(P, L, Q, K, nn, part, nparts, s);
+  };
+  if (K <= 2) go(std::integral_constant<int, 2>());
+  else go(std::integral_constant<int, kCtrKT>());
 }
 }  // namespace
 
@@ -1253,11 +1315,11 @@ cudaError_t launch_contract(const void* P, int64_t L, const void* Q, int64_t K, 
                                                     nparts, y0);
     }
   } else if (dtype == SP2_F64) {
-    if (al && nn % 2 == 0) contract_dense<double, 2>(P, L, Q, K, nn, part, nparts, s);
-    else contract_dense<double, 1>(P, L, Q, K, nn, part, nparts, s);
+    if (al && nn % 2 == 0) contract_dense<double, true>(P, L, Q, K, nn, part, nparts, s);
+    else contract_dense<double, false>(P, L, Q, K, nn, part, nparts, s);
   } else {
-    if (al && nn % 4 == 0) contract_dense<float, 4>(P, L, Q, K, nn, part, nparts, s);
-    else contract_dense<float, 1>(P, L, Q, K, nn, part, nparts, s);
+    if (al && nn % 4 == 0) contract_dense<float, true>(P, L, Q, K, nn, part, nparts, s);
+    else contract_dense<float, false>(P, L, Q, K, nn, part, nparts, s);
   }
   launch_dep(k_contract_final, (unsigned)(L * K), 256, 0, s, part, nparts, out);
   return cudaGetLastError();

@@ -233,3 +233,39 @@ def test_dense_incoming_gradient(sp2, mode, n):
         (grad,) = torch.autograd.grad((w * d).sum(), x)
         out.append(grad)
     assert torch.equal(out[0], out[1]) and out[0].abs().max() > 0
+
+
+@pytest.mark.parametrize("L,K,n,shift", [(1, 1, 45, 0), (2, 2, 33, 0), (5, 3, 77, 0), (7, 5, 131, 0),
+                                         (1, 6, 65, 1), (6, 7, 32, 1), (3, 15, 91, 0), (8, 4, 37, 0),
+                                         (1, 23, 701, 0), (5, 12, 701, 0), (3, 17, 702, 1)])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
+def test_contraction_remainders(sp2, L, K, n, shift, dtype):
+    """Every count of perturbations and rows that a block can be left with, of matrices on
+    16-byte boundaries and not, N^2 of every remainder: bounds as in test_contraction_forms."""
+    test_contraction_forms(sp2, L, K, n, shift, dtype)
+
+
+@pytest.mark.parametrize("L", [1, 3])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
+def test_offset_contractions_cost_what_aligned_ones_do(sp2, L, dtype):
+    """The same bytes and operations, with single-entry copies in place of 16-byte ones
+    (4 or 2 times their number, beside 16 arithmetic operations or more per entry): less
+    than twice the time. The best of several runs of each, in turn."""
+    n, K = 2000, 40
+    h = sp2.Handle()
+    def make(rows, shift):
+        buf = torch.randn(rows * n * n + 1, dtype=dtype, device="cuda")
+        return buf[shift:shift + rows * n * n].view(rows, n, n)
+    forms = [(make(L, s), make(K, s)) for s in (0, 1)]
+    best = [float("inf")] * 2
+    for _ in range(6):
+        for i, (P, Q) in enumerate(forms):
+            t0, t1 = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            sp2.response_contract(P, Q, handle=h)
+            t0.record()
+            for _ in range(4):
+                sp2.response_contract(P, Q, handle=h)
+            t1.record()
+            t1.synchronize()
+            best[i] = min(best[i], t0.elapsed_time(t1))
+    assert best[1] <= 2.0 * best[0]
