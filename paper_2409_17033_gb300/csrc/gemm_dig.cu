@@ -52,6 +52,7 @@
 #include <string.h>
 
 #include "decide.cuh"
+#include "per_device.h"
 #include "sp2_internal.h"
 #include "tc_ptx.cuh"
 
@@ -744,38 +745,43 @@ k_dig_plain(const Sums q, int64_t rows, const int* __restrict__ ea,
   st4d(out + (i0 + r) * np + j0 + c4, w);
 }
 
+// CTA pairs of k_gemm_dig<BN> resident at a time on the current device, whose
+// shared-memory limit for the kernel is set with it.
 template <int BN>
-int resident_pairs() {
-  static int n = 0;
-  if (n) return n;
-  auto kern = k_gemm_dig<BN>;
-  int dev = 0, nsm = 0, nc = 0;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           Geo<BN>::SMEM_BYTES) != cudaSuccess ||
-      cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-    return 0;
-  cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = 2;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  cfg.gridDim = dim3((unsigned)(2 * (nsm / 2)));
-  cfg.blockDim = dim3(NUM_THREADS);
-  cfg.dynamicSmemBytes = Geo<BN>::SMEM_BYTES;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  if (cudaOccupancyMaxActiveClusters(&nc, kern, &cfg) != cudaSuccess || nc < 1) return 0;
-  n = nc;
-  return n;
+cudaError_t resident_pairs(int* n) {
+  static PerDevice kept;
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  return kept.get(dev, cudaErrorInvalidDevice, n, [&](int* pairs) {
+    auto kern = k_gemm_dig<BN>;
+    int nsm = 0;
+    cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         Geo<BN>::SMEM_BYTES);
+    if (r == cudaSuccess) r = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    if (r != cudaSuccess) return r;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 2;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3((unsigned)(2 * (nsm / 2)));
+    cfg.blockDim = dim3(NUM_THREADS);
+    cfg.dynamicSmemBytes = Geo<BN>::SMEM_BYTES;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    r = cudaOccupancyMaxActiveClusters(pairs, kern, &cfg);
+    return r == cudaSuccess && *pairs < 1 ? cudaErrorNotSupported : r;
+  });
 }
 
 template <int BN>
 cudaError_t launch_bn(const CUtensorMap& am, const CUtensorMap& bm, const DParams& p,
                       cudaStream_t s) {
-  const int res = resident_pairs<BN>();
-  if (res < 1) return cudaErrorNotSupported;
+  int res = 0;
+  const cudaError_t e = resident_pairs<BN>(&res);
+  if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute at[2];
   at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;

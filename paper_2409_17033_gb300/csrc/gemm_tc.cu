@@ -67,6 +67,7 @@
 #include <mutex>
 
 #include "decide.cuh"
+#include "per_device.h"
 #include "sp2_internal.h"
 #include "tc_ptx.cuh"
 
@@ -952,37 +953,36 @@ bool cached_maps(const MapKey& k, KMaps* out) {
 // count queried once
 template <int KIND, int EPI, int CG, int BN = BN_FULL, bool SPARSE = false>
 cudaError_t launch_kind(const KMaps& maps, const KParams& p, int units, cudaStream_t s) {
-  static int resident = 0;
   auto kern = k_gemm_tc<KIND, EPI, CG, BN, SPARSE>;
   constexpr int smem = Ring<CG, BN>::SMEM_BYTES;
-  if (!resident) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
-    int dev = 0, nsm = 0;
-    e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
+  static PerDevice kept;   // CTAs (pairs) resident at a time
+  int dev = 0, resident = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  e = kept.get(dev, cudaErrorInvalidDevice, &resident, [&](int* res) {
+    int nsm = 0;
+    cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (r == cudaSuccess) r = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    if (r != cudaSuccess) return r;
     if (CG == 1) {
-      resident = nsm;   // one CTA per SM: the ring leaves no room for a second
-    } else {
-      cudaLaunchConfig_t cfg = {};
-      cudaLaunchAttribute at[1];
-      at[0].id = cudaLaunchAttributeClusterDimension;
-      at[0].val.clusterDim.x = CG;
-      at[0].val.clusterDim.y = 1;
-      at[0].val.clusterDim.z = 1;
-      cfg.gridDim = dim3((unsigned)(CG * (nsm / CG)));
-      cfg.blockDim = dim3(NUM_THREADS);
-      cfg.dynamicSmemBytes = smem;
-      cfg.attrs = at;
-      cfg.numAttrs = 1;
-      int nc = 0;
-      e = cudaOccupancyMaxActiveClusters(&nc, kern, &cfg);
-      if (e != cudaSuccess) return e;
-      if (nc < 1) return cudaErrorNotSupported;
-      resident = nc;
+      *res = nsm;   // one CTA per SM: the ring leaves no room for a second
+      return cudaSuccess;
     }
-  }
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = CG;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3((unsigned)(CG * (nsm / CG)));
+    cfg.blockDim = dim3(NUM_THREADS);
+    cfg.dynamicSmemBytes = smem;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    r = cudaOccupancyMaxActiveClusters(res, kern, &cfg);
+    return r == cudaSuccess && *res < 1 ? cudaErrorNotSupported : r;
+  });
+  if (e != cudaSuccess) return e;
   const int n = units < resident ? units : resident;
   if (CG == 1) return launch_dep(kern, n, NUM_THREADS, smem, s, maps, p);
   cudaLaunchConfig_t cfg = {};
