@@ -17,6 +17,17 @@
 
 using namespace sp2;
 
+// What every call needs, in one allocation of the handle that does not count as
+// workspace: the step state, its copies for the adjoint, the squares' completion counter
+// and the partials of all but the largest products (more of them than a product's tiles
+// once had, so that a workspace limit holds what it held).
+constexpr int64_t kFixedParts = 16384;
+struct HandleBlock {
+  DevState state, hist, adj;
+  unsigned done;
+  Part3 part[kFixedParts];
+};
+
 struct sp2_handle_s {
   int device = 0;
   cudaStream_t stream = nullptr;
@@ -33,7 +44,8 @@ struct sp2_handle_s {
     int n = 0;
   };
   std::map<std::string, TileList> tiles;
-  DevState* d_state = nullptr;
+  HandleBlock* block = nullptr;  // device
+  DevState* d_state = nullptr;   // &block->state
   DevState* h_state = nullptr;  // pinned mirror
   TcTuning tune;                // product-kernel launch settings (sp2_set_option)
   // The digit buffers of FP64 products ("dig.*") are optional: when device memory or
@@ -456,13 +468,12 @@ double dig_flops(const Ctx& c, const DigBufs& b) {
   return 2.0 * 256.0 * b.plan.bn * (double)c.np * 36.0 * b.ntiles;
 }
 
-int decide_args(Ctx& c, const DecideParams& dec, SimtDecide* sd) {
-  void* dn;
-  TRY(ws(c.h, "decide.done", sizeof(unsigned), &dn));
-  sd->p = dec;
-  sd->st = c.st;
-  sd->done = static_cast<unsigned*>(dn);
-  return SP2_OK;
+SimtDecide decide_args(const Ctx& c, const DecideParams& dec) {
+  SimtDecide sd;
+  sd.p = dec;
+  sd.st = c.st;
+  sd.done = &c.h->block->done;
+  return sd;
 }
 
 // One FP64 step with responses by digits, Y_n X_n and X_n^2 in one product launch, and
@@ -475,8 +486,7 @@ int dig_step(Ctx& c, const MatBuf& xin, const MatBuf& xout, const MatBuf& yin, c
   DigBufs db;
   if (!dig_mode(c, rows + c.np) || h->dig_apart || dig_chunk(c.np, batch + 1) <= batch) return SP2_OK;
   if (!dig_bufs(c, rows, false, &db, true)) return SP2_OK;
-  SimtDecide sd;
-  TRY(decide_args(c, *dec, &sd));
+  SimtDecide sd = decide_args(c, *dec);
   sd.p.nparts = (int)dig_square_nparts(c.np);
   const double *x = static_cast<const double*>(xin.master), *y = static_cast<const double*>(yin.master);
   const int64_t left = rows + c.np;
@@ -510,7 +520,7 @@ int square_step(Ctx& c, const MatBuf& xin, const MatBuf& xout, int step,
   sp2_handle_t h = c.h;
   DigBufs db;
   SimtDecide sd;
-  if (dec) TRY(decide_args(c, *dec, &sd));
+  if (dec) sd = decide_args(c, *dec);
   if (dig_mode(c, c.np)) {
     sd.p.nparts = (int)dig_square_nparts(c.np);
     if (dig_bufs(c, 0, true, &db)) {
@@ -1060,12 +1070,8 @@ int run_sp2(sp2_handle_t h, const void* Hd, int64_t n, int dtype, double nocc, c
     TRY(ws(h, "Xbest.m", xbytes, &xbest.master));
     if (ybatch > 0) TRY(ws(h, "Ybest.m", (size_t)ybatch * xbytes, &ybest.master));
   }
-  if (!sparse) {
-    // the completion counter of the squares' last-block decision starts at zero
-    void* dn;
-    TRY(ws(h, "decide.done", sizeof(unsigned), &dn));
-    CK(cudaMemsetAsync(dn, 0, sizeof(unsigned), h->stream));
-  }
+  // the completion counter of the squares' last-block decision starts at zero
+  if (!sparse) CK(cudaMemsetAsync(&h->block->done, 0, sizeof(unsigned), h->stream));
   // a small candidate is kept by the block that takes the decision (see keep_candidate)
   const bool keep_small = track && mode == SP2_MODE_FP64 && xbytes <= kKeepSmall;
   const HostSnap* seen = nullptr;   // the snapshot of the recursion's end
@@ -1225,9 +1231,12 @@ int make_ctx(sp2_handle_t h, int mode, int64_t n, int64_t np, bool timing, Ctx* 
   h->dig_apart = false;
   h->dig_x = nullptr;
   if (dig_mode(*c, np) && maxp < dig_square_nparts(np)) maxp = dig_square_nparts(np);
-  void* p;
-  TRY(ws(h, "part", (size_t)maxp * sizeof(Part3), &p));
-  c->part = static_cast<Part3*>(p);
+  c->part = h->block->part;
+  if (maxp > kFixedParts) {
+    void* p;
+    TRY(ws(h, "part", (size_t)maxp * sizeof(Part3), &p));
+    c->part = static_cast<Part3*>(p);
+  }
   return SP2_OK;
 }
 
@@ -1241,12 +1250,8 @@ int run_adjoint(sp2_handle_t h, const void* Bd, int64_t batch, int b_diag, int s
   const int mode = hs.mode, M = hs.M, k = hs.k;
   // the adjoint's own state: the branch signs of the kept forward recursion (a
   // device copy), with nothing to stop and no floor candidate to keep
-  void* stp;
-  void* hst;
-  TRY(ws(h, "adj.state", sizeof(DevState), &stp));
-  TRY(ws(h, "hist.state", sizeof(DevState), &hst));
-  DevState* ast = static_cast<DevState*>(stp);
-  CK(cudaMemcpyAsync(ast, hst, sizeof(DevState), cudaMemcpyDeviceToDevice, h->stream));
+  DevState* ast = &h->block->adj;
+  CK(cudaMemcpyAsync(ast, &h->block->hist, sizeof(DevState), cudaMemcpyDeviceToDevice, h->stream));
   CK(launch_adjoint_state(ast, h->stream));
   c.kernels++;
   c.st = ast;
@@ -1325,9 +1330,7 @@ int run_adjoint(sp2_handle_t h, const void* Bd, int64_t batch, int b_diag, int s
 // keep the forward recursion's device state (branch signs) for a later adjoint
 int keep_history(sp2_handle_t h, const Sp2Out& r, int64_t n, int64_t np, int mode, int k,
                  int tail) {
-  void* hst;
-  TRY(ws(h, "hist.state", sizeof(DevState), &hst));
-  CK(cudaMemcpyAsync(hst, h->d_state, sizeof(DevState), cudaMemcpyDeviceToDevice, h->stream));
+  CK(cudaMemcpyAsync(&h->block->hist, h->d_state, sizeof(DevState), cudaMemcpyDeviceToDevice, h->stream));
   auto& hs = h->hist;
   hs.valid = true;
   hs.n = n;
@@ -1410,9 +1413,8 @@ int complete_pending(sp2_handle_t h, sp2_info* info) {
         info->M = hs.M;
         info->converged = 1;
         info->beta = hs.beta;
-        void* hst;
-        if (ws(h, "hist.state", sizeof(DevState), &hst) == SP2_OK &&
-            cudaMemcpy(h->h_state, hst, sizeof(DevState), cudaMemcpyDeviceToHost) == cudaSuccess)
+        if (cudaMemcpy(h->h_state, &h->block->hist, sizeof(DevState), cudaMemcpyDeviceToHost) ==
+            cudaSuccess)
           for (int i = 1; i <= hs.M; ++i) info->sigma[i - 1] = (int8_t)h->h_state->sigma[i];
       }
     }
@@ -1629,7 +1631,7 @@ int sp2_create(sp2_handle_t* out, void* stream, size_t limit) {
   h->limit = limit;
   int code = SP2_OK;
   if (cudaGetDevice(&h->device) != cudaSuccess ||
-      cudaMalloc(&h->d_state, sizeof(DevState)) != cudaSuccess ||
+      cudaMalloc(&h->block, sizeof(HandleBlock)) != cudaSuccess ||
       cudaMallocHost(&h->h_state, sizeof(DevState)) != cudaSuccess) {
     cudaGetLastError();
     code = SP2_ECUDA;
@@ -1642,10 +1644,11 @@ int sp2_create(sp2_handle_t* out, void* stream, size_t limit) {
   if (code != SP2_OK) {
     if (h->ring) cudaFreeHost(h->ring);
     if (h->h_state) cudaFreeHost(h->h_state);
-    if (h->d_state) cudaFree(h->d_state);
+    if (h->block) cudaFree(h->block);
     delete h;
     return code;
   }
+  h->d_state = &h->block->state;
   memset(h->h_state, 0, sizeof(DevState));
   memset(h->ring, 0, sizeof(HostSnap) * sp2_handle_s::kRing);
   *out = h;
@@ -1658,7 +1661,7 @@ int sp2_destroy(sp2_handle_t h) {
   for (auto& kv : h->bufs)
     if (kv.second.p) cudaFree(kv.second.p);
   for (auto& kv : h->tiles) cudaFree(kv.second.d);
-  if (h->d_state) cudaFree(h->d_state);
+  if (h->block) cudaFree(h->block);
   if (h->h_state) cudaFreeHost(h->h_state);
   if (h->ring) cudaFreeHost(h->ring);
   if (h->side) {

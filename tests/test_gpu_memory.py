@@ -1,0 +1,84 @@
+"""What a handle asks for: limits that hold a call by its least form, what earlier calls
+leave, and the optional buffers (digits of FP64 products, batches of responses)."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def sp2():
+    import __graft_entry__ as g
+    g.build()
+    import paper_2409_17033_gb300 as m
+    return m
+
+
+def _gapped(n, seed=0):
+    rng = np.random.default_rng(seed)
+    q, _ = np.linalg.qr(rng.standard_normal((n, n)))
+    e = np.concatenate([rng.uniform(-1, -.2, n // 2), rng.uniform(.2, 1, n - n // 2)])
+    h = (q * e) @ q.T
+    return 0.5 * (h + h.T)
+
+
+def _inputs(n, mode):
+    dt = torch.float64 if mode == "fp64" else torch.float32
+    H = torch.from_numpy(_gapped(n)).to(dt).cuda()
+    return H, torch.from_numpy(np.stack([_gapped(n, s) for s in (1, 2, 3)])).to(dt).cuda()
+
+
+def _call(sp2, name, n, mode, H, B, handle):
+    """One call; its outputs."""
+    kw = dict(mode=mode, idem_tol=1e-10 if mode == "fp64" else 0.0, handle=handle)
+    if name == "density":
+        return sp2.sp2_density(H, n // 2, **kw)[0]
+    if name == "response":
+        return sp2.sp2_response(H, n // 2, B, **kw)[0]
+    if name == "chi":
+        return sp2.sp2_susceptibility(H, n // 2, B[:2], direction="backward", **kw)[0]
+    if name == "chi_k1":
+        return sp2.sp2_susceptibility(H, n // 2, B[:1], direction="backward", ckpt_k=1, **kw)[0]
+    if name == "fermi":
+        del kw["idem_tol"]
+        return sp2.sp2_fermi(H, 0.0, 0.05, B, n_doublings=12, **kw)[0]
+    sp2.sp2_density(H, n // 2, keep_history=True, **kw)
+    return sp2.sp2_adjoint(B[0].contiguous(), handle)
+
+
+# Bytes that each call takes with its matrices at the least padding (64 in FP64), one
+# response at a time and no digits: the limit that has to be enough for it.
+LEAST = {
+    **{("fp64", 128, k): v for k, v in dict(density=398340, response=1971204, chi=2778436,
+            chi_k1=5268804, fermi=4986896, adjoint=2385220).items()},
+    **{("fp64", 190, k): v for k, v in dict(density=892388, response=4431332, chi=6221604,
+            chi_k1=11824932, fermi=11215840, adjoint=5336868).items()},
+    **{("fp64", 256, k): v for k, v in dict(density=1583300, response=7874756, chi=11041284,
+            chi_k1=22051332, fermi=19935440, adjoint=9468420).items()},
+    **{("fp32", 300, k): v for k, v in dict(density=1783492, response=8861380, chi=13600772,
+            chi_k1=28936196, fermi=22428544, adjoint=11831300).items()},
+    **{("fp32", 1000, k): v for k, v in dict(density=12623492, response=62955140, chi=96530372,
+            chi_k1=209776580, fermi=159428144, adjoint=83947460).items()},
+    **{("fp16x2", 300, k): v for k, v in dict(density=5259968, response=24134396, chi=33592360,
+            chi_k1=52466708, fermi=79710384, adjoint=28349460).items()},
+    **{("fp16x2", 1000, k): v for k, v in dict(density=21012096, response=96509628, chi=138473448,
+            chi_k1=213970900, fermi=318812000, adjoint=117501908).items()},
+    **{("bf16x3", 300, k): v for k, v in dict(density=6308544, response=28328640, chi=38835200,
+            chi_k1=56136704, fermi=99633024, adjoint=32543744).items()},
+}
+
+
+@pytest.mark.parametrize("mode,n,name", sorted(LEAST))
+def test_least_limit_is_enough(sp2, mode, n, name):
+    """With the same result as without a limit (other products in FP64: digits or sums)."""
+    H, B = _inputs(n, mode)
+    free = _call(sp2, name, n, mode, H, B, sp2.Handle())
+    h = sp2.Handle(LEAST[mode, n, name])
+    got = _call(sp2, name, n, mode, H, B, h)
+    assert h.workspace_bytes() <= LEAST[mode, n, name]
+    if mode == "fp64":
+        # some 30 steps of sums whose rounding, relative to the norms, each at most doubles
+        assert (got - free).norm() <= 1e-8 * free.norm()
+    else:
+        assert torch.equal(got, free)
