@@ -2036,19 +2036,28 @@ int fermi_batch(Ctx& c, FermiState& fs, int64_t want, int64_t* B) {
   const Buf bufs[] = {{"ft.dd0", &fs.dd[0]}, {"ft.dd1", &fs.dd[1]}, {"ft.E", &fs.E}, {"ft.F1", &fs.F1},
                       {"ft.dW", &fs.dW}, {"ft.G1", &fs.G1}, {"ft.P", &fs.P}, {"ft.T", &fs.T},
                       {"ft.U", &fs.U}};
-  for (;; b = (b + 1) / 2) {
+  for (; b > 1; b = (b + 1) / 2) {
+    // larger batches take free room only: neither the digits' nor what earlier calls left
     int r = SP2_OK;
-    for (const Buf& q : bufs)
-      if (r == SP2_OK) r = fmat(h, q.name, c.np, c.mode, q.f, b);
-    if (r == SP2_OK) r = ws(h, "ft.tr", (size_t)b * sizeof(double), &fs.tr);
+    const size_t el = (size_t)c.np * c.np * b;
+    void* p;
+    for (const Buf& q : bufs) {
+      const std::string nm = q.name;
+      if (r == SP2_OK) r = ws_try(h, nm + ".m", el * master_size(c.mode), &p);
+      for (const char* part : {".h", ".l", ".d"})
+        if (r == SP2_OK && split_mode(c.mode) && (n_planes(c.mode) == 3 || part[1] != 'd'))
+          r = ws_try(h, nm + part, el * 2, &p);
+    }
     if (r == SP2_OK) break;
-    if (r != SP2_ENOMEM || b == 1) return r;
+    if (r != SP2_ENOMEM) return r;
     // (all of them: some may have grown)
     CK(cudaStreamSynchronize(h->stream));
     for (const Buf& q : bufs)
-      for (const char* part : {".m", ".h", ".l", ".d", ".s"}) ws_free(h, std::string(q.name) + part);
+      for (const char* part : {".m", ".h", ".l", ".d"}) ws_free(h, std::string(q.name) + part);
     h->err.clear();
   }
+  for (const Buf& q : bufs) TRY(fmat(h, q.name, c.np, c.mode, q.f, b));
+  TRY(ws(h, "ft.tr", (size_t)b * sizeof(double), &fs.tr));
   *B = b;
   return SP2_OK;
 }

@@ -82,3 +82,28 @@ def test_least_limit_is_enough(sp2, mode, n, name):
         assert (got - free).norm() <= 1e-8 * free.norm()
     else:
         assert torch.equal(got, free)
+
+
+def test_batch_growth_keeps_the_digits(sp2):
+    """FP64 finite-T responses on a GPU that is nearly full: the scratch of a larger batch
+    does not fit, and the products keep their digit buffers."""
+    n, k, dbl = 2000, 6, 12
+    mat = 8 * 2048 * 2048
+    g = torch.Generator(device="cuda").manual_seed(0)
+    H = torch.randn(n, n, generator=g, device="cuda", dtype=torch.float64)
+    H = (H + H.T) * 0.2 / n ** 0.5
+    B = torch.randn(k, n, generator=g, device="cuda", dtype=torch.float64)
+    kw = dict(diag_only=True, mode="fp64", n_doublings=dbl)
+    h = sp2.Handle()
+    least = (2 * dbl + 1 + 6 + 6 + 1) * mat + 8 * mat      # history, scratch, R_I; digits and sums
+    torch.cuda.empty_cache()
+    fill = torch.cuda.mem_get_info()[0] - least - (n * n * 8 * (k + 1)) - 24 * mat
+    filler = torch.empty(max(fill, 0), dtype=torch.uint8, device="cuda")
+    try:
+        D1, _, _ = sp2.sp2_fermi(H, 0.0, 0.1, B, handle=h, **kw)
+    finally:
+        del filler
+        torch.cuda.empty_cache()
+    assert h.workspace_bytes() > least - mat
+    ref, _, _ = sp2.sp2_fermi(H, 0.0, 0.1, B, handle=sp2.Handle(), **kw)
+    assert (D1 - ref).norm() <= 1e-9 * ref.norm()
