@@ -57,7 +57,9 @@
  * Internal working storage (padded copies, X ping-pong buffers, split planes,
  * the X_n checkpoints of the adjoint, reduction partials) is owned by the
  * handle, grows on demand up to `workspace_limit_bytes` (0 = no limit; beside a
- * fixed half megabyte for step states and partials) and is freed by sp2_destroy.
+ * fixed half megabyte for step states and partials) and is freed by sp2_destroy;
+ * what earlier calls left, but for the X_n history, is given back before a call fails
+ * for want of room.
  *
  * Return value: an sp2_status. On failure nothing is guaranteed about the
  * outputs; sp2_last_error(h) gives a message (handle-owned string, valid

@@ -37,8 +37,12 @@ struct sp2_handle_s {
   struct Buf {
     void* p = nullptr;
     size_t bytes = 0;
+    unsigned long long call = 0;   // the last call that asked for it
   };
   std::map<std::string, Buf> bufs;
+  unsigned long long call = 0;     // calls so far (CallScope)
+  int depth = 0;
+  bool ft_single = false;          // room was short: finite-T responses one at a time
   struct TileList {
     Tile* d = nullptr;
     int n = 0;
@@ -109,11 +113,23 @@ int fail(sp2_handle_t h, int code, const char* fmt, ...) {
   } while (0)
 
 // --------------------------------------------------------------- workspace
+// One call through the ABI (calls that a call makes count as part of it).
+struct CallScope {
+  sp2_handle_t h;
+  explicit CallScope(sp2_handle_t hh) : h(hh) {
+    if (h && h->depth++ == 0) ++h->call;
+  }
+  ~CallScope() {
+    if (h) --h->depth;
+  }
+};
+
 // A named device buffer of at least `bytes`; SP2_ENOMEM with h->err set when there
 // is no room.
 int ws_try(sp2_handle_t h, const std::string& name, size_t bytes, void** out) {
   if (bytes == 0) bytes = 256;
   auto& b = h->bufs[name];
+  b.call = h->call;
   if (b.bytes >= bytes) {
     *out = b.p;
     return SP2_OK;
@@ -157,8 +173,31 @@ bool drop_digits(sp2_handle_t h) {
   return any;
 }
 
+// gives back what earlier calls left and this one has not asked for (but the X_n history
+// kept for sp2_adjoint); true if there was anything
+bool drop_idle(sp2_handle_t h) {
+  bool any = false;
+  for (auto& kv : h->bufs) {
+    auto& b = kv.second;
+    if (!b.p || b.call == h->call || (h->hist.valid && kv.first.rfind("ckpt.", 0) == 0)) continue;
+    if (!any) cudaStreamSynchronize(h->stream);
+    any = true;
+    // (or the next finite-T call would grow its batches into the room that is short)
+    if (kv.first.rfind("ft.", 0) == 0) h->ft_single = true;
+    cudaFree(b.p);
+    h->held -= b.bytes;
+    b.p = nullptr;
+    b.bytes = 0;
+  }
+  return any;
+}
+
+// A buffer that the call cannot do without. Where there is no room, what earlier calls
+// left goes first (a call may leave more than it needs, padded matrices and batches, and
+// the next one must find what it would have found beside the least), then the digits.
 int ws(sp2_handle_t h, const std::string& name, size_t bytes, void** out) {
   int r = ws_try(h, name, bytes, out);
+  if (r == SP2_ENOMEM && drop_idle(h)) r = ws_try(h, name, bytes, out);
   if (r == SP2_ENOMEM && drop_digits(h)) {
     h->dig_off = true;
     r = ws_try(h, name, bytes, out);
@@ -1715,6 +1754,7 @@ size_t sp2_workspace_bytes(sp2_handle_t h) { return h ? h->held : 0; }
 
 int sp2_density(sp2_handle_t h, const void* H, int64_t N, int dtype, double nocc,
                 const sp2_opts* opts_in, void* D, sp2_info* info) {
+  CallScope scope(h);
   TRY(check_common(h, H, N, dtype, nocc));
   if (N > 0 && !D) return fail(h, SP2_EINVAL, "D is NULL");
   sp2_opts o = resolve(opts_in);
@@ -1760,6 +1800,7 @@ int sp2_density(sp2_handle_t h, const void* H, int64_t N, int dtype, double nocc
 int sp2_response(sp2_handle_t h, const void* H, int64_t N, int dtype, double nocc, const void* H1,
                  int64_t K, int h1_diag_only, const sp2_opts* opts_in, void* D, void* D1,
                  sp2_info* info) {
+  CallScope scope(h);
   TRY(check_common(h, H, N, dtype, nocc));
   if (K < 0) return fail(h, SP2_EINVAL, "K < 0");
   if (N > 0 && K > 0 && (!H1 || !D1)) return fail(h, SP2_EINVAL, "H1 or D1 is NULL");
@@ -1810,6 +1851,7 @@ int sp2_adjoint(sp2_handle_t h, const void* G, int64_t N, int dtype, void* grad,
 int sp2_susceptibility(sp2_handle_t h, const void* H, int64_t N, int dtype, double nocc,
                        const void* A, int64_t L, int a_diag_only, int direction,
                        const sp2_opts* opts_in, void* D, void* chi, sp2_info* info) {
+  CallScope scope(h);
   TRY(check_common(h, H, N, dtype, nocc));
   if (L < 0) return fail(h, SP2_EINVAL, "L < 0");
   if (direction != 0 && direction != 1) return fail(h, SP2_EINVAL, "direction must be 0 or 1");
@@ -1866,6 +1908,7 @@ int sp2_susceptibility(sp2_handle_t h, const void* H, int64_t N, int dtype, doub
 }
 
 int sp2_adjoint(sp2_handle_t h, const void* G, int64_t N, int dtype, void* grad, sp2_info* info) {
+  CallScope scope(h);
   if (!h) return SP2_EINVAL;
   if (!h->hist.valid) return fail(h, SP2_ENOSTATE, "no X_n history kept on this handle");
   if (N != h->hist.n) return fail(h, SP2_ENOSTATE, "N = %lld differs from the kept history (%lld)",
@@ -2028,7 +2071,7 @@ int fermi_batch(Ctx& c, FermiState& fs, int64_t want, int64_t* B) {
   const int64_t cap = ((int64_t)1 << 25) / (c.np * c.np);
   int64_t b = want < cap ? want : cap;
   // (under a workspace limit FP64 leaves the room to the digits of its products)
-  if (b < 1 || (h->limit && c.mode == SP2_MODE_FP64)) b = 1;
+  if (b < 1 || h->ft_single || (h->limit && c.mode == SP2_MODE_FP64)) b = 1;
   struct Buf {
     const char* name;
     FMat* f;
@@ -2144,6 +2187,7 @@ extern "C" {
 int sp2_fermi(sp2_handle_t h, const void* H, int64_t N, int dtype, double mu, double kT,
               const void* B, int64_t K, int b_diag_only, int canonical, int n_doublings,
               const sp2_opts* opts_in, void* D, void* D1, sp2_info* info) {
+  CallScope scope(h);
   if (h) drop_pending(h);   // this call completes before it returns
   if (!h) return SP2_EINVAL;
   if (N < 0 || K < 0) return fail(h, SP2_EINVAL, "negative size");
@@ -2270,6 +2314,7 @@ extern "C" {
 int sp2_nonorth_susceptibility(sp2_handle_t h, const void* H, const void* S, int64_t N, int dtype,
                                double nocc, const void* A, const sp2_opts* opts_in, void* D,
                                void* WH, void* WS, void* Zout, sp2_info* info) {
+  CallScope scope(h);
   if (h) drop_pending(h);   // this call completes before it returns
   TRY(check_common(h, H, N, dtype, nocc));
   if (N > 0 && (!S || !A || !D || !WH || !WS)) return fail(h, SP2_EINVAL, "null pointer");
@@ -2427,6 +2472,7 @@ int sp2_nonorth_susceptibility(sp2_handle_t h, const void* H, const void* S, int
 
 int response_contract(sp2_handle_t h, const void* P, int64_t L, const void* Q, int64_t K, int64_t N,
                       int dtype, int q_diag_only, double* out) {
+  CallScope scope(h);
   if (!h) return SP2_EINVAL;
   if (L < 0 || K < 0 || N < 0) return fail(h, SP2_EINVAL, "negative size");
   if (dtype != SP2_F64 && dtype != SP2_F32) return fail(h, SP2_EINVAL, "unknown dtype %d", dtype);
@@ -2549,6 +2595,7 @@ extern "C" {
 
 int sp2_mlp_forward(sp2_handle_t h, const float* W1, const float* W2, int din, int dh,
                     const float* X, int64_t P, float* Y, int bf16) {
+  CallScope scope(h);
   if (!h) return SP2_EINVAL;
   if (din <= 0 || dh <= 0 || P < 0) return fail(h, SP2_EINVAL, "bad MLP sizes");
   if (P == 0) return SP2_OK;
@@ -2563,6 +2610,7 @@ int sp2_mlp_forward(sp2_handle_t h, const float* W1, const float* W2, int din, i
 int sp2_mlp_loss_grad(sp2_handle_t h, const float* W1, const float* W2, int din, int dh,
                       const float* X, const float* T, int64_t P, double* loss, float* dW1,
                       float* dW2) {
+  CallScope scope(h);
   if (!h) return SP2_EINVAL;
   if (din <= 0 || dh <= 0 || P <= 0) return fail(h, SP2_EINVAL, "bad MLP sizes");
   if (!W1 || !W2 || !X || !T || !dW1 || !dW2 || !loss) return fail(h, SP2_EINVAL, "null pointer");
@@ -2578,6 +2626,7 @@ int sp2_mlp_loss_grad(sp2_handle_t h, const float* W1, const float* W2, int din,
 
 int sp2_mlp_train(sp2_handle_t h, float* W1, float* W2, int din, int dh, const float* X,
                   const float* T, int64_t P, int steps, double lr, double* loss_hist) {
+  CallScope scope(h);
   if (!h) return SP2_EINVAL;
   if (din <= 0 || dh <= 0 || P <= 0 || steps < 0) return fail(h, SP2_EINVAL, "bad MLP sizes");
   if (!W1 || !W2 || !X || !T) return fail(h, SP2_EINVAL, "null pointer");
@@ -2612,6 +2661,7 @@ int sp2_scf_response(sp2_handle_t h, const void* H, int64_t N, int dtype, double
                      const double* Ksite, const double* Vext, int64_t F, const sp2_scf_opts* so,
                      const sp2_opts* opts_in, double* q_out, double* residuals, int* iterations,
                      double* traj_r, double* traj_q, sp2_info* info) {
+  CallScope scope(h);
   if (h) drop_pending(h);   // this call completes before it returns
   TRY(check_common(h, H, N, dtype, nocc));
   if (!so) return fail(h, SP2_EINVAL, "null sp2_scf_opts");

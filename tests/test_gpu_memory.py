@@ -107,3 +107,17 @@ def test_batch_growth_keeps_the_digits(sp2):
     assert h.workspace_bytes() > least - mat
     ref, _, _ = sp2.sp2_fermi(H, 0.0, 0.1, B, handle=sp2.Handle(), **kw)
     assert (D1 - ref).norm() <= 1e-9 * ref.norm()
+
+
+def test_batches_leave_room_for_the_next_call(sp2):
+    """Finite-T responses by batches take free room under a limit; the density that follows
+    finds the room it would have found beside one response at a time."""
+    mode = "fp16x2"
+    Hs, Bs = _inputs(300, mode)
+    Hl, _ = _inputs(1000, mode)
+    h = sp2.Handle(LEAST[mode, 300, "fermi"] + LEAST[mode, 1000, "density"])
+    want = _call(sp2, "fermi", 300, mode, Hs, Bs, sp2.Handle())
+    dens = _call(sp2, "density", 1000, mode, Hl, None, sp2.Handle())
+    for _ in range(2):
+        assert torch.equal(_call(sp2, "fermi", 300, mode, Hs, Bs, h), want)
+        assert torch.equal(_call(sp2, "density", 1000, mode, Hl, None, h), dens)
