@@ -451,12 +451,57 @@ bool dig_mode(const Ctx& c, int64_t rows) {
          (c.np > kPad || rows >= 2 * kPad);
 }
 
-// Batch entries whose digits and sums are formed at a time (48 bytes per entry of a
-// stacked factor): at most 4 GiB of them, at least one.
-int64_t dig_chunk(int64_t np, int64_t batch) {
-  const int64_t per = 48 * np * np;
-  const int64_t m = ((int64_t)4 << 30) / per;
-  return m < 1 ? 1 : (m < batch ? m : batch);
+// The digit buffers of one product, in bytes, of a rows x np left factor (0: the square of
+// the right factor; with_x: the right factor stacked below the left one): 16 an entry of a
+// factor, and 32 of the sums for every part that the plan cuts the K axis into.
+struct DigBytes {
+  DigPlan plan;
+  size_t x = 0, xe = 0, G = 0, a = 0, ae = 0;
+};
+DigBytes dig_bytes(int64_t np, int64_t rows, bool upper, bool with_x = false) {
+  DigBytes d;
+  const int64_t left = rows + (with_x ? np : 0);   // rows of the stacked left factor
+  d.plan = dig_plan(rows ? rows : np, np, upper, with_x);
+  d.G = (size_t)(rows ? left : np) * np * 4 * kDigPlanes * d.plan.ksplit;
+  if (!with_x) d.x = (size_t)np * np * 2 * kDigPlanes, d.xe = (size_t)np * sizeof(int);
+  if (rows) d.a = (size_t)left * np * 2 * kDigPlanes, d.ae = (size_t)left * sizeof(int);
+  return d;
+}
+
+// Batch entries whose digits and sums are formed at a time: at most 4 GiB of them, at
+// least one (with_x: X_n's below them as well, 0 when that is more).
+int64_t dig_chunk(int64_t np, int64_t batch, bool with_x = false) {
+  constexpr size_t cap = (size_t)4 << 30;
+  for (int64_t m = batch; m > 0; m = m > 16 ? m - m / 16 : m - 1) {
+    const DigBytes d = dig_bytes(np, m * np, false, with_x);
+    if (d.G + d.a <= cap) return m;
+  }
+  return with_x ? 0 : 1;
+}
+
+// The buffers a call will ask for, by name.
+struct Room {
+  std::map<std::string, size_t> need;
+  void add(const std::string& name, size_t bytes) {
+    size_t& n = need[name];
+    n = std::max(n, bytes);
+  }
+  void add(const DigBytes& d) {
+    add("dig.x", d.x);
+    add("dig.xe", d.xe);
+    add("dig.G", d.G);
+    add("dig.a", d.a);
+    add("dig.ae", d.ae);
+  }
+};
+
+// digits of the FP64 steps of a recursion with `ybatch` responses and of an adjoint of `adj`
+void dig_room(Room& r, int64_t np, int64_t ybatch, int64_t adj) {
+  const int64_t bc = ybatch > 0 ? dig_chunk(np, ybatch, true) : 0;
+  if (bc == ybatch && ybatch > 0) r.add(dig_bytes(np, bc * np, false, true));
+  if (bc != ybatch) r.add(dig_bytes(np, dig_chunk(np, ybatch) * np, false));
+  if (bc != ybatch || ybatch == 0) r.add(dig_bytes(np, 0, true));
+  if (adj > 0) r.add(dig_bytes(np, dig_chunk(np, adj) * np, false));
 }
 
 struct DigBufs {
@@ -473,18 +518,16 @@ struct DigBufs {
 // as the rest of the call does.
 bool dig_bufs(Ctx& c, int64_t rows, bool upper, DigBufs* b, bool with_x = false) {
   sp2_handle_t h = c.h;
-  const int64_t left = rows + (with_x ? c.np : 0);   // rows of the stacked left factor
-  const size_t el = (size_t)c.np * c.np, ra = (size_t)left * c.np;
-  const size_t nt = rows ? ra : el;
+  const int64_t left = rows + (with_x ? c.np : 0);
   void *xd = nullptr, *xe = nullptr, *G, *ad = nullptr, *ae = nullptr;
-  b->plan = dig_plan(rows ? rows : c.np, c.np, upper, with_x);
+  const DigBytes n = dig_bytes(c.np, rows, upper, with_x);
+  b->plan = n.plan;
   const void* old_x = h->bufs["dig.x"].p;
-  bool ok = (with_x || (ws_try(h, "dig.x", el * 2 * kDigPlanes, &xd) == SP2_OK &&
-                        ws_try(h, "dig.xe", (size_t)c.np * sizeof(int), &xe) == SP2_OK)) &&
-            ws_try(h, "dig.G", nt * 4 * kDigPlanes * b->plan.ksplit, &G) == SP2_OK;
+  bool ok = (with_x || (ws_try(h, "dig.x", n.x, &xd) == SP2_OK &&
+                        ws_try(h, "dig.xe", n.xe, &xe) == SP2_OK)) &&
+            ws_try(h, "dig.G", n.G, &G) == SP2_OK;
   if (ok && rows)
-    ok = ws_try(h, "dig.a", ra * 2 * kDigPlanes, &ad) == SP2_OK &&
-         ws_try(h, "dig.ae", (size_t)left * sizeof(int), &ae) == SP2_OK;
+    ok = ws_try(h, "dig.a", n.a, &ad) == SP2_OK && ws_try(h, "dig.ae", n.ae, &ae) == SP2_OK;
   if (ok)
     ok = tile_list(h, c.mode, rows ? left : c.np, c.np, upper, &b->tiles, &b->ntiles, 256, b->plan.bn,
                    with_x ? rows : -1) == SP2_OK;
@@ -523,7 +566,7 @@ int dig_step(Ctx& c, const MatBuf& xin, const MatBuf& xout, const MatBuf& yin, c
   sp2_handle_t h = c.h;
   const int64_t rows = batch * c.np;
   DigBufs db;
-  if (!dig_mode(c, rows + c.np) || h->dig_apart || dig_chunk(c.np, batch + 1) <= batch) return SP2_OK;
+  if (!dig_mode(c, rows + c.np) || h->dig_apart || dig_chunk(c.np, batch, true) < batch) return SP2_OK;
   if (!dig_bufs(c, rows, false, &db, true)) return SP2_OK;
   SimtDecide sd = decide_args(c, *dec);
   sd.p.nparts = (int)dig_square_nparts(c.np);
@@ -880,18 +923,24 @@ int resolve_ckpt(sp2_handle_t h, sp2_opts* o, int64_t np, int64_t batch) {
   const double ms = (double)master_size(o->mode), mat_b = el * (ms + 2.0 * n_planes(o->mode));
   const double b = (double)(batch > 0 ? batch : 1);
   avail -= 2.0 * mat_b + 2.0 * b * mat_b + b * el * ms + (double)(1ull << 30);
-  if (o->mode == SP2_MODE_FP64 && np % kPad == 0)   // digit buffers
-    avail -= el * (16.0 + 48.0 * (double)dig_chunk(np, batch > 0 ? batch + 1 : 1));
   const int cap = o->fixed_m > 0 ? o->fixed_m : o->max_iter;
-  int k = cap;
-  for (int kk = 1; kk <= cap; ++kk) {
-    const double need = (double)((cap + kk - 1) / kk) * el * ms + (double)(kk - 1) * mat_b;
-    if (need <= avail) {
-      k = kk;
-      break;
-    }
+  auto interval = [&](double room) {   // 0: none fits
+    for (int kk = 1; kk <= cap; ++kk)
+      if ((double)((cap + kk - 1) / kk) * el * ms + (double)(kk - 1) * mat_b <= room) return kk;
+    return 0;
+  };
+  int k = 0;
+  if (o->mode == SP2_MODE_FP64 && np % kPad == 0) {
+    // beside the digit buffers if possible (an interval above 1 costs one square per step,
+    // whatever its length; FP64 products on the CUDA cores many times more)
+    Room r;
+    dig_room(r, np, 0, batch > 0 ? batch : 1);
+    double digits = 0.0;
+    for (auto& kv : r.need) digits += (double)kv.second;
+    k = interval(avail - digits);
   }
-  o->ckpt_k = k;
+  if (k == 0) k = interval(avail);
+  o->ckpt_k = k ? k : cap;
   return SP2_OK;
 }
 

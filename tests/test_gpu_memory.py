@@ -121,3 +121,21 @@ def test_batches_leave_room_for_the_next_call(sp2):
     for _ in range(2):
         assert torch.equal(_call(sp2, "fermi", 300, mode, Hs, Bs, h), want)
         assert torch.equal(_call(sp2, "density", 1000, mode, Hl, None, h), dens)
+
+
+def test_history_leaves_room_for_the_digits(sp2):
+    """From K = 8193 on the sums of a product come in parts along K, two or three here, of 32
+    bytes an entry each: the automatic checkpoint interval counts them (by one part it would
+    choose the interval 1, and 2 + 9 + 2 matrices beside 16 of digits and sums do not fit)."""
+    n = 8300
+    mat = 8 * 8448 * 8448
+    g = torch.Generator(device="cuda").manual_seed(0)
+    H = torch.randn(n, n, generator=g, device="cuda", dtype=torch.float64)
+    H = (H + H.T) * 0.002
+    b = torch.ones(1, n, device="cuda", dtype=torch.float64)
+    h = sp2.Handle(27 * mat + (1 << 30))
+    chi, _, info = sp2.sp2_susceptibility(H, n // 2, b, direction="backward", diag_only=True, mode="fp64",
+                                          sigma=[1, -1] * 4 + [1], bounds=(-1.0, 1.0), ckpt_k="auto",
+                                          handle=h, allow_noconv=True)
+    assert info["ckpt_k"] > 1 and bool(torch.isfinite(chi).all())
+    assert h.workspace_bytes() > 18 * mat      # without the digits: 9 to 14 of them
