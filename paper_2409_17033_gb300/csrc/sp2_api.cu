@@ -42,7 +42,9 @@ struct sp2_handle_s {
   std::map<std::string, Buf> bufs;
   unsigned long long call = 0;     // calls so far (CallScope)
   int depth = 0;
+  bool narrow = false;             // this call pads FP64 matrices to 64 (pick_np)
   bool ft_single = false;          // room was short: finite-T responses one at a time
+  size_t fit_extra = 0;            // device memory found free for a call (pick_np)
   struct TileList {
     Tile* d = nullptr;
     int n = 0;
@@ -117,7 +119,10 @@ int fail(sp2_handle_t h, int code, const char* fmt, ...) {
 struct CallScope {
   sp2_handle_t h;
   explicit CallScope(sp2_handle_t hh) : h(hh) {
-    if (h && h->depth++ == 0) ++h->call;
+    if (h && h->depth++ == 0) {
+      ++h->call;
+      h->narrow = false;
+    }
   }
   ~CallScope() {
     if (h) --h->depth;
@@ -479,7 +484,7 @@ int64_t dig_chunk(int64_t np, int64_t batch, bool with_x = false) {
   return with_x ? 0 : 1;
 }
 
-// The buffers a call will ask for, by name.
+// The buffers a call will ask for: at most how many bytes more than the handle holds.
 struct Room {
   std::map<std::string, size_t> need;
   void add(const std::string& name, size_t bytes) {
@@ -492,6 +497,15 @@ struct Room {
     add("dig.G", d.G);
     add("dig.a", d.a);
     add("dig.ae", d.ae);
+  }
+  size_t extra(sp2_handle_t h) const {
+    size_t e = 0;
+    for (auto& kv : need) {
+      auto it = h->bufs.find(kv.first);
+      const size_t have = it == h->bufs.end() ? 0 : it->second.bytes;
+      if (kv.second > have) e += kv.second - have;
+    }
+    return e;
   }
 };
 
@@ -941,6 +955,51 @@ int resolve_ckpt(sp2_handle_t h, sp2_opts* o, int64_t np, int64_t batch) {
   }
   if (k == 0) k = interval(avail);
   o->ckpt_k = k ? k : cap;
+  return SP2_OK;
+}
+
+// The padded size of an FP64 call. From kDigMinN on products run by digits, on matrices
+// padded to 256; where that padding and the digits do not certainly fit beside what the
+// handle holds (N = 300 takes 2.6 times the memory of a padding to 64, and the CUDA cores
+// 4.1 times its work), to 64. room(np, Room&): the most the call may ask for.
+template <typename F>
+int pick_np(sp2_handle_t h, int64_t n, int mode, F room, int64_t* np) {
+  *np = pad_n(n, mode);
+  const int64_t least = (n + 63) / 64 * 64;
+  if (mode != SP2_MODE_FP64 || *np == least) return SP2_OK;
+  if (!h->narrow) {
+    Room r;
+    TRY(room(*np, r));
+    const size_t extra = r.extra(h);
+    h->narrow = h->limit && h->held + extra > h->limit;
+    if (!h->narrow && extra > h->fit_extra) {
+      size_t fr = 0, tot = 0;
+      CK(cudaMemGetInfo(&fr, &tot));
+      h->narrow = extra + extra / 8 + ((size_t)64 << 20) > fr;
+      if (!h->narrow) h->fit_extra = extra;
+    }
+  }
+  if (h->narrow) *np = least;
+  return SP2_OK;
+}
+
+// FP64 buffers of a recursion with `ybatch` responses, and with `adj` > 0 those of its
+// history and an adjoint of that many matrices
+int sp2_room(sp2_handle_t h, Room& r, sp2_opts o, int64_t np, int64_t ybatch, int64_t adj) {
+  const size_t el = (size_t)np * np * sizeof(double);
+  const int cap = o.fixed_m > 0 ? o.fixed_m : o.max_iter;
+  for (const char* x : {"X0.m", "X1.m", "Xbest.m"}) r.add(x, el);
+  for (const char* y : {"Y0.m", "Y1.m", "Ybest.m"})
+    if (ybatch > 0) r.add(y, (size_t)ybatch * el);
+  if (adj > 0) {
+    TRY(resolve_ckpt(h, &o, np, adj));
+    for (int i = 0; i < (cap + o.ckpt_k - 1) / o.ckpt_k; ++i) r.add("ckpt." + std::to_string(i), el);
+    for (int i = 1; i < o.ckpt_k; ++i) r.add("seg." + std::to_string(i) + ".m", el);
+    r.add("G0.m", (size_t)adj * el);
+    r.add("G1.m", (size_t)adj * el);
+  }
+  dig_room(r, np, ybatch, adj);
+  r.add("call", (size_t)1 << 16);   // bounds and other small buffers
   return SP2_OK;
 }
 
@@ -1818,12 +1877,13 @@ int sp2_density(sp2_handle_t h, const void* H, int64_t N, int dtype, double nocc
   TRY(stage_in(h, "H", H, mb, &Hd));
   OutStage od;
   TRY(stage_out(h, "D", D, mb, &od));
-  const int64_t np = pad_n(N, o.mode);
+  const bool keep = o.keep_history != 0;
+  int64_t np;
+  TRY(pick_np(h, N, o.mode, [&](int64_t w, Room& q) { return sp2_room(h, q, o, w, 0, keep ? 1 : 0); }, &np));
   Ctx c;
   TRY(make_ctx(h, o.mode, N, np, o.time_kernels != 0, &c));
   MatBuf X[2], Y[2];
   Sp2Out r;
-  const bool keep = o.keep_history != 0;
   if (keep) {
     h->hist.valid = false;
     TRY(resolve_ckpt(h, &o, np, 1));
@@ -1868,7 +1928,8 @@ int sp2_response(sp2_handle_t h, const void* H, int64_t N, int dtype, double noc
   OutStage od, oy;
   if (D) TRY(stage_out(h, "D", D, mb, &od));
   if (K > 0) TRY(stage_out(h, "Y", D1, (size_t)K * mb, &oy));
-  const int64_t np = pad_n(N, o.mode);
+  int64_t np;
+  TRY(pick_np(h, N, o.mode, [&](int64_t w, Room& q) { return sp2_room(h, q, o, w, K, 0); }, &np));
   Ctx c;
   TRY(make_ctx(h, o.mode, N, np, o.time_kernels != 0, &c));
   MatBuf X[2], Y[2];
@@ -1923,12 +1984,14 @@ int sp2_susceptibility(sp2_handle_t h, const void* H, int64_t N, int dtype, doub
   OutStage od, oy;
   if (D) TRY(stage_out(h, "D", D, mb, &od));
   if (L > 0) TRY(stage_out(h, "Y", chi, (size_t)L * mb, &oy));
-  const int64_t np = pad_n(N, o.mode);
+  h->hist.valid = false;
+  int64_t np;
+  TRY(pick_np(h, N, o.mode,
+              [&](int64_t w, Room& q) { return sp2_room(h, q, o, w, 0, L > 0 ? L : 1); }, &np));
   Ctx c;
   TRY(make_ctx(h, o.mode, N, np, o.time_kernels != 0, &c));
   MatBuf X[2], Y[2];
   Sp2Out r;
-  h->hist.valid = false;
   TRY(resolve_ckpt(h, &o, np, L));
   TRY(run_sp2(h, Hd, N, dtype, nocc, o, nullptr, 0, 0, true, X, Y, c, &r));
   if (D) {
@@ -2109,6 +2172,19 @@ int fermi_setup(Ctx& c, FermiState& fs, const void* Hd, int64_t N, int dtype, do
   return SP2_OK;
 }
 
+// FP64 buffers of fermi_setup and of one response at a time
+void fermi_room(Room& r, int64_t np, int n, bool canonical, bool responses) {
+  const size_t el = (size_t)np * np * sizeof(double);
+  for (int j = 0; j <= n; ++j) r.add("ft.d" + std::to_string(j) + ".m", el);
+  for (int j = 0; j < n; ++j) r.add("ft.W" + std::to_string(j) + ".m", el);
+  for (const char* x : {"ft.P.m", "ft.S.m", "ft.T.m", "ft.U.m", "ft.Z0.m", "ft.Z1.m"}) r.add(x, el);
+  for (const char* x : {"ft.dd0.m", "ft.dd1.m", "ft.E.m", "ft.F1.m", "ft.dW.m", "ft.G1.m"})
+    if (responses) r.add(x, el);
+  if (responses && canonical) r.add("ft.RI.m", el);
+  r.add(dig_bytes(np, np, false));
+  r.add("call", ((size_t)1 << 16) + (size_t)np * 8);
+}
+
 // Scratch for batches of up to `want` responses; *B: how many fit. A batch shares each
 // product's launch (one 2048 x 2048 product keeps 64 of 76 CTA pairs busy for one tile:
 // 42 us) and the launches of the passes between them: 4 perturbations at N = 2048,
@@ -2253,7 +2329,6 @@ int sp2_fermi(sp2_handle_t h, const void* H, int64_t N, int dtype, double mu, do
     return SP2_OK;
   }
   const int mode = o.mode;
-  const int64_t np = pad_n(N, mode);
   const size_t mb = (size_t)N * N * dsize(dtype);
   const void *Hd, *Bd = nullptr;
   TRY(stage_in(h, "H", H, mb, &Hd));
@@ -2261,6 +2336,11 @@ int sp2_fermi(sp2_handle_t h, const void* H, int64_t N, int dtype, double mu, do
   OutStage od, oy;
   if (D) TRY(stage_out(h, "D", D, mb, &od));
   if (K > 0) TRY(stage_out(h, "Y", D1, (size_t)K * mb, &oy));
+  int64_t np;
+  TRY(pick_np(h, N, mode, [&](int64_t w, Room& q) {
+    fermi_room(q, w, n_doublings, canonical != 0, K > 0);
+    return SP2_OK;
+  }, &np));
   Ctx c;
   TRY(make_ctx(h, mode, N, np, o.time_kernels != 0, &c));
   FermiState fs;
@@ -2377,7 +2457,6 @@ int sp2_nonorth_susceptibility(sp2_handle_t h, const void* H, const void* S, int
     return SP2_OK;
   }
   const int mode = o.mode;
-  const int64_t np = pad_n(N, mode);
   const size_t mb = (size_t)N * N * dsize(dtype);
   const void *Hd, *Sd, *Ad;
   TRY(stage_in(h, "H", H, mb, &Hd));
@@ -2388,6 +2467,16 @@ int sp2_nonorth_susceptibility(sp2_handle_t h, const void* H, const void* S, int
   TRY(stage_out(h, "no.WH", WH, mb, &oh));
   TRY(stage_out(h, "no.WS", WS, mb, &os));
   if (Zout) TRY(stage_out(h, "no.Z", Zout, mb, &oz));
+  int64_t np;
+  TRY(pick_np(h, N, mode, [&](int64_t w, Room& q) {
+    const size_t el = (size_t)w * w * sizeof(double);
+    for (const char* x : {"Y", "Zk", "T", "P", "Q", "Q2", "Z", "Sinv", "H", "A", "Hp", "Ap", "Dp", "Cp",
+                          "Dm", "Wh", "Ws"})
+      q.add(std::string("no.") + x + ".m", el);
+    for (const char* x : {"no.Hpn", "no.Apn", "no.Dpn", "no.Cpn"}) q.add(x, mb);
+    q.add(dig_bytes(w, w, false));
+    return sp2_room(h, q, o, w, 0, 1);
+  }, &np));
   Ctx c;
   TRY(make_ctx(h, mode, N, np, o.time_kernels != 0, &c));
   CK(cudaMemsetAsync(h->d_state, 0, sizeof(DevState), h->stream));

@@ -56,6 +56,10 @@ LEAST = {
             chi_k1=11824932, fermi=11215840, adjoint=5336868).items()},
     **{("fp64", 256, k): v for k, v in dict(density=1583300, response=7874756, chi=11041284,
             chi_k1=22051332, fermi=19935440, adjoint=9468420).items()},
+    **{("fp64", 300, k): v for k, v in dict(density=2472196, response=12302596, chi=17238596,
+            chi_k1=34441796, fermi=31146608, adjoint=14780996).items()},
+    **{("fp64", 520, k): v for k, v in dict(density=8002244, response=39852740, chi=58452996,
+            chi_k1=116845572, fermi=100903696, adjoint=50490372).items()},
     **{("fp32", 300, k): v for k, v in dict(density=1783492, response=8861380, chi=13600772,
             chi_k1=28936196, fermi=22428544, adjoint=11831300).items()},
     **{("fp32", 1000, k): v for k, v in dict(density=12623492, response=62955140, chi=96530372,
@@ -84,6 +88,40 @@ def test_least_limit_is_enough(sp2, mode, n, name):
         assert torch.equal(got, free)
 
 
+def test_wide_fp64_padding_needs_its_room(sp2):
+    """Matrices of N = 300 are padded for the digits without a limit or under one with room
+    for them, to 64 otherwise, and a call gives back nothing that another still needs."""
+    n = 300
+    H, B = _inputs(n, "fp64")
+    wide, tight = sp2.Handle(64 << 20), sp2.Handle(16 << 20)
+    d1, d2 = (_call(sp2, "density", n, "fp64", H, B, h) for h in (wide, tight))
+    assert (d1 - d2).norm() <= 1e-10 * d1.norm()
+    assert wide.workspace_bytes() > 16 * 512 * 512 + 3 * 8 * 512 * 512
+    assert tight.workspace_bytes() < 4 * 8 * 320 * 320
+    # a kept history outlives calls that are short of room
+    sp2.sp2_density(H, n // 2, mode="fp64", keep_history=True, handle=tight, idem_tol=1e-10)
+    want = sp2.sp2_adjoint(B[0].contiguous(), tight)
+    try:
+        sp2.sp2_density(_inputs(700, "fp32")[0], 350, mode="fp32", handle=tight)
+    except sp2.SP2Error:
+        pass
+    assert torch.equal(sp2.sp2_adjoint(B[0].contiguous(), tight), want)
+
+
+def test_batches_leave_room_for_the_next_call(sp2):
+    """Finite-T responses by batches take free room under a limit; the density that follows
+    finds the room it would have found beside one response at a time."""
+    mode = "fp16x2"
+    Hs, Bs = _inputs(300, mode)
+    Hl, _ = _inputs(1000, mode)
+    h = sp2.Handle(LEAST[mode, 300, "fermi"] + LEAST[mode, 1000, "density"])
+    want = _call(sp2, "fermi", 300, mode, Hs, Bs, sp2.Handle())
+    dens = _call(sp2, "density", 1000, mode, Hl, None, sp2.Handle())
+    for _ in range(2):
+        assert torch.equal(_call(sp2, "fermi", 300, mode, Hs, Bs, h), want)
+        assert torch.equal(_call(sp2, "density", 1000, mode, Hl, None, h), dens)
+
+
 def test_batch_growth_keeps_the_digits(sp2):
     """FP64 finite-T responses on a GPU that is nearly full: the scratch of a larger batch
     does not fit, and the products keep their digit buffers."""
@@ -107,20 +145,6 @@ def test_batch_growth_keeps_the_digits(sp2):
     assert h.workspace_bytes() > least - mat
     ref, _, _ = sp2.sp2_fermi(H, 0.0, 0.1, B, handle=sp2.Handle(), **kw)
     assert (D1 - ref).norm() <= 1e-9 * ref.norm()
-
-
-def test_batches_leave_room_for_the_next_call(sp2):
-    """Finite-T responses by batches take free room under a limit; the density that follows
-    finds the room it would have found beside one response at a time."""
-    mode = "fp16x2"
-    Hs, Bs = _inputs(300, mode)
-    Hl, _ = _inputs(1000, mode)
-    h = sp2.Handle(LEAST[mode, 300, "fermi"] + LEAST[mode, 1000, "density"])
-    want = _call(sp2, "fermi", 300, mode, Hs, Bs, sp2.Handle())
-    dens = _call(sp2, "density", 1000, mode, Hl, None, sp2.Handle())
-    for _ in range(2):
-        assert torch.equal(_call(sp2, "fermi", 300, mode, Hs, Bs, h), want)
-        assert torch.equal(_call(sp2, "density", 1000, mode, Hl, None, h), dens)
 
 
 def test_history_leaves_room_for_the_digits(sp2):
