@@ -69,7 +69,7 @@ struct sp2_handle_s {
   unsigned long long run_id = 0;    // recursions run on this handle (part of the tokens)
   // side stream for host copies that overlap later work of the same call
   cudaStream_t side = nullptr;
-  cudaEvent_t side_ev[2] = {};
+  cudaEvent_t side_ev[3] = {};
   bool side_pending = false;
   std::vector<cudaEvent_t> events;  // pool for time_kernels (start/stop pairs)
 
@@ -298,16 +298,20 @@ int finish_out(sp2_handle_t h, const OutStage& o) {
   return SP2_OK;
 }
 
+int side_stream(sp2_handle_t h) {
+  if (h->side) return SP2_OK;
+  for (cudaEvent_t& e : h->side_ev)
+    if (!e) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+  CK(cudaStreamCreateWithFlags(&h->side, cudaStreamNonBlocking));
+  return SP2_OK;
+}
+
 // The host copy of an output that is final while later work of the call still
 // runs: on the handle's side stream, after what the main stream has enqueued so
 // far; join_beside makes the main stream wait for it.
 int finish_out_beside(sp2_handle_t h, const OutStage& o) {
   if (!o.host) return SP2_OK;
-  if (!h->side) {
-    CK(cudaStreamCreateWithFlags(&h->side, cudaStreamNonBlocking));
-    CK(cudaEventCreateWithFlags(&h->side_ev[0], cudaEventDisableTiming));
-    CK(cudaEventCreateWithFlags(&h->side_ev[1], cudaEventDisableTiming));
-  }
+  TRY(side_stream(h));
   CK(cudaEventRecord(h->side_ev[0], h->stream));
   CK(cudaStreamWaitEvent(h->side, h->side_ev[0], 0));
   CK(cudaMemcpyAsync(o.user, o.dev, o.bytes, cudaMemcpyDeviceToHost, h->side));
@@ -1065,12 +1069,15 @@ void ring_slot(sp2_handle_t h, int step, DecideParams* dp) {
 
 // Wait for the word of `step`; *out stays null while the recursion goes on, else it is
 // the snapshot of its end. Words are read in step order, none past the end (a
-// stopped recursion's later decisions may not run). When the stream has drained
-// without it (an aborted product never reached its decision), the state itself is
-// read.
+// stopped recursion's later decisions may not run). When the work enqueued so far has
+// ended without it (an aborted product never reached its decision), the state itself is
+// read. A wait that lasts marks the end of that work by an event, and the state comes over
+// the side stream: the stream may have other users, who need never leave it idle.
 int ring_read(sp2_handle_t h, int step, const HostSnap** out) {
   HostSnap* s = h->ring + step % sp2_handle_s::kRing;
   const unsigned long long token = h->run_id * 1024ull + (unsigned long long)step;
+  constexpr int kPatience = 64;   // polls (a millisecond or more) before the event
+  int polls = 0;
   *out = nullptr;
   for (unsigned it = 1;; ++it) {
     const unsigned long long w = __atomic_load_n(&s->word, __ATOMIC_ACQUIRE);
@@ -1079,7 +1086,12 @@ int ring_read(sp2_handle_t h, int step, const HostSnap** out) {
       return SP2_OK;
     }
     if (it % 16384 != 0) continue;
-    const cudaError_t e = cudaStreamQuery(h->stream);
+    if (++polls == kPatience) {
+      TRY(side_stream(h));
+      CK(cudaEventRecord(h->side_ev[2], h->stream));
+    }
+    const cudaError_t e =
+        polls < kPatience ? cudaStreamQuery(h->stream) : cudaEventQuery(h->side_ev[2]);
     if (e == cudaErrorNotReady) {
       cudaGetLastError();
       std::this_thread::yield();
@@ -1087,8 +1099,9 @@ int ring_read(sp2_handle_t h, int step, const HostSnap** out) {
     }
     CK(e);
     if (__atomic_load_n(&s->word, __ATOMIC_ACQUIRE) >> 1 == token) continue;
-    CK(cudaMemcpyAsync(h->h_state, h->d_state, sizeof(DevState), cudaMemcpyDeviceToHost, h->stream));
-    CK(cudaStreamSynchronize(h->stream));
+    TRY(side_stream(h));
+    CK(cudaMemcpyAsync(h->h_state, h->d_state, sizeof(DevState), cudaMemcpyDeviceToHost, h->side));
+    CK(cudaStreamSynchronize(h->side));
     const DevState& d = *h->h_state;
     h->late = HostSnap{2ull * token + 1ull, d.stop_at, d.nonfinite, d.abort_flag, d.backtracked,
                        d.stop_step, 0, {d.bounds[0], d.bounds[1]}, d.alpha, d.beta, d.work_kblocks};
@@ -1814,9 +1827,9 @@ int sp2_destroy(sp2_handle_t h) {
   if (h->side) {
     cudaStreamSynchronize(h->side);
     cudaStreamDestroy(h->side);
-    cudaEventDestroy(h->side_ev[0]);
-    cudaEventDestroy(h->side_ev[1]);
   }
+  for (cudaEvent_t e : h->side_ev)
+    if (e) cudaEventDestroy(e);
   for (auto e : h->events) cudaEventDestroy(e);
   delete h->pending;
   delete h;
