@@ -460,7 +460,8 @@ def run_ours(args, ws, rank):
             line["plain_fp64"] = {"ms_per_solve_extrapolated": est,
                                   "tflops_effective": lflops / (est * 1e-3) / 1e12,
                                   "square_ms": sq_ms, "response_product_ms": y_ms,
-                                  "note": "FP64 CUDA-core products, per-product event times x product count"}
+                                  "note": "FP64 products by digits on the tensor cores (digits, product and "
+                                          "the pass over its sums), per-product event times x product count"}
             line["speedup_vs_plain_fp64"] = est / ms
         except Exception as ex:
             line["plain_fp64"] = {"error": str(ex)}

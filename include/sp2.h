@@ -163,7 +163,9 @@ typedef struct {
                           set, so X_n is recomputed only when the history outgrows HBM. */
   int keep_history;    /* sp2_density: keep the X_n checkpoints for a later sp2_adjoint */
   int time_kernels;    /* 1: bracket every product-kernel launch with CUDA events on the
-                          handle's stream and report their summed duration in sp2_info */
+                          handle's stream and report their summed duration in sp2_info
+                          (FP64 products by digits: with the passes that form the digits and
+                          turn the sums into the result, the response's update among them) */
   double tail_f;       /* split modes, > 0: split-tail arithmetic (the mixed-precision use the
                           paper suggests in Sec. VI.B: low precision in the bulk of the
                           iterations, higher precision in the last ones). Step n uses the hi

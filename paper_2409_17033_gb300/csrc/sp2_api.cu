@@ -413,6 +413,22 @@ int ev_pair(Ctx& c, cudaEvent_t* a, cudaEvent_t* b) {
   return SP2_OK;
 }
 
+// with c.timing: the events around one product of `step`
+int time_from(Ctx& c, cudaEvent_t* a, cudaEvent_t* b) {
+  sp2_handle_t h = c.h;
+  if (!c.timing) return SP2_OK;
+  TRY(ev_pair(c, a, b));
+  CK(cudaEventRecord(*a, h->stream));
+  return SP2_OK;
+}
+int time_to(Ctx& c, cudaEvent_t b, int step) {
+  sp2_handle_t h = c.h;
+  if (!c.timing) return SP2_OK;
+  CK(cudaEventRecord(b, h->stream));
+  c.timed.push_back({step, 0});
+  return SP2_OK;
+}
+
 // summed duration of the timed product launches of steps <= m
 double timed_ms(Ctx& c, int m) {
   double tot = 0.0;
@@ -590,20 +606,14 @@ int dig_step(Ctx& c, const MatBuf& xin, const MatBuf& xout, const MatBuf& yin, c
   sd.p.nparts = (int)dig_square_nparts(c.np);
   const double *x = static_cast<const double*>(xin.master), *y = static_cast<const double*>(yin.master);
   const int64_t left = rows + c.np;
-  CK(launch_digits(y, rows, x, c.np, c.np, db.a, c.st, step, h->stream));
   cudaEvent_t e0 = nullptr, e1 = nullptr;
-  if (c.timing) {
-    TRY(ev_pair(c, &e0, &e1));
-    CK(cudaEventRecord(e0, h->stream));
-  }
+  TRY(time_from(c, &e0, &e1));
+  CK(launch_digits(y, rows, x, c.np, c.np, db.a, c.st, step, h->stream));
   CK(launch_gemm_dig(db.a, left, db.x, c.np, db.G, db.tiles, db.ntiles, db.plan, c.st, step, h->tune,
                      h->stream));
-  if (c.timing) {
-    CK(cudaEventRecord(e1, h->stream));
-    c.timed.push_back({step, 0});
-  }
   CK(launch_dig_step(db.G, db.plan.ksplit, batch, db.a.ex, y, static_cast<double*>(yout.master), x,
                      static_cast<double*>(xout.master), c.np, c.st, step, c.part, &sd, h->stream));
+  TRY(time_to(c, e1, step));
   c.launches++;
   c.kernels += 3;
   c.flops += dig_flops(c, db);
@@ -625,25 +635,19 @@ int square_step(Ctx& c, const MatBuf& xin, const MatBuf& xout, int step,
     sd.p.nparts = (int)dig_square_nparts(c.np);
     if (dig_bufs(c, 0, true, &db)) {
       const double* x = static_cast<const double*>(xin.master);
+      cudaEvent_t e0 = nullptr, e1 = nullptr;
+      TRY(time_from(c, &e0, &e1));
       // (the response product of this step has left X_n's digits)
       if (h->dig_x != xin.master) {
         CK(launch_digits(x, c.np, nullptr, 0, c.np, db.x, c.st, step, h->stream));
         c.kernels++;
       }
       h->dig_x = nullptr;
-      cudaEvent_t e0 = nullptr, e1 = nullptr;
-      if (c.timing) {
-        TRY(ev_pair(c, &e0, &e1));
-        CK(cudaEventRecord(e0, h->stream));
-      }
       CK(launch_gemm_dig(db.x, c.np, db.x, c.np, db.G, db.tiles, db.ntiles, db.plan, c.st, step,
                          h->tune, h->stream));
-      if (c.timing) {
-        CK(cudaEventRecord(e1, h->stream));
-        c.timed.push_back({step, 0});
-      }
       CK(launch_dig_square(db.G, db.plan.ksplit, db.x.ex, x, static_cast<double*>(xout.master), c.np, c.st, step,
                            c.part, dec ? &sd : nullptr, h->stream));
+      TRY(time_to(c, e1, step));
       c.launches++;
       c.kernels += 2;
       c.flops += dig_flops(c, db);
@@ -781,6 +785,8 @@ int response_step(Ctx& c, const MatBuf& x, const MatBuf& yin, const MatBuf& yout
     if (dig_bufs(c, bc * c.np, false, &db)) {
       const double* y = static_cast<const double*>(yin.master);
       double* yo = static_cast<double*>(yout.master);
+      cudaEvent_t e0 = nullptr, e1 = nullptr;
+      TRY(time_from(c, &e0, &e1));
       CK(launch_digits(static_cast<const double*>(x.master), c.np, nullptr, 0, c.np, db.x, c.st, step,
                        h->stream));
       h->dig_x = x.master;
@@ -795,20 +801,13 @@ int response_step(Ctx& c, const MatBuf& x, const MatBuf& yin, const MatBuf& yout
           db.plan.kseg = kseg;
           TRY(tile_list(h, c.mode, r, c.np, false, &db.tiles, &db.ntiles, 256, db.plan.bn));
         }
+        if (b0 > 0) TRY(time_from(c, &e0, &e1));
         CK(launch_digits(y + off, r, nullptr, 0, c.np, db.a, c.st, step, h->stream));
-        cudaEvent_t e0 = nullptr, e1 = nullptr;
-        if (c.timing) {
-          TRY(ev_pair(c, &e0, &e1));
-          CK(cudaEventRecord(e0, h->stream));
-        }
         CK(launch_gemm_dig(db.a, r, db.x, c.np, db.G, db.tiles, db.ntiles, db.plan, c.st, step,
                            h->tune, h->stream));
-        if (c.timing) {
-          CK(cudaEventRecord(e1, h->stream));
-          c.timed.push_back({step, 0});
-        }
         CK(launch_dig_symm(db.G, db.plan.ksplit, r, db.a.ex, db.x.ex, y + off, yo + off, c.np, c.st, step,
                            h->stream));
+        TRY(time_to(c, e1, step));
         c.launches++;
         c.kernels += 3;
         c.flops += dig_flops(c, db);
@@ -1661,24 +1660,18 @@ int fprod(Ctx& c, FMat& C, const FMat& L, const FMat& R, bool trans = false) {
   const int64_t rows = L.B * c.np;
   if (dig_mode(c, rows) && dig_bufs(c, same ? 0 : rows, false, &db)) {
     const double* l = static_cast<const double*>(L.m.master);
+    cudaEvent_t e0 = nullptr, e1 = nullptr;
+    TRY(time_from(c, &e0, &e1));
     CK(launch_digits(l, rows, nullptr, 0, c.np, db.a, c.st, 0, h->stream));
     if (!same)
       CK(launch_digits(static_cast<const double*>(R.m.master), c.np, nullptr, 0, c.np, db.x, c.st, 0,
                        h->stream));
     h->dig_x = nullptr;
-    cudaEvent_t e0 = nullptr, e1 = nullptr;
-    if (c.timing) {
-      TRY(ev_pair(c, &e0, &e1));
-      CK(cudaEventRecord(e0, h->stream));
-    }
     CK(launch_gemm_dig(db.a, rows, db.x, c.np, db.G, db.tiles, db.ntiles, db.plan, c.st, 0, h->tune,
                        h->stream));
-    if (c.timing) {
-      CK(cudaEventRecord(e1, h->stream));
-      c.timed.push_back({0, 0});
-    }
     CK(launch_dig_plain(db.G, db.plan.ksplit, rows, db.a.ex, db.x.ex, static_cast<double*>(C.m.master), c.np, c.st,
                         0, h->stream));
+    TRY(time_to(c, e1, 0));
     c.launches++;
     c.kernels += same ? 3 : 4;
     c.flops += dig_flops(c, db);
