@@ -43,6 +43,7 @@ struct sp2_handle_s {
   unsigned long long call = 0;     // calls so far (CallScope)
   int depth = 0;
   bool narrow = false;             // this call pads FP64 matrices to 64 (pick_np)
+  int64_t narrow_n = 0;            // the size whose history did not fit otherwise
   bool ft_single = false;          // room was short: finite-T responses one at a time
   size_t fit_extra = 0;            // device memory found free for a call (pick_np)
   struct TileList {
@@ -504,7 +505,8 @@ int64_t dig_chunk(int64_t np, int64_t batch, bool with_x = false) {
   return with_x ? 0 : 1;
 }
 
-// The buffers a call will ask for: at most how many bytes more than the handle holds.
+// The large buffers a call will ask for, and how many bytes more than the handle holds they
+// take (what else it asks for, some KB, has a place in that of the digits).
 struct Room {
   std::map<std::string, size_t> need;
   void add(const std::string& name, size_t bytes) {
@@ -961,48 +963,73 @@ int resolve_ckpt(sp2_handle_t h, sp2_opts* o, int64_t np, int64_t batch) {
   return SP2_OK;
 }
 
-// The padded size of an FP64 call. From kDigMinN on products run by digits, on matrices
-// padded to 256; where that padding and the digits do not certainly fit beside what the
-// handle holds (N = 300 takes 2.6 times the memory of a padding to 64, and the CUDA cores
-// 4.1 times its work), to 64. room(np, Room&): the most the call may ask for.
-template <typename F>
-int pick_np(sp2_handle_t h, int64_t n, int mode, F room, int64_t* np) {
-  *np = pad_n(n, mode);
-  const int64_t least = (n + 63) / 64 * 64;
-  if (mode != SP2_MODE_FP64 || *np == least) return SP2_OK;
-  if (!h->narrow) {
-    Room r;
-    TRY(room(*np, r));
-    const size_t extra = r.extra(h);
-    h->narrow = h->limit && h->held + extra > h->limit;
-    if (!h->narrow && extra > h->fit_extra) {
-      size_t fr = 0, tot = 0;
-      CK(cudaMemGetInfo(&fr, &tot));
-      h->narrow = extra + extra / 8 + ((size_t)64 << 20) > fr;
-      if (!h->narrow) h->fit_extra = extra;
-    }
+// Is there room for what the call will ask for, beside what the handle holds?
+int has_room(sp2_handle_t h, const Room& r, bool* room) {
+  const size_t extra = r.extra(h);
+  *room = !h->limit || h->held + extra <= h->limit;
+  if (*room && extra > h->fit_extra) {
+    size_t fr = 0, tot = 0;
+    CK(cudaMemGetInfo(&fr, &tot));
+    *room = extra + extra / 64 + ((size_t)64 << 20) <= fr;   // (buffers take whole pages)
+    if (*room) h->fit_extra = extra;
   }
-  if (h->narrow) *np = least;
   return SP2_OK;
 }
 
-// FP64 buffers of a recursion with `ybatch` responses, and with `adj` > 0 those of its
-// history and an adjoint of that many matrices
-int sp2_room(sp2_handle_t h, Room& r, sp2_opts o, int64_t np, int64_t ybatch, int64_t adj) {
+int64_t least_np(int64_t n) { return (n + 63) / 64 * 64; }
+
+// Does the padding to np cost enough that it only pays with the digits? (At 5 % more rows
+// the CUDA cores have 16 % more work; from N = 5000 on it is always less.)
+bool dear_padding(int64_t n, int64_t np) { return 20 * np > 21 * least_np(n); }
+
+// The padded size of an FP64 call. From kDigMinN on products run by digits, on matrices
+// padded to 256; where that padding and the digits do not fit beside what the handle
+// holds (N = 300 takes 2.6 times the memory of a padding to 64, and the CUDA cores 4.1
+// times its work), to 64. Where the two paddings are nearly the same the digits may come
+// and go. room(np, Room&, digits): what the call will ask for, with or without digits.
+template <typename F>
+int pick_np(sp2_handle_t h, int64_t n, int mode, F room, int64_t* np) {
+  *np = pad_n(n, mode);
+  if (mode != SP2_MODE_FP64 || *np == least_np(n)) return SP2_OK;
+  if (h->narrow_n == n) h->narrow = true;
+  if (!h->narrow) {
+    Room r;
+    bool ok;
+    TRY(room(*np, r, dear_padding(n, *np)));
+    TRY(has_room(h, r, &ok));
+    h->narrow = !ok;
+  }
+  if (h->narrow) *np = least_np(n);
+  return SP2_OK;
+}
+
+// FP64 buffers of an adjoint of `adj` matrices, beside the history
+void adjoint_room(Room& r, const sp2_opts& o, int64_t np, int64_t adj, bool digits) {
   const size_t el = (size_t)np * np * sizeof(double);
-  const int cap = o.fixed_m > 0 ? o.fixed_m : o.max_iter;
+  for (int i = 1; i < o.ckpt_k; ++i) r.add("seg." + std::to_string(i) + ".m", el);
+  r.add("G0.m", (size_t)adj * el);
+  r.add("G1.m", (size_t)adj * el);
+  if (digits) dig_room(r, np, 0, adj);
+  else r.add("Z", (size_t)adj * el);
+}
+
+// FP64 buffers of a recursion with `ybatch` responses, and with `adj` > 0 those of its
+// history, of at most `steps` steps, and of an adjoint of that many matrices (20: few
+// recursions take fewer; see run_forward for those that take more)
+int sp2_room(sp2_handle_t h, Room& r, sp2_opts o, int64_t np, int64_t ybatch, int64_t adj,
+             bool digits, int steps = 20) {
+  const size_t el = (size_t)np * np * sizeof(double);
+  const int cap = std::min(steps, o.fixed_m > 0 ? o.fixed_m : o.max_iter);
   for (const char* x : {"X0.m", "X1.m", "Xbest.m"}) r.add(x, el);
   for (const char* y : {"Y0.m", "Y1.m", "Ybest.m"})
     if (ybatch > 0) r.add(y, (size_t)ybatch * el);
   if (adj > 0) {
     TRY(resolve_ckpt(h, &o, np, adj));
     for (int i = 0; i < (cap + o.ckpt_k - 1) / o.ckpt_k; ++i) r.add("ckpt." + std::to_string(i), el);
-    for (int i = 1; i < o.ckpt_k; ++i) r.add("seg." + std::to_string(i) + ".m", el);
-    r.add("G0.m", (size_t)adj * el);
-    r.add("G1.m", (size_t)adj * el);
+    adjoint_room(r, o, np, adj, digits);
   }
-  dig_room(r, np, ybatch, adj);
-  r.add("call", (size_t)1 << 16);   // bounds and other small buffers
+  if (digits) dig_room(r, np, ybatch, adj);
+  else if (ybatch > 0) r.add("Z", (size_t)ybatch * el);
   return SP2_OK;
 }
 
@@ -1397,6 +1424,46 @@ int make_ctx(sp2_handle_t h, int mode, int64_t n, int64_t np, bool timing, Ctx* 
     c->part = static_cast<Part3*>(p);
   }
   return SP2_OK;
+}
+
+// A recursion without responses; adj > 0: with its history, for an adjoint of that many
+// matrices. The number of checkpoints shows only as it runs: where an FP64 recursion whose
+// matrices are padded for the digits finds no room for them, or leaves none for the
+// adjoint, it runs again on the least padding (and calls of this size start there).
+int run_forward(sp2_handle_t h, const void* Hd, int64_t n, int dtype, double nocc, sp2_opts* o, int64_t adj,
+                int64_t* np, Ctx& c, Sp2Out* r) {
+  for (const int k = o->ckpt_k;;) {
+    c = Ctx();
+    *r = Sp2Out();
+    TRY(make_ctx(h, o->mode, n, *np, o->time_kernels != 0, &c));
+    o->ckpt_k = k;
+    if (adj > 0) TRY(resolve_ckpt(h, o, *np, adj));
+    MatBuf X[2], Y[2];
+    const int code = run_sp2(h, Hd, n, dtype, nocc, *o, nullptr, 0, 0, adj > 0, X, Y, c, r);
+    if (o->mode != SP2_MODE_FP64 || adj == 0 || *np == least_np(n)) return code;
+    bool room = code != SP2_ENOMEM;
+    if (code == SP2_OK) {
+      const bool dear = dear_padding(n, *np);
+      Room q;
+      adjoint_room(q, *o, *np, adj, dear);
+      TRY(has_room(h, q, &room));
+      if (dear && h->dig_off) room = false;
+    }
+    if (room) return code;
+    CK(cudaStreamSynchronize(h->stream));
+    for (auto& kv : h->bufs)
+      for (const char* own : {"X", "ckpt.", "seg.", "G", "dig.", "Z"})
+        if (kv.first.rfind(own, 0) == 0 && kv.second.p) {
+          cudaFree(kv.second.p);
+          h->held -= kv.second.bytes;
+          kv.second.p = nullptr;
+          kv.second.bytes = 0;
+        }
+    h->err.clear();
+    h->narrow = true;
+    h->narrow_n = n;
+    *np = least_np(n);
+  }
 }
 
 // Eq. DM2 over the kept history: G_{M+1} = B, G_n = (1 - s_n) G_{n+1} + s_n (G_{n+1} X_n + X_n G_{n+1}),
@@ -1885,16 +1952,11 @@ int sp2_density(sp2_handle_t h, const void* H, int64_t N, int dtype, double nocc
   TRY(stage_out(h, "D", D, mb, &od));
   const bool keep = o.keep_history != 0;
   int64_t np;
-  TRY(pick_np(h, N, o.mode, [&](int64_t w, Room& q) { return sp2_room(h, q, o, w, 0, keep ? 1 : 0); }, &np));
+  TRY(pick_np(h, N, o.mode, [&](int64_t w, Room& q, bool dig) { return sp2_room(h, q, o, w, 0, keep ? 1 : 0, dig); }, &np));
   Ctx c;
-  TRY(make_ctx(h, o.mode, N, np, o.time_kernels != 0, &c));
-  MatBuf X[2], Y[2];
   Sp2Out r;
-  if (keep) {
-    h->hist.valid = false;
-    TRY(resolve_ckpt(h, &o, np, 1));
-  }
-  TRY(run_sp2(h, Hd, N, dtype, nocc, o, nullptr, 0, 0, keep, X, Y, c, &r));
+  if (keep) h->hist.valid = false;
+  TRY(run_forward(h, Hd, N, dtype, nocc, &o, keep ? 1 : 0, &np, c, &r));
   CK(launch_copy_out(r.xout, N, np, 1, o.mode, 1.0, od.dev, dtype, h->stream));
   c.kernels++;
   TRY(finish_out(h, od));
@@ -1935,7 +1997,7 @@ int sp2_response(sp2_handle_t h, const void* H, int64_t N, int dtype, double noc
   if (D) TRY(stage_out(h, "D", D, mb, &od));
   if (K > 0) TRY(stage_out(h, "Y", D1, (size_t)K * mb, &oy));
   int64_t np;
-  TRY(pick_np(h, N, o.mode, [&](int64_t w, Room& q) { return sp2_room(h, q, o, w, K, 0); }, &np));
+  TRY(pick_np(h, N, o.mode, [&](int64_t w, Room& q, bool dig) { return sp2_room(h, q, o, w, K, 0, dig); }, &np));
   Ctx c;
   TRY(make_ctx(h, o.mode, N, np, o.time_kernels != 0, &c));
   MatBuf X[2], Y[2];
@@ -1993,13 +2055,10 @@ int sp2_susceptibility(sp2_handle_t h, const void* H, int64_t N, int dtype, doub
   h->hist.valid = false;
   int64_t np;
   TRY(pick_np(h, N, o.mode,
-              [&](int64_t w, Room& q) { return sp2_room(h, q, o, w, 0, L > 0 ? L : 1); }, &np));
+              [&](int64_t w, Room& q, bool dig) { return sp2_room(h, q, o, w, 0, L > 0 ? L : 1, dig); }, &np));
   Ctx c;
-  TRY(make_ctx(h, o.mode, N, np, o.time_kernels != 0, &c));
-  MatBuf X[2], Y[2];
   Sp2Out r;
-  TRY(resolve_ckpt(h, &o, np, L));
-  TRY(run_sp2(h, Hd, N, dtype, nocc, o, nullptr, 0, 0, true, X, Y, c, &r));
+  TRY(run_forward(h, Hd, N, dtype, nocc, &o, L > 0 ? L : 1, &np, c, &r));
   if (D) {
     CK(launch_copy_out(r.xout, N, np, 1, o.mode, 1.0, od.dev, dtype, h->stream));
     c.kernels++;
@@ -2056,6 +2115,7 @@ int sp2_adjoint(sp2_handle_t h, const void* G, int64_t N, int dtype, void* grad,
 int sp2_release_history(sp2_handle_t h) {
   if (!h) return SP2_EINVAL;
   h->hist.valid = false;
+  h->narrow_n = 0;
   std::vector<std::string> names;
   for (auto& kv : h->bufs)
     if (kv.first.rfind("ckpt.", 0) == 0 || kv.first.rfind("seg.", 0) == 0) names.push_back(kv.first);
@@ -2179,7 +2239,7 @@ int fermi_setup(Ctx& c, FermiState& fs, const void* Hd, int64_t N, int dtype, do
 }
 
 // FP64 buffers of fermi_setup and of one response at a time
-void fermi_room(Room& r, int64_t np, int n, bool canonical, bool responses) {
+void fermi_room(Room& r, int64_t np, int n, bool canonical, bool responses, bool digits) {
   const size_t el = (size_t)np * np * sizeof(double);
   for (int j = 0; j <= n; ++j) r.add("ft.d" + std::to_string(j) + ".m", el);
   for (int j = 0; j < n; ++j) r.add("ft.W" + std::to_string(j) + ".m", el);
@@ -2187,8 +2247,7 @@ void fermi_room(Room& r, int64_t np, int n, bool canonical, bool responses) {
   for (const char* x : {"ft.dd0.m", "ft.dd1.m", "ft.E.m", "ft.F1.m", "ft.dW.m", "ft.G1.m"})
     if (responses) r.add(x, el);
   if (responses && canonical) r.add("ft.RI.m", el);
-  r.add(dig_bytes(np, np, false));
-  r.add("call", ((size_t)1 << 16) + (size_t)np * 8);
+  if (digits) r.add(dig_bytes(np, np, false));
 }
 
 // Scratch for batches of up to `want` responses; *B: how many fit. A batch shares each
@@ -2343,8 +2402,8 @@ int sp2_fermi(sp2_handle_t h, const void* H, int64_t N, int dtype, double mu, do
   if (D) TRY(stage_out(h, "D", D, mb, &od));
   if (K > 0) TRY(stage_out(h, "Y", D1, (size_t)K * mb, &oy));
   int64_t np;
-  TRY(pick_np(h, N, mode, [&](int64_t w, Room& q) {
-    fermi_room(q, w, n_doublings, canonical != 0, K > 0);
+  TRY(pick_np(h, N, mode, [&](int64_t w, Room& q, bool dig) {
+    fermi_room(q, w, n_doublings, canonical != 0, K > 0, dig);
     return SP2_OK;
   }, &np));
   Ctx c;
@@ -2474,14 +2533,14 @@ int sp2_nonorth_susceptibility(sp2_handle_t h, const void* H, const void* S, int
   TRY(stage_out(h, "no.WS", WS, mb, &os));
   if (Zout) TRY(stage_out(h, "no.Z", Zout, mb, &oz));
   int64_t np;
-  TRY(pick_np(h, N, mode, [&](int64_t w, Room& q) {
+  TRY(pick_np(h, N, mode, [&](int64_t w, Room& q, bool dig) {
     const size_t el = (size_t)w * w * sizeof(double);
     for (const char* x : {"Y", "Zk", "T", "P", "Q", "Q2", "Z", "Sinv", "H", "A", "Hp", "Ap", "Dp", "Cp",
                           "Dm", "Wh", "Ws"})
       q.add(std::string("no.") + x + ".m", el);
     for (const char* x : {"no.Hpn", "no.Apn", "no.Dpn", "no.Cpn"}) q.add(x, mb);
-    q.add(dig_bytes(w, w, false));
-    return sp2_room(h, q, o, w, 0, 1);
+    if (dig) q.add(dig_bytes(w, w, false));
+    return sp2_room(h, q, o, w, 0, 1, dig, SP2_MAX_ITER);
   }, &np));
   Ctx c;
   TRY(make_ctx(h, mode, N, np, o.time_kernels != 0, &c));

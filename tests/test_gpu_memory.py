@@ -108,6 +108,21 @@ def test_wide_fp64_padding_needs_its_room(sp2):
     assert torch.equal(sp2.sp2_adjoint(B[0].contiguous(), tight), want)
 
 
+@pytest.mark.parametrize("extra", [0, 1, 3, 6, 12])
+@pytest.mark.parametrize("name", ["chi", "chi_k1", "adjoint"])
+def test_history_that_outgrows_the_room_runs_again(sp2, name, extra):
+    """Limits between the least and what digits, the wide padding and the history take: the
+    call returns its result under each of them (on the least padding where the number of
+    checkpoints shows that the wide one has no room), and so does a second one."""
+    n = 300
+    H, B = _inputs(n, "fp64")
+    want = _call(sp2, name, n, "fp64", H, B, sp2.Handle())
+    h = sp2.Handle(LEAST["fp64", n, name] + extra * (8 << 20))
+    for _ in range(2):
+        got = _call(sp2, name, n, "fp64", H, B, h)
+        assert (got - want).norm() <= 1e-8 * want.norm()
+
+
 def test_batches_leave_room_for_the_next_call(sp2):
     """Finite-T responses by batches take free room under a limit; the density that follows
     finds the room it would have found beside one response at a time."""
