@@ -45,7 +45,7 @@ struct sp2_handle_s {
   bool narrow = false;             // this call pads FP64 matrices to 64 (pick_np)
   int64_t narrow_n = 0;            // the size whose history did not fit otherwise
   bool ft_single = false;          // room was short: finite-T responses one at a time
-  size_t fit_extra = 0;            // device memory found free for a call (pick_np)
+  size_t fit_extra = 0;            // device memory found free for a call (has_room)
   struct TileList {
     Tile* d = nullptr;
     int n = 0;
@@ -398,7 +398,9 @@ struct Ctx {
   int64_t kernels = 0;    // every kernel launched
   bool timing = false;
   int tail = 0;           // split-tail mode (product kernels read st->plane1)
-  std::vector<std::pair<int, int>> timed;  // (step, event-pair index) per timed product launch
+  // per event pair the step and the number of products between its events
+  std::vector<std::pair<int, int>> timed;
+  bool span = false;      // the last pair's second event is still to be recorded
 };
 
 int ev_pair(Ctx& c, cudaEvent_t* a, cudaEvent_t* b) {
@@ -414,19 +416,29 @@ int ev_pair(Ctx& c, cudaEvent_t* a, cudaEvent_t* b) {
   return SP2_OK;
 }
 
-// with c.timing: the events around one product of `step`
-int time_from(Ctx& c, cudaEvent_t* a, cudaEvent_t* b) {
+// With c.timing: events around products by digits, of several launches each. Products that
+// follow one another directly share a pair: an event between them would keep the digits'
+// launch from overlapping with the pass before (adjoint at N = 300 1.79 -> 1.88 ms).
+int time_from(Ctx& c, int step) {
   sp2_handle_t h = c.h;
-  if (!c.timing) return SP2_OK;
-  TRY(ev_pair(c, a, b));
-  CK(cudaEventRecord(*a, h->stream));
+  if (!c.timing || c.span) return SP2_OK;
+  cudaEvent_t a, b;
+  TRY(ev_pair(c, &a, &b));
+  CK(cudaEventRecord(a, h->stream));
+  c.timed.push_back({step, 0});
+  c.span = true;
   return SP2_OK;
 }
-int time_to(Ctx& c, cudaEvent_t b, int step) {
+void time_product(Ctx& c, int kernels) {
+  c.launches++;
+  c.kernels += kernels;
+  if (c.span) c.timed.back().second++;
+}
+// before any other work
+int time_to(Ctx& c) {
   sp2_handle_t h = c.h;
-  if (!c.timing) return SP2_OK;
-  CK(cudaEventRecord(b, h->stream));
-  c.timed.push_back({step, 0});
+  if (c.span) CK(cudaEventRecord(h->events[2 * c.timed.size() - 1], h->stream));
+  c.span = false;
   return SP2_OK;
 }
 
@@ -446,7 +458,7 @@ double timed_ms(Ctx& c, int m) {
 
 int64_t timed_count(const Ctx& c, int m) {
   int64_t k = 0;
-  for (auto& t : c.timed) k += t.first <= m ? 1 : 0;
+  for (auto& t : c.timed) k += t.first <= m ? t.second : 0;
   return k;
 }
 
@@ -498,6 +510,8 @@ DigBytes dig_bytes(int64_t np, int64_t rows, bool upper, bool with_x = false) {
 // least one (with_x: X_n's below them as well, 0 when that is more).
 int64_t dig_chunk(int64_t np, int64_t batch, bool with_x = false) {
   constexpr size_t cap = (size_t)4 << 30;
+  // (the K axis is cut into at most np / 256 parts)
+  if ((size_t)(batch + (with_x ? 1 : 0)) * np * np * (16 + 32 * (np / 256)) <= cap) return batch;
   for (int64_t m = batch; m > 0; m = m > 16 ? m - m / 16 : m - 1) {
     const DigBytes d = dig_bytes(np, m * np, false, with_x);
     if (d.G + d.a <= cap) return m;
@@ -608,16 +622,13 @@ int dig_step(Ctx& c, const MatBuf& xin, const MatBuf& xout, const MatBuf& yin, c
   sd.p.nparts = (int)dig_square_nparts(c.np);
   const double *x = static_cast<const double*>(xin.master), *y = static_cast<const double*>(yin.master);
   const int64_t left = rows + c.np;
-  cudaEvent_t e0 = nullptr, e1 = nullptr;
-  TRY(time_from(c, &e0, &e1));
+  TRY(time_from(c, step));
   CK(launch_digits(y, rows, x, c.np, c.np, db.a, c.st, step, h->stream));
   CK(launch_gemm_dig(db.a, left, db.x, c.np, db.G, db.tiles, db.ntiles, db.plan, c.st, step, h->tune,
                      h->stream));
   CK(launch_dig_step(db.G, db.plan.ksplit, batch, db.a.ex, y, static_cast<double*>(yout.master), x,
                      static_cast<double*>(xout.master), c.np, c.st, step, c.part, &sd, h->stream));
-  TRY(time_to(c, e1, step));
-  c.launches++;
-  c.kernels += 3;
+  time_product(c, 3);
   c.flops += dig_flops(c, db);
   c.alg += (double)c.n * (double)c.n * (2.0 * (double)batch * (double)c.n + (double)(c.n + 1));
   *done = true;
@@ -637,26 +648,22 @@ int square_step(Ctx& c, const MatBuf& xin, const MatBuf& xout, int step,
     sd.p.nparts = (int)dig_square_nparts(c.np);
     if (dig_bufs(c, 0, true, &db)) {
       const double* x = static_cast<const double*>(xin.master);
-      cudaEvent_t e0 = nullptr, e1 = nullptr;
-      TRY(time_from(c, &e0, &e1));
+      TRY(time_from(c, step));
       // (the response product of this step has left X_n's digits)
-      if (h->dig_x != xin.master) {
-        CK(launch_digits(x, c.np, nullptr, 0, c.np, db.x, c.st, step, h->stream));
-        c.kernels++;
-      }
+      const int made = h->dig_x != xin.master;
+      if (made) CK(launch_digits(x, c.np, nullptr, 0, c.np, db.x, c.st, step, h->stream));
       h->dig_x = nullptr;
       CK(launch_gemm_dig(db.x, c.np, db.x, c.np, db.G, db.tiles, db.ntiles, db.plan, c.st, step,
                          h->tune, h->stream));
       CK(launch_dig_square(db.G, db.plan.ksplit, db.x.ex, x, static_cast<double*>(xout.master), c.np, c.st, step,
                            c.part, dec ? &sd : nullptr, h->stream));
-      TRY(time_to(c, e1, step));
-      c.launches++;
-      c.kernels += 2;
+      time_product(c, 2 + made);
       c.flops += dig_flops(c, db);
       c.alg += (double)c.n * (double)(c.n + 1) * (double)c.n;
       return SP2_OK;
     }
   }
+  TRY(time_to(c));
   const Tile* tl;
   int nt;
   int bm, bn;
@@ -689,7 +696,7 @@ int square_step(Ctx& c, const MatBuf& xin, const MatBuf& xout, int step,
   }
   if (c.timing) {
     CK(cudaEventRecord(e1, h->stream));
-    c.timed.push_back({step, 0});
+    c.timed.push_back({step, 1});
   }
   c.launches++;
   c.kernels++;
@@ -761,7 +768,7 @@ int sparse_square(Ctx& c, const MatBuf& xin, const MatBuf& xout, int step, const
   if (e != cudaSuccess) return fail(h, SP2_ECUDA, "block-sparse square: %s %s", cudaGetErrorString(e), eb);
   if (c.timing) {
     CK(cudaEventRecord(e1, h->stream));
-    c.timed.push_back({step, 0});
+    c.timed.push_back({step, 1});
   }
   c.launches++;
   c.kernels++;
@@ -787,12 +794,10 @@ int response_step(Ctx& c, const MatBuf& x, const MatBuf& yin, const MatBuf& yout
     if (dig_bufs(c, bc * c.np, false, &db)) {
       const double* y = static_cast<const double*>(yin.master);
       double* yo = static_cast<double*>(yout.master);
-      cudaEvent_t e0 = nullptr, e1 = nullptr;
-      TRY(time_from(c, &e0, &e1));
+      TRY(time_from(c, step));
       CK(launch_digits(static_cast<const double*>(x.master), c.np, nullptr, 0, c.np, db.x, c.st, step,
                        h->stream));
       h->dig_x = x.master;
-      c.kernels++;
       for (int64_t b0 = 0; b0 < batch; b0 += bc) {
         const int64_t nb = batch - b0 < bc ? batch - b0 : bc, r = nb * c.np, off = b0 * c.np * c.np;
         if (nb != bc) {   // the last, smaller chunk has its own tiles (and the same K parts:
@@ -803,21 +808,19 @@ int response_step(Ctx& c, const MatBuf& x, const MatBuf& yin, const MatBuf& yout
           db.plan.kseg = kseg;
           TRY(tile_list(h, c.mode, r, c.np, false, &db.tiles, &db.ntiles, 256, db.plan.bn));
         }
-        if (b0 > 0) TRY(time_from(c, &e0, &e1));
         CK(launch_digits(y + off, r, nullptr, 0, c.np, db.a, c.st, step, h->stream));
         CK(launch_gemm_dig(db.a, r, db.x, c.np, db.G, db.tiles, db.ntiles, db.plan, c.st, step,
                            h->tune, h->stream));
         CK(launch_dig_symm(db.G, db.plan.ksplit, r, db.a.ex, db.x.ex, y + off, yo + off, c.np, c.st, step,
                            h->stream));
-        TRY(time_to(c, e1, step));
-        c.launches++;
-        c.kernels += 3;
+        time_product(c, b0 > 0 ? 3 : 4);
         c.flops += dig_flops(c, db);
       }
       c.alg += 2.0 * (double)batch * (double)c.n * (double)c.n * (double)c.n;
       return SP2_OK;
     }
   }
+  TRY(time_to(c));
   const Tile* tl;
   int nt;
   int bm, bn;
@@ -858,7 +861,7 @@ int response_step(Ctx& c, const MatBuf& x, const MatBuf& yin, const MatBuf& yout
     if (e != cudaSuccess) return fail(h, SP2_ECUDA, "response product: %s %s", cudaGetErrorString(e), eb);
     if (c.timing) {
       CK(cudaEventRecord(e1, h->stream));
-      c.timed.push_back({step, 0});
+      c.timed.push_back({step, 1});
     }
     if (f16) {
       CK(launch_sym_scale(static_cast<Part3*>(yp), parts_per_tile(h, c.mode), tl, nt, c.np, batch,
@@ -899,7 +902,7 @@ int response_step(Ctx& c, const MatBuf& x, const MatBuf& yin, const MatBuf& yout
   }
   if (c.timing) {
     CK(cudaEventRecord(e1, h->stream));
-    c.timed.push_back({step, 0});
+    c.timed.push_back({step, 1});
   }
   CK(launch_symm_update(z, yin, yout, c.np, batch, c.mode, c.st, step, sc, slot_in, slot_out,
                         h->stream));
@@ -1304,6 +1307,7 @@ int run_sp2(sp2_handle_t h, const void* Hd, int64_t n, int dtype, double nocc, c
     } else {
       TRY(square_step(c, xin, xo, step, &dp));
     }
+    TRY(time_to(c));
     if (track) {
       if (!keep_small) {
         CK(launch_keep_best(xin.master, xbest.master, np * np, mode, c.st, step, h->stream));
@@ -1544,6 +1548,7 @@ int run_adjoint(sp2_handle_t h, const void* Bd, int64_t batch, int b_diag, int s
       gs = 1 - gs;
     }
   }
+  TRY(time_to(c));
   // gs now holds G_1
   CK(launch_copy_out(G[gs], n, np, batch, mode, hs.beta, outd, out_dtype, h->stream));
   c.kernels++;
@@ -1727,8 +1732,7 @@ int fprod(Ctx& c, FMat& C, const FMat& L, const FMat& R, bool trans = false) {
   const int64_t rows = L.B * c.np;
   if (dig_mode(c, rows) && dig_bufs(c, same ? 0 : rows, false, &db)) {
     const double* l = static_cast<const double*>(L.m.master);
-    cudaEvent_t e0 = nullptr, e1 = nullptr;
-    TRY(time_from(c, &e0, &e1));
+    TRY(time_from(c, 0));
     CK(launch_digits(l, rows, nullptr, 0, c.np, db.a, c.st, 0, h->stream));
     if (!same)
       CK(launch_digits(static_cast<const double*>(R.m.master), c.np, nullptr, 0, c.np, db.x, c.st, 0,
@@ -1738,9 +1742,8 @@ int fprod(Ctx& c, FMat& C, const FMat& L, const FMat& R, bool trans = false) {
                        h->stream));
     CK(launch_dig_plain(db.G, db.plan.ksplit, rows, db.a.ex, db.x.ex, static_cast<double*>(C.m.master), c.np, c.st,
                         0, h->stream));
-    TRY(time_to(c, e1, 0));
-    c.launches++;
-    c.kernels += same ? 3 : 4;
+    time_product(c, same ? 3 : 4);
+    TRY(time_to(c));
     c.flops += dig_flops(c, db);
     c.alg += 2.0 * (double)L.B * (double)c.n * (double)c.n * (double)c.n;
     return SP2_OK;
@@ -1782,7 +1785,7 @@ int fprod(Ctx& c, FMat& C, const FMat& L, const FMat& R, bool trans = false) {
   }
   if (c.timing) {
     CK(cudaEventRecord(e1, h->stream));
-    c.timed.push_back({0, 0});
+    c.timed.push_back({0, 1});
   }
   c.launches++;
   c.kernels++;
@@ -1952,7 +1955,8 @@ int sp2_density(sp2_handle_t h, const void* H, int64_t N, int dtype, double nocc
   TRY(stage_out(h, "D", D, mb, &od));
   const bool keep = o.keep_history != 0;
   int64_t np;
-  TRY(pick_np(h, N, o.mode, [&](int64_t w, Room& q, bool dig) { return sp2_room(h, q, o, w, 0, keep ? 1 : 0, dig); }, &np));
+  TRY(pick_np(h, N, o.mode,
+              [&](int64_t w, Room& q, bool dig) { return sp2_room(h, q, o, w, 0, keep ? 1 : 0, dig); }, &np));
   Ctx c;
   Sp2Out r;
   if (keep) h->hist.valid = false;
@@ -1997,7 +2001,8 @@ int sp2_response(sp2_handle_t h, const void* H, int64_t N, int dtype, double noc
   if (D) TRY(stage_out(h, "D", D, mb, &od));
   if (K > 0) TRY(stage_out(h, "Y", D1, (size_t)K * mb, &oy));
   int64_t np;
-  TRY(pick_np(h, N, o.mode, [&](int64_t w, Room& q, bool dig) { return sp2_room(h, q, o, w, K, 0, dig); }, &np));
+  TRY(pick_np(h, N, o.mode,
+              [&](int64_t w, Room& q, bool dig) { return sp2_room(h, q, o, w, K, 0, dig); }, &np));
   Ctx c;
   TRY(make_ctx(h, o.mode, N, np, o.time_kernels != 0, &c));
   MatBuf X[2], Y[2];
