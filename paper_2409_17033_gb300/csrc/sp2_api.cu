@@ -23,9 +23,11 @@ using namespace sp2;
 // once had, so that a workspace limit holds what it held).
 constexpr int64_t kFixedParts = 16384;
 struct HandleBlock {
-  DevState state, hist, adj;
-  unsigned done;
-  Part3 part[kFixedParts];
+  alignas(256) DevState state;
+  alignas(256) DevState hist;
+  alignas(256) DevState adj;
+  alignas(256) unsigned done;   // (blocks count on it while others store partials)
+  alignas(256) Part3 part[kFixedParts];
 };
 
 struct sp2_handle_s {
