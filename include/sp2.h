@@ -95,11 +95,14 @@ typedef enum { SP2_F64 = 0, SP2_F32 = 1 } sp2_dtype;
 
 /* Arithmetic of the matrix products (Sec. VI.B).
  *   SP2_MODE_FP64    FP64. Products of matrices from N = 257 on (in steps with responses
- *                    from N = 193, where they are padded to 256) are formed on the tensor
- *                    cores from 8 error-free digits of 8 bits per entry (36 exact
- *                    products summed in integers), with errors below those of an
- *                    FP64 dot product relative to the norms of its row and column;
- *                    smaller ones by CUDA-core DFMA.
+ *                    from N = 193, in sp2_scf_response from N = 1, as these pad to 256) are
+ *                    formed on the tensor cores from 8 error-free digits of 8 bits per
+ *                    entry (36 exact products summed in integers), with errors below
+ *                    those of an FP64 dot product relative to the norms of its row and
+ *                    column. (Entries more than 2^10 below their row's norm keep fewer
+ *                    than 53 bits: results far below these norms are accurate to 2^-60
+ *                    of them, not relative to themselves.) Smaller products, and all where
+ *                    the digits' buffers do not fit, by CUDA-core DFMA.
  *   SP2_MODE_FP32    plain FP32 (CUDA-core FFMA): the paper's "GPU FP32" form.
  *   SP2_MODE_BF16X2  Eq. doubleHalf / Eq. MixPrecMult with bfloat16 hi/lo planes:
  *                    three tensor-core products (hi*hi + hi*lo + lo*hi, lo*lo
