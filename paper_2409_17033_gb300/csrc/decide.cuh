@@ -1,7 +1,8 @@
 // The SP2 branch and stop decision of one step (Eq. DM0 with the readings of
 // the stop rule in sp2.h): one block of threads reduces the step's trace
 // partials in a fixed order and one thread updates the device state. Shared by
-// the decision kernel and by the CUDA-core square, whose last block takes it.
+// the decision kernel and by the squares whose last block takes it: on the CUDA cores, by
+// digits, and on the tensor cores with tiles below 256 columns.
 #pragma once
 #include "sp2_internal.h"
 

@@ -339,7 +339,9 @@ k_gemm_f32(const float* __restrict__ A, const float* __restrict__ X, int64_t np,
   const int sg = st->sigma[step];
   // sums of this thread's entries in FP32 with their rounding errors (FP64
   // instructions on all 64 entries took 34 us of a tile): entries above the diagonal
-  // (counted twice) and on it
+  // (counted twice) and on it. Tr X - ||X||_F^2 comes within 6 units in the last place of
+  // the sums (N = 100 to 4096); a third word per sum would make it 1, and a step of N = 96 to
+  // 2000 5 to 18 % longer.
   SumF32 t1, t2, f, e2, ef;
 #pragma unroll
   for (int ih = 0; ih < 2; ++ih)

@@ -31,7 +31,9 @@ inline int64_t pad_n(int64_t n, int mode) {
 }
 
 // Device-resident SP2 control state: traces of every X_n, the branch signs
-// and the stop decision. Written only by k_decide; read by the step kernels
+// and the stop decision. Written by the step decisions (decide.cuh: k_decide, or the last
+// block of a square), the kernels that start a recursion (bounds, given branches) and the
+// block-sparse plan, and by products whose wait runs out; read by the step kernels
 // (which become no-ops once the recursion has stopped) and by the host.
 struct DevState {
   double t1[SP2_MAX_ITER + 2];   // Tr[X_n], index n = 1..M+1

@@ -170,8 +170,8 @@ __device__ __forceinline__ uint64_t sdesc_sw128(uint32_t addr) {
 
 // The MMA issuer runs as a whole warp in uniform control flow, and one elected lane
 // issues: the descriptors then live in uniform registers. Issued from inside a
-// branch on the lane, every tcgen05.mma first moved its operands there, which took
-// about 78 clocks an instruction, 310 of the 640 clocks of a 64-wide k-block.
+// branch on the lane, every tcgen05.mma first moved its operands there (N = 16384 solve
+// 823 -> 735 ms without).
 //
 // One k-block: four K = 16 instructions over a stage's swizzled rows (the K advance
 // of 32 bytes is 2 in the descriptors' 16-byte units). CG = 2: instructions of
