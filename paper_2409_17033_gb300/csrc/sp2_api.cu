@@ -2487,8 +2487,11 @@ int fsandwich(Ctx& c, FMat& C, const FMat& L, const FMat& Mid, const FMat& R, FM
   return fcomb(c, C, &T2, 0.5, nullptr, 0.0, nullptr, 0.0, 0.0, true);
 }
 
-// ||T - I||_F^2 of the padded master (zero outside the caller's block), FP64
-int dist_to_identity(Ctx& c, const FMat& T, double* out) {
+// ||T - I||_F^2 of the padded master (zero outside the caller's block), FP64, through W = T - I:
+// as Tr T^2 - 2 Tr T + N it has an error of N 2^-52, which decided whether it was below the
+// residuals of 1e-26 N that end the FP64 iteration, one step early for some overlap
+// matrices (D off by 2.5e-9 at N = 1100, 8e-15 with the step).
+int dist_to_identity(Ctx& c, const FMat& T, FMat& W, double* out) {
   sp2_handle_t h = c.h;
   void* p;
   TRY(ws(h, "no.red", 4 * sizeof(double), &p));
@@ -2497,14 +2500,12 @@ int dist_to_identity(Ctx& c, const FMat& T, double* out) {
   const int np_ = contract_nparts(c.np, 0);
   void* part;
   TRY(ws(h, "no.part", (size_t)np_ * sizeof(double), &part));
-  CK(launch_contract(T.m.master, 1, T.m.master, 1, c.np, mdt, 0, static_cast<double*>(part), np_,
+  TRY(fcomb(c, W, nullptr, 0.0, nullptr, 0.0, &T, 1.0, -1.0, false));
+  CK(launch_contract(W.m.master, 1, W.m.master, 1, c.np, mdt, 0, static_cast<double*>(part), np_,
                      d, h->stream));
-  CK(launch_trace(c.mode, T.m.master, c.np, c.n, 1, d + 1, h->stream));
-  double hv[2];
-  CK(cudaMemcpyAsync(hv, d, 2 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+  CK(cudaMemcpyAsync(out, d, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
   CK(cudaStreamSynchronize(h->stream));
   c.kernels += 2;
-  *out = hv[0] - 2.0 * hv[1] + (double)c.n;
   return SP2_OK;
 }
 
@@ -2582,9 +2583,17 @@ int sp2_nonorth_susceptibility(sp2_handle_t h, const void* H, const void* S, int
     TRY(fprod(c, P, Zk, Y));
     TRY(fcomb(c, T, &P, -0.25, nullptr, 0.0, nullptr, 0.0, 1.5, true));
     double e;
-    TRY(dist_to_identity(c, T, &e));  // ||T - I||^2 = ||I - Zk Yk||^2 / 4
+    TRY(dist_to_identity(c, T, Q, &e));  // ||T - I||^2 = ||I - Zk Yk||^2 / 4
     if (!std::isfinite(e)) return fail(h, SP2_ENONFINITE, "non-finite Newton-Schulz residual");
-    if (e <= tol) break;
+    if (e <= tol) {
+      // Z_k still has an error of the residual's size: FP64 applies the last T to it
+      if (mode == SP2_MODE_FP64) {
+        TRY(fprod(c, Q2, T, Zk));
+        TRY(fcomb(c, Zk, &Q2, 0.5, nullptr, 0.0, nullptr, 0.0, 0.0, true));
+        ++its;
+      }
+      break;
+    }
     // below 1e-6 an iteration that does not halve the residual has reached the
     // rounding floor of the mode (twice in a row ends the iteration)
     if (its > 0 && e < 1e-6 * (double)N && e > 0.25 * prev) {
