@@ -45,7 +45,8 @@ struct sp2_handle_s {
   unsigned long long call = 0;     // calls so far (CallScope)
   int depth = 0;
   bool narrow = false;             // this call pads FP64 matrices to 64 (pick_np)
-  int64_t narrow_n = 0;            // the size whose history did not fit otherwise
+  // the recursion whose history did not fit otherwise: size, interval asked for, adjoints
+  int64_t narrow_n = 0, narrow_k = 0, narrow_adj = 0;
   bool ft_single = false;          // room was short: finite-T responses one at a time
   size_t fit_extra = 0;            // device memory found free for a call (has_room)
   struct TileList {
@@ -983,6 +984,11 @@ int has_room(sp2_handle_t h, const Room& r, bool* room) {
 
 int64_t least_np(int64_t n) { return (n + 63) / 64 * 64; }
 
+// has a recursion like this one run out of room for its history (run_forward)?
+void known_narrow(sp2_handle_t h, int64_t n, int64_t k, int64_t adj) {
+  if (h->narrow_n == n && h->narrow_k == k && h->narrow_adj == adj) h->narrow = true;
+}
+
 // Does the padding to np cost enough that it only pays with the digits? (At 5 % more rows
 // the CUDA cores have 16 % more work; from N = 5000 on it is always less.)
 bool dear_padding(int64_t n, int64_t np) { return 20 * np > 21 * least_np(n); }
@@ -996,7 +1002,6 @@ template <typename F>
 int pick_np(sp2_handle_t h, int64_t n, int mode, F room, int64_t* np) {
   *np = pad_n(n, mode);
   if (mode != SP2_MODE_FP64 || *np == least_np(n)) return SP2_OK;
-  if (h->narrow_n == n) h->narrow = true;
   if (!h->narrow) {
     Room r;
     bool ok;
@@ -1435,7 +1440,7 @@ int make_ctx(sp2_handle_t h, int mode, int64_t n, int64_t np, bool timing, Ctx* 
 // A recursion without responses; adj > 0: with its history, for an adjoint of that many
 // matrices. The number of checkpoints shows only as it runs: where an FP64 recursion whose
 // matrices are padded for the digits finds no room for them, or leaves none for the
-// adjoint, it runs again on the least padding (and calls of this size start there).
+// adjoint, it runs again on the least padding (and such recursions start there).
 int run_forward(sp2_handle_t h, const void* Hd, int64_t n, int dtype, double nocc, sp2_opts* o, int64_t adj,
                 int64_t* np, Ctx& c, Sp2Out* r) {
   for (const int k = o->ckpt_k;;) {
@@ -1467,7 +1472,7 @@ int run_forward(sp2_handle_t h, const void* Hd, int64_t n, int dtype, double noc
         }
     h->err.clear();
     h->narrow = true;
-    h->narrow_n = n;
+    h->narrow_n = n, h->narrow_k = k, h->narrow_adj = adj;
     *np = least_np(n);
   }
 }
@@ -1956,6 +1961,7 @@ int sp2_density(sp2_handle_t h, const void* H, int64_t N, int dtype, double nocc
   OutStage od;
   TRY(stage_out(h, "D", D, mb, &od));
   const bool keep = o.keep_history != 0;
+  if (keep) known_narrow(h, N, o.ckpt_k, 1);
   int64_t np;
   TRY(pick_np(h, N, o.mode,
               [&](int64_t w, Room& q, bool dig) { return sp2_room(h, q, o, w, 0, keep ? 1 : 0, dig); }, &np));
@@ -2060,6 +2066,7 @@ int sp2_susceptibility(sp2_handle_t h, const void* H, int64_t N, int dtype, doub
   if (D) TRY(stage_out(h, "D", D, mb, &od));
   if (L > 0) TRY(stage_out(h, "Y", chi, (size_t)L * mb, &oy));
   h->hist.valid = false;
+  known_narrow(h, N, o.ckpt_k, L > 0 ? L : 1);
   int64_t np;
   TRY(pick_np(h, N, o.mode,
               [&](int64_t w, Room& q, bool dig) { return sp2_room(h, q, o, w, 0, L > 0 ? L : 1, dig); }, &np));

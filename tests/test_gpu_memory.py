@@ -123,6 +123,23 @@ def test_history_that_outgrows_the_room_runs_again(sp2, name, extra):
         assert (got - want).norm() <= 1e-8 * want.norm()
 
 
+def test_short_room_of_one_call_leaves_the_digits_to_others(sp2):
+    """A history that ran again on the least padding does not keep a density of the same size,
+    which has room, from the wide one and its digits."""
+    n = 300
+    H, B = _inputs(n, "fp64")
+    limit = LEAST["fp64", n, "chi"] + (44 << 20)      # 63.4 MB; chi with its digits takes 67.1
+    h = sp2.Handle(limit)
+    want = _call(sp2, "chi", n, "fp64", H, B, sp2.Handle())
+    for _ in range(2):
+        assert (_call(sp2, "chi", n, "fp64", H, B, h) - want).norm() <= 1e-8 * want.norm()
+        held = h.workspace_bytes()
+        assert held < 2 * LEAST["fp64", n, "chi"]
+        _call(sp2, "density", n, "fp64", H, B, h)
+        assert h.workspace_bytes() - held > 16 * 512 * 512      # the digits of X alone
+        h = sp2.Handle(limit)
+
+
 def test_batches_leave_room_for_the_next_call(sp2):
     """Finite-T responses by batches take free room under a limit; the density that follows
     finds the room it would have found beside one response at a time."""
